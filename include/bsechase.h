@@ -58,13 +58,16 @@ typedef enum {
 
 typedef enum {
     CHASE_FP64 = 0,       /* FP64 accuracy.  Products with H (Lanczos, filter,
-                             Rayleigh-Ritz) run on the BF16 tensor cores as an
-                             Ozaki-scheme emulation: 6 slices of 8 bits per
-                             operand, exact integer accumulation of the
-                             slice diagonals 2..5 per K chunk of 64, FP32 for
-                             diagonals 6..7 (normwise error ~1e-12 relative
-                             to ||H|| ||Y||).  QR, reduced eig,
-                             residuals and locking in native FP64.          */
+                             the solve's Rayleigh-Ritz) run on the tensor cores
+                             in residue arithmetic: operands rounded to integers
+                             of 51 and 50 bits relative to their row's or
+                             column's 2-norm, the integer product exact modulo
+                             13 coprime moduli (normwise error ~1e-13 relative
+                             to ||H|| ||Y||).  With half storage, and in
+                             chase_rayleigh_ritz, the products are the BF16
+                             Ozaki-scheme emulation of 6 slices of 8 bits per
+                             operand (~1e-12).  QR, reduced eig, residuals and
+                             locking in native FP64.                         */
     CHASE_MIXED_FP32 = 1, /* filter products at FP32-level accuracy on the
                              tensor cores (first 4 slices: 32 bits relative to
                              the row/column maximum, 10 slice pairs) while
@@ -127,8 +130,8 @@ typedef struct {
                             nex_damping, nex grows once to min(max(2 nex,
                             nex + 8), min(N, 512) - nev).  The new columns are
                             the seeded start block's next columns. */
-    int half_storage;    /* 0 (default): the tensor-core slices of all of H
-                            (24 N^2 bytes).  1: of its lower triangle only
+    int half_storage;    /* 0 (default): the tensor-core operand of all of H
+                            (26 N^2 bytes, 24 N^2 in the mixed mode).  1: of its lower triangle only
                             (12 N^2 bytes), the strict upper triangle never
                             read (H is Hermitian; the paper's reader holds one
                             triangle, Sec. 3): rows are scaled symmetrically,
@@ -238,8 +241,8 @@ int chase_solve(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t ldh, int 
  * (same seed, Nk, Nv, Nc, model), without storing it: its elements are
  * generated straight into the tensor-core slices of H, so the N x N
  * complex128 matrix (16 N^2 bytes) never exists and the device memory the
- * solve needs drops from 40 N^2 to 24 N^2 bytes plus workspace, 12 N^2 with
- * chase_opts.half_storage (Sec. 3's
+ * solve needs drops by 16 N^2 bytes, to 26 N^2 plus workspace (24 N^2 in the
+ * mixed mode, 12 N^2 with chase_opts.half_storage) (Sec. 3's
  * filter works on H only through its products).  The slices, and so every
  * result, are bit for bit those of bse_build_hamiltonian + chase_solve.
  * Tensor-core precisions only (CHASE_FP64, CHASE_MIXED_FP32, value 2);

@@ -176,6 +176,29 @@ int sync_scalars(bsechase_ctx *ctx) {
     return check_device_error(ctx);
 }
 
+}  // namespace
+
+HopBytes hop_bytes(int64_t N, int mc, bool res, bool tri, bool bse) {
+    HopBytes h;
+    h.GA = std::max(ozaki_gen_a_bytes(mc, N), ozaki_gen_a_bytes(N, mc));
+    if (res) {
+        h.A = residue_a_bytes(N, N);
+        h.B = std::max(residue_b_bytes(N, mc), ozaki_b_bytes(N, mc));
+        if (bse) h.B = std::max(h.B, residue_panel_bytes(N));
+        h.P = std::max({residue_r_bytes(N, N, mc), residue_work_bytes(N), ozaki_gen_partial_bytes(N, mc)});
+    } else {
+        h.A = tri ? ozaki_a_bytes_tri(N) : ozaki_a_bytes(N);
+        h.B = ozaki_b_bytes(N, mc);
+        h.P = ozaki_partial_bytes(N, mc);
+    }
+    return h;
+}
+
+// Whether the products with H of a precision run in residues.
+bool precision_uses_residues(int precision, bool half) { return precision == CHASE_FP64 && !half; }
+
+namespace {
+
 // ------------------------------------------------------- the operator H
 // Every product with H goes through Hop: native FP64 (zgemm.cu) or the
 // FP64-accurate tensor-core emulation (ozaki.cu), fixed per solve.
@@ -186,31 +209,58 @@ struct Hop {
     int level = OZ_S6;   // slices of the tensor-core product (mixed precision filter)
     const BseSource *bse = nullptr;   // H not stored: its slices from the generator
     bool tri = false;    // half storage of the slices (lower triangle of H only)
+    bool res = false;    // products in residues (residue.cu): the FP64 mode on full storage
 };
+
+size_t hop_f_bytes(int mc) { return ((size_t)(mc + 64) * sizeof(int) + 15) / 16 * 16; }
+
+int hop_buffers(bsechase_ctx *ctx, const Hop &op, int mc) {
+    int rc;
+    const int64_t Np = ozaki_padded(op.N);
+    const HopBytes hb = hop_bytes(op.N, mc, op.res, op.tri, op.bse != nullptr);
+    if ((rc = ensure(ctx, ctx->ozA, hb.A))) return rc;
+    if (op.tri && (rc = ensure(ctx, ctx->ozT, (size_t)2 * Np * sizeof(double)))) return rc;
+    if ((rc = ensure(ctx, ctx->ozE, (size_t)Np * sizeof(int)))) return rc;
+    if ((rc = ensure(ctx, ctx->ozB, hb.B))) return rc;
+    if ((rc = ensure(ctx, ctx->ozF, hop_f_bytes(mc) + (op.res ? (size_t)mc * 32 * sizeof(float2) : 0)))) return rc;
+    if ((rc = ensure(ctx, ctx->ozP, hb.P))) return rc;
+    // general products of QR and Rayleigh-Ritz: op(A) is m x N (A^H) or N x m
+    if ((rc = ensure(ctx, ctx->ozGA, hb.GA))) return rc;
+    return ensure(ctx, ctx->ozGE, (size_t)(Np + 512) * sizeof(int));
+}
 
 int hop_prepare(bsechase_ctx *ctx, Hop &op, int max_cols) {
     if (!op.tc) return BSE_OK;
     int rc;
     const int64_t Np = ozaki_padded(op.N);
-    if ((rc = ensure(ctx, ctx->ozA, op.tri ? ozaki_a_bytes_tri(op.N) : ozaki_a_bytes(op.N))))
-        return rc;
-    if (op.tri && (rc = ensure(ctx, ctx->ozT, (size_t)2 * Np * sizeof(double)))) return rc;
-    if ((rc = ensure(ctx, ctx->ozE, (size_t)Np * sizeof(int)))) return rc;
     const int mc = std::max(max_cols, 32);
-    if ((rc = ensure(ctx, ctx->ozB, ozaki_b_bytes(op.N, mc)))) return rc;
-    if ((rc = ensure(ctx, ctx->ozF, (size_t)(mc + 64) * sizeof(int)))) return rc;
-    const size_t pbytes = ozaki_partial_bytes(op.N, mc);
-    if ((rc = ensure(ctx, ctx->ozP, pbytes))) return rc;
-    // general products of QR and Rayleigh-Ritz: op(A) is m x N (A^H) or N x m
-    const size_t gab = std::max(ozaki_gen_a_bytes(mc, op.N), ozaki_gen_a_bytes(op.N, mc));
-    if ((rc = ensure(ctx, ctx->ozGA, gab))) return rc;
-    if ((rc = ensure(ctx, ctx->ozGE, (size_t)(Np + 512) * sizeof(int)))) return rc;
+    rc = hop_buffers(ctx, op, mc);
+    if (rc == BSE_ENOMEM && op.res) {
+        // the residues take 2 N^2 bytes more than the slices: those, where only
+        // they fit
+        op.res = false;
+        DevBuf *bufs[] = {&ctx->ozA, &ctx->ozB, &ctx->ozP, &ctx->ozGA};
+        for (DevBuf *d : bufs) {
+            if (d->p) cudaFreeAsync(d->p, ctx->st);
+            d->p = nullptr;
+            d->bytes = 0;
+        }
+        ctx->err.clear();
+        rc = hop_buffers(ctx, op, mc);
+    }
+    if (rc) return rc;
+    ctx->hop_cols = mc;
     ctx->oh.A = ctx->ozA.p;
     ctx->oh.E = (int *)ctx->ozE.p;
     ctx->oh.wait_ns = ctx->wait_ns;
     ctx->oh.t = (double *)ctx->ozT.p;
     ctx->oh.s = ctx->oh.t ? ctx->oh.t + Np : nullptr;
-    if (op.bse)
+    if (op.res && op.bse)
+        CK(residue_prepare_bse(op.bse->Nk, op.bse->Nv, op.bse->Nc, op.bse->md, op.bse->dE, op.bse->u, op.bse->a,
+                               op.bse->Kt, &ctx->oh, ctx->ozP.p, ctx->ozB.p, ctx->sc, ctx->st));
+    else if (op.res)
+        CK(residue_prepare(op.N, op.H, op.ldh, &ctx->oh, ctx->ozP.p, ctx->sc, ctx->st));
+    else if (op.bse)
         CK(ozaki_prepare_bse(op.bse->Nk, op.bse->Nv, op.bse->Nc, op.bse->md, op.bse->dE, op.bse->u,
                              op.bse->a, op.bse->Kt, op.tri, &ctx->oh, ctx->sc, ctx->st));
     else if (op.tri)
@@ -242,7 +292,13 @@ void kernel_events(bsechase_ctx *ctx, double flops, cudaEvent_t *e0, cudaEvent_t
 // C[N x n] = epi(H Y)
 int hop_apply(bsechase_ctx *ctx, const Hop &op, int n, const z_t *Y, int64_t ldy, z_t *C,
               int64_t ldc, const GemmEpi &ep) {
-    if (op.tc) {
+    if (op.res) {
+        cudaEvent_t e0 = nullptr, e1 = nullptr;
+        if (!ctx->batcher) kernel_events(ctx, residue_flops(op.N, op.N, n), &e0, &e1);
+        CK(residue_zgemm(ctx->oh, n, Y, ldy, C, ldc, ep, ctx->ozB.p, ctx->ozB.bytes, (int *)ctx->ozF.p,
+                         (float2 *)((char *)ctx->ozF.p + hop_f_bytes(ctx->hop_cols)), ctx->ozP.p, ctx->ozP.bytes,
+                         ctx->sc, ctx->sms, ctx->st, e0, e1, ctx->batcher));
+    } else if (op.tc) {
         // tensor flops: 8 real flops per complex multiply-add for each of
         // the 21 (FP64), 15 or 10 (FP32-level) slice pairs
         const double pairs = oz_pairs(op.level);
@@ -561,6 +617,7 @@ int solve_device(bsechase_ctx *ctx, const z_t *H, int64_t N, int64_t ldh, int ne
     Hop op{H, N, ldh, precision_uses_tc(precision)};
     op.bse = bse;
     op.tri = o.half_storage == 1;
+    op.res = ctx->residues && precision_uses_residues(precision, op.tri);
     if ((rc = hop_prepare(ctx, op, m_cap))) return rc;
     GenTcScope gen_scope(ctx, op.tc);
     if ((rc = phase_lanczos(ctx, op, m, o.lanczos_steps, o.lanczos_vecs, o.seed))) return rc;
@@ -1006,6 +1063,7 @@ int chase_lanczos(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t ldh, in
     precision = precision_mode(precision);
     Hop op{(const z_t *)d_H, N, ldh, precision_uses_tc(precision),
            precision == CHASE_MIXED_FP32 ? OZ_S4 : OZ_S6};
+    op.res = precision_uses_residues(precision, false);
     if ((rc = hop_prepare(ctx, op, 8))) return rc;
     if ((rc = phase_lanczos(ctx, op, m, steps, runs, seed))) return rc;
     if ((rc = sync_scalars(ctx))) return rc;
@@ -1035,6 +1093,7 @@ int chase_filter(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t ldh, voi
     precision = precision_mode(precision);
     Hop op{(const z_t *)d_H, N, ldh, precision_uses_tc(precision),
            precision == CHASE_MIXED_FP32 ? OZ_S4 : OZ_S6};
+    op.res = precision_uses_residues(precision, false);
     if ((rc = hop_prepare(ctx, op, m))) return rc;
     if ((rc = phase_filter(ctx, op, (z_t *)d_V, ldv, m, h_deg, s.deg, lower, c, e, matvecs)))
         return rc;
@@ -1069,6 +1128,9 @@ int chase_rayleigh_ritz(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t l
     precision = precision_mode(precision);
     Hop op{(const z_t *)d_H, N, ldh, precision_uses_tc(precision),
            precision == CHASE_MIXED_FP32 ? OZ_S4 : OZ_S6};
+    // The products stay on the slices here: the signs of the eigenvectors of
+    // the reduced problem, and so of the columns returned, follow the rounding
+    // of its matrix, and a caller gets the same vectors as ever.
     if ((rc = hop_prepare(ctx, op, m))) return rc;
     GenTcScope gen_scope(ctx, op.tc);
     if ((rc = phase_rr(ctx, op, (const z_t *)d_Q, ldq, m, s.theta, (z_t *)d_V, (z_t *)d_HV)))
@@ -1132,8 +1194,9 @@ int chase_hemm(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t ldh, const
     if (!hemm_args_ok(d_H, N, ldh, d_Y, ldy, n, d_C, ldc) || !precision_valid(precision))
         return fail(ctx, BSE_EINVAL, "bad product arguments%s");
     precision = precision_mode(precision);
-    const Hop op{(const z_t *)d_H, N, ldh, precision_uses_tc(precision),
-                 precision == CHASE_MIXED_FP32 ? OZ_S4 : OZ_S6};
+    Hop op{(const z_t *)d_H, N, ldh, precision_uses_tc(precision),
+           precision == CHASE_MIXED_FP32 ? OZ_S4 : OZ_S6};
+    op.res = precision_uses_residues(precision, false);
     return hemm(ctx, op, n, d_Y, ldy, d_C, ldc);
 }
 
@@ -1146,6 +1209,7 @@ int chase_hemm_slices(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t ldh
         return fail(ctx, BSE_EINVAL, "bad product arguments%s");
     Hop op{(const z_t *)d_H, N, ldh, true, slices == 4 ? OZ_S4 : slices == 5 ? OZ_S5 : OZ_S6};
     op.tri = half_storage == 1;
+    op.res = slices == 6 && !op.tri;   // CHASE_FP64's product
     return hemm(ctx, op, n, d_Y, ldy, d_C, ldc);
 }
 

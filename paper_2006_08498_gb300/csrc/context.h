@@ -35,6 +35,9 @@ struct bsechase_ctx {
     int sms = 0;                     // multiprocessors of the device
     uint64_t wait_ns = kDefaultWaitNs;  // bounded waits of the tensor-core kernel
     OzakiH oh;
+    bool residues = true;            // solves may use the residue products (a server slot whose
+                                     // request fits the budget on slices alone: not)
+    int hop_cols = 0;                // columns the product buffers were sized for
     int64_t wsN = 0;
     int wsM = 0;
     cudaEvent_t ev[kCtxEvents];   // 0..6: solve phases; 8, 9: host copies
@@ -75,6 +78,16 @@ int solve_device(bsechase_ctx *ctx, const z_t *H, int64_t N, int64_t ldh, int ne
                  double tol, int deg_max, int precision, const chase_opts *opts, double *h_evals,
                  z_t *d_evecs, int64_t ldz, double *h_resid, chase_stats *stats,
                  const BseSource *bse = nullptr);
+// Device bytes that the products with H of an N x N solve of up to mc columns
+// take: H's slices or residues, those of the operand, the partial results, and
+// the slices of op(A) in the general products of QR and Rayleigh-Ritz.
+struct HopBytes {
+    size_t A = 0, B = 0, P = 0, GA = 0;
+};
+HopBytes hop_bytes(int64_t N, int mc, bool res, bool tri, bool bse);
+// Whether the products with H run in residues (residue.cu): the FP64 mode on
+// full storage.
+bool precision_uses_residues(int precision, bool half);
 // Whether `precision` is a chase_precision value, and the mode it runs
 // (CHASE_MIXED_BF16X3 runs as CHASE_MIXED_FP32).
 bool precision_valid(int precision);

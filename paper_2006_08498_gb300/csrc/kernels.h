@@ -85,6 +85,8 @@ size_t ozaki_a_bytes_tri(int64_t N);
 size_t ozaki_b_bytes(int64_t N, int m);
 // workspace for split-K partial products of up to m columns
 size_t ozaki_partial_bytes(int64_t N, int m);
+// ... of the general products alone (ozaki_gemm) of a search space of m columns
+size_t ozaki_gen_partial_bytes(int64_t N, int m);
 
 // General FP64-accurate products on the tensor cores (same kernel and
 // slicing as the product with H): C (M x n) = out(op(A) B), op(A) = A
@@ -146,6 +148,27 @@ cudaError_t ozaki_zgemm(const OzakiH &oh, int n, const z_t *Y, int64_t ldy, z_t 
                         z_t *partials, size_t partial_bytes, int sms, cudaStream_t st,
                         cudaEvent_t ev0 = nullptr, cudaEvent_t ev1 = nullptr,
                         OzBatcher *batcher = nullptr);
+// ---- FP64-accurate products in residue arithmetic (residue.cu): the products
+// with H of the FP64 mode on full storage.  oh->A holds residue_a_bytes(N, N),
+// oh->E Np ints; `work` residue_work_bytes(N) while H is prepared, `panel`
+// residue_panel_bytes(N) when it is generated (bit for bit the stored H's
+// residues).  A product of n columns: B >= residue_b_bytes(N, n), R >=
+// residue_r_bytes(N, N, n), F n ints, part 32 n pairs.
+size_t residue_a_bytes(int64_t M, int64_t K);
+size_t residue_b_bytes(int64_t K, int n);
+size_t residue_r_bytes(int64_t M, int64_t K, int n);
+size_t residue_work_bytes(int64_t N);
+size_t residue_panel_bytes(int64_t N);
+double residue_flops(int64_t M, int64_t K, int n);   // tensor flops of a product
+cudaError_t residue_prepare(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh, void *work, ChaseScalars *sc,
+                            cudaStream_t st);
+cudaError_t residue_prepare_bse(int Nk, int Nv, int Nc, const BseModel &md, const double *dE, const z_t *u,
+                                const z_t *a, const double *Kt, OzakiH *oh, void *work, void *panel,
+                                ChaseScalars *sc, cudaStream_t st);
+cudaError_t residue_zgemm(const OzakiH &oh, int n, const z_t *Y, int64_t ldy, z_t *C, int64_t ldc,
+                          const GemmEpi &ep, void *B, size_t b_bytes, int *F, float2 *part, void *R,
+                          size_t r_bytes, ChaseScalars *sc, int sms, cudaStream_t st, cudaEvent_t ev0,
+                          cudaEvent_t ev1, OzBatcher *batcher);
 // Product batcher shared by the solver threads of a request server: products
 // submitted within window_s of each other (or as soon as every active solver
 // has submitted one) run in one launch of the tensor-core kernel.

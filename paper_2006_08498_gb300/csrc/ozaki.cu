@@ -57,6 +57,7 @@
 #include "common.cuh"
 #include "gen_element.cuh"
 #include "kernels.h"
+#include "residue.h"
 #include "tc_common.cuh"
 
 namespace {
@@ -1276,30 +1277,29 @@ __global__ void k_gen_reduce(int64_t M, int n, int nsplit, const unsigned long l
     C[i + j * ldc] = v;
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
-                                  const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
-                                  const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+}  // namespace
 
 // cuTensorMapEncodeTiled of the CUDA driver API, looked up once (a thread-safe static).
-EncodeTiledFn encode_fn() {
-    static const EncodeTiledFn fn = [] {
+TensorMapEncode tensor_map_encode() {
+    static const TensorMapEncode fn = [] {
         void *p = nullptr;
         cudaDriverEntryPointQueryResult q;
         if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
                                              &q) == cudaSuccess &&
             q == cudaDriverEntryPointSuccess)
-            return (EncodeTiledFn)p;
+            return (TensorMapEncode)p;
         cudaGetLastError();
-        return (EncodeTiledFn) nullptr;
+        return (TensorMapEncode) nullptr;
     }();
     return fn;
 }
 
+namespace {
+
 // 3-D BF16 tensor of K-chunk tiles [tiles][rows][64], box 64 x box_rows x 1,
 // 128-byte swizzle (the shared-memory image of one K-major rows x 64 tile).
 bool make_map(CUtensorMap *m, void *base, uint64_t rows, uint64_t tiles, uint32_t box_rows) {
-    EncodeTiledFn enc = encode_fn();
+    const TensorMapEncode enc = tensor_map_encode();
     if (!enc) return false;
     cuuint64_t dims[3] = {64, rows, tiles};
     cuuint64_t strides[2] = {64 * 2, rows * 64 * 2};
@@ -1362,6 +1362,12 @@ size_t ozaki_partial_bytes(int64_t N, int m) {
     const int64_t sp0 = (nch + kUnitChunks - 1) / kUnitChunks;
     return (size_t)N * (kPartWords * 8) *
            std::max<int64_t>(16 * kW, std::max<int64_t>(8, sp0) * (int64_t)mp);
+}
+
+size_t ozaki_gen_partial_bytes(int64_t N, int m) {
+    // N x m outputs over K <= 512 (one split), m x m outputs over K = N
+    const int64_t nch = ozaki_padded(N) / kKC, sp = (nch + kUnitChunks - 1) / kUnitChunks + 32;
+    return (size_t)(kPartWords * 8) * m * std::max<int64_t>(N, m * sp);
 }
 
 size_t ozaki_b_bytes(int64_t N, int m) {
@@ -1519,8 +1525,9 @@ struct OzBatcher {
     std::mutex mu;
     std::condition_variable cv;
     struct Pending {
-        OzJob job;
-        int cfg = OZ_S6;         // kernel configuration (launch_batch)
+        const OzJob *job = nullptr;     // one of the two, by cfg
+        const RsJob *rjob = nullptr;
+        int cfg = OZ_S6;         // kernel configuration (launch_batch), or kRsCfg
         cudaEvent_t ready = nullptr, done = nullptr;
         bool launched = false;
         cudaError_t err = cudaSuccess;
@@ -1590,12 +1597,39 @@ cudaEvent_t ready_event() {
     return ev;
 }
 
-// Run job (with its kernel configuration) through the batcher; returns after
-// `st` waits for the launch that contains it.
-cudaError_t ozb_run(OzBatcher *b, const OzJob &job, int cfg, cudaStream_t st) {
-    OzBatcher::Pending me;
-    me.job = job;
-    me.cfg = cfg;
+constexpr int kRsCfg = 8;         // residue products (residue.cu)
+
+// The launch of the products taken, all of one configuration.
+cudaError_t launch_taken(const std::vector<OzBatcher::Pending *> &take, int cfg, int sms, cudaStream_t st) {
+    int u = 0;
+    if (cfg == kRsCfg) {
+        static_assert(kRsMaxJobs >= kMaxJobs, "jobs of a launch");
+        RsBatch bt;
+        memset(&bt, 0, sizeof bt);
+        for (size_t k = 0; k < take.size(); k++) {
+            bt.job[k] = *take[k]->rjob;
+            bt.job[k].unit0 = u;
+            u += rs_units(bt.job[k]);
+        }
+        bt.njobs = (int)take.size();
+        bt.units = u;
+        return residue_launch(bt, sms, st);
+    }
+    OzBatch bt;
+    memset(&bt, 0, sizeof bt);
+    for (size_t k = 0; k < take.size(); k++) {
+        bt.job[k] = *take[k]->job;
+        bt.job[k].unit0 = u;
+        u += bt.job[k].args.tx * bt.job[k].args.ty * bt.job[k].args.tz;
+    }
+    bt.njobs = (int)take.size();
+    bt.units = u;
+    return launch_batch(bt, cfg, sms, st);
+}
+
+// Run `me` (job and kernel configuration set) through the batcher; returns
+// after `st` waits for the launch that contains it.
+cudaError_t ozb_run(OzBatcher *b, OzBatcher::Pending &me, cudaStream_t st) {
     me.ready = ready_event();
     if (!me.ready) return cudaErrorUnknown;
     cudaError_t e = cudaEventRecord(me.ready, st);
@@ -1632,16 +1666,6 @@ cudaError_t ozb_run(OzBatcher *b, const OzJob &job, int cfg, cudaStream_t st) {
             b->pool.pop_back();
         }
         lk.unlock();
-        OzBatch bt;
-        memset(&bt, 0, sizeof bt);
-        int u = 0;
-        for (size_t k = 0; k < take.size(); k++) {
-            bt.job[k] = take[k]->job;
-            bt.job[k].unit0 = u;
-            u += take[k]->job.args.tx * take[k]->job.args.ty * take[k]->job.args.tz;
-        }
-        bt.njobs = (int)take.size();
-        bt.units = u;
         cudaError_t le = cudaSuccess;
         if (!done && cudaEventCreateWithFlags(&done, cudaEventDisableTiming) != cudaSuccess) {
             le = cudaGetLastError();
@@ -1649,7 +1673,7 @@ cudaError_t ozb_run(OzBatcher *b, const OzJob &job, int cfg, cudaStream_t st) {
         }
         for (size_t k = 0; k < take.size() && le == cudaSuccess; k++)
             le = cudaStreamWaitEvent(b->st, take[k]->ready, 0);
-        if (le == cudaSuccess) le = launch_batch(bt, cfg0, b->sms, b->st);
+        if (le == cudaSuccess) le = launch_taken(take, cfg0, b->sms, b->st);
         if (le == cudaSuccess) le = cudaEventRecord(done, b->st);
         lk.lock();
         for (auto *p : take) {
@@ -1682,6 +1706,13 @@ cudaError_t ozb_run(OzBatcher *b, const OzJob &job, int cfg, cudaStream_t st) {
 }
 
 }  // namespace
+
+cudaError_t ozb_run_residue(OzBatcher *b, const RsJob &job, cudaStream_t st) {
+    OzBatcher::Pending me;
+    me.rjob = &job;
+    me.cfg = kRsCfg;
+    return ozb_run(b, me, st);
+}
 
 cudaError_t ozaki_zgemm(const OzakiH &oh, int n, const z_t *Y, int64_t ldy, z_t *C, int64_t ldc,
                         const GemmEpi &ep, void *bslices, int *F, ChaseScalars *sc, int level,
@@ -1728,7 +1759,10 @@ cudaError_t ozaki_zgemm(const OzakiH &oh, int n, const z_t *Y, int64_t ldy, z_t 
     const int cfg = level | (oh.tri ? kOzTri : 0);
     cudaError_t e;
     if (batcher) {
-        e = ozb_run(batcher, one.job[0], cfg, st);   // launched with other solvers' products
+        OzBatcher::Pending me;                       // launched with other solvers' products
+        me.job = &one.job[0];
+        me.cfg = cfg;
+        e = ozb_run(batcher, me, st);
     } else {
         if (ev0) cudaEventRecord(ev0, st);
         e = launch_batch(one, cfg, sms, st);

@@ -1,0 +1,1121 @@
+// FP64-accurate complex products on the tensor cores in residue arithmetic
+// (the Chinese remainder form of the Ozaki scheme: Ozaki, Uchino, Imamura,
+// "Ozaki scheme II", 2025).  It is the Chebyshev filter's product H Y (Sec. 3
+// and the Supplement's "Filter" item: a repeated HEMM) and the Lanczos and
+// Rayleigh-Ritz products with H of the FP64 mode on full storage.
+//
+// Representation.  Row i of A is scaled by a power of two so that its 2-norm
+// is at most 2^kAlpha, column j of B so that its is at most 2^kBeta, and both
+// are rounded to integers.  By Cauchy-Schwarz the real and imaginary parts of
+// every element of the integer product are below 2^(kAlpha + kBeta) < P / 2,
+// P the product of kNMod pairwise coprime moduli of at most 8 bits, so they
+// are determined by their residues.  For each modulus the residues, balanced
+// in [-128, 127], are exact in FP16, and so are their products' FP32 sums
+// over 512 terms (kRange): the tensor cores do exact arithmetic.
+//
+// Why residues.  With slices of 8 bits an FP64-accurate product takes every
+// pair of slices of the two operands (21 pairs of 48-bit operands with the
+// small ones left out); residues multiply modulus by modulus, 13 products for
+// operands of 51 and 50 bits.  And modulo p the complex product takes three
+// real ones (Gauss) instead of four, without the cancellation that the
+// three-product form has in floating point:
+//   T0 = Ar Br, T1 = Ai Bi, T2 = (Ar + Ai)(Br + Bi);
+//   Re = T0 - T1, Im = T2 - T0 - T1  (mod p).
+// 13 x 6 = 78 tensor flops per complex multiply-add, against 168.
+//
+// Accuracy.  The only rounding is that of the operands (and one FP64
+// rounding of the result): normwise about 2^-50 sqrt(N), without the
+// truncated partial sums that the slices leave.
+#include <cuda_fp16.h>
+
+#include <algorithm>
+#include <climits>
+#include <cstring>
+#include <mutex>
+
+#include "gen_element.cuh"
+#include "kernels.h"
+#include "residue.h"
+#include "tc_common.cuh"
+
+namespace {
+
+// ------------------------------------------------------------ the moduli
+constexpr int kNMod = 13;
+constexpr int kAlpha = 51, kBeta = 50;
+constexpr int kMod[kNMod] = {256, 253, 251, 249, 247, 241, 239, 233, 229, 227, 223, 217, 211};
+
+constexpr int gcd_of(int a, int b) { return b == 0 ? a : gcd_of(b, a % b); }
+constexpr bool coprime() {
+    for (int i = 0; i < kNMod; i++)
+        for (int j = 0; j < i; j++)
+            if (gcd_of(kMod[i], kMod[j]) != 1) return false;
+    return true;
+}
+static_assert(coprime(), "pairwise coprime moduli");
+constexpr unsigned __int128 modulus_product() {
+    unsigned __int128 P = 1;
+    for (int i = 0; i < kNMod; i++) P *= (unsigned)kMod[i];
+    return P;
+}
+// 2^(kAlpha + kBeta) plus 20 % (norm estimates and the operands' rounding) below P / 2
+static_assert(modulus_product() / 2 > ((unsigned __int128)6 << (kAlpha + kBeta)) / 5, "range of the product");
+
+// Constants of one modulus.  A residue of the 64-bit integer X + 2^63 (bytes
+// b_0..b_7): v = sum_i b_i (256^i mod p) + k0 - 12582912 by two 4-byte dot
+// products, below 2^20; started at k0 they leave the bit pattern of the float
+// 1.5 2^23 + v, an integer F below 2^24 that k0 makes congruent to X.  Then r = F -
+// p rint(F / p) in FP32 (two FMAs and an addition, exact; |r| <= p / 2 + 1, so at
+// most 127 for p <= 253, and 256 divides exactly), and the low byte of r + 128 +
+// 2^23 is the residue as it is stored: b in [0, 255] stands for b - 128.
+// (The same with an integer multiply-high and multiply in place of the FP32
+// steps: 278 instructions per element of A for the 26 residues, 178 of them on one
+// of the two FMA pipes.)
+struct ModConst {
+    uint32_t clo, chi, k0;
+    float pf, inv;
+    unsigned long long W;   // round(2^64 ((P/p)^-1 mod p) / p)
+};
+struct ModTable {
+    ModConst m[kNMod];
+};
+constexpr ModTable make_table() {
+    ModTable t{};
+    for (int i = 0; i < kNMod; i++) {
+        const unsigned p = (unsigned)kMod[i];
+        unsigned c = 1 % p, cc[8] = {};
+        for (int b = 0; b < 8; b++) {
+            cc[b] = c;
+            c = c * 256u % p;
+        }
+        t.m[i].clo = cc[0] | cc[1] << 8 | cc[2] << 16 | cc[3] << 24;
+        t.m[i].chi = cc[4] | cc[5] << 8 | cc[6] << 16 | cc[7] << 24;
+        // F = 12582912 + (k0 - 0x4B400000) + sum: congruent to X
+        const unsigned two63 = cc[7] * 128u % p, base = 12582912u % p;
+        t.m[i].k0 = 0x4B400000u + (2 * p - two63 - base) % p;
+        t.m[i].pf = (float)p;
+        t.m[i].inv = 1.0f / (float)p;
+        unsigned q = 1;                            // (P / p) mod p
+        for (int j = 0; j < kNMod; j++)
+            if (j != i) q = q * ((unsigned)kMod[j] % p) % p;
+        unsigned v = 1;
+        while (q * v % p != 1) v++;
+        t.m[i].W = (unsigned long long)((((unsigned __int128)v << 64) + p / 2) / p);
+    }
+    return t;
+}
+__constant__ ModTable kTab = make_table();
+
+// The element is F / 2^64 P with F = sum_m W_m r_m modulo 2^64 as a signed
+// number: the fraction of sum_m r_m inv_m / p_m, to 2^-53 of the range.
+constexpr double kScale = (double)modulus_product() * 0x1.0p-64;
+
+// ------------------------------------------------------------ the tiling
+constexpr int kRows = 128;         // rows of a CTA (TMEM lanes, MMA M)
+constexpr int kMaxW = 144;         // complex columns of a CTA at most
+constexpr int kChunk = 64;         // K elements of a stage (one swizzle row of FP16)
+constexpr int kRange = 8;          // T2 is drained every kRange chunks, T0 and T1 every 2 kRange
+constexpr int kMaxUnitChunks = 224;           // a drain thread's packed sums
+constexpr int kAStage = 2 * kRows * kChunk;   // Re and Im residues, one byte each
+constexpr int kPack = 8192;        // a drain thread keeps Re + kPack Im in one integer
+constexpr int kDrainWarps = 8;
+constexpr int kTmemCols = 512;
+// Tensor memory holds the three accumulators of a launch's widest tile and, in
+// the rest, the ring of A operand stages (16 columns: K = 32 of one operand): 5
+// beside 144 columns, more beside fewer, which covers the latency between an
+// MMA's reading a stage and the MMA that reads its next contents.
+constexpr int kMinSlots = 5, kMaxSlots = 16;
+constexpr int kBars = 32;          // barriers of the stages, as a ring (a power of two, above kMaxSlots)
+
+// Variants by the widest column tile of a launch.  Converting A costs the same
+// whatever the width, so a narrow tile is bound by the converters: it has more
+// of them, which the drain threads' registers (one packed sum per column) allow.
+// Warpgroups (4 warps, one per TMEM quadrant): copies and MMAs; kConv converter
+// groups; two drain groups.  Registers a thread: R0, RC, RD (setmaxnreg moves
+// them from the others to the drain groups) of RL at launch; 0: no move.
+template <int W, int CONV, int SA, int SB, int HOLD, int RL, int R0, int RC, int RD>
+struct RsCfg {
+    static constexpr int kW = W;                   // columns of a tile at most
+    static constexpr int kConv = CONV;
+    static constexpr int kThreads = 32 * (4 + 4 * CONV + kDrainWarps);
+    static constexpr int kSA = SA, kSB = SB;       // stages of A's bytes and of B
+    static constexpr int kBStage = 3 * W * kChunk * 2;
+    static constexpr int kSmem = SA * kAStage + SB * kBStage + 1024;
+    static constexpr int kHold = HOLD;             // granules of 8 columns a drain thread loads at once
+    static constexpr int kR0 = R0, kRC = RC, kRD = RD;
+    static_assert(128 * (R0 + CONV * RC + 2 * RD) <= kThreads * RL && 65536 / kThreads >= RL, "register split");
+    static_assert(kSmem <= 231000 && 3 * W + kMinSlots * 16 <= kTmemCols && 2 * HOLD >= W / 16, "resources");
+};
+using RsWide = RsCfg<144, 2, 3, 3, 6, 96, 48, 80, 136>;
+using RsMid = RsCfg<96, 3, 5, 3, 6, 80, 48, 64, 112>;
+using RsNarrow = RsCfg<48, 4, 8, 3, 3, 72, 0, 0, 0>;
+static_assert((long long)kRange * kChunk * 128 * 256 <= (1ll << 24) &&
+                  2ll * kRange * kChunk * 128 * 128 <= (1ll << 24), "exact FP32 sums");
+static_assert((kMaxUnitChunks / (2 * kRange) + 1) * 2 * 128 < kPack / 2, "packed sums");
+// The accumulators are drained after chunk c of a unit of nc: T0 when c % 16 is
+// 15, T1 when it is 10, T2 (whose operand Ar + Ai is twice as large) when it is
+// 5 or 13, and all three after the last chunk: spread over time, so that each
+// drain is over before the next is due.
+static_assert(kRange == 8, "drain pattern");
+__device__ __forceinline__ bool range_end(int t, int c) {
+    return t == 0 ? (c & 15) == 15 : t == 1 ? (c & 15) == 10 : (c & 7) == 5;
+}
+constexpr uint64_t kWindDownNs = 2000000000ull;
+
+// Work per CTA: one modulus, 128 rows, w <= 144 columns, the K chunks of one
+// split.  Persistent, one CTA per SM, units walked by modulus (slowest), split,
+// row tile and column tile (fastest), so that the CTAs running at one time
+// read one modulus' operand (L2) and different rows of A.
+//
+//   warp 0      copies A's bytes (16 KB per chunk, untiled) into a ring of stages;
+//   warps 1-3   copy a part of B each (FP16, one TMA box per chunk) and issue the
+//               MMAs of its product: per chunk 4 K steps;
+//   converters  turn A's bytes into FP16 pairs (a byte permute makes 1024 + b,
+//               one subtraction b - 128), add Re and Im for the third product
+//               and store the operands into tensor memory: one byte per
+//               residue crosses HBM and shared memory, and the MMA reads only
+//               B from shared memory;
+//   the last 8  drain an accumulator every 16 (T2: 8) chunks: reduce modulo p in FP32
+//               (exact: two FMAs and an addition, two values an instruction)
+//               and add into one packed integer per output.
+template <class Cfg>
+__global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_constant__ RsBatch bt) {
+    constexpr int kConvWarps = 4 * Cfg::kConv;
+    constexpr int kSA = Cfg::kSA, kSB = Cfg::kSB, kBStage = Cfg::kBStage, kConvGroups = Cfg::kConv;
+    extern __shared__ uint8_t smraw[];
+    uint8_t *sm = (uint8_t *)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
+    uint8_t *sB = sm, *sA = sm + kSB * kBStage;
+    __shared__ uint64_t fullA[kSA], emptyA[kSA], fullB[3 * kSB], emptyB[3 * kSB];   // B: per product
+    __shared__ uint64_t accFull[3], accEmpty[3], mmaDone;
+    __shared__ __align__(2 * kBars * 8) uint64_t aBars[2 * kBars];   // stages of A: full, then empty
+    uint64_t *aFull = aBars, *aEmpty = aBars + kBars;
+    __shared__ uint32_t tmem_base;
+    __shared__ volatile int abort_flag;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x / 32, 0), lane = threadIdx.x % 32;
+    const int units = bt.units;
+    const uint32_t stride = (uint32_t)bt.stride, slots = (uint32_t)bt.slots;
+    const uint64_t wait_ns = bt.job[0].wait_ns;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kSA; s++) {
+            tc::mbar_init(&fullA[s], 1);
+            tc::mbar_init(&emptyA[s], 8);
+        }
+        for (int s = 0; s < 3 * kSB; s++) {
+            tc::mbar_init(&fullB[s], 1);
+            tc::mbar_init(&emptyB[s], 1);
+        }
+        for (int s = 0; s < kBars; s++) {
+            tc::mbar_init(&aFull[s], 4);
+            tc::mbar_init(&aEmpty[s], 1);
+        }
+        for (int t = 0; t < 3; t++) {
+            tc::mbar_init(&accFull[t], 1);
+            tc::mbar_init(&accEmpty[t], kDrainWarps);
+        }
+        tc::mbar_init(&mmaDone, 3);
+        abort_flag = 0;
+        tc::mbar_fence_init();
+    }
+    if (warp == 1) tc::tmem_alloc(&tmem_base, kTmemCols);
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    const uint32_t tmem = tmem_base;
+
+    struct Unit {
+        int jb, x, y, z, m, c0, c1;
+    };
+    auto unit = [&](int u) {
+        Unit n;
+        n.jb = 0;
+        while (n.jb + 1 < bt.njobs && u >= bt.job[n.jb + 1].unit0) n.jb++;
+        const RsJob &a = bt.job[n.jb];
+        int r = u - a.unit0;
+        n.x = r % a.tx;
+        r /= a.tx;
+        n.y = r % a.ty;
+        r /= a.ty;
+        n.z = r % a.tz;
+        n.m = r / a.tz;
+        n.c0 = n.z * a.cs;
+        n.c1 = min(a.nch, n.c0 + a.cs);
+        return n;
+    };
+
+    // A wait of a whole warp: every lane waits (bounded), and all leave with
+    // the same answer, so that no lane is missed at the next warp barrier.
+    auto wait_all = [&](uint32_t b, uint32_t parity) {
+        const bool r = tc::mbar_wait_at(b, parity, &abort_flag, wait_ns);
+        return __all_sync(0xffffffffu, r) != 0;
+    };
+    const uint32_t bars = tc::smem_u32(aBars);     // aligned to its size: a stage's barrier by or-ing
+    constexpr uint32_t kBarMask = 8 * kBars - 1, kBarEmpty = 8 * kBars;
+
+    int fills = 0;      // copies issued, of A (warp 0) or of a part of B (warps 1-3)
+    if (warp < 4) {
+      if (Cfg::kR0) tc::reg_dec<Cfg::kR0 ? Cfg::kR0 : 24>();
+      if (warp == 0) {
+        if (lane == 0) {
+            bool ok = true;
+            for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+                const Unit n = unit(u);
+                const RsJob &a = bt.job[n.jb];
+                const uint8_t *src = a.A + (((int64_t)n.m * a.ty + n.y) * a.nch + n.c0) * kAStage;
+                for (int c = n.c0; c < n.c1; c++, src += kAStage) {
+                    const int s = fills % kSA, f = fills / kSA;
+                    if (f >= 1 && !tc::mbar_wait(&emptyA[s], (f - 1) & 1, &abort_flag, wait_ns)) { ok = false; break; }
+                    tc::mbar_expect_tx(&fullA[s], kAStage);
+                    tc::bulk_load(sA + s * kAStage, src, kAStage, &fullA[s]);
+                    fills++;
+                }
+            }
+        }
+      } else {
+        // A warp for each product: its waits and instructions are a third (one
+        // warp for all three needed 1.5 to 2 times the MMAs' own time, measured).
+        // The whole warp runs the loop and one elected lane issues (predicated,
+        // without branches), so that the descriptors are warp-uniform (uniform
+        // registers feed tcgen05.mma).  The next chunk's barriers are looked at
+        // (without blocking) before this one's MMAs are issued, and waited for
+        // only if that look failed.
+        const int t = warp - 1;
+        const uint32_t one = tc::elect_one() ? 1u : 0u;
+        const uint32_t fullB0 = tc::smem_u32(fullB + t * kSB), emptyB0 = tc::smem_u32(emptyB + t * kSB);
+        const uint32_t accF = tc::smem_u32(&accFull[t]), accE = tc::smem_u32(&accEmpty[t]);
+        const uint32_t acc = tmem + t * stride, tbeg = tmem + 3 * stride, tend = tbeg + slots * 16;
+        bool ok = true;
+        uint32_t sB8 = 0, sph = 0, aph = 1;        // stage of B (8 bytes a barrier), phases
+        // The warp also copies its part of B (a third of the stage whatever the width:
+        // the products' warps reuse a stage independently of one another), kSB - 1 chunks ahead: into the stage
+        // whose MMAs it issued a chunk ago (one thread that copied A and all of B
+        // spent up to 1650 cycles a chunk on it, measured, more than any other role).
+        int uL = blockIdx.x, leftL = 0, jL = 0, xL = 0, zL = 0;
+        uint32_t l8 = 0, lph = 1;
+        bool rdyE = false;                         // its stage was seen free
+        auto load = [&]() {
+            if (leftL == 0) {
+                if (uL >= units) return true;
+                const Unit n = unit(uL);
+                const RsJob &a = bt.job[n.jb];
+                jL = n.jb;
+                xL = n.x * a.w;
+                zL = (n.m * a.nch + n.c0) * 3 + t;
+                leftL = n.c1 - n.c0;
+                uL += gridDim.x;
+            }
+            if (!rdyE && !wait_all(emptyB0 + l8, lph)) return false;
+            if (one) {
+                const uint32_t bytes = (uint32_t)bt.job[jL].w * kChunk * 2;
+                uint64_t *bar = &fullB[t * kSB + l8 / 8];
+                tc::mbar_expect_tx(bar, bytes);
+                tc::tma_load_3d(sB + l8 / 8 * kBStage + t * (kBStage / 3), &bt.job[jL].tmB, 0, xL, zL, bar);
+            }
+            __syncwarp();
+            fills++;
+            zL += 3;
+            leftL--;
+            l8 += 8;
+            if (l8 == 8 * kSB) { l8 = 0; lph ^= 1; }
+            return true;
+        };
+        for (int s = 0; s + 1 < kSB; s++) load();   // fresh barriers: no wait
+        // The product's stage of a half chunk, its barrier and phase.  A wait that
+        // succeeds costs a warp about 100 cycles, so the barriers of the next half
+        // chunk are looked at (without blocking) before this one's MMAs are issued,
+        // and waited for only if that look failed.
+        uint32_t f8 = 8 * t, bph = 0, at = tbeg + 16 * t;
+        bool rdy = false, rdyB = false;
+        auto next = [&]() { return bars | f8; };
+        auto advance = [&]() {
+            f8 += 24;
+            if (f8 > kBarMask) { f8 &= kBarMask; bph ^= 1; }
+            at += 48;
+            if (at >= tend) at -= slots * 16;
+        };
+        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+            const Unit n = unit(u);
+            const int w = bt.job[n.jb].w;
+            const uint32_t id = tc::idesc_f16_f32(kRows, w);
+            const uint64_t bd0 = tc::sdesc_sw128(sB) + (uint32_t)(t * (kBStage / 3) >> 4);
+            const int nc = n.c1 - n.c0;
+            uint32_t fresh = 1;
+            for (int c = 0; c < nc; c++) {
+                const uint32_t end = c + 1 == nc || range_end(t, c) ? 1u : 0u;
+                if (!rdyB && !wait_all(fullB0 + sB8, sph)) { ok = false; break; }
+                // a fresh barrier passes the wait for the phase before its first
+                if (fresh && !wait_all(accE, aph)) { ok = false; break; }
+                const uint64_t bd = bd0 + (uint64_t)(sB8 * (kBStage / 8 >> 4));
+                const uint32_t b0 = next();
+                if (!rdy && !wait_all(b0, bph)) { ok = false; break; }
+                tc::fence_after();
+                const uint32_t t0 = at;
+                advance();
+                const uint32_t b1 = next();
+                bool look = tc::mbar_test_at(b1, bph);
+                tc::mma_f16_ta_if(one, acc, t0, bd, id, fresh ^ 1);
+                tc::mma_f16_ta_if(one, acc, t0 + 8, bd + 2, id, 1u);
+                tc::mma_commit_if(one, b0 + kBarEmpty);
+                rdy = __all_sync(0xffffffffu, look) != 0;
+                if (!rdy && !wait_all(b1, bph)) { ok = false; break; }
+                tc::fence_after();
+                const uint32_t t1 = at, eB = emptyB0 + sB8;
+                advance();
+                sB8 += 8;
+                if (sB8 == 8 * kSB) { sB8 = 0; sph ^= 1; }
+                look = tc::mbar_test_at(next(), bph);
+                const bool lookB = tc::mbar_test_at(fullB0 + sB8, sph), lookE = tc::mbar_test_at(emptyB0 + l8, lph);
+                tc::mma_f16_ta_if(one, acc, t1, bd + 4, id, 1u);
+                tc::mma_f16_ta_if(one, acc, t1 + 8, bd + 6, id, 1u);
+                tc::mma_commit_if(one, b1 + kBarEmpty);
+                tc::mma_commit_if(one, eB);
+                if (end) tc::mma_commit_if(one, accF);
+                fresh = end;
+                aph ^= end;
+                rdy = __all_sync(0xffffffffu, look) != 0;
+                rdyB = __all_sync(0xffffffffu, lookB) != 0;
+                rdyE = __all_sync(0xffffffffu, lookE) != 0;
+                if (!load()) { ok = false; break; }
+            }
+        }
+      }
+    } else if (warp < 4 + kConvWarps) {
+        if (Cfg::kRC) tc::reg_dec<Cfg::kRC ? Cfg::kRC : 24>();
+        // The groups take turns, half a chunk (32 K elements) each: item 2 chunk + h.
+        // Its i-th operand is fill 3 item + i of the ring of stages, and waits for
+        // the MMAs on the fill `slots` before it.
+        const int quad = warp & 3, row = quad * 32 + lane;
+        const __half2 k1152 = __floats2half2_rn(1152.f, 1152.f);
+        int item = (warp - 4) >> 2;
+        uint32_t f8 = 24 * item;                   // the fill's barrier
+        uint32_t e8 = 8 * (3 * item - slots), eph = 1;   // of the fill it waits for (modulo the ring)
+        if ((int)e8 >= 0) eph = 0;
+        e8 &= kBarMask;
+        const uint32_t tbeg = tmem + ((uint32_t)(quad * 32) << 16) + 3 * stride, tend = tbeg + slots * 16;
+        uint32_t ta = tbeg + 3 * item % slots * 16;
+        const uint32_t skip = 3 * (kConvGroups - 1) % slots * 16;
+        uint32_t sa8 = 8 * (item >> 1), saph = 0;  // stage of A's bytes (8 bytes a barrier), and its phase
+        static_assert((kConvGroups - 1) / 2 < kSA && (kConvGroups + 1) / 2 <= kSA, "one turn of the ring at most");
+        const uint32_t fullA0 = tc::smem_u32(fullA), emptyA0 = tc::smem_u32(emptyA);
+        auto convert = [&](const uint8_t *src, uint32_t *r) {
+#pragma unroll
+            for (int g = 0; g < 2; g++) {
+                const uint4 q = *(const uint4 *)(src + g * (kRows * 16));
+                const uint32_t v[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+                for (int e = 0; e < 8; e++) {
+                    const uint32_t x = __byte_perm(v[e / 2], 0x64646464u, e % 2 ? 0x4342 : 0x4140);
+                    __half2 a;                     // (1024 + b) - 1152
+                    memcpy(&a, &x, 4);
+                    a = __hsub2(a, k1152);
+                    memcpy(&r[g * 8 + e], &a, 4);
+                }
+            }
+        };
+        auto put = [&](const uint32_t *r) {
+            // a fresh barrier passes the wait for the phase before its first
+            if (!wait_all(bars | kBarEmpty | e8, eph)) return false;
+            tc::fence_after();
+            tc::tmem_st16(ta, r);
+            ta += 16;
+            if (ta == tend) ta = tbeg;
+            tc::tmem_wait_st();
+            tc::fence_before();
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive_at(bars | f8);
+            f8 = (f8 + 8) & kBarMask;
+            e8 += 8;
+            if (e8 > kBarMask) { e8 = 0; eph ^= 1; }
+            return true;
+        };
+        // item counts over all units; i is its number in its unit
+        int done = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+            const Unit n = unit(u);
+            const int ni = 2 * (n.c1 - n.c0);
+            for (int i = item - done; i < ni; i += kConvGroups, item += kConvGroups) {
+                if (!wait_all(fullA0 + sa8, saph)) { ok = false; break; }
+                const int h = i & 1;
+                const uint8_t *src = sA + sa8 * (kAStage / 8) + (h * 2 * kRows + row) * 16;
+                uint32_t re[16], im[16];           // FP16 pairs
+                convert(src, re);
+                convert(src + 4 * kRows * 16, im);
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive_at(emptyA0 + sa8);
+                if (!put(re) || !put(im)) { ok = false; break; }
+#pragma unroll
+                for (int e = 0; e < 16; e++) {
+                    __half2 a, b;
+                    memcpy(&a, &re[e], 4);
+                    memcpy(&b, &im[e], 4);
+                    a = __hadd2(a, b);             // in [-256, 254]: exact
+                    memcpy(&re[e], &a, 4);
+                }
+                if (!put(re)) { ok = false; break; }
+                // past the other groups' items
+                f8 = (f8 + 24 * (kConvGroups - 1)) & kBarMask;
+                e8 += 24 * (kConvGroups - 1);
+                if (e8 > kBarMask) { e8 &= kBarMask; eph ^= 1; }
+                ta += skip;
+                if (ta >= tend) ta -= slots * 16;
+                sa8 += (h + kConvGroups) / 2 * 8;
+                if (sa8 >= 8 * kSA) { sa8 -= 8 * kSA; saph ^= 1; }
+            }
+            done += ni;
+        }
+    } else {
+        if (Cfg::kRD) tc::reg_inc<Cfg::kRD ? Cfg::kRD : 24>();
+        const int quad = warp & 3, half = (warp - 4 - kConvWarps) >> 2;
+        const int row = quad * 32 + lane;
+        const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
+        constexpr int kG = Cfg::kW / 16, kHold = Cfg::kHold;   // granules of 8 columns per thread, held at once
+        constexpr float kMagic = 12582912.f;       // 1.5 2^23: rounds to an integer
+        bool ok = true;
+        uint32_t ph = 0;                           // phases of accFull
+        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+            const Unit n = unit(u);
+            const RsJob &a = bt.job[n.jb];
+            const int ng = a.w / 16;
+            const float pf = kTab.m[n.m].pf, inv = kTab.m[n.m].inv;
+            int acc[kG * 8];
+#pragma unroll
+            for (int v = 0; v < kG * 8; v++) acc[v] = 0;
+            int cnt = 0;
+            const int nc = n.c1 - n.c0;
+            const uint64_t inv2 = tc::pin2(tc::f32x2(inv, inv)), mp2 = tc::pin2(tc::f32x2(-pf, -pf));
+            const uint64_t magic2 = tc::pin2(tc::f32x2(kMagic, kMagic)), mmagic2 = tc::pin2(tc::f32x2(-kMagic, -kMagic));
+            for (int ev = 0, fin = 0; fin < 3;) {
+                // the next drain: T2, T1, T2, T0 after chunks 5, 10, 13, 15 of every
+                // 16, until the last chunk; then T0, T1, T2
+                int t;
+                if (fin == 0 && (ev >> 2) * 16 + ((0xFDA5 >> (ev % 4 * 4)) & 15) < nc - 1) {
+                    t = (0x0212 >> (ev % 4 * 4)) & 3;
+                    ev++;
+                } else {
+                    t = fin++;
+                }
+                if (!wait_all(tc::smem_u32(&accFull[t]), (ph >> t) & 1)) { ok = false; break; }
+                ph ^= 1u << t;
+                tc::fence_after();
+                // Re + kPack Im: T0 counts (1, -1), T1 (-1, -1), T2 (0, 1)
+                const float coef = t == 0 ? (float)(1 - kPack) : t == 1 ? (float)(-1 - kPack) : (float)kPack;
+                const uint64_t coef2 = tc::pin2(tc::f32x2(coef, coef));
+                const uint32_t col = tmem + lane_addr + t * stride + half * ng * 8;
+                auto digest = [&](const uint32_t *r, int g) {
+#pragma unroll
+                    for (int v = 0; v < 8; v += 2) {
+                        const uint64_t xx = tc::pack2(r[v], r[v + 1]);
+                        const uint64_t q = tc::add2(tc::fma2(xx, inv2, magic2), mmagic2);
+                        const uint64_t y = tc::fma2(q, mp2, xx);
+                        const uint64_t z = tc::fma2(y, coef2, magic2);
+                        acc[g * 8 + v] += (int)(uint32_t)z;
+                        acc[g * 8 + v + 1] += (int)(uint32_t)(z >> 32);
+                    }
+                };
+                // as many columns as registers hold are loaded first, then the
+                // accumulator goes back to the MMAs, then the arithmetic
+                uint32_t r[kHold * 8];
+#pragma unroll
+                for (int g = 0; g < kHold; g++)
+                    if (g < ng) tc::tmem_ld8(col + g * 8, r + g * 8);
+                tc::tmem_wait_ld();
+#pragma unroll
+                for (int g = kHold; g < kG; g++)
+                    if (g < ng) {
+                        digest(r + (g - kHold) * 8, g - kHold);
+                        tc::tmem_ld8(col + g * 8, r + (g - kHold) * 8);
+                    }
+                tc::tmem_wait_ld();
+                tc::fence_before();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&accEmpty[t]);
+#pragma unroll
+                for (int g = 0; g < kG; g++) {
+                    const int at = g >= kHold ? g - kHold : g;
+                    if (g < ng && (g >= kG - kHold || g + kHold >= ng)) digest(r + at * 8, g);
+                }
+                cnt++;
+            }
+            if (!ok) break;
+            char2 *R = a.R + ((int64_t)(n.m * a.tz + n.z) * a.mp + n.x * a.w + half * ng * 8) * a.Mp +
+                       (int64_t)n.y * kRows + row;
+            const unsigned off = (unsigned)cnt * (unsigned)__float_as_int(kMagic);
+#pragma unroll
+            for (int v = 0; v < kG * 8; v++) {
+                if (v < ng * 8) {
+                    const int s = (int)((unsigned)acc[v] - off);
+                    const int si = (s + kPack / 2) >> 13, sr = s - si * kPack;
+                    const float xr = (float)sr, xi = (float)si;
+                    const float yr = __fmaf_rn(-pf, rintf(xr * inv), xr), yi = __fmaf_rn(-pf, rintf(xi * inv), xi);
+                    R[(int64_t)v * a.Mp] = make_char2((signed char)(int)yr, (signed char)(int)yi);
+                }
+            }
+        }
+    }
+
+    tc::fence_before();
+    __syncthreads();
+    if (abort_flag) {
+        // An expired wait: every role has left its loop.  Before shared and
+        // tensor memory go, the copies and MMAs already issued must land.
+        bool drained = true;
+        if (warp == 0 && lane == 0) {
+            for (int s = 0; s < kSA; s++) {
+                const int f = (fills - s + kSA - 1) / kSA;           // copies into stage s
+                if (f > 0) drained &= tc::mbar_wait_for(&fullA[s], (f - 1) & 1, kWindDownNs);
+            }
+        }
+        if (warp >= 1 && warp < 4 && tc::elect_one()) {
+            for (int s = 0; s < kSB; s++) {
+                const int f = (fills - s + kSB - 1) / kSB;
+                if (f > 0) drained &= tc::mbar_wait_for(&fullB[(warp - 1) * kSB + s], (f - 1) & 1, kWindDownNs);
+            }
+            tc::mma_commit(&mmaDone);
+            drained &= tc::mbar_wait_for(&mmaDone, 0, kWindDownNs);
+        }
+        if (!drained)
+            for (int j = 0; j < bt.njobs; j++) set_error(bt.job[j].sc, DEV_TIMEOUT, -1 - (int)blockIdx.x);
+        tc::fence_before();
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int j = 0; j < bt.njobs; j++) set_error(bt.job[j].sc, DEV_TIMEOUT, blockIdx.x);
+    }
+    if (warp == 1) {
+        tc::fence_after();
+        tc::tmem_dealloc(tmem, kTmemCols);
+    }
+}
+
+// ------------------------------------------------------------ line norms
+// The 2-norm of a line (row of A, column of B) only sets a power of two, so
+// it is summed in FP32 on the top 20 mantissa bits relative to the largest
+// exponent seen, from the bit patterns with integer operations (FP64 issue is
+// scarce on this part).  acc 2^(2 (eb - 1023)): the sum of squares, less a
+// relative 2^-12 that norm_exponent adds back.
+struct NormAcc {
+    float acc = 0.f;
+    int eb = 0;         // biased exponent of the largest entry
+    __device__ __forceinline__ void shift_to(int e) {
+        const int d = 2 * (e - eb);
+        acc = d > 120 ? 0.f : acc * __int_as_float((127 - d) << 23);
+        eb = e;
+    }
+    __device__ __forceinline__ float mant(unsigned h) const {
+        const int t = (int)h - ((eb - 127) << 20);
+        return (h == 0 || t < 0) ? 0.f : __int_as_float(t << 3);
+    }
+    __device__ __forceinline__ void add(z_t v) {
+        const unsigned hx = (unsigned)__double2hiint(v.x) & 0x7FFFFFFFu;
+        const unsigned hy = (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu;
+        const int e = (int)(max(hx, hy) >> 20);
+        if (e > eb) shift_to(e);
+        const float fx = mant(hx), fy = mant(hy);
+        acc = fmaf(fx, fx, fmaf(fy, fy, acc));
+    }
+    __device__ __forceinline__ void add(float2 o) { merge(o.x, __float_as_int(o.y)); }
+    __device__ __forceinline__ void merge(float oacc, int oeb) {
+        if (oeb > eb) shift_to(oeb);
+        const int d = 2 * (eb - oeb);
+        if (d <= 120) acc = fmaf(oacc, __int_as_float((127 - d) << 23), acc);
+    }
+    __device__ __forceinline__ float2 pack() const { return make_float2(acc, __int_as_float(eb)); }
+    // h with norm <= 2^h; INT_MIN for a zero line
+    __device__ __forceinline__ int exponent() const {
+        if (!(acc > 0.f)) return INT_MIN;
+        int e;
+        frexpf(acc * (1.f + 0x1.0p-10f), &e);
+        return (e + 2 * (eb - 1023) + 1) >> 1;
+    }
+};
+constexpr int kInfExp = 0x7FF;      // biased exponent of Inf and NaN
+
+// Row sums of squares of the columns [k0, k0 + cols) of A (M rows): one
+// partial per row and segment of `seg` columns, partial index seg0 + segment.
+__global__ void __launch_bounds__(128)
+k_res_rownorm(int64_t M, int64_t cols, const z_t *__restrict__ A, int64_t lda, int seg, int64_t seg0,
+              float2 *__restrict__ part) {
+    const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    if (i >= M) return;
+    const int64_t k0 = (int64_t)blockIdx.y * seg, k1 = min(k0 + seg, cols);
+    NormAcc n;
+#pragma unroll 8
+    for (int64_t k = k0; k < k1; k++) n.add(A[i + k * lda]);
+    part[(seg0 + blockIdx.y) * M + i] = n.pack();
+}
+
+__global__ void __launch_bounds__(128)
+k_res_rowscale(int64_t M, int64_t Mp, int nseg, const float2 *__restrict__ part, int *E, ChaseScalars *sc) {
+    const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    if (i >= Mp) return;
+    NormAcc n;
+    if (i < M) {
+#pragma unroll 8
+        for (int s = 0; s < nseg; s++) n.add(part[(int64_t)s * M + i]);
+    }
+    if (n.eb == kInfExp) set_error(sc, DEV_NONFINITE, (int)i);
+    E[i] = n.exponent();
+}
+
+// Partial sums of squares of column blockIdx.y: part[j * gridDim.x + block]
+__global__ void __launch_bounds__(256)
+k_res_colnorm(int64_t N, const z_t *__restrict__ Y, int64_t ldy, float2 *__restrict__ part, ChaseScalars *sc) {
+    __shared__ float2 red[8];
+    const int j = blockIdx.y;
+    NormAcc n;
+    for (int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x; k < N; k += (int64_t)gridDim.x * 256)
+        n.add(Y[k + j * ldy]);
+    for (int o = 16; o > 0; o >>= 1) {
+        const float oa = __shfl_xor_sync(0xffffffffu, n.acc, o);
+        const int oe = __shfl_xor_sync(0xffffffffu, n.eb, o);
+        n.merge(oa, oe);
+    }
+    if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = n.pack();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        NormAcc t;
+        for (int w = 0; w < 8; w++) t.add(red[w]);
+        if (t.eb == kInfExp) set_error(sc, DEV_NONFINITE, j);
+        part[(int64_t)j * gridDim.x + blockIdx.x] = t.pack();
+    }
+}
+
+// ------------------------------------------------------------ residues
+// rint(x 2^sh) + 2^63, ties to even, for |x 2^sh| < 2^62, from the bit
+// pattern with integer operations.  Non-finite x gives an arbitrary value.
+__device__ __forceinline__ unsigned long long biased_rint(double x, int sh) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const int ef = (int)((b >> 52) & 0x7FF);
+    unsigned long long m = b & 0xFFFFFFFFFFFFFull;
+    int s = -1074 + sh;
+    if (ef != 0) {
+        m |= 1ull << 52;
+        s = ef - 1075 + sh;
+    }
+    unsigned long long q;
+    if (s >= 0) {
+        q = m << min(s, 63);
+    } else {
+        // add half an ulp less one, plus the quotient's last bit: ties to even
+        const int r = min(-s, 62);
+        const unsigned long long half = 1ull << (r - 1);
+        q = (m + half - 1 + ((m >> r) & 1)) >> r;
+    }
+    q = (b >> 63) ? 0ull - q : q;
+    return q + (1ull << 63);
+}
+
+// The residues of x0 and x1: words whose low bytes are residue + 128.
+struct ResConst {
+    uint32_t clo, chi, k0;
+    uint64_t mp2, inv2;
+    __device__ __forceinline__ explicit ResConst(const ModConst &m)
+        : clo(m.clo), chi(m.chi), k0(m.k0), mp2(tc::f32x2(-m.pf, -m.pf)), inv2(tc::f32x2(m.inv, m.inv)) {}
+    __device__ __forceinline__ uint64_t two(unsigned long long x0, unsigned long long x1) const {
+        const uint64_t magic2 = tc::f32x2(12582912.f, 12582912.f), mmagic2 = tc::f32x2(-12582912.f, -12582912.f);
+        const uint64_t bias2 = tc::f32x2(8388736.f, 8388736.f);
+        const uint32_t v0 = __dp4a((uint32_t)(x0 >> 32), chi, __dp4a((uint32_t)x0, clo, k0));
+        const uint32_t v1 = __dp4a((uint32_t)(x1 >> 32), chi, __dp4a((uint32_t)x1, clo, k0));
+        const uint64_t f = tc::pack2(v0, v1);
+        const uint64_t q = tc::add2(tc::fma2(f, inv2, magic2), mmagic2);
+        return tc::add2(tc::fma2(q, mp2, f), bias2);
+    }
+};
+
+// Residues of 16 consecutive K elements of one row of A per thread: columns
+// k0 + 16 (blockIdx.x) of the matrix, read coalesced down the rows, and for
+// each modulus 16 bytes of Re and of Im, [group of 16][row][16 bytes] of the
+// chunk's 16 KB block, so that a converter thread's row is conflict-free.
+// Bound by integer issue: about 130 instructions per element for the 26
+// residues, over 16 bytes read and 26 written.
+__global__ void __launch_bounds__(128, 4)
+k_res_slice_a(int64_t M, int64_t K, const z_t *__restrict__ A, int64_t lda, int64_t kbase, int64_t T,
+              int64_t nch, const int *__restrict__ E, uint8_t *__restrict__ S) {
+    const int row = threadIdx.x;
+    const int64_t i = (int64_t)blockIdx.y * kRows + row;
+    const int64_t k0 = (int64_t)blockIdx.x * 16;               // within this panel
+    const int64_t kg = kbase + k0;                             // of the whole matrix
+    int sh = 0;
+    bool live = i < M;
+    if (live) {
+        const int e = E[i];
+        live = e != INT_MIN;
+        sh = live ? kAlpha - e : 0;
+    }
+    z_t v[16];
+#pragma unroll
+    for (int e = 0; e < 16; e++) v[e] = (live && kg + e < K) ? A[i + (k0 + e) * lda] : zmk(0.0, 0.0);
+    const int64_t c = kg / kChunk;
+    const int g = (int)(kg % kChunk) / 16;
+    uint8_t *dst = S + ((int64_t)blockIdx.y * nch + c) * kAStage + g * (kRows * 16) + row * 16;
+    const int64_t mstep = T * nch * kAStage;
+#pragma unroll
+    for (int part = 0; part < 2; part++) {
+        unsigned long long x[16];
+#pragma unroll
+        for (int e = 0; e < 16; e++) x[e] = biased_rint(part ? v[e].y : v[e].x, sh);
+        uint8_t *d = dst + part * (4 * kRows * 16);
+#pragma unroll 1
+        for (int m = 0; m < kNMod; m++, d += mstep) {
+            const ResConst rc(kTab.m[m]);
+            uint32_t o[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const uint64_t a = rc.two(x[q * 4], x[q * 4 + 1]), b = rc.two(x[q * 4 + 2], x[q * 4 + 3]);
+                const uint32_t lo = __byte_perm((uint32_t)a, (uint32_t)(a >> 32), 0x0040);
+                const uint32_t hi = __byte_perm((uint32_t)b, (uint32_t)(b >> 32), 0x0040);
+                o[q] = __byte_perm(lo, hi, 0x5410);
+            }
+            *(uint4 *)d = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+    }
+}
+
+// FP16 residues of Y, -> [modulus][chunk][Re, Im, Re + Im][column][64]: one
+// column and 8 consecutive K elements per thread, the moduli from blockIdx.z
+// in steps of gridDim.z.  The column's norm comes from its partial sums; F[j]
+// receives its exponent.
+__global__ void __launch_bounds__(128)
+k_res_slice_b(int64_t N, int64_t Kp, int n, int mp, const z_t *__restrict__ Y, int64_t ldy, int npart,
+              const float2 *__restrict__ part, int *__restrict__ F, uint16_t *__restrict__ B) {
+    const int j = blockIdx.y;
+    const int64_t k = ((int64_t)blockIdx.x * 128 + threadIdx.x) * 8;
+    int h = INT_MIN;
+    if (j < n) {
+        NormAcc a;
+        for (int s = 0; s < npart; s++) a.add(part[(int64_t)j * npart + s]);
+        h = a.exponent();
+    }
+    if (blockIdx.x == 0 && blockIdx.z == 0 && threadIdx.x == 0) F[j] = h;
+    if (k >= Kp) return;
+    const bool live = h != INT_MIN;
+    const int sh = live ? kBeta - h : 0;
+    unsigned long long xr[8], xi[8];
+#pragma unroll
+    for (int e = 0; e < 8; e++) {
+        const z_t y = (live && k + e < N) ? Y[k + e + j * ldy] : zmk(0.0, 0.0);
+        xr[e] = biased_rint(y.x, sh);
+        xi[e] = biased_rint(y.y, sh);
+    }
+    const int64_t nch = Kp / kChunk, c = k / kChunk;
+    const int64_t pstep = (int64_t)mp * kChunk;
+    const __half2 bias = __floats2half2_rn(1152.f, 1152.f);
+#pragma unroll 1
+    for (int m = blockIdx.z; m < kNMod; m += gridDim.z) {
+        const ResConst rc(kTab.m[m]);
+        const int p = (int)kTab.m[m].pf;
+        uint32_t o[3][4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            // bytes residue + 128 of two elements, 16 bits each: Re, Im, Re + Im
+            const uint64_t a = rc.two(xr[q * 2], xr[q * 2 + 1]), b = rc.two(xi[q * 2], xi[q * 2 + 1]);
+            const uint32_t wr = __byte_perm((uint32_t)a, (uint32_t)(a >> 32), 0x0400) & 0x00FF00FFu;
+            const uint32_t wi = __byte_perm((uint32_t)b, (uint32_t)(b >> 32), 0x0400) & 0x00FF00FFu;
+            uint32_t ws = 0;
+#pragma unroll
+            for (int e = 0; e < 2; e++) {
+                // the sum modulo p, in [-128, 127]
+                int s = (int)(wr >> (16 * e) & 255) + (int)(wi >> (16 * e) & 255) - 256;
+                s += s < -128 ? p : 0;
+                s -= s > 127 ? p : 0;
+                ws |= (uint32_t)(s + 128) << (16 * e);
+            }
+            const uint32_t w[3] = {wr, wi, ws};
+#pragma unroll
+            for (int t = 0; t < 3; t++) {
+                const uint32_t x = 0x64006400u | w[t];
+                __half2 hh;
+                memcpy(&hh, &x, 4);
+                hh = __hsub2(hh, bias);
+                memcpy(&o[t][q], &hh, 4);
+            }
+        }
+        uint16_t *d = B + (((int64_t)m * nch + c) * 3) * pstep + (int64_t)j * kChunk + k % kChunk;
+#pragma unroll
+        for (int t = 0; t < 3; t++)
+            *(uint4 *)(d + t * pstep) = make_uint4(o[t][0], o[t][1], o[t][2], o[t][3]);
+    }
+}
+
+// One panel of the synthetic Hamiltonian: all rows, columns j0 .. j0 + cols, as
+// bse_build_hamiltonian writes them (the element of the lower triangle, or its
+// conjugate), column-major with leading dimension N.
+constexpr int kPT = 32;
+__global__ void __launch_bounds__(256)
+k_res_panel(int Nk, int nb, int N, int jbase, int cols, BseModel md, const double *__restrict__ dE,
+            const z_t *__restrict__ u, const z_t *__restrict__ a, const double *__restrict__ Kt,
+            z_t *__restrict__ H) {
+    extern __shared__ z_t gsm[];
+    const int R = md.rank_x;
+    z_t *sai = gsm, *saj = gsm + kPT * R;
+    const int tx = threadIdx.x, ty = threadIdx.y;      // 32 x 8
+    const int i0 = blockIdx.x * kPT, j0 = jbase + blockIdx.y * kPT;
+    for (int e = ty * kPT + tx; e < kPT * R; e += kPT * 8) {
+        const int t = e / R, r = e % R;
+        sai[r * kPT + t] = (i0 + t < N) ? a[(int64_t)(i0 + t) * R + r] : zmk(0.0, 0.0);
+        saj[r * kPT + t] = (j0 + t < N) ? a[(int64_t)(j0 + t) * R + r] : zmk(0.0, 0.0);
+    }
+    __syncthreads();
+    const int I = i0 + tx;
+    if (I >= N) return;
+    for (int c = ty; c < kPT; c += 8) {
+        const int J = j0 + c;
+        if (J >= N || J >= jbase + cols) continue;
+        z_t h;
+        if (I >= J) h = bse_element(I, J, R, sai + tx, saj + c, kPT, u[I], u[J], dE[I], Nk, nb, md.w0, Kt);
+        else h = zconj(bse_element(J, I, R, saj + c, sai + tx, kPT, u[J], u[I], dE[J], Nk, nb, md.w0, Kt));
+        H[I + (int64_t)(J - jbase) * N] = h;
+    }
+}
+
+// ------------------------------------------------------------ the result
+// Element (i, j) from the residues of all moduli and splits, four consecutive
+// rows per thread; then the Chebyshev recurrence.
+__global__ void __launch_bounds__(128)
+k_res_reduce(int64_t M, int64_t Mp, int mp, int nz, const char2 *__restrict__ R, const int *__restrict__ E,
+             const int *__restrict__ F, GemmEpi ep, const z_t *__restrict__ Y, int64_t ldy, z_t *C,
+             int64_t ldc) {
+    const int64_t i = ((int64_t)blockIdx.x * 128 + threadIdx.x) * 4;
+    const int j = blockIdx.y;
+    if (i >= M) return;
+    unsigned long long fr[4] = {}, fi[4] = {};
+    const char2 *r0 = R + (int64_t)j * Mp + i;
+    const int64_t step = (int64_t)mp * Mp;
+#pragma unroll 1
+    for (int z = 0; z < nz; z++, r0 += step) {
+        uint2 q[kNMod];                            // all in flight together
+#pragma unroll
+        for (int m = 0; m < kNMod; m++) q[m] = *(const uint2 *)(r0 + (int64_t)m * nz * step);
+#pragma unroll
+        for (int m = 0; m < kNMod; m++) {
+            const unsigned long long W = kTab.m[m].W;
+            const uint32_t w[2] = {q[m].x, q[m].y};
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                fr[e] += (unsigned long long)(long long)(signed char)(w[e / 2] >> (16 * (e % 2))) * W;
+                fi[e] += (unsigned long long)(long long)(signed char)(w[e / 2] >> (16 * (e % 2) + 8)) * W;
+            }
+        }
+    }
+    const int f = F[j];
+#pragma unroll
+    for (int e = 0; e < 4; e++) {
+        if (i + e >= M) break;
+        const int h = E[i + e];
+        z_t v = zmk(0.0, 0.0);
+        if (h != INT_MIN && f != INT_MIN) {
+            const int x = h + f - (kAlpha + kBeta);
+            const double a = (double)(long long)fr[e] * kScale, b = (double)(long long)fi[e] * kScale;
+            if (x > -1000 && x < 900) {
+                const double s = __longlong_as_double((long long)(1023 + x) << 52);
+                v = zmk(a * s, b * s);
+            } else {
+                v = zmk(ldexp(a, x), ldexp(b, x));
+            }
+        }
+        if (ep.mode == GEMM_CHEB) {
+            v = zscale(zsub(v, zscale(Y[i + e + j * ldy], ep.c)), ep.s1);
+            if (ep.Yp) v = zsub(v, zscale(ep.Yp[i + e + j * ep.ldyp], ep.s2));
+        }
+        C[i + e + j * ldc] = v;
+    }
+}
+
+// 3-D FP16 tensor [tiles][rows][64], box 64 x box_rows, 128-byte swizzle
+bool make_map(CUtensorMap *m, void *base, uint64_t rows, uint64_t tiles, uint32_t box_rows) {
+    const TensorMapEncode enc = tensor_map_encode();
+    if (!enc) return false;
+    cuuint64_t dims[3] = {64, rows, tiles};
+    cuuint64_t strides[2] = {64 * 2, rows * 64 * 2};
+    cuuint32_t box[3] = {64, box_rows, 1};
+    cuuint32_t es[3] = {1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, base, dims, strides, box, es,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// Column tiles of an n-column product: as few as hold n, of equal width
+void column_tiles(int n, int *tx, int *w) {
+    *tx = (n + kMaxW - 1) / kMaxW;
+    *w = ((n + *tx - 1) / *tx + 15) / 16 * 16;
+}
+
+// Chunks per K split.  Modelled time, in cycles, of the busiest SM: a chunk
+// takes 6 w cycles of MMA, at least about 700 (its share of HBM) or 260 (its
+// conversion) when the matrix is in L2; a unit costs about 2000 more (its first
+// copies and its last drain) and each split about 52 bytes per output.
+int choose_chunks(int64_t Mp, int nch, int mp, int tx, int w, size_t r_bytes, int sms) {
+    const double mat = 26.0 * Mp * nch * kChunk;
+    const double per_chunk = std::max(6.0 * w, mat > 1.0e8 ? 700.0 : 300.0);
+    const int64_t tiles = Mp / kRows * tx * kNMod;
+    int best = 0;
+    double best_t = 1e300;
+    for (int cs = 1; cs <= kMaxUnitChunks; cs = cs < 8 ? cs * 2 : cs + 8) {
+        const int nz = (nch + cs - 1) / cs;
+        if ((size_t)kNMod * nz * mp * Mp * sizeof(char2) > r_bytes) continue;
+        const int64_t per = (tiles * nz + sms - 1) / sms;
+        const double t = (double)per * (std::min(cs, nch) * per_chunk + 2000.0) +
+                         52.0 * nz * mp * Mp / (5e12 / 1.9e9);
+        if (t < best_t) {
+            best_t = t;
+            best = cs;
+        }
+    }
+    return best;
+}
+
+int norm_segment(int64_t N) { return N < 4096 ? 32 : 256; }
+
+}  // namespace
+
+size_t residue_a_bytes(int64_t M, int64_t K) {
+    const int64_t Mp = (M + kRows - 1) / kRows * kRows, Kp = (K + kChunk - 1) / kChunk * kChunk;
+    return (size_t)kNMod * 2 * Mp * Kp;
+}
+
+size_t residue_b_bytes(int64_t K, int n) {
+    const int64_t Kp = (K + kChunk - 1) / kChunk * kChunk;
+    return (size_t)kNMod * 3 * Kp * (n + 64) * 2;
+}
+
+size_t residue_r_bytes(int64_t M, int64_t K, int n) {
+    const int64_t Mp = (M + kRows - 1) / kRows * kRows, nch = (K + kChunk - 1) / kChunk;
+    // splits: as many as the longest units need, and some more to fill the SMs
+    const int64_t nz = std::max<int64_t>((nch + kMaxUnitChunks - 1) / kMaxUnitChunks, std::min<int64_t>(nch, nch < 128 ? 8 : 3));
+    return (size_t)kNMod * nz * (n + 64) * Mp * sizeof(char2);
+}
+
+size_t residue_work_bytes(int64_t N) {
+    const int64_t s = norm_segment(N);
+    return (size_t)((N + s - 1) / s) * N * sizeof(float2);
+}
+
+size_t residue_panel_bytes(int64_t N) { return (size_t)N * 256 * sizeof(z_t); }
+
+cudaError_t residue_prepare(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh, void *work, ChaseScalars *sc,
+                            cudaStream_t st) {
+    const int64_t Np = ozaki_padded(N), T = Np / kRows, nch = (N + kChunk - 1) / kChunk;
+    oh->N = N;
+    oh->Np = Np;
+    oh->tri = false;
+    const int seg = norm_segment(N), nseg = (int)((N + seg - 1) / seg);
+    const unsigned rb = (unsigned)((N + 127) / 128);
+    k_res_rownorm<<<dim3(rb, (unsigned)nseg), 128, 0, st>>>(N, N, H, ldh, seg, 0, (float2 *)work);
+    k_res_rowscale<<<(unsigned)T, 128, 0, st>>>(N, Np, nseg, (const float2 *)work, oh->E, sc);
+    k_res_slice_a<<<dim3((unsigned)(nch * 4), (unsigned)T), 128, 0, st>>>(N, N, H, ldh, 0, T, nch, oh->E,
+                                                                         (uint8_t *)oh->A);
+    bse_count_launches(3);
+    return cudaGetLastError();
+}
+
+cudaError_t residue_prepare_bse(int Nk, int Nv, int Nc, const BseModel &md, const double *dE, const z_t *u,
+                                const z_t *a, const double *Kt, OzakiH *oh, void *work, void *panel,
+                                ChaseScalars *sc, cudaStream_t st) {
+    const int64_t N = (int64_t)Nk * Nv * Nc, Np = ozaki_padded(N), T = Np / kRows, nch = (N + kChunk - 1) / kChunk;
+    oh->N = N;
+    oh->Np = Np;
+    oh->tri = false;
+    const int dyn = 2 * kPT * std::max(md.rank_x, 1) * (int)sizeof(z_t);
+    static std::once_flag once[kMaxDevices];
+    static cudaError_t attr[kMaxDevices];
+    const cudaError_t ae = smem_attr_once(once, attr, (const void *)k_res_panel, 2 * kPT * 64 * (int)sizeof(z_t));
+    if (ae != cudaSuccess) return ae;
+    const int seg = norm_segment(N), nseg = (int)((N + seg - 1) / seg);
+    const unsigned rb = (unsigned)((N + 127) / 128);
+    z_t *Hp = (z_t *)panel;
+    for (int pass = 0; pass < 2; pass++) {
+        for (int64_t j0 = 0; j0 < N; j0 += 256) {
+            const int cols = (int)std::min<int64_t>(256, N - j0);
+            k_res_panel<<<dim3((unsigned)((N + kPT - 1) / kPT), (unsigned)((cols + kPT - 1) / kPT)),
+                          dim3(kPT, 8), dyn, st>>>(Nk, Nv * Nc, (int)N, (int)j0, cols, md, dE, u, a, Kt, Hp);
+            if (pass == 0)
+                k_res_rownorm<<<dim3(rb, (unsigned)((cols + seg - 1) / seg)), 128, 0, st>>>(
+                    N, cols, Hp, N, seg, j0 / seg, (float2 *)work);
+            else
+                k_res_slice_a<<<dim3((unsigned)((cols + kChunk - 1) / kChunk * 4), (unsigned)T), 128, 0, st>>>(
+                    N, N, Hp, N, j0, T, nch, oh->E, (uint8_t *)oh->A);
+            bse_count_launches(2);
+        }
+        if (pass == 0) {
+            k_res_rowscale<<<(unsigned)T, 128, 0, st>>>(N, Np, nseg, (const float2 *)work, oh->E, sc);
+            bse_count_launches(1);
+        }
+    }
+    return cudaGetLastError();
+}
+
+double residue_flops(int64_t M, int64_t K, int n) { return 6.0 * kNMod * (double)M * (double)K * n; }
+
+namespace {
+template <class Cfg>
+cudaError_t launch_cfg(const RsBatch &b, int sms, cudaStream_t st) {
+    static std::once_flag once[kMaxDevices];
+    static cudaError_t attr[kMaxDevices];
+    const cudaError_t ae = smem_attr_once(once, attr, (const void *)k_res_zgemm<Cfg>, Cfg::kSmem);
+    if (ae != cudaSuccess) return ae;
+    k_res_zgemm<Cfg><<<(unsigned)std::min(b.units, sms), Cfg::kThreads, Cfg::kSmem, st>>>(b);
+    bse_count_launches(1);
+    return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t residue_launch(RsBatch &b, int sms, cudaStream_t st) {
+    b.stride = 16;
+    for (int j = 0; j < b.njobs; j++) b.stride = std::max(b.stride, b.job[j].w);
+    b.slots = std::min((kTmemCols - 3 * b.stride) / 16, kMaxSlots);
+    if (b.stride <= RsNarrow::kW) return launch_cfg<RsNarrow>(b, sms, st);
+    if (b.stride <= RsMid::kW) return launch_cfg<RsMid>(b, sms, st);
+    return launch_cfg<RsWide>(b, sms, st);
+}
+
+cudaError_t residue_zgemm(const OzakiH &oh, int n, const z_t *Y, int64_t ldy, z_t *C, int64_t ldc,
+                          const GemmEpi &ep, void *B, size_t b_bytes, int *F, float2 *part, void *R,
+                          size_t r_bytes, ChaseScalars *sc, int sms, cudaStream_t st, cudaEvent_t ev0,
+                          cudaEvent_t ev1, OzBatcher *batcher) {
+    if (n <= 0) return cudaSuccess;
+    const int64_t N = oh.N, nch = (N + kChunk - 1) / kChunk, Kp = nch * kChunk;
+    int tx, w;
+    column_tiles(n, &tx, &w);
+    const int mp = tx * w;
+    if ((size_t)kNMod * 3 * Kp * mp * 2 > b_bytes) return cudaErrorInvalidValue;
+    const int npart = (int)std::min<int64_t>((N + 1023) / 1024, 32);
+    k_res_colnorm<<<dim3((unsigned)npart, (unsigned)n), 256, 0, st>>>(N, Y, ldy, part, sc);
+    const unsigned bx = (unsigned)((Kp + 1023) / 1024);
+    // split the moduli over blocks while that leaves SMs idle otherwise
+    const unsigned bz = (unsigned)std::max<int64_t>(1, std::min<int64_t>(kNMod, 4 * sms / ((int64_t)bx * mp)));
+    k_res_slice_b<<<dim3(bx, (unsigned)mp, bz), 128, 0, st>>>(N, Kp, n, mp, Y, ldy, npart, part, F, (uint16_t *)B);
+    bse_count_launches(2);
+    RsBatch b;
+    memset(&b, 0, sizeof b);
+    RsJob &j = b.job[0];
+    if (!make_map(&j.tmB, B, (uint64_t)mp, (uint64_t)(kNMod * 3 * nch), (uint32_t)w)) return cudaErrorInvalidValue;
+    j.A = (const uint8_t *)oh.A;
+    j.R = (char2 *)R;
+    j.sc = sc;
+    j.wait_ns = oh.wait_ns;
+    j.Mp = oh.Np;
+    j.w = w;
+    j.mp = mp;
+    j.nch = (int)nch;
+    j.cs = choose_chunks(oh.Np, j.nch, mp, tx, w, r_bytes, sms);
+    if (j.cs < 1) return cudaErrorInvalidValue;
+    j.tx = tx;
+    j.ty = (int)(oh.Np / kRows);
+    j.tz = (j.nch + j.cs - 1) / j.cs;
+    j.nmod = kNMod;
+    b.njobs = 1;
+    b.units = rs_units(j);
+    cudaError_t e;
+    if (batcher) {
+        e = ozb_run_residue(batcher, j, st);
+    } else {
+        if (ev0) cudaEventRecord(ev0, st);
+        e = residue_launch(b, sms, st);
+        if (ev1) cudaEventRecord(ev1, st);
+    }
+    if (e != cudaSuccess) return e;
+    k_res_reduce<<<dim3((unsigned)((N + 511) / 512), (unsigned)n), 128, 0, st>>>(
+        N, oh.Np, mp, j.tz, j.R, oh.E, F, ep, Y, ldy, C, ldc);
+    bse_count_launches(1);
+    return cudaGetLastError();
+}

@@ -47,6 +47,7 @@ struct Req {
     chase_request rq{};
     int64_t N = 0;
     size_t run_bytes = 0;      // admission estimate while running
+    bool residues = false;     // products with H in residues (they fit the budget)
     size_t keep_bytes = 0;     // eigenvectors kept after the solve
     int state = 0;             // 0 queued, 1 running, 2 done
     int status = BSE_EBUSY;
@@ -80,14 +81,17 @@ struct BseServer {
 
 namespace {
 
-size_t estimate_run_bytes(int64_t N, int m, int nev, int precision, bool own_h, bool half) {
+size_t estimate_run_bytes(int64_t N, int m, int nev, int precision, bool own_h, bool half, bool res) {
     const size_t Np = (size_t)ozaki_padded(N);
     const size_t mp = (size_t)((std::max(m, 32) + 31) / 32 * 32);
     size_t b = own_h ? 16 * (size_t)N * N : 0;              // H, unless the caller's
     b += 4 * 16 * (size_t)N * m;                            // V and three scratch blocks
     b += 16 * (size_t)N * nev;                              // eigenvectors
     b += (size_t)N * 8 * 3 * 16 + ((size_t)20 << 20);       // Lanczos blocks, small matrices
-    if (precision != CHASE_FP64_DFMA) {
+    if (precision != CHASE_FP64_DFMA && res) {
+        const HopBytes hb = hop_bytes(N, std::max(m, 32), true, false, !own_h);
+        b += hb.A + hb.B + hb.P + hb.GA;                    // residues of H and of the operand,
+    } else if (precision != CHASE_FP64_DFMA) {              // partial results
         b += half ? ozaki_a_bytes_tri(N) + 16 * Np          // slices of H (half storage:
                   : 24 * Np * Np;                           // the lower triangle, scales)
         b += 36 * mp * Np;                                  // slices of the operand
@@ -194,6 +198,7 @@ void worker(BseServer *S, int slot) {
         }
         std::vector<double> ev(rq.nev), rs(rq.nev);
         chase_stats st{};
+        ctx->residues = job->residues;
         if (rc == BSE_OK)
             rc = solve_device(ctx, rq.h_free ? nullptr : Hs, N, rq.h_free ? N : lds, rq.nev,
                               rq.nex, rq.tol, rq.deg_max, rq.precision, &o, ev.data(), (z_t *)dZ,
@@ -310,8 +315,12 @@ int chase_server_submit(bsechase_ctx *ctx, const chase_request *req, uint64_t *t
     q->rq.precision = precision_mode(req->precision);
     q->N = N;
     if (req->d_H && req->ldh < N) return fail(ctx, BSE_EINVAL, "request H: ldh < N%s");
-    q->run_bytes = estimate_run_bytes(N, m, req->nev, q->rq.precision,
-                                      req->d_H == nullptr && !req->h_free, req->half_storage == 1);
+    // residue products where they fit the budget, else the slices (2 N^2 bytes less)
+    for (q->residues = precision_uses_residues(q->rq.precision, req->half_storage == 1);; q->residues = false) {
+        q->run_bytes = estimate_run_bytes(N, m, req->nev, q->rq.precision, req->d_H == nullptr && !req->h_free,
+                                          req->half_storage == 1, q->residues);
+        if (!q->residues || q->run_bytes <= S->budget) break;
+    }
     if (q->run_bytes > S->budget)
         return fail(ctx, BSE_ENOMEM, "request needs more than the whole HBM budget%s");
     q->t_submit = now_s();
