@@ -12,7 +12,7 @@
 struct RsJob {
     CUtensorMap tmB;       // operand residues, box 64 x w
     const uint8_t *A;      // residues of A: [modulus][row tile][chunk][16 KB]
-    char2 *R;              // residues of C: [modulus][split][column < mp][row < Mp]
+    uchar2 *R;             // residues of C + 128: [modulus][split][column < mp][row < Mp]
     ChaseScalars *sc;
     uint64_t wait_ns;      // limit of each bounded mbarrier wait
     int64_t Mp;            // rows, padded to whole row tiles

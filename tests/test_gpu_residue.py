@@ -68,6 +68,15 @@ def test_rows_and_chunks(ctx, N):
     _check(A, Y, _hemm(ctx, A, Y))
 
 
+@pytest.mark.parametrize("N,n", [(4095, 97), (4095, 98), (4096, 97), (4096, 98), (4097, 98), (6001, 1)])
+def test_rules_on_sizes(ctx, N, n):
+    """Both sides of the lines between one row of the result per thread and four
+    (N n = 400000), of column norms of their own (N = 4096), of row exponents in
+    one launch (N = 4096)."""
+    A, Y = _hermitian(N, 11), _block(N, n, 12)
+    _check(A, Y, _hemm(ctx, A, Y))
+
+
 def test_longest_unit(ctx):
     """More K chunks than one unit sums (224): K splits."""
     A, Y = _hermitian(14400, 5), _block(14400, 40, 6)
