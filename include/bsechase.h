@@ -190,7 +190,7 @@ const char *bsechase_last_error(const bsechase_ctx *ctx);
 
 /* Time limit, in seconds (0 < seconds <= 60, default 2), of every bounded
  * wait inside the context's tensor-core kernels (a wait for a copy, an MMA or
- * a drained accumulator).  When a wait runs out, the kernel stops issuing
+ * a drained accumulator; chase_qr and chase_gram keep the default).  When a wait runs out, the kernel stops issuing
  * work, waits for the copies and MMAs it already issued, releases its tensor
  * memory and returns; the call then fails with BSE_ETIMEOUT and the context
  * stays usable.  A short limit makes that path run on purpose (failure
@@ -288,7 +288,8 @@ int chase_filter(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t ldh, voi
 /* QR phase (Supplement, "QR" item): d_V (N x m) becomes an orthonormal
  * basis of span(d_V) projected off span(d_L) (d_L: N x k orthonormal, may
  * be NULL with k = 0): two projections, column scaling, shifted Cholesky QR
- * and two Cholesky QR passes each after a projection. */
+ * and two Cholesky QR passes each after a projection.  Its products run as
+ * chase_gram's do. */
 int chase_qr(bsechase_ctx *ctx, const void *d_L, int64_t ldl, int k, void *d_V, int64_t ldv,
              int64_t N, int m);
 
@@ -301,9 +302,12 @@ int chase_rayleigh_ritz(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t l
 
 /* Gram product of the QR and Rayleigh-Ritz phases (Supplement, "QR" and
  * "RR" items): d_G (m1 x m2, ldg >= m1) = A^H B for A: K x m1 (lda), B: K x m2
- * (ldb), 1 <= m1, m2 <= 512.  Split over K with a fixed partition and a
- * fixed-order sum (run-to-run deterministic); partial sums live in the
- * context's workspace. */
+ * (ldb), 1 <= m1, m2 <= 512.  Run-to-run deterministic.  For K >= 64 in
+ * residue arithmetic on the tensor cores (operands of 58 bits against each
+ * column's 2-norm, exact sums, one rounding; its workspace, up to 30 bytes per
+ * element of the wider block and 90 of the other, stays in the context), in
+ * native FP64 below, where that workspace cannot be had, and for non-finite
+ * operands, whose product is what IEEE arithmetic makes of them. */
 int chase_gram(bsechase_ctx *ctx, const void *d_A, int64_t lda, const void *d_B, int64_t ldb,
                int64_t K, int m1, int m2, void *d_G, int64_t ldg);
 
@@ -311,7 +315,7 @@ int chase_gram(bsechase_ctx *ctx, const void *d_A, int64_t lda, const void *d_B,
  * memory (their memory manager owns the device, they cannot afford the
  * allocator's synchronisation, or they cannot create a context, which
  * allocates workspace).  The paper has no counterpart: it is a service entry
- * point.  Same result as chase_gram (G = A^H B, m1 x m2, ldg >= m1, for A: K x
+ * point.  The result of chase_gram to FP64 rounding (native FP64; G = A^H B, m1 x m2, ldg >= m1, for A: K x
  * m1, B: K x m2) computed on the current device and on `cuda_stream` (NULL =
  * the default stream); the call returns once the work is enqueued.  The
  * split-K partial sums live in a fixed 4 MiB device array inside the library

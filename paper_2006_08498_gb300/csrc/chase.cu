@@ -229,23 +229,31 @@ int hop_buffers(bsechase_ctx *ctx, const Hop &op, int mc) {
     return ensure(ctx, ctx->ozGE, (size_t)(Np + 512) * sizeof(int));
 }
 
+void free_product_buffers(bsechase_ctx *ctx) {
+    DevBuf *bufs[] = {&ctx->ozA, &ctx->ozB, &ctx->ozP, &ctx->ozGA};
+    for (DevBuf *d : bufs) {
+        if (d->p) cudaFreeAsync(d->p, ctx->st);
+        d->p = nullptr;
+        d->bytes = 0;
+    }
+    ctx->err.clear();
+}
+
 int hop_prepare(bsechase_ctx *ctx, Hop &op, int max_cols) {
     if (!op.tc) return BSE_OK;
     int rc;
     const int64_t Np = ozaki_padded(op.N);
     const int mc = std::max(max_cols, 32);
     rc = hop_buffers(ctx, op, mc);
+    if (rc == BSE_ENOMEM) {
+        free_product_buffers(ctx);     // what other calls left in them
+        rc = hop_buffers(ctx, op, mc);
+    }
     if (rc == BSE_ENOMEM && op.res) {
         // the residues take 2 N^2 bytes more than the slices: those, where only
         // they fit
         op.res = false;
-        DevBuf *bufs[] = {&ctx->ozA, &ctx->ozB, &ctx->ozP, &ctx->ozGA};
-        for (DevBuf *d : bufs) {
-            if (d->p) cudaFreeAsync(d->p, ctx->st);
-            d->p = nullptr;
-            d->bytes = 0;
-        }
-        ctx->err.clear();
+        free_product_buffers(ctx);
         rc = hop_buffers(ctx, op, mc);
     }
     if (rc) return rc;
@@ -405,8 +413,7 @@ int phase_filter(bsechase_ctx *ctx, const Hop &op, z_t *V, int64_t ldv, int m, c
     return BSE_OK;
 }
 
-// V -= L (L^H V)
-// The N x m products of QR and Rayleigh-Ritz: on the tensor cores with
+// The N x m products of a solve's QR and Rayleigh-Ritz: on the tensor cores with
 // FP64-level accuracy when the solve's products with H are (ctx->gen_tc),
 // else native FP64.  The operands here are orthonormal or unit-norm
 // columns, so the per-row/per-column scaling of the slices keeps the error
@@ -489,6 +496,94 @@ int cholqr_pass(bsechase_ctx *ctx, z_t *V, int64_t ldv, int64_t N, int m, double
     return BSE_OK;
 }
 
+// The general products in residues (residue.cu): their buffers, shared with the
+// products with H, for left operands of at most m columns of N, a kept block of
+// k columns in both roles, and right operands of m columns.
+struct ResBufs {
+    RsSide VA, VB, LA, LB;
+    void *R;
+    size_t r_bytes;
+};
+int residue_buffers(bsechase_ctx *ctx, int64_t N, int m, int k, bool tall, ResBufs *b) {
+    auto up = [](size_t x) { return (x + 1023) / 1024 * 1024; };
+    const int64_t Np = ozaki_padded(N), mk = std::max(m, k);
+    const size_t va = up(std::max(residue_left_bytes(m, N), tall ? residue_left_bytes(N, m) : 0));
+    const size_t la = k > 0 && tall ? residue_left_bytes(N, k) : 0;
+    const size_t vb = up(residue_right_bytes(N, tall ? m : k)), lb = k > 0 && tall ? residue_right_bytes(N, k) : 0;
+    size_t r = residue_out_bytes(m, N, (int)mk);
+    if (tall) r = std::max(r, residue_out_bytes(N, mk, m));
+    const size_t ne = (size_t)(Np + 512), parts = (size_t)kMaxM * kRsColParts;
+    int rc;
+    if ((rc = ensure(ctx, ctx->ozGA, va + la)) || (rc = ensure(ctx, ctx->ozB, vb + lb)) ||
+        (rc = ensure(ctx, ctx->ozP, r)) || (rc = ensure(ctx, ctx->ozGE, 2 * ne * sizeof(int))) ||
+        (rc = ensure(ctx, ctx->ozF, 2 * parts * sizeof(float2) + 2 * kMaxM * sizeof(int))))
+        return rc;
+    float2 *part = (float2 *)ctx->ozF.p;
+    int *f = (int *)(part + 2 * parts), *e = (int *)ctx->ozGE.p;
+    b->VA = RsSide{ctx->ozGA.p, va, e, part};
+    b->LA = RsSide{(char *)ctx->ozGA.p + va, la, e + ne, nullptr};
+    b->VB = RsSide{ctx->ozB.p, vb, f, part + parts};
+    b->LB = RsSide{(char *)ctx->ozB.p + vb, lb, f + kMaxM, part + parts};
+    b->R = ctx->ozP.p;
+    b->r_bytes = ctx->ozP.bytes;
+    return BSE_OK;
+}
+
+// phase_qr in residues.  L is turned into residues once for the four
+// projections, in both its roles; a projection multiplies V^H L (the wide block
+// on the left, a byte a residue) and stores its adjoint; the results go to V
+// itself.
+int phase_qr_residues(bsechase_ctx *ctx, const ResBufs &b, const z_t *L, int64_t ldl, int k, z_t *V, int64_t ldv,
+                      int64_t N, int m) {
+    cudaStream_t st = ctx->st;
+    const int sms = ctx->sms;
+    ChaseScalars *sc = ctx->sc;
+    z_t *X = (z_t *)ctx->R.p, *G = (z_t *)ctx->G.p, *Ri = (z_t *)ctx->Ri.p;
+    auto product = [&](int64_t M, int n, int64_t K, const RsSide &A, const RsSide &B, const RsOut &o) {
+        return residue_product(M, n, K, A, B, o, b.R, b.r_bytes, kDefaultWaitNs, sc, sms, st);
+    };
+    auto proj = [&]() -> int {
+        if (k <= 0) return BSE_OK;
+        RsOut x{X, k}, v{V, ldv, V, ldv};
+        x.adjoint = 1;
+        CK(residue_left(m, N, V, ldv, true, b.VA, sc, st));
+        CK(product(m, k, N, b.VA, b.LB, x));
+        CK(residue_right(k, m, X, k, nullptr, b.VB, sc, sms, st));
+        CK(product(N, m, k, b.LA, b.VB, v));
+        return BSE_OK;
+    };
+    auto cholqr = [&](double shift) -> int {
+        RsOut g{G, m}, v{V, ldv};
+        g.shift = shift;
+        g.mirror = 1;
+        CK(residue_left(m, N, V, ldv, true, b.VA, sc, st));
+        CK(residue_right(N, m, V, ldv, b.VA.part, b.VB, sc, sms, st));
+        CK(product(m, m, N, b.VA, b.VB, g));
+        CK(launch_cholesky(m, G, m, sc, st));
+        CK(launch_trinv(m, G, m, Ri, m, st));
+        CK(residue_left(N, m, V, ldv, false, b.VA, sc, st));
+        CK(residue_right(m, m, Ri, m, nullptr, b.VB, sc, sms, st));
+        CK(product(N, m, m, b.VA, b.VB, v));
+        return BSE_OK;
+    };
+    int rc;
+    Small s = small_layout(ctx, m);
+    if (k > 0) {
+        CK(residue_right(N, k, L, ldl, nullptr, b.LB, sc, sms, st));
+        CK(residue_left(N, k, L, ldl, false, b.LA, sc, st));
+    }
+    if ((rc = proj())) return rc;
+    if ((rc = proj())) return rc;
+    CK(launch_normalize_cols(N, m, V, ldv, (double *)ctx->part.p, s.norms, sc, st));
+    // columns have unit norm, so ||V||_F^2 = m
+    if ((rc = cholqr(11.0 * ((double)N * m + (double)m * (m + 1)) * kU * (double)m))) return rc;
+    for (int pass = 0; pass < 2; pass++) {
+        if ((rc = proj())) return rc;
+        if ((rc = cholqr(0.0))) return rc;
+    }
+    return BSE_OK;
+}
+
 int phase_qr(bsechase_ctx *ctx, const z_t *L, int64_t ldl, int k, z_t *V, int64_t ldv, int64_t N,
              int m) {
     int rc;
@@ -505,6 +600,36 @@ int phase_qr(bsechase_ctx *ctx, const z_t *L, int64_t ldl, int k, z_t *V, int64_
         if ((rc = cholqr_pass(ctx, V, ldv, N, m, 0.0))) return rc;
     }
     return BSE_OK;
+}
+
+// Sums over K = N of a chunk or more go in residues, whatever the widths.  us,
+// native FP64 against residues: Gram K = 7 (3 x 2) 70, 73; K = 64 (1 x 1) 104,
+// 74; K = 2000 (40 x 20) 309, 87; K = 20000 (140 x 40) 1816, 214; QR N = 7 (3
+// after 2) 467, 503; N = 64 (1) 340, 285; N = 2000 (40 after 20) 3247, 1049;
+// N = 20000 (100 after 40) 21832, 3714.  Below one chunk every split of the FP64
+// kernel is short, and the residues' padding and launches cost more.
+bool sums_in_residues(int64_t K) { return K >= 64; }
+
+// G = A^H B in residues, the wider block on the left; synchronises.
+int gram_residues(bsechase_ctx *ctx, const z_t *A, int64_t lda, const z_t *B, int64_t ldb, int64_t K, int m1, int m2,
+                  z_t *G, int64_t ldg) {
+    const bool same = A == B && lda == ldb && m1 == m2;
+    RsOut o{G, ldg};
+    o.mirror = same ? 1 : 0;
+    if (m2 > m1) {
+        std::swap(A, B);
+        std::swap(lda, ldb);
+        std::swap(m1, m2);
+        o.adjoint = 1;
+    }
+    ResBufs b;
+    int rc;
+    if ((rc = residue_buffers(ctx, K, m1, m2, false, &b))) return rc;
+    CK(cudaMemsetAsync(ctx->sc, 0, sizeof(ChaseScalars), ctx->st));
+    CK(residue_left(m1, K, A, lda, true, b.VA, ctx->sc, ctx->st));
+    CK(residue_right(K, m2, B, ldb, same ? b.VA.part : nullptr, b.VB, ctx->sc, ctx->sms, ctx->st));
+    CK(residue_product(m1, m2, K, b.VA, b.VB, o, b.R, b.r_bytes, kDefaultWaitNs, ctx->sc, ctx->sms, ctx->st));
+    return sync_scalars(ctx);
 }
 
 // Rayleigh-Ritz: theta (device), Vout = Q Y (ld N), HVout = H Q Y (ld N)
@@ -1109,7 +1234,16 @@ int chase_qr(bsechase_ctx *ctx, const void *d_L, int64_t ldl, int k, void *d_V, 
     int rc;
     if ((rc = ensure_workspace(ctx, N, k + m))) return rc;
     CK(cudaMemsetAsync(ctx->sc, 0, sizeof(ChaseScalars), ctx->st));
-    if ((rc = phase_qr(ctx, (const z_t *)d_L, ldl, k, (z_t *)d_V, ldv, N, m))) return rc;
+    bool res = sums_in_residues(N);
+    ResBufs b;
+    if (res && (rc = residue_buffers(ctx, N, m, k, true, &b))) {
+        if (rc != BSE_ENOMEM) return rc;
+        free_product_buffers(ctx);      // native FP64 needs no more workspace
+        res = false;
+    }
+    if (res) rc = phase_qr_residues(ctx, b, (const z_t *)d_L, ldl, k, (z_t *)d_V, ldv, N, m);
+    else rc = phase_qr(ctx, (const z_t *)d_L, ldl, k, (z_t *)d_V, ldv, N, m);
+    if (rc) return rc;
     return sync_scalars(ctx);
 }
 
@@ -1156,6 +1290,14 @@ int chase_gram(bsechase_ctx *ctx, const void *d_A, int64_t lda, const void *d_B,
         return fail(ctx, BSE_EINVAL, "bad Gram arguments%s");
     DeviceGuard g(ctx->device);
     int rc;
+    if (sums_in_residues(K)) {
+        rc = gram_residues(ctx, (const z_t *)d_A, lda, (const z_t *)d_B, ldb, K, m1, m2, (z_t *)d_G, ldg);
+        if (rc == BSE_OK) return rc;
+        // no memory for the residues, or non-finite operands, whose product is
+        // what IEEE arithmetic makes of them: native FP64
+        if (rc == BSE_ENOMEM) free_product_buffers(ctx);
+        ctx->err.clear();
+    }
     if ((rc = ensure(ctx, ctx->part, (size_t)kCnWork * sizeof(z_t)))) return rc;
     CK(launch_zgemm_cn(m1, m2, K, (const z_t *)d_A, lda, (const z_t *)d_B, ldb, (z_t *)d_G, ldg,
                        0.0, 0, (z_t *)ctx->part.p, kCnWork, ctx->st));

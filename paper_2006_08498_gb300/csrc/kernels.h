@@ -169,6 +169,40 @@ cudaError_t residue_zgemm(const OzakiH &oh, int n, const z_t *Y, int64_t ldy, z_
                           const GemmEpi &ep, void *B, size_t b_bytes, int *F, float2 *part, void *R,
                           size_t r_bytes, ChaseScalars *sc, int sms, cudaStream_t st, cudaEvent_t ev0,
                           cudaEvent_t ev1, OzBatcher *batcher);
+// General products C = out(op(A) B), op(A) M x K, B K x n, at native FP64's
+// accuracy or better (operands of 58 bits against each line's 2-norm): the left
+// operand's rows (A, K <= 512, or A^H with ah and A K x M) and the right
+// operand's columns are turned into residues once and multiplied as often as
+// wanted.  A side's buffers: p of residue_left_bytes or residue_right_bytes, e
+// M (to whole 128s) or n exponents, part kRsColParts pairs a column.  norms: the right
+// operand's column norms where residue_left (ah) has left them already.
+constexpr int kRsColParts = 32;
+struct RsSide {
+    void *p = nullptr;
+    size_t bytes = 0;
+    int *e = nullptr;
+    float2 *part = nullptr;
+};
+// S = op(A) B goes to C as D - S (D may be C) or as its conjugate transpose; with
+// mirror (S = A^H A) its upper triangle gives both halves and the diagonal is
+// real.  shift is added to the diagonal.
+struct RsOut {
+    z_t *C;
+    int64_t ldc;
+    const z_t *D = nullptr;
+    int64_t ldd = 0;
+    double shift = 0.0;
+    int mirror = 0, adjoint = 0;
+};
+size_t residue_left_bytes(int64_t M, int64_t K);
+size_t residue_right_bytes(int64_t K, int n);
+size_t residue_out_bytes(int64_t M, int64_t K, int n);   // the splits' residues
+cudaError_t residue_left(int64_t M, int64_t K, const z_t *A, int64_t lda, bool ah, const RsSide &s, ChaseScalars *sc,
+                         cudaStream_t st);
+cudaError_t residue_right(int64_t K, int n, const z_t *B, int64_t ldb, const float2 *norms, const RsSide &s,
+                          ChaseScalars *sc, int sms, cudaStream_t st);
+cudaError_t residue_product(int64_t M, int n, int64_t K, const RsSide &A, const RsSide &B, const RsOut &out, void *R,
+                            size_t r_bytes, uint64_t wait_ns, ChaseScalars *sc, int sms, cudaStream_t st);
 // Product batcher shared by the solver threads of a request server: products
 // submitted within window_s of each other (or as soon as every active solver
 // has submitted one) run in one launch of the tensor-core kernel.

@@ -41,25 +41,28 @@
 namespace {
 
 // ------------------------------------------------------------ the moduli
-constexpr int kNMod = 13;
-constexpr int kAlpha = 51, kBeta = 50;
-constexpr int kMod[kNMod] = {256, 253, 251, 249, 247, 241, 239, 233, 229, 227, 223, 217, 211};
+// The product with H takes the first kNMod; the general products (kGMod below),
+// which stand in for native FP64, two more and operands of kGBits bits.
+constexpr int kNMod = 13, kGMod = 15;
+constexpr int kAlpha = 51, kBeta = 50, kGBits = 58;
+constexpr int kMod[kGMod] = {256, 253, 251, 249, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197};
 
 constexpr int gcd_of(int a, int b) { return b == 0 ? a : gcd_of(b, a % b); }
 constexpr bool coprime() {
-    for (int i = 0; i < kNMod; i++)
+    for (int i = 0; i < kGMod; i++)
         for (int j = 0; j < i; j++)
             if (gcd_of(kMod[i], kMod[j]) != 1) return false;
     return true;
 }
 static_assert(coprime(), "pairwise coprime moduli");
-constexpr unsigned __int128 modulus_product() {
+constexpr unsigned __int128 modulus_product(int n) {
     unsigned __int128 P = 1;
-    for (int i = 0; i < kNMod; i++) P *= (unsigned)kMod[i];
+    for (int i = 0; i < n; i++) P *= (unsigned)kMod[i];
     return P;
 }
 // 2^(kAlpha + kBeta) plus 20 % (norm estimates and the operands' rounding) below P / 2
-static_assert(modulus_product() / 2 > ((unsigned __int128)6 << (kAlpha + kBeta)) / 5, "range of the product");
+static_assert(modulus_product(kNMod) / 2 > ((unsigned __int128)6 << (kAlpha + kBeta)) / 5 &&
+                  modulus_product(kGMod) / 2 > ((unsigned __int128)6 << (2 * kGBits)) / 5, "range of the product");
 
 // Constants of one modulus.  A residue of the 64-bit integer X + 2^63 (bytes
 // b_0..b_7): v = sum_i b_i (256^i mod p) + k0 - 12582912 by two 4-byte dot
@@ -74,15 +77,26 @@ static_assert(modulus_product() / 2 > ((unsigned __int128)6 << (kAlpha + kBeta))
 struct ModConst {
     uint32_t clo, chi, k0;
     float pf, inv;
-    uint32_t w0, w1;        // W = round(2^64 ((P/p)^-1 mod p) / p), low and high word
+    uint32_t w[2], g[3];    // W = round(2^64 ((P/p)^-1 mod p) / p), low word first; of all kGMod with 2^96
 };
 struct ModTable {
-    ModConst m[kNMod];
-    unsigned long long bias;   // 128 sum_m W_m
+    ModConst m[kGMod];
+    unsigned long long bias;           // 128 sum_m W_m
+    unsigned long long gbias, gbias2;  // the same of all kGMod: low and high 64 bits
 };
+constexpr unsigned inverse_of_rest(int i, int n) {     // (P / p_i)^-1 mod p_i, P of the first n
+    const unsigned p = (unsigned)kMod[i];
+    unsigned q = 1;
+    for (int j = 0; j < n; j++)
+        if (j != i) q = q * ((unsigned)kMod[j] % p) % p;
+    unsigned v = 1;
+    while (q * v % p != 1) v++;
+    return v;
+}
 constexpr ModTable make_table() {
     ModTable t{};
-    for (int i = 0; i < kNMod; i++) {
+    unsigned __int128 gb = 0;
+    for (int i = 0; i < kGMod; i++) {
         const unsigned p = (unsigned)kMod[i];
         unsigned c = 1 % p, cc[8] = {};
         for (int b = 0; b < 8; b++) {
@@ -96,23 +110,32 @@ constexpr ModTable make_table() {
         t.m[i].k0 = 0x4B400000u + (2 * p - two63 - base) % p;
         t.m[i].pf = (float)p;
         t.m[i].inv = 1.0f / (float)p;
-        unsigned q = 1;                            // (P / p) mod p
-        for (int j = 0; j < kNMod; j++)
-            if (j != i) q = q * ((unsigned)kMod[j] % p) % p;
-        unsigned v = 1;
-        while (q * v % p != 1) v++;
-        const unsigned long long W = (unsigned long long)((((unsigned __int128)v << 64) + p / 2) / p);
-        t.m[i].w0 = (uint32_t)W;
-        t.m[i].w1 = (uint32_t)(W >> 32);
-        t.bias += 128 * W;
+        if (i < kNMod) {
+            const unsigned v = inverse_of_rest(i, kNMod);
+            const unsigned long long W = (unsigned long long)((((unsigned __int128)v << 64) + p / 2) / p);
+            t.m[i].w[0] = (uint32_t)W;
+            t.m[i].w[1] = (uint32_t)(W >> 32);
+            t.bias += 128 * W;
+        }
+        const unsigned __int128 G = (((unsigned __int128)inverse_of_rest(i, kGMod) << 96) + p / 2) / p;
+        for (int k = 0; k < 3; k++) t.m[i].g[k] = (uint32_t)(G >> (32 * k));
+        gb += 128 * G;
     }
+    t.gbias = (unsigned long long)gb;
+    t.gbias2 = (unsigned long long)(gb >> 64);
     return t;
 }
 __constant__ ModTable kTab = make_table();
 
 // The element is F / 2^64 P with F = sum_m W_m r_m modulo 2^64 as a signed
-// number: the fraction of sum_m r_m inv_m / p_m, to 2^-53 of the range.
-constexpr double kScale = (double)modulus_product() * 0x1.0p-64;
+// number: the fraction of sum_m r_m inv_m / p_m, to 2^-53 of the range.  The
+// general products keep 96 bits, to 2^-84: an element far below its norms'
+// product keeps its FP64 digits.
+constexpr double kScale = (double)modulus_product(kNMod) * 0x1.0p-64;
+// P of the general products as a 64-bit mantissa, P = kGMant 2^kGExp
+constexpr int kGExp = 54;
+constexpr unsigned long long kGMant = (unsigned long long)((modulus_product(kGMod) + ((unsigned __int128)1 << (kGExp - 1))) >> kGExp);
+static_assert(kGMant >> 63 == 1, "normalised");
 
 // ------------------------------------------------------------ the tiling
 constexpr int kRows = 128;         // rows of a CTA (TMEM lanes, MMA M)
@@ -666,11 +689,14 @@ k_res_rowscale(int64_t M, int64_t Mp, int nseg, const float2 *__restrict__ part,
 // order as the two kernels above.  For short segments only (N < 4096): 17 us
 // against 16 + 14 at N = 2000, but with one block for 8 whole rows 1056 us
 // against 940 + 17 at N = 20000.
-constexpr int kSmallSegs = 128, kRowsBlock = 8, kSegThreads = 64;
+// With 32 rows and 8 segments at a time: the rows of a tall A of at most
+// kMaxTallCols columns (the general products).
+constexpr int kSmallSegs = 128, kMaxTallCols = 512, kTallSegs = kMaxTallCols / 32;
+template <int kRowsBlock, int kSegThreads, int kSegs>
 __global__ void __launch_bounds__(kRowsBlock *kSegThreads)
 k_res_rowexp(int64_t M, int64_t Mp, int64_t K, const z_t *__restrict__ A, int64_t lda, int seg, int nseg, int *E,
              ChaseScalars *sc) {
-    __shared__ float2 part[kSmallSegs][kRowsBlock];
+    __shared__ float2 part[kSegs][kRowsBlock];
     const int row = threadIdx.x % kRowsBlock;
     const int64_t i = (int64_t)blockIdx.x * kRowsBlock + row;
     for (int s = threadIdx.x / kRowsBlock; s < nseg; s += kSegThreads) {
@@ -763,34 +789,10 @@ struct ResConst {
     }
 };
 
-// Residues of 16 consecutive K elements of one row of A per thread: columns
-// k0 + 16 (blockIdx.x) of the matrix, read coalesced down the rows, and for
-// each modulus 16 bytes of Re and of Im, [group of 16][row][16 bytes] of the
-// chunk's 16 KB block, so that a converter thread's row is conflict-free.
-// Bound by integer issue: about 130 instructions per element for the 26
-// residues, over 16 bytes read and 26 written.
-template <int EL>   // K elements of a thread: 16, or 4 to fill the SMs from a small matrix
-__global__ void __launch_bounds__(128, 4)
-k_res_slice_a(int64_t M, int64_t K, const z_t *__restrict__ A, int64_t lda, int64_t kbase, int64_t T,
-              int64_t nch, const int *__restrict__ E, uint8_t *__restrict__ S) {
-    const int row = threadIdx.x;
-    const int64_t i = (int64_t)blockIdx.y * kRows + row;
-    const int64_t k0 = (int64_t)blockIdx.x * EL;               // within this panel
-    const int64_t kg = kbase + k0;                             // of the whole matrix
-    int sh = 0;
-    bool live = i < M;
-    if (live) {
-        const int e = E[i];
-        live = e != INT_MIN;
-        sh = live ? kAlpha - e : 0;
-    }
-    z_t v[EL];
-#pragma unroll
-    for (int e = 0; e < EL; e++) v[e] = (live && kg + e < K) ? A[i + (k0 + e) * lda] : zmk(0.0, 0.0);
-    const int64_t c = kg / kChunk;
-    const int g = (int)(kg % kChunk) / 16;
-    uint8_t *dst = S + ((int64_t)blockIdx.y * nch + c) * kAStage + g * (kRows * 16) + row * 16 + (int)(kg % 16);
-    const int64_t mstep = T * nch * kAStage;
+// The residues of EL consecutive K elements of a row: EL bytes of Re, and of Im
+// half a chunk's block on, for each modulus mstep apart.
+template <int EL>
+__device__ __forceinline__ void residues_of_row(const z_t *v, int sh, int nmod, int64_t mstep, uint8_t *dst) {
 #pragma unroll
     for (int part = 0; part < 2; part++) {
         unsigned long long x[EL];
@@ -798,7 +800,7 @@ k_res_slice_a(int64_t M, int64_t K, const z_t *__restrict__ A, int64_t lda, int6
         for (int e = 0; e < EL; e++) x[e] = biased_rint(part ? v[e].y : v[e].x, sh);
         uint8_t *d = dst + part * (4 * kRows * 16);
 #pragma unroll 1
-        for (int m = 0; m < kNMod; m++, d += mstep) {
+        for (int m = 0; m < nmod; m++, d += mstep) {
             const ResConst rc(kTab.m[m]);
             uint32_t o[EL / 4];
 #pragma unroll
@@ -814,13 +816,75 @@ k_res_slice_a(int64_t M, int64_t K, const z_t *__restrict__ A, int64_t lda, int6
     }
 }
 
+// Residues of 16 consecutive K elements of one row of A per thread: columns
+// k0 + 16 (blockIdx.x) of the matrix, read coalesced down the rows, and for
+// each modulus 16 bytes of Re and of Im, [group of 16][row][16 bytes] of the
+// chunk's 16 KB block, so that a converter thread's row is conflict-free.
+// Bound by integer issue: about 130 instructions per element for the 26
+// residues, over 16 bytes read and 26 written.
+template <int EL>   // K elements of a thread: 16, or 4 to fill the SMs from a small matrix
+__global__ void __launch_bounds__(128, 4)
+k_res_slice_a(int64_t M, int64_t K, const z_t *__restrict__ A, int64_t lda, int64_t kbase, int64_t T,
+              int64_t nch, const int *__restrict__ E, int nmod, int bits, uint8_t *__restrict__ S) {
+    const int row = threadIdx.x;
+    const int64_t i = (int64_t)blockIdx.y * kRows + row;
+    const int64_t k0 = (int64_t)blockIdx.x * EL;               // within this panel
+    const int64_t kg = kbase + k0;                             // of the whole matrix
+    int sh = 0;
+    bool live = i < M;
+    if (live) {
+        const int e = E[i];
+        live = e != INT_MIN;
+        sh = live ? bits - e : 0;
+    }
+    z_t v[EL];
+#pragma unroll
+    for (int e = 0; e < EL; e++) v[e] = (live && kg + e < K) ? A[i + (k0 + e) * lda] : zmk(0.0, 0.0);
+    const int64_t c = kg / kChunk;
+    const int g = (int)(kg % kChunk) / 16;
+    uint8_t *dst = S + ((int64_t)blockIdx.y * nch + c) * kAStage + g * (kRows * 16) + row * 16 + (int)(kg % 16);
+    residues_of_row<EL>(v, sh, nmod, T * nch * kAStage, dst);
+}
+
+// The same of A^H for A with long columns (K x M): 32 columns by 64 elements a
+// block, read along the columns and turned in shared memory.  E[i] receives
+// column i's exponent, from its partial sums of squares.  K = 20000, 100 columns:
+// 46 us, 32 MB read and 60 written.
+__global__ void __launch_bounds__(128, 4)
+k_res_slice_ah(int64_t M, int64_t K, const z_t *__restrict__ A, int64_t lda, int64_t T, int64_t nch, int npart,
+               const float2 *__restrict__ part, int *__restrict__ E, int nmod, int bits, uint8_t *__restrict__ S) {
+    __shared__ z_t tile[32][kChunk + 1];
+    const int64_t i0 = (int64_t)blockIdx.y * 32, c = blockIdx.x;
+    for (int e = threadIdx.x; e < 32 * kChunk; e += 128) {
+        const int64_t k = c * kChunk + e % kChunk, i = i0 + e / kChunk;
+        tile[e / kChunk][e % kChunk] = (k < K && i < M) ? A[k + i * lda] : zmk(0.0, 0.0);
+    }
+    const int r = threadIdx.x % 32, g = threadIdx.x / 32;
+    const int64_t i = i0 + r;
+    NormAcc n;
+    if (i < M)
+        for (int s = 0; s < npart; s++) n.add(part[i * npart + s]);
+    const int h = n.exponent();
+    if (blockIdx.x == 0 && g == 0 && i < M) E[i] = h;
+    __syncthreads();
+    z_t v[16];
+#pragma unroll
+    for (int e = 0; e < 16; e++) {
+        const z_t x = tile[r][g * 16 + e];
+        v[e] = h != INT_MIN ? zmk(x.x, -x.y) : zmk(0.0, 0.0);
+    }
+    uint8_t *dst = S + (i / kRows * nch + c) * kAStage + g * (kRows * 16) + (int)(i % kRows) * 16;
+    residues_of_row<16>(v, h != INT_MIN ? bits - h : 0, nmod, T * nch * kAStage, dst);
+}
+
 // FP16 residues of Y, -> [modulus][chunk][Re, Im, Re + Im][column][64]: one
 // column and 8 consecutive K elements per thread, the moduli from blockIdx.z
 // in steps of gridDim.z.  The column's norm comes from its partial sums, or with
 // npart = 0 from the column itself; F[j] receives its exponent.
 __global__ void __launch_bounds__(128)
 k_res_slice_b(int64_t N, int64_t Kp, int n, int mp, const z_t *__restrict__ Y, int64_t ldy, int npart,
-              const float2 *__restrict__ part, int *__restrict__ F, uint16_t *__restrict__ B, ChaseScalars *sc) {
+              const float2 *__restrict__ part, int *__restrict__ F, int nmod, int bits, uint16_t *__restrict__ B,
+              ChaseScalars *sc) {
     const int j = blockIdx.y;
     const int64_t k = ((int64_t)blockIdx.x * 128 + threadIdx.x) * 8;
     int h = INT_MIN;
@@ -842,7 +906,7 @@ k_res_slice_b(int64_t N, int64_t Kp, int n, int mp, const z_t *__restrict__ Y, i
     if (blockIdx.x == 0 && blockIdx.z == 0 && threadIdx.x == 0) F[j] = h;
     if (k >= Kp) return;
     const bool live = h != INT_MIN;
-    const int sh = live ? kBeta - h : 0;
+    const int sh = live ? bits - h : 0;
     unsigned long long xr[8], xi[8];
 #pragma unroll
     for (int e = 0; e < 8; e++) {
@@ -854,7 +918,7 @@ k_res_slice_b(int64_t N, int64_t Kp, int n, int mp, const z_t *__restrict__ Y, i
     const int64_t pstep = (int64_t)mp * kChunk;
     const __half2 bias = __floats2half2_rn(1152.f, 1152.f);
 #pragma unroll 1
-    for (int m = blockIdx.z; m < kNMod; m += gridDim.z) {
+    for (int m = blockIdx.z; m < nmod; m += gridDim.z) {
         const ResConst rc(kTab.m[m]);
         const int p = (int)kTab.m[m].pf;
         uint32_t o[3][4];
@@ -923,24 +987,69 @@ k_res_panel(int Nk, int nb, int N, int jbase, int cols, BseModel md, const doubl
 
 // ------------------------------------------------------------ the result
 // Element (i, j) from the residues of all moduli and splits, ROWS consecutive
-// rows per thread (4, or 1 to fill the SMs from a small result); then the
-// Chebyshev recurrence.  The splits' bytes (residue + 128) are summed two to a
+// rows per thread (4, or 1 to fill the SMs from a small result).  The splits' bytes (residue + 128) are summed two to a
 // word first, then F = sum_m W_m u_m - nz bias, a multiply-add per word of W:
 // 10 us at N = 2000, 75 columns (15 with four rows per thread, and 20 with a
 // 64-bit product per split and value before), 7 us at N = 256 (14).  At N =
 // 20000, 140 columns four rows take 82 us, with one 8-byte load per modulus.
-template <int ROWS>
-__global__ void __launch_bounds__(128)
-k_res_reduce(int64_t M, int64_t Mp, int mp, int nz, const uchar2 *__restrict__ R, const int *__restrict__ E,
-             const int *__restrict__ F, GemmEpi ep, const z_t *__restrict__ Y, int64_t ldy, z_t *C,
-             int64_t ldc) {
+struct WithH {                                     // the product with H
+    static constexpr int kMods = kNMod, kWords = 2, kBits = kAlpha + kBeta;
+    static __device__ __forceinline__ unsigned long long word(int m, int i) { return kTab.m[m].w[i]; }
+    // F P 2^(x - 64)
+    static __device__ __forceinline__ double value(const unsigned long long *s, int nz, int x) {
+        const double a = (double)(long long)(s[0] + (s[1] << 32) - kTab.bias * (unsigned)nz) * kScale;
+        if (x > -1000 && x < 900) return a * __longlong_as_double((long long)(1023 + x) << 52);
+        return ldexp(a, x);
+    }
+};
+// m 2^e, m >= 2^62, rounded once
+__device__ __forceinline__ double to_double(unsigned long long m, int e, bool neg) {
+    if (!(m >> 63)) {
+        m <<= 1;
+        e--;
+    }
+    const unsigned long long q = (m >> 11) + (m >> 10 & 1);    // 53 bits, or 2^53
+    const int be = e + 63 + 1023;
+    double v;
+    if (be >= 1 && be <= 2045) v = __longlong_as_double((long long)(((unsigned long long)(be - 1) << 52) + q));
+    else v = ldexp((double)m, e);
+    return neg ? -v : v;
+}
+struct General {                                   // the general products
+    static constexpr int kMods = kGMod, kWords = 3, kBits = 2 * kGBits;
+    static __device__ __forceinline__ unsigned long long word(int m, int i) { return kTab.m[m].g[i]; }
+    // |F| P in integers, 64 bits of each, and one rounding to FP64 (whose issue
+    // is scarce: with conversions and products in FP64 these took longer than the loads)
+    static __device__ __forceinline__ double value(const unsigned long long *s, int nz, int x) {
+        const unsigned __int128 b = ((unsigned __int128)kTab.gbias2 << 64 | kTab.gbias) * (unsigned)nz;
+        unsigned __int128 t = s[0] + ((unsigned __int128)s[1] << 32) + ((unsigned __int128)s[2] << 64) - b;
+        const bool neg = (uint32_t)(t >> 64) >> 31;            // F: 96 bits, signed
+        if (neg) t = 0 - t;
+        unsigned long long hi = (unsigned long long)(t >> 32), lo = (unsigned long long)(uint32_t)t << 32;
+        int lz = __clzll((long long)hi);
+        if (lz == 64) {
+            if (lo == 0) return 0.0;
+            hi = lo;
+            lo = 0;
+            lz = __clzll((long long)hi);
+            hi <<= lz;
+            lz += 64;
+        } else if (lz > 0) {
+            hi = hi << lz | lo >> (64 - lz);
+        }
+        return to_double(__umul64hi(hi, kGMant), kGExp - lz + x, neg);   // |F| = hi 2^(32 - lz)
+    }
+};
+// v[e]: elements (i + e, j), e < ROWS, where i + e < M (i a multiple of ROWS)
+template <class Set, int ROWS>
+__device__ __forceinline__ void recombine(int64_t i, int j, int64_t M, int64_t Mp, int mp, int nz,
+                                          const uchar2 *__restrict__ R, const int *__restrict__ E,
+                                          const int *__restrict__ F, z_t *v) {
+    constexpr int kMods = Set::kMods;
     constexpr int kW2 = (ROWS + 1) / 2;            // words of two rows
-    const int64_t i = ((int64_t)blockIdx.x * 128 + threadIdx.x) * ROWS;
-    const int j = blockIdx.y;
-    if (i >= M) return;
     const uchar2 *r0 = R + (int64_t)j * Mp + i;
     const int64_t step = (int64_t)mp * Mp;
-    unsigned long long s[ROWS][2][2] = {};         // [row][Re, Im][word of W]
+    unsigned long long s[ROWS][2][Set::kWords] = {};   // [row][Re, Im][word of W]
     auto load = [](const uchar2 *p, uint32_t *q) {
         if constexpr (ROWS == 4) {
             const uint2 v = *(const uint2 *)p;
@@ -951,36 +1060,36 @@ k_res_reduce(int64_t M, int64_t Mp, int mp, int nz, const uchar2 *__restrict__ R
         }
     };
     auto digest = [&](int m, const uint32_t *ur, const uint32_t *ui) {   // sums, 16 bits a row
-        const unsigned long long w0 = kTab.m[m].w0, w1 = kTab.m[m].w1;
 #pragma unroll
-        for (int e = 0; e < ROWS; e++) {
-            const uint32_t a = ur[e / 2] >> (16 * (e % 2)) & 0xFFFFu, b = ui[e / 2] >> (16 * (e % 2)) & 0xFFFFu;
-            s[e][0][0] += a * w0;
-            s[e][0][1] += a * w1;
-            s[e][1][0] += b * w0;
-            s[e][1][1] += b * w1;
+        for (int k = 0; k < Set::kWords; k++) {
+            const unsigned long long w = Set::word(m, k);
+#pragma unroll
+            for (int e = 0; e < ROWS; e++) {
+                s[e][0][k] += (ur[e / 2] >> (16 * (e % 2)) & 0xFFFFu) * w;
+                s[e][1][k] += (ui[e / 2] >> (16 * (e % 2)) & 0xFFFFu) * w;
+            }
         }
     };
     if constexpr (ROWS == 1) {
         // few threads: the loads of all moduli in flight together
-        uint32_t ur[kNMod] = {}, ui[kNMod] = {};
+        uint32_t ur[kMods] = {}, ui[kMods] = {};
 #pragma unroll 1
         for (int z = 0; z < nz; z++, r0 += step) {
-            uint32_t q[kNMod];
+            uint32_t q[kMods];
 #pragma unroll
-            for (int m = 0; m < kNMod; m++) load(r0 + (int64_t)m * nz * step, &q[m]);
+            for (int m = 0; m < kMods; m++) load(r0 + (int64_t)m * nz * step, &q[m]);
 #pragma unroll
-            for (int m = 0; m < kNMod; m++) {
+            for (int m = 0; m < kMods; m++) {
                 ur[m] += q[m] & 255;
                 ui[m] += q[m] >> 8;
             }
         }
 #pragma unroll
-        for (int m = 0; m < kNMod; m++) digest(m, &ur[m], &ui[m]);
+        for (int m = 0; m < kMods; m++) digest(m, &ur[m], &ui[m]);
     } else {
         // many threads hide the loads, and few registers each leave room for them
 #pragma unroll 2
-        for (int m = 0; m < kNMod; m++) {
+        for (int m = 0; m < kMods; m++) {
             uint32_t ur[kW2] = {}, ui[kW2] = {};
             for (int z = 0; z < nz; z++, r0 += step) {
                 uint32_t q[kW2];
@@ -995,28 +1104,61 @@ k_res_reduce(int64_t M, int64_t Mp, int mp, int nz, const uchar2 *__restrict__ R
         }
     }
     const int f = F[j];
-    const unsigned long long bias = kTab.bias * (unsigned)nz;
+#pragma unroll
+    for (int e = 0; e < ROWS; e++) {
+        v[e] = zmk(0.0, 0.0);
+        if (i + e >= M) continue;
+        const int h = E[i + e];
+        if (h == INT_MIN || f == INT_MIN) continue;
+        const int x = h + f - Set::kBits;
+        v[e] = zmk(Set::value(s[e][0], nz, x), Set::value(s[e][1], nz, x));
+    }
+}
+
+template <int ROWS>
+__global__ void __launch_bounds__(128)
+k_res_reduce(int64_t M, int64_t Mp, int mp, int nz, const uchar2 *__restrict__ R, const int *__restrict__ E,
+             const int *__restrict__ F, GemmEpi ep, const z_t *__restrict__ Y, int64_t ldy, z_t *C,
+             int64_t ldc) {
+    const int64_t i = ((int64_t)blockIdx.x * 128 + threadIdx.x) * ROWS;
+    const int j = blockIdx.y;
+    if (i >= M) return;
+    z_t r[ROWS];
+    recombine<WithH, ROWS>(i, j, M, Mp, mp, nz, R, E, F, r);
 #pragma unroll
     for (int e = 0; e < ROWS; e++) {
         if (i + e >= M) break;
-        const int h = E[i + e];
-        z_t v = zmk(0.0, 0.0);
-        if (h != INT_MIN && f != INT_MIN) {
-            const int x = h + f - (kAlpha + kBeta);
-            const double a = (double)(long long)(s[e][0][0] + (s[e][0][1] << 32) - bias) * kScale;
-            const double b = (double)(long long)(s[e][1][0] + (s[e][1][1] << 32) - bias) * kScale;
-            if (x > -1000 && x < 900) {
-                const double sc = __longlong_as_double((long long)(1023 + x) << 52);
-                v = zmk(a * sc, b * sc);
-            } else {
-                v = zmk(ldexp(a, x), ldexp(b, x));
-            }
-        }
+        z_t v = r[e];
         if (ep.mode == GEMM_CHEB) {
             v = zscale(zsub(v, zscale(Y[i + e + j * ldy], ep.c)), ep.s1);
             if (ep.Yp) v = zsub(v, zscale(ep.Yp[i + e + j * ep.ldyp], ep.s2));
         }
         C[i + e + j * ldc] = v;
+    }
+}
+
+// The general products' results (RsOut).  N = 20000, 100 columns: 60 us (76 with
+// the conversions to FP64 on the FP64 pipe).
+template <int ROWS>
+__global__ void __launch_bounds__(128)
+k_res_out(int64_t M, int64_t Mp, int mp, int nz, const uchar2 *__restrict__ R, const int *__restrict__ E,
+          const int *__restrict__ F, RsOut o) {
+    const int64_t i = ((int64_t)blockIdx.x * 128 + threadIdx.x) * ROWS;
+    const int j = blockIdx.y;
+    if (i >= M) return;
+    z_t r[ROWS];
+    const bool lower = ROWS == 1 && o.mirror && i > j;
+    recombine<General, ROWS>(lower ? j : i, lower ? (int)i : j, M, Mp, mp, nz, R, E, F, r);
+    if (lower) r[0] = zconj(r[0]);
+    if (ROWS == 1 && o.mirror && i == j) r[0].y = 0.0;
+#pragma unroll
+    for (int e = 0; e < ROWS; e++) {
+        if (i + e >= M) break;
+        z_t v = r[e];
+        if (o.D) v = zsub(o.D[i + e + j * o.ldd], v);
+        if (i + e == j) v.x += o.shift;
+        if (o.adjoint) o.C[j + (i + e) * o.ldc] = zconj(v);
+        else o.C[i + e + j * o.ldc] = v;
     }
 }
 
@@ -1043,19 +1185,19 @@ void column_tiles(int n, int *tx, int *w) {
 // takes 6 w cycles of MMA, at least about 700 (its share of HBM) or 260 (its
 // conversion) when the matrix is in L2; a unit costs about 2000 more (its first
 // copies and its last drain) and each split about 52 bytes per output.
-int choose_chunks(int64_t Mp, int nch, int mp, int tx, int w, size_t r_bytes, int sms) {
-    const double mat = 26.0 * Mp * nch * kChunk;
+int choose_chunks(int64_t Mp, int nch, int mp, int tx, int w, int nmod, size_t r_bytes, int sms) {
+    const double mat = 2.0 * nmod * Mp * nch * kChunk;
     const double per_chunk = std::max(6.0 * w, mat > 1.0e8 ? 700.0 : 300.0);
-    const int64_t tiles = Mp / kRows * tx * kNMod;
+    const int64_t tiles = Mp / kRows * tx * nmod;
     int best = 0;
     double best_t = 1e300;
     for (int cs = 1; cs <= kMaxUnitChunks; cs = cs < 8 ? cs * 2 : cs + 8) {
         const int nz = (nch + cs - 1) / cs;
         if (nz > 250) continue;                    // 16-bit sums of the splits' bytes
-        if ((size_t)kNMod * nz * mp * Mp * sizeof(uchar2) > r_bytes) continue;
+        if ((size_t)nmod * nz * mp * Mp * sizeof(uchar2) > r_bytes) continue;
         const int64_t per = (tiles * nz + sms - 1) / sms;
         const double t = (double)per * (std::min(cs, nch) * per_chunk + 2000.0) +
-                         52.0 * nz * mp * Mp / (5e12 / 1.9e9);
+                         4.0 * nmod * nz * mp * Mp / (5e12 / 1.9e9);
         if (t < best_t) {
             best_t = t;
             best = cs;
@@ -1069,15 +1211,20 @@ constexpr int64_t kShortColumn = 4096;
 
 }  // namespace
 
-size_t residue_a_bytes(int64_t M, int64_t K) {
+namespace {
+size_t a_bytes_of(int64_t M, int64_t K, int nmod) {
     const int64_t Mp = (M + kRows - 1) / kRows * kRows, Kp = (K + kChunk - 1) / kChunk * kChunk;
-    return (size_t)kNMod * 2 * Mp * Kp;
+    return (size_t)nmod * 2 * Mp * Kp;
 }
-
-size_t residue_b_bytes(int64_t K, int n) {
+size_t b_bytes_of(int64_t K, int n, int nmod) {
     const int64_t Kp = (K + kChunk - 1) / kChunk * kChunk;
-    return (size_t)kNMod * 3 * Kp * (n + 64) * 2;
+    return (size_t)nmod * 3 * Kp * (n + 64) * 2;
 }
+}  // namespace
+
+size_t residue_a_bytes(int64_t M, int64_t K) { return a_bytes_of(M, K, kNMod); }
+
+size_t residue_b_bytes(int64_t K, int n) { return b_bytes_of(K, n, kNMod); }
 
 size_t residue_r_bytes(int64_t M, int64_t K, int n) {
     const int64_t Mp = (M + kRows - 1) / kRows * kRows, nch = (K + kChunk - 1) / kChunk;
@@ -1102,8 +1249,7 @@ cudaError_t residue_prepare(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh, vo
     const int seg = norm_segment(N), nseg = (int)((N + seg - 1) / seg);
     const unsigned rb = (unsigned)((N + 127) / 128);
     if (seg == 32 && nseg <= kSmallSegs) {
-        k_res_rowexp<<<(unsigned)(Np / kRowsBlock), kRowsBlock * kSegThreads, 0, st>>>(N, Np, N, H, ldh, seg, nseg,
-                                                                                       oh->E, sc);
+        k_res_rowexp<8, 64, kSmallSegs><<<(unsigned)(Np / 8), 512, 0, st>>>(N, Np, N, H, ldh, seg, nseg, oh->E, sc);
         bse_count_launches(1);
     } else {
         k_res_rownorm<<<dim3(rb, (unsigned)nseg), 128, 0, st>>>(N, N, H, ldh, seg, 0, (float2 *)work);
@@ -1111,11 +1257,11 @@ cudaError_t residue_prepare(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh, vo
         bse_count_launches(2);
     }
     if (nch * 4 * T < 608)                         // too few blocks for four on every SM (N = 256: 9.2 us, 6.5 here)
-        k_res_slice_a<4><<<dim3((unsigned)(nch * 16), (unsigned)T), 128, 0, st>>>(N, N, H, ldh, 0, T, nch, oh->E,
-                                                                                 (uint8_t *)oh->A);
+        k_res_slice_a<4><<<dim3((unsigned)(nch * 16), (unsigned)T), 128, 0, st>>>(N, N, H, ldh, 0, T, nch, oh->E, kNMod,
+                                                                                 kAlpha, (uint8_t *)oh->A);
     else
-        k_res_slice_a<16><<<dim3((unsigned)(nch * 4), (unsigned)T), 128, 0, st>>>(N, N, H, ldh, 0, T, nch, oh->E,
-                                                                                 (uint8_t *)oh->A);
+        k_res_slice_a<16><<<dim3((unsigned)(nch * 4), (unsigned)T), 128, 0, st>>>(N, N, H, ldh, 0, T, nch, oh->E, kNMod,
+                                                                                 kAlpha, (uint8_t *)oh->A);
     bse_count_launches(1);
     return cudaGetLastError();
 }
@@ -1145,7 +1291,7 @@ cudaError_t residue_prepare_bse(int Nk, int Nv, int Nc, const BseModel &md, cons
                     N, cols, Hp, N, seg, j0 / seg, (float2 *)work);
             else
                 k_res_slice_a<16><<<dim3((unsigned)((cols + kChunk - 1) / kChunk * 4), (unsigned)T), 128, 0, st>>>(
-                    N, N, Hp, N, j0, T, nch, oh->E, (uint8_t *)oh->A);
+                    N, N, Hp, N, j0, T, nch, oh->E, kNMod, kAlpha, (uint8_t *)oh->A);
             bse_count_launches(2);
         }
         if (pass == 0) {
@@ -1180,6 +1326,34 @@ cudaError_t residue_launch(RsBatch &b, int sms, cudaStream_t st) {
     return launch_cfg<RsWide>(b, sms, st);
 }
 
+namespace {
+// A launch of one product: the residues of A (Mp rows) and of B (tx tiles of w columns)
+bool single_job(RsBatch *b, const void *A, void *B, int64_t Mp, int nch, int tx, int w, int nmod, void *R,
+                size_t r_bytes, ChaseScalars *sc, uint64_t wait_ns, int sms) {
+    memset(b, 0, sizeof *b);
+    RsJob &j = b->job[0];
+    const int mp = tx * w;
+    if (!make_map(&j.tmB, B, (uint64_t)mp, (uint64_t)nmod * 3 * nch, (uint32_t)w)) return false;
+    j.A = (const uint8_t *)A;
+    j.R = (uchar2 *)R;
+    j.sc = sc;
+    j.wait_ns = wait_ns;
+    j.Mp = Mp;
+    j.w = w;
+    j.mp = mp;
+    j.nch = nch;
+    j.cs = choose_chunks(Mp, nch, mp, tx, w, nmod, r_bytes, sms);
+    if (j.cs < 1) return false;
+    j.tx = tx;
+    j.ty = (int)(Mp / kRows);
+    j.tz = (nch + j.cs - 1) / j.cs;
+    j.nmod = nmod;
+    b->njobs = 1;
+    b->units = rs_units(j);
+    return true;
+}
+}  // namespace
+
 cudaError_t residue_zgemm(const OzakiH &oh, int n, const z_t *Y, int64_t ldy, z_t *C, int64_t ldc,
                           const GemmEpi &ep, void *B, size_t b_bytes, int *F, float2 *part, void *R,
                           size_t r_bytes, ChaseScalars *sc, int sms, cudaStream_t st, cudaEvent_t ev0,
@@ -1200,28 +1374,13 @@ cudaError_t residue_zgemm(const OzakiH &oh, int n, const z_t *Y, int64_t ldy, z_
     const unsigned bx = (unsigned)((Kp + 1023) / 1024);
     // split the moduli over blocks while that leaves SMs idle otherwise
     const unsigned bz = (unsigned)std::max<int64_t>(1, std::min<int64_t>(kNMod, 4 * sms / ((int64_t)bx * mp)));
-    k_res_slice_b<<<dim3(bx, (unsigned)mp, bz), 128, 0, st>>>(N, Kp, n, mp, Y, ldy, npart, part, F, (uint16_t *)B, sc);
+    k_res_slice_b<<<dim3(bx, (unsigned)mp, bz), 128, 0, st>>>(N, Kp, n, mp, Y, ldy, npart, part, F, kNMod, kBeta,
+                                                              (uint16_t *)B, sc);
     bse_count_launches(1);
     RsBatch b;
-    memset(&b, 0, sizeof b);
     RsJob &j = b.job[0];
-    if (!make_map(&j.tmB, B, (uint64_t)mp, (uint64_t)(kNMod * 3 * nch), (uint32_t)w)) return cudaErrorInvalidValue;
-    j.A = (const uint8_t *)oh.A;
-    j.R = (uchar2 *)R;
-    j.sc = sc;
-    j.wait_ns = oh.wait_ns;
-    j.Mp = oh.Np;
-    j.w = w;
-    j.mp = mp;
-    j.nch = (int)nch;
-    j.cs = choose_chunks(oh.Np, j.nch, mp, tx, w, r_bytes, sms);
-    if (j.cs < 1) return cudaErrorInvalidValue;
-    j.tx = tx;
-    j.ty = (int)(oh.Np / kRows);
-    j.tz = (j.nch + j.cs - 1) / j.cs;
-    j.nmod = kNMod;
-    b.njobs = 1;
-    b.units = rs_units(j);
+    if (!single_job(&b, oh.A, B, oh.Np, (int)nch, tx, w, kNMod, R, r_bytes, sc, oh.wait_ns, sms))
+        return cudaErrorInvalidValue;
     cudaError_t e;
     if (batcher) {
         e = ozb_run_residue(batcher, j, st);
@@ -1237,6 +1396,87 @@ cudaError_t residue_zgemm(const OzakiH &oh, int n, const z_t *Y, int64_t ldy, z_
     else
         k_res_reduce<4><<<dim3((unsigned)((N + 511) / 512), (unsigned)n), 128, 0, st>>>(
             N, oh.Np, mp, j.tz, j.R, oh.E, F, ep, Y, ldy, C, ldc);
+    bse_count_launches(1);
+    return cudaGetLastError();
+}
+
+// ------------------------------------------------------------ general products
+// A^H B and A B of the QR and Gram entries, for tall A and B.  In native FP64
+// (1.2 TFLOP/s on this part) they were bound by its issue: Gram K = 20000,
+// 140 x 40: 1805 us, here 187 (55 left residues, 24 right, 23 norms, 47 product,
+// 17 result); QR N = 20000, 100 columns after 40: 21.8 ms, here 3.5.
+size_t residue_left_bytes(int64_t M, int64_t K) { return a_bytes_of(M, K, kGMod); }
+size_t residue_right_bytes(int64_t K, int n) { return b_bytes_of(K, n, kGMod); }
+size_t residue_out_bytes(int64_t M, int64_t K, int n) {
+    const int64_t Mp = (M + kRows - 1) / kRows * kRows, nch = (K + kChunk - 1) / kChunk;
+    // splits of a long sum: enough to fill the SMs from one row tile
+    const int64_t nz = std::max<int64_t>((nch + kMaxUnitChunks - 1) / kMaxUnitChunks, std::min<int64_t>(nch, Mp <= 512 ? 24 : 4));
+    return (size_t)kGMod * nz * (n + 64) * Mp * sizeof(uchar2);
+}
+
+namespace {
+int col_parts(int64_t K) { return (int)std::min<int64_t>((K + 1023) / 1024, kRsColParts); }
+
+void col_norms(int64_t K, int64_t n, const z_t *A, int64_t lda, float2 *part, ChaseScalars *sc, cudaStream_t st) {
+    k_res_colnorm<<<dim3((unsigned)col_parts(K), (unsigned)n), 256, 0, st>>>(K, A, lda, part, sc);
+    bse_count_launches(1);
+}
+}  // namespace
+
+cudaError_t residue_left(int64_t M, int64_t K, const z_t *A, int64_t lda, bool ah, const RsSide &s, ChaseScalars *sc,
+                         cudaStream_t st) {
+    const int64_t T = (M + kRows - 1) / kRows, nch = (K + kChunk - 1) / kChunk;
+    if (M < 1 || K < 1 || residue_left_bytes(M, K) > s.bytes || (!ah && K > kMaxTallCols)) return cudaErrorInvalidValue;
+    if (ah) {
+        col_norms(K, M, A, lda, s.part, sc, st);
+        k_res_slice_ah<<<dim3((unsigned)nch, (unsigned)((M + 31) / 32)), 128, 0, st>>>(
+            M, K, A, lda, T, nch, col_parts(K), s.part, s.e, kGMod, kGBits, (uint8_t *)s.p);
+    } else {
+        k_res_rowexp<32, 8, kTallSegs><<<(unsigned)(T * kRows / 32), 256, 0, st>>>(
+            M, T * kRows, K, A, lda, 32, (int)((K + 31) / 32), s.e, sc);
+        k_res_slice_a<16><<<dim3((unsigned)(nch * 4), (unsigned)T), 128, 0, st>>>(M, K, A, lda, 0, T, nch, s.e, kGMod,
+                                                                                 kGBits, (uint8_t *)s.p);
+        bse_count_launches(1);
+    }
+    bse_count_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t residue_right(int64_t K, int n, const z_t *B, int64_t ldb, const float2 *norms, const RsSide &s,
+                          ChaseScalars *sc, int sms, cudaStream_t st) {
+    if (n < 1 || K < 1 || residue_right_bytes(K, n) > s.bytes) return cudaErrorInvalidValue;
+    const int64_t Kp = (K + kChunk - 1) / kChunk * kChunk;
+    int tx, w;
+    column_tiles(n, &tx, &w);
+    const int mp = tx * w;
+    int npart = 0;
+    if (norms || K > kShortColumn) {
+        if (!norms) col_norms(K, n, B, ldb, s.part, sc, st);
+        npart = col_parts(K);
+    }
+    const unsigned bx = (unsigned)((Kp + 1023) / 1024);
+    const unsigned bz = (unsigned)std::max<int64_t>(1, std::min<int64_t>(kGMod, 4 * sms / ((int64_t)bx * mp)));
+    k_res_slice_b<<<dim3(bx, (unsigned)mp, bz), 128, 0, st>>>(K, Kp, n, mp, B, ldb, npart, norms ? norms : s.part, s.e,
+                                                              kGMod, kGBits, (uint16_t *)s.p, sc);
+    bse_count_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t residue_product(int64_t M, int n, int64_t K, const RsSide &A, const RsSide &B, const RsOut &out, void *R,
+                            size_t r_bytes, uint64_t wait_ns, ChaseScalars *sc, int sms, cudaStream_t st) {
+    if (out.mirror && (M != n || out.adjoint || out.D)) return cudaErrorInvalidValue;
+    const int64_t Mp = (M + kRows - 1) / kRows * kRows, nch = (K + kChunk - 1) / kChunk;
+    int tx, w;
+    column_tiles(n, &tx, &w);
+    RsBatch b;
+    if (!single_job(&b, A.p, B.p, Mp, (int)nch, tx, w, kGMod, R, r_bytes, sc, wait_ns, sms)) return cudaErrorInvalidValue;
+    const RsJob &j = b.job[0];
+    const cudaError_t e = residue_launch(b, sms, st);
+    if (e != cudaSuccess) return e;
+    if (M * n < 400000 || out.mirror)
+        k_res_out<1><<<dim3((unsigned)((M + 127) / 128), (unsigned)n), 128, 0, st>>>(M, Mp, j.mp, j.tz, j.R, A.e, B.e, out);
+    else
+        k_res_out<4><<<dim3((unsigned)((M + 511) / 512), (unsigned)n), 128, 0, st>>>(M, Mp, j.mp, j.tz, j.R, A.e, B.e, out);
     bse_count_launches(1);
     return cudaGetLastError();
 }

@@ -118,3 +118,74 @@ def test_nonfinite_is_reported(ctx):
         with pytest.raises(pkg.BseError) as ei:
             _hemm(ctx, A, Y)
         assert ei.value.status == pkg.BSE_ENONFINITE
+
+
+# ---- the general products (Gram and QR entries)
+
+def _integers(rows, cols, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    r = torch.randint(-2 ** 17, 2 ** 17 + 1, (2, cols, rows), device="cuda", generator=g).double()
+    return torch.complex(r[0], r[1]).T
+
+
+@pytest.mark.parametrize("K,m1,m2", [(63, 4, 3), (64, 4, 3), (65, 1, 1), (64, 33, 40), (127, 129, 16), (1025, 17, 145),
+                                     (4096, 31, 5), (4097, 97, 128), (20000, 140, 40), (4097, 512, 512)])
+def test_gram_of_integers(ctx, K, m1, m2):
+    """Integers of 18 bits are exact in the operands' 58 bits, so only the
+    result's own rounding is left (one FP64 product of the 96-bit fraction:
+    2^-52 of the element, and the fraction's 2^-70 of the norms); the FP64
+    reference is exact: sums of 2 K products of 34 bits stay below 2^53."""
+    A, B = _integers(K, m1, 5), _integers(K, m2, 6)
+    A[:, 0] = 0.0
+    torch.cuda.synchronize()
+    for X, Y in ((A, B), (A, A)):
+        G, ref = ctx.gram(X, Y), X.conj().T @ Y
+        norms = torch.linalg.vector_norm(X, dim=0)[:, None] * torch.linalg.vector_norm(Y, dim=0)[None, :]
+        assert torch.all((G - ref).abs() <= 2.0 ** -52 * ref.abs() + 2.0 ** -70 * norms)
+    assert torch.equal(G, G.conj().T)
+
+
+def test_gram_scales_and_nonfinite(ctx):
+    """Column norms over the exponent range; non-finite entries give what IEEE
+    arithmetic gives (native FP64), and the context stays usable."""
+    K, m = 300, 6
+    A = _integers(K, m, 7)
+    s = 2.0 ** torch.tensor([-1060, -300, 0, 1, 300, 490], device="cuda", dtype=torch.float64)
+    B = (A * s).T.contiguous().T
+    torch.cuda.synchronize()
+    G, ref = ctx.gram(A, B), (A.conj().T @ A) * s
+    norms = torch.linalg.vector_norm(A, dim=0)[:, None] * torch.linalg.vector_norm(A, dim=0)[None, :]
+    tol = (2.0 ** -52 * (A.conj().T @ A).abs() + 2.0 ** -70 * norms) * s + 2.0 ** -1073
+    # the first column's entries lose bits below 2^-1074
+    assert torch.all(((G - ref).abs() <= tol)[:, 1:])
+    for bad in (float("nan"), float("inf")):
+        C = A.clone(memory_format=torch.preserve_format)
+        C[7, 2] = bad
+        torch.cuda.synchronize()
+        G = ctx.gram(C, A)
+        fine = torch.isfinite(torch.view_as_real(G)).all(dim=-1)
+        assert not fine[2].any() and fine[[0, 1, 3, 4, 5]].all()
+    torch.cuda.synchronize()
+    assert torch.all((ctx.gram(A, A) - A.conj().T @ A).abs() <= 2.0 ** -52 * norms)
+
+
+@pytest.mark.parametrize("N,m,k", [(63, 5, 3), (64, 5, 3), (64, 64, 0), (65, 1, 1), (129, 17, 33), (1000, 97, 16),
+                                   (4097, 100, 40), (1030, 290, 222)])
+def test_qr_of_sizes(ctx, N, m, k):
+    """Orthonormal to the bound of CholeskyQR2, 6 (N m + m (m + 1)) 2^-53 (its
+    products are at least FP64's here), against L to the same; V R = the
+    projected block to 2^-40 of its norm (three passes, each a product to FP64
+    rounding over at most m = 290 columns)."""
+    V0 = _block(N, m, 8)
+    L = torch.linalg.qr(_block(N, k, 9))[0].T.contiguous().T if k else None
+    V = V0.clone(memory_format=torch.preserve_format)
+    torch.cuda.synchronize()
+    out = ctx.qr(V, L)
+    V = V if out is None else out
+    bound = 6 * (N * m + m * (m + 1)) * 2.0 ** -53
+    assert torch.linalg.matrix_norm(V.conj().T @ V - torch.eye(m, device="cuda")) <= bound
+    P = V0
+    if k:
+        assert torch.linalg.matrix_norm(L.conj().T @ V) <= bound
+        P = V0 - L @ (L.conj().T @ V0)
+    assert torch.linalg.matrix_norm(V @ (V.conj().T @ P) - P) <= 2.0 ** -40 * torch.linalg.matrix_norm(P)
