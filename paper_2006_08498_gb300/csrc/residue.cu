@@ -130,12 +130,13 @@ __constant__ ModTable kTab = make_table();
 // The element is F / 2^64 P with F = sum_m W_m r_m modulo 2^64 as a signed
 // number: the fraction of sum_m r_m inv_m / p_m, to 2^-53 of the range.  The
 // general products keep 96 bits, to 2^-84: an element far below its norms'
-// product keeps its FP64 digits.
-constexpr double kScale = (double)modulus_product(kNMod) * 0x1.0p-64;
-// P of the general products as a 64-bit mantissa, P = kGMant 2^kGExp
-constexpr int kGExp = 54;
-constexpr unsigned long long kGMant = (unsigned long long)((modulus_product(kGMod) + ((unsigned __int128)1 << (kGExp - 1))) >> kGExp);
-static_assert(kGMant >> 63 == 1, "normalised");
+// product keeps its FP64 digits.  P as a 64-bit mantissa: P = mant 2^exp.
+constexpr unsigned long long mantissa(int n, int e) {
+    return (unsigned long long)((modulus_product(n) + ((unsigned __int128)1 << (e - 1))) >> e);
+}
+constexpr int kHExp = 39, kGExp = 54;
+constexpr unsigned long long kHMant = mantissa(kNMod, kHExp), kGMant = mantissa(kGMod, kGExp);
+static_assert(kHMant >> 63 == 1 && kGMant >> 63 == 1, "normalised");
 
 // ------------------------------------------------------------ the tiling
 constexpr int kRows = 128;         // rows of a CTA (TMEM lanes, MMA M)
@@ -568,14 +569,17 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
             uchar2 *R = a.R + ((int64_t)(n.m * a.tz + n.z) * a.mp + n.x * a.w + half * ng * 8) * a.Mp +
                        (int64_t)n.y * kRows + row;
             const unsigned off = (unsigned)cnt * (unsigned)__float_as_int(kMagic);
+            const uint64_t byte2 = tc::pin2(tc::f32x2(8388736.f, 8388736.f));
 #pragma unroll
             for (int v = 0; v < kG * 8; v++) {
                 if (v < ng * 8) {
                     const int s = (int)((unsigned)acc[v] - off);
                     const int si = (s + kPack / 2) >> 13, sr = s - si * kPack;
-                    const float xr = (float)sr, xi = (float)si;
-                    const float yr = __fmaf_rn(-pf, rintf(xr * inv), xr), yi = __fmaf_rn(-pf, rintf(xi * inv), xi);
-                    R[(int64_t)v * a.Mp] = make_uchar2((uint8_t)((int)yr + 128), (uint8_t)((int)yi + 128));
+                    // to FP32 and back by the bit patterns of 1.5 2^23 + x and 2^23 + 128 + r
+                    const uint64_t xx = tc::add2(tc::pack2(0x4B400000u + (uint32_t)sr, 0x4B400000u + (uint32_t)si), mmagic2);
+                    const uint64_t q = tc::add2(tc::fma2(xx, inv2, magic2), mmagic2);
+                    const uint64_t z = tc::add2(tc::fma2(q, mp2, xx), byte2);
+                    R[(int64_t)v * a.Mp] = make_uchar2((uint8_t)z, (uint8_t)(z >> 32));
                 }
             }
         }
@@ -990,18 +994,10 @@ k_res_panel(int Nk, int nb, int N, int jbase, int cols, BseModel md, const doubl
 // rows per thread (4, or 1 to fill the SMs from a small result).  The splits' bytes (residue + 128) are summed two to a
 // word first, then F = sum_m W_m u_m - nz bias, a multiply-add per word of W:
 // 10 us at N = 2000, 75 columns (15 with four rows per thread, and 20 with a
-// 64-bit product per split and value before), 7 us at N = 256 (14).  At N =
-// 20000, 140 columns four rows take 82 us, with one 8-byte load per modulus.
-struct WithH {                                     // the product with H
-    static constexpr int kMods = kNMod, kWords = 2, kBits = kAlpha + kBeta;
-    static __device__ __forceinline__ unsigned long long word(int m, int i) { return kTab.m[m].w[i]; }
-    // F P 2^(x - 64)
-    static __device__ __forceinline__ double value(const unsigned long long *s, int nz, int x) {
-        const double a = (double)(long long)(s[0] + (s[1] << 32) - kTab.bias * (unsigned)nz) * kScale;
-        if (x > -1000 && x < 900) return a * __longlong_as_double((long long)(1023 + x) << 52);
-        return ldexp(a, x);
-    }
-};
+// 64-bit product per split and value before; 23 with the moduli shared out over
+// four warps), 7 us at N = 256 (14).  At N = 20000, 140 columns four rows take 65
+// us (82 with the loads of two moduli in flight, and the conversion and the
+// scaling on the FP64 pipe).
 // m 2^e, m >= 2^62, rounded once
 __device__ __forceinline__ double to_double(unsigned long long m, int e, bool neg) {
     if (!(m >> 63)) {
@@ -1015,6 +1011,19 @@ __device__ __forceinline__ double to_double(unsigned long long m, int e, bool ne
     else v = ldexp((double)m, e);
     return neg ? -v : v;
 }
+struct WithH {                                     // the product with H
+    static constexpr int kMods = kNMod, kWords = 2, kBits = kAlpha + kBeta;
+    static __device__ __forceinline__ unsigned long long word(int m, int i) { return kTab.m[m].w[i]; }
+    // F P 2^(x - 64)
+    static __device__ __forceinline__ double value(const unsigned long long *s, int nz, int x) {
+        const unsigned long long t = s[0] + (s[1] << 32) - kTab.bias * (unsigned)nz;
+        if (t == 0) return 0.0;
+        const bool neg = t >> 63;
+        const unsigned long long a = neg ? 0 - t : t;
+        const int lz = __clzll((long long)a);
+        return to_double(__umul64hi(a << lz, kHMant), kHExp - lz + x, neg);
+    }
+};
 struct General {                                   // the general products
     static constexpr int kMods = kGMod, kWords = 3, kBits = 2 * kGBits;
     static __device__ __forceinline__ unsigned long long word(int m, int i) { return kTab.m[m].g[i]; }
@@ -1040,67 +1049,58 @@ struct General {                                   // the general products
         return to_double(__umul64hi(hi, kGMant), kGExp - lz + x, neg);   // |F| = hi 2^(32 - lz)
     }
 };
-// v[e]: elements (i + e, j), e < ROWS, where i + e < M (i a multiple of ROWS)
+// v[e]: elements (i + e, j), e < ROWS, where i + e < M (i a multiple of ROWS).
+// The loads of kAhead moduli are in flight together: all of them where one row
+// a thread leaves few threads, four with four rows, whose sums need the registers.
 template <class Set, int ROWS>
 __device__ __forceinline__ void recombine(int64_t i, int j, int64_t M, int64_t Mp, int mp, int nz,
                                           const uchar2 *__restrict__ R, const int *__restrict__ E,
                                           const int *__restrict__ F, z_t *v) {
-    constexpr int kMods = Set::kMods;
-    constexpr int kW2 = (ROWS + 1) / 2;            // words of two rows
-    const uchar2 *r0 = R + (int64_t)j * Mp + i;
+    constexpr int kMods = Set::kMods, kW = Set::kWords, kW2 = (ROWS + 1) / 2;   // kW2: words of two rows
+    constexpr int kAhead = ROWS == 1 ? kMods : 4;
     const int64_t step = (int64_t)mp * Mp;
-    unsigned long long s[ROWS][2][Set::kWords] = {};   // [row][Re, Im][word of W]
-    auto load = [](const uchar2 *p, uint32_t *q) {
-        if constexpr (ROWS == 4) {
-            const uint2 v = *(const uint2 *)p;
-            q[0] = v.x;
-            q[1] = v.y;
-        } else {
-            q[0] = *(const uint16_t *)p;
-        }
-    };
-    auto digest = [&](int m, const uint32_t *ur, const uint32_t *ui) {   // sums, 16 bits a row
+    unsigned long long s[ROWS][2][kW] = {};        // [row][Re, Im][word of W]
 #pragma unroll
-        for (int k = 0; k < Set::kWords; k++) {
-            const unsigned long long w = Set::word(m, k);
-#pragma unroll
-            for (int e = 0; e < ROWS; e++) {
-                s[e][0][k] += (ur[e / 2] >> (16 * (e % 2)) & 0xFFFFu) * w;
-                s[e][1][k] += (ui[e / 2] >> (16 * (e % 2)) & 0xFFFFu) * w;
-            }
-        }
-    };
-    if constexpr (ROWS == 1) {
-        // few threads: the loads of all moduli in flight together
-        uint32_t ur[kMods] = {}, ui[kMods] = {};
+    for (int m0 = 0; m0 < kMods; m0 += kAhead) {
+        uint32_t ur[kAhead][kW2] = {}, ui[kAhead][kW2] = {};   // sums, 16 bits a row
+        const uchar2 *r = R + (int64_t)j * Mp + i + (int64_t)m0 * nz * step;
 #pragma unroll 1
-        for (int z = 0; z < nz; z++, r0 += step) {
-            uint32_t q[kMods];
+        for (int z = 0; z < nz; z++, r += step) {
+            uint32_t q[kAhead][kW2];
 #pragma unroll
-            for (int m = 0; m < kMods; m++) load(r0 + (int64_t)m * nz * step, &q[m]);
-#pragma unroll
-            for (int m = 0; m < kMods; m++) {
-                ur[m] += q[m] & 255;
-                ui[m] += q[m] >> 8;
-            }
-        }
-#pragma unroll
-        for (int m = 0; m < kMods; m++) digest(m, &ur[m], &ui[m]);
-    } else {
-        // many threads hide the loads, and few registers each leave room for them
-#pragma unroll 2
-        for (int m = 0; m < kMods; m++) {
-            uint32_t ur[kW2] = {}, ui[kW2] = {};
-            for (int z = 0; z < nz; z++, r0 += step) {
-                uint32_t q[kW2];
-                load(r0, q);
-#pragma unroll
-                for (int e = 0; e < kW2; e++) {
-                    ur[e] += q[e] & 0x00FF00FFu;
-                    ui[e] += q[e] >> 8 & 0x00FF00FFu;
+            for (int m = 0; m < kAhead; m++) {
+                if (m0 + m >= kMods) break;
+                const uchar2 *p = r + (int64_t)m * nz * step;
+                if constexpr (ROWS == 4) {
+                    const uint2 w = *(const uint2 *)p;
+                    q[m][0] = w.x;
+                    q[m][kW2 - 1] = w.y;
+                } else {
+                    q[m][0] = *(const uint16_t *)p;
                 }
             }
-            digest(m, ur, ui);
+#pragma unroll
+            for (int m = 0; m < kAhead; m++) {
+                if (m0 + m >= kMods) break;
+#pragma unroll
+                for (int e = 0; e < kW2; e++) {
+                    ur[m][e] += q[m][e] & 0x00FF00FFu;
+                    ui[m][e] += q[m][e] >> 8 & 0x00FF00FFu;
+                }
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < kAhead; m++) {
+            if (m0 + m >= kMods) break;
+#pragma unroll
+            for (int k = 0; k < kW; k++) {
+                const unsigned long long w = Set::word(m0 + m, k);
+#pragma unroll
+                for (int e = 0; e < ROWS; e++) {
+                    s[e][0][k] += (ur[m][e / 2] >> (16 * (e % 2)) & 0xFFFFu) * w;
+                    s[e][1][k] += (ui[m][e / 2] >> (16 * (e % 2)) & 0xFFFFu) * w;
+                }
+            }
         }
     }
     const int f = F[j];
@@ -1137,8 +1137,8 @@ k_res_reduce(int64_t M, int64_t Mp, int mp, int nz, const uchar2 *__restrict__ R
     }
 }
 
-// The general products' results (RsOut).  N = 20000, 100 columns: 60 us (76 with
-// the conversions to FP64 on the FP64 pipe).
+// The general products' results (RsOut).  N = 20000, 100 columns: 45 us (60 with
+// the loads of two moduli in flight, 76 with conversions on the FP64 pipe too).
 template <int ROWS>
 __global__ void __launch_bounds__(128)
 k_res_out(int64_t M, int64_t Mp, int mp, int nz, const uchar2 *__restrict__ R, const int *__restrict__ E,
