@@ -158,10 +158,16 @@ constexpr int kBars = 32;          // barriers of the stages, as a ring (a power
 // Variants by the widest column tile of a launch.  Converting A costs the same
 // whatever the width, so a narrow tile is bound by the converters: it has more
 // of them, which the drain threads' registers (one packed sum per column) allow.
+// Up to 96 columns tensor memory has room for stages of a whole chunk (kH = 1):
+// half the barriers and commits, and with 4 or 5 stages of B (3: the MMA warps
+// waited 150 cycles a chunk for it) N = 8000 takes 299, 319, 361, 386 us at 16, 48,
+// 80, 96 columns against 348, 374, 404, 420 with half chunks throughout; the
+// MMA warps' own instructions, about 800 cycles a chunk, set the pace (H's
+// residues cross HBM in 248 us).
 // Warpgroups (4 warps, one per TMEM quadrant): copies and MMAs; kConv converter
 // groups; two drain groups.  Registers a thread: R0, RC, RD (setmaxnreg moves
 // them from the others to the drain groups) of RL at launch; 0: no move.
-template <int W, int CONV, int SA, int SB, int HOLD, int RL, int R0, int RC, int RD>
+template <int W, int CONV, int SA, int SB, int HOLD, int H, int RL, int R0, int RC, int RD>
 struct RsCfg {
     static constexpr int kW = W;                   // columns of a tile at most
     static constexpr int kConv = CONV;
@@ -170,13 +176,14 @@ struct RsCfg {
     static constexpr int kBStage = 3 * W * kChunk * 2;
     static constexpr int kSmem = SA * kAStage + SB * kBStage + 1024;
     static constexpr int kHold = HOLD;             // granules of 8 columns a drain thread loads at once
+    static constexpr int kH = H, kCols = 32 / H;   // stages of A a chunk and product takes, their columns
     static constexpr int kR0 = R0, kRC = RC, kRD = RD;
     static_assert(128 * (R0 + CONV * RC + 2 * RD) <= kThreads * RL && 65536 / kThreads >= RL, "register split");
-    static_assert(kSmem <= 231000 && 3 * W + kMinSlots * 16 <= kTmemCols && 2 * HOLD >= W / 16, "resources");
+    static_assert(kSmem <= 231000 && 3 * W + kMinSlots * kCols <= kTmemCols && 2 * HOLD >= W / 16, "resources");
 };
-using RsWide = RsCfg<144, 2, 3, 3, 6, 96, 48, 80, 136>;
-using RsMid = RsCfg<96, 3, 5, 3, 6, 80, 48, 64, 112>;
-using RsNarrow = RsCfg<48, 4, 8, 3, 3, 72, 0, 0, 0>;
+using RsWide = RsCfg<144, 2, 3, 3, 6, 2, 96, 48, 80, 136>;
+using RsMid = RsCfg<96, 3, 5, 4, 6, 1, 80, 48, 64, 112>;
+using RsNarrow = RsCfg<48, 4, 8, 5, 3, 1, 72, 0, 0, 0>;
 static_assert((long long)kRange * kChunk * 128 * 256 <= (1ll << 24) &&
                   2ll * kRange * kChunk * 128 * 128 <= (1ll << 24), "exact FP32 sums");
 static_assert((kMaxUnitChunks / (2 * kRange) + 1) * 2 * 128 < kPack / 2, "packed sums");
@@ -209,6 +216,7 @@ constexpr uint64_t kWindDownNs = 2000000000ull;
 template <class Cfg>
 __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_constant__ RsBatch bt) {
     constexpr int kConvWarps = 4 * Cfg::kConv;
+    constexpr int kH = Cfg::kH, kCols = Cfg::kCols;
     constexpr int kSA = Cfg::kSA, kSB = Cfg::kSB, kBStage = Cfg::kBStage, kConvGroups = Cfg::kConv;
     extern __shared__ uint8_t smraw[];
     uint8_t *sm = (uint8_t *)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
@@ -234,7 +242,7 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
             tc::mbar_init(&emptyB[s], 1);
         }
         for (int s = 0; s < kBars; s++) {
-            tc::mbar_init(&aFull[s], 4);
+            tc::mbar_init(&aFull[s], kH == 1 ? 8 : 4);
             tc::mbar_init(&aEmpty[s], 1);
         }
         for (int t = 0; t < 3; t++) {
@@ -311,14 +319,17 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
         const uint32_t one = tc::elect_one() ? 1u : 0u;
         const uint32_t fullB0 = tc::smem_u32(fullB + t * kSB), emptyB0 = tc::smem_u32(emptyB + t * kSB);
         const uint32_t accF = tc::smem_u32(&accFull[t]), accE = tc::smem_u32(&accEmpty[t]);
-        const uint32_t acc = tmem + t * stride, tbeg = tmem + 3 * stride, tend = tbeg + slots * 16;
+        const uint32_t acc = tmem + t * stride, tbeg = tmem + 3 * stride, tend = tbeg + slots * kCols;
         bool ok = true;
         uint32_t sB8 = 0, sph = 0, aph = 1;        // stage of B (8 bytes a barrier), phases
         // The warp also copies its part of B (a third of the stage whatever the width:
         // the products' warps reuse a stage independently of one another), kSB - 1 chunks ahead: into the stage
         // whose MMAs it issued a chunk ago (one thread that copied A and all of B
         // spent up to 1650 cycles a chunk on it, measured, more than any other role).
-        int uL = blockIdx.x, leftL = 0, jL = 0, xL = 0, zL = 0;
+        int uL = blockIdx.x, leftL = 0, xL = 0, zL = 0;
+        const CUtensorMap *mapL = nullptr;
+        uint32_t bytesL = 0;
+        const uint32_t sB0 = tc::smem_u32(sB) + t * (kBStage / 3);
         uint32_t l8 = 0, lph = 1;
         bool rdyE = false;                         // its stage was seen free
         auto load = [&]() {
@@ -326,20 +337,15 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                 if (uL >= units) return true;
                 const Unit n = unit(uL);
                 const RsJob &a = bt.job[n.jb];
-                jL = n.jb;
+                mapL = &a.tmB;
+                bytesL = (uint32_t)a.w * kChunk * 2;
                 xL = n.x * a.w;
                 zL = (n.m * a.nch + n.c0) * 3 + t;
                 leftL = n.c1 - n.c0;
                 uL += gridDim.x;
             }
             if (!rdyE && !wait_all(emptyB0 + l8, lph)) return false;
-            if (one) {
-                const uint32_t bytes = (uint32_t)bt.job[jL].w * kChunk * 2;
-                uint64_t *bar = &fullB[t * kSB + l8 / 8];
-                tc::mbar_expect_tx(bar, bytes);
-                tc::tma_load_3d(sB + l8 / 8 * kBStage + t * (kBStage / 3), &bt.job[jL].tmB, 0, xL, zL, bar);
-            }
-            __syncwarp();
+            tc::tma_load_3d_if(one, sB0 + l8 * (kBStage / 8), mapL, 0, xL, zL, fullB0 + l8, bytesL);
             fills++;
             zL += 3;
             leftL--;
@@ -348,18 +354,18 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
             return true;
         };
         for (int s = 0; s + 1 < kSB; s++) load();   // fresh barriers: no wait
-        // The product's stage of a half chunk, its barrier and phase.  A wait that
-        // succeeds costs a warp about 100 cycles, so the barriers of the next half
-        // chunk are looked at (without blocking) before this one's MMAs are issued,
+        // The product's stage of a chunk (or half of it), its barrier and phase.  A wait that
+        // succeeds costs a warp about 100 cycles, so the barriers of the next
+        // stage are looked at (without blocking) before this one's MMAs are issued,
         // and waited for only if that look failed.
-        uint32_t f8 = 8 * t, bph = 0, at = tbeg + 16 * t;
+        uint32_t f8 = 8 * t, bph = 0, at = tbeg + kCols * t;
         bool rdy = false, rdyB = false;
         auto next = [&]() { return bars | f8; };
         auto advance = [&]() {
             f8 += 24;
             if (f8 > kBarMask) { f8 &= kBarMask; bph ^= 1; }
-            at += 48;
-            if (at >= tend) at -= slots * 16;
+            at += 3 * kCols;
+            if (at >= tend) at -= slots * kCols;
         };
         for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
             const Unit n = unit(u);
@@ -374,33 +380,35 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                 // a fresh barrier passes the wait for the phase before its first
                 if (fresh && !wait_all(accE, aph)) { ok = false; break; }
                 const uint64_t bd = bd0 + (uint64_t)(sB8 * (kBStage / 8 >> 4));
-                const uint32_t b0 = next();
-                if (!rdy && !wait_all(b0, bph)) { ok = false; break; }
-                tc::fence_after();
-                const uint32_t t0 = at;
-                advance();
-                const uint32_t b1 = next();
-                bool look = tc::mbar_test_at(b1, bph);
-                tc::mma_f16_ta_if(one, acc, t0, bd, id, fresh ^ 1);
-                tc::mma_f16_ta_if(one, acc, t0 + 8, bd + 2, id, 1u);
-                tc::mma_commit_if(one, b0 + kBarEmpty);
-                rdy = __all_sync(0xffffffffu, look) != 0;
-                if (!rdy && !wait_all(b1, bph)) { ok = false; break; }
-                tc::fence_after();
-                const uint32_t t1 = at, eB = emptyB0 + sB8;
-                advance();
-                sB8 += 8;
-                if (sB8 == 8 * kSB) { sB8 = 0; sph ^= 1; }
-                look = tc::mbar_test_at(next(), bph);
-                const bool lookB = tc::mbar_test_at(fullB0 + sB8, sph), lookE = tc::mbar_test_at(emptyB0 + l8, lph);
-                tc::mma_f16_ta_if(one, acc, t1, bd + 4, id, 1u);
-                tc::mma_f16_ta_if(one, acc, t1 + 8, bd + 6, id, 1u);
-                tc::mma_commit_if(one, b1 + kBarEmpty);
-                tc::mma_commit_if(one, eB);
-                if (end) tc::mma_commit_if(one, accF);
+                bool lookB = false, lookE = false;
+#pragma unroll
+                for (int h = 0; h < kH; h++) {
+                    const uint32_t b0 = next();
+                    if (!rdy && !wait_all(b0, bph)) { ok = false; break; }
+                    tc::fence_after();
+                    const uint32_t t0 = at, eB = emptyB0 + sB8;
+                    advance();
+                    const bool look = tc::mbar_test_at(next(), bph);
+                    if (h == kH - 1) {
+                        sB8 += 8;
+                        if (sB8 == 8 * kSB) { sB8 = 0; sph ^= 1; }
+                        lookB = tc::mbar_test_at(fullB0 + sB8, sph);
+                        lookE = tc::mbar_test_at(emptyB0 + l8, lph);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4 / kH; k++)
+                        tc::mma_f16_ta_if(one, acc, t0 + 8 * k, bd + 2 * (h * (4 / kH) + k), id,
+                                          h + k == 0 ? fresh ^ 1 : 1u);
+                    tc::mma_commit_if(one, b0 + kBarEmpty);
+                    if (h == kH - 1) {
+                        tc::mma_commit_if(one, eB);
+                        if (end) tc::mma_commit_if(one, accF);
+                    }
+                    rdy = __all_sync(0xffffffffu, look) != 0;
+                }
+                if (!ok) break;
                 fresh = end;
                 aph ^= end;
-                rdy = __all_sync(0xffffffffu, look) != 0;
                 rdyB = __all_sync(0xffffffffu, lookB) != 0;
                 rdyE = __all_sync(0xffffffffu, lookE) != 0;
                 if (!load()) { ok = false; break; }
@@ -410,20 +418,23 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
     } else if (warp < 4 + kConvWarps) {
         if (Cfg::kRC) tc::reg_dec<Cfg::kRC ? Cfg::kRC : 24>();
         // The groups take turns, half a chunk (32 K elements) each: item 2 chunk + h.
-        // Its i-th operand is fill 3 item + i of the ring of stages, and waits for
-        // the MMAs on the fill `slots` before it.
+        // (Publishing the three operands one by one costs nothing with kH = 2, whose
+        // few stages the MMAs wait for.)
+        // Its i-th operand is (with kH = 1 its half of) fill 3 item + i (3 chunk + i)
+        // of the ring of stages, and waits for the MMAs on the fill `slots` before it.
         const int quad = warp & 3, row = quad * 32 + lane;
         const __half2 k1152 = __floats2half2_rn(1152.f, 1152.f);
         int item = (warp - 4) >> 2;
-        uint32_t f8 = 24 * item;                   // the fill's barrier
-        uint32_t e8 = 8 * (3 * item - slots), eph = 1;   // of the fill it waits for (modulo the ring)
+        const int first = kH == 1 ? item >> 1 : item;
+        uint32_t f8 = 24 * first;                  // the fill's barrier
+        uint32_t e8 = 8 * (3 * first - slots), eph = 1;   // of the fill it waits for (modulo the ring)
         if ((int)e8 >= 0) eph = 0;
         e8 &= kBarMask;
-        const uint32_t tbeg = tmem + ((uint32_t)(quad * 32) << 16) + 3 * stride, tend = tbeg + slots * 16;
-        uint32_t ta = tbeg + 3 * item % slots * 16;
-        const uint32_t skip = 3 * (kConvGroups - 1) % slots * 16;
+        const uint32_t tbeg = tmem + ((uint32_t)(quad * 32) << 16) + 3 * stride, tend = tbeg + slots * kCols;
+        uint32_t ta = tbeg + 3 * first % slots * kCols;
         uint32_t sa8 = 8 * (item >> 1), saph = 0;  // stage of A's bytes (8 bytes a barrier), and its phase
-        static_assert((kConvGroups - 1) / 2 < kSA && (kConvGroups + 1) / 2 <= kSA, "one turn of the ring at most");
+        static_assert((kConvGroups - 1) / 2 < kSA && (kConvGroups + 1) / 2 <= kSA && kConvGroups >= 2 &&
+                          3 * ((kH == 1 ? (kConvGroups + 1) / 2 : kConvGroups) - 1) <= kMinSlots, "one turn of the ring at most");
         const uint32_t fullA0 = tc::smem_u32(fullA), emptyA0 = tc::smem_u32(emptyA);
         auto convert = [&](const uint8_t *src, uint32_t *r) {
 #pragma unroll
@@ -440,21 +451,27 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                 }
             }
         };
-        auto put = [&](const uint32_t *r) {
+        // store an operand's columns: waits for the stage; publish tells the MMAs of
+        // the last n stored
+        auto put = [&](const uint32_t *r, int h) {
             // a fresh barrier passes the wait for the phase before its first
             if (!wait_all(bars | kBarEmpty | e8, eph)) return false;
             tc::fence_after();
-            tc::tmem_st16(ta, r);
-            ta += 16;
+            tc::tmem_st16(kH == 1 ? ta + 16 * h : ta, r);
+            ta += kCols;
             if (ta == tend) ta = tbeg;
-            tc::tmem_wait_st();
-            tc::fence_before();
-            __syncwarp();
-            if (lane == 0) tc::mbar_arrive_at(bars | f8);
-            f8 = (f8 + 8) & kBarMask;
             e8 += 8;
             if (e8 > kBarMask) { e8 = 0; eph ^= 1; }
             return true;
+        };
+        auto publish = [&](int n) {
+            tc::tmem_wait_st();
+            tc::fence_before();
+            __syncwarp();
+            for (int k = 0; k < n; k++) {
+                if (lane == 0) tc::mbar_arrive_at(bars | f8);
+                f8 = (f8 + 8) & kBarMask;
+            }
         };
         // item counts over all units; i is its number in its unit
         int done = 0;
@@ -471,7 +488,10 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                 convert(src + 4 * kRows * 16, im);
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive_at(emptyA0 + sa8);
-                if (!put(re) || !put(im)) { ok = false; break; }
+                if (!put(re, h)) { ok = false; break; }
+                if (kH == 2) publish(1);
+                if (!put(im, h)) { ok = false; break; }
+                if (kH == 2) publish(1);
 #pragma unroll
                 for (int e = 0; e < 16; e++) {
                     __half2 a, b;
@@ -480,14 +500,16 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                     a = __hadd2(a, b);             // in [-256, 254]: exact
                     memcpy(&re[e], &a, 4);
                 }
-                if (!put(re)) { ok = false; break; }
+                if (!put(re, h)) { ok = false; break; }
+                publish(kH == 2 ? 1 : 3);
                 // past the other groups' items
-                f8 = (f8 + 24 * (kConvGroups - 1)) & kBarMask;
-                e8 += 24 * (kConvGroups - 1);
+                const int chunks = (h + kConvGroups) / 2, over = (kH == 1 ? chunks : kConvGroups) - 1;
+                f8 = (f8 + 24 * over) & kBarMask;
+                e8 += 24 * over;
                 if (e8 > kBarMask) { e8 &= kBarMask; eph ^= 1; }
-                ta += skip;
-                if (ta >= tend) ta -= slots * 16;
-                sa8 += (h + kConvGroups) / 2 * 8;
+                ta += 3 * kCols * over;            // at most one turn of the ring
+                if (ta >= tend) ta -= slots * kCols;
+                sa8 += chunks * 8;
                 if (sa8 >= 8 * kSA) { sa8 -= 8 * kSA; saph ^= 1; }
             }
             done += ni;
@@ -1306,7 +1328,8 @@ double residue_flops(int64_t M, int64_t K, int n) { return 6.0 * kNMod * (double
 
 namespace {
 template <class Cfg>
-cudaError_t launch_cfg(const RsBatch &b, int sms, cudaStream_t st) {
+cudaError_t launch_cfg(RsBatch &b, int sms, cudaStream_t st) {
+    b.slots = std::min((kTmemCols - 3 * b.stride) / Cfg::kCols, kMaxSlots);
     static std::once_flag once[kMaxDevices];
     static cudaError_t attr[kMaxDevices];
     const cudaError_t ae = smem_attr_once(once, attr, (const void *)k_res_zgemm<Cfg>, Cfg::kSmem);
@@ -1320,7 +1343,6 @@ cudaError_t launch_cfg(const RsBatch &b, int sms, cudaStream_t st) {
 cudaError_t residue_launch(RsBatch &b, int sms, cudaStream_t st) {
     b.stride = 16;
     for (int j = 0; j < b.njobs; j++) b.stride = std::max(b.stride, b.job[j].w);
-    b.slots = std::min((kTmemCols - 3 * b.stride) / 16, kMaxSlots);
     if (b.stride <= RsNarrow::kW) return launch_cfg<RsNarrow>(b, sms, st);
     if (b.stride <= RsMid::kW) return launch_cfg<RsMid>(b, sms, st);
     return launch_cfg<RsWide>(b, sms, st);

@@ -140,6 +140,19 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, i
         : "memory");
 }
 
+// The copy with its barrier's expected bytes, by the lane whose `one` is set
+// (predicated, without a branch around it).
+__device__ __forceinline__ void tma_load_3d_if(uint32_t one, uint32_t dst, const CUtensorMap *map, int x, int y, int z,
+                                               uint32_t bar, uint32_t bytes) {
+    asm volatile(
+        "{\n .reg .pred q;\n setp.ne.b32 q, %7, 0;\n"
+        " @q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%5], %6;\n"
+        " @q cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4}], [%5];\n}\n" ::"r"(dst),
+        "l"((uint64_t)map), "r"(x), "r"(y), "r"(z), "r"(bar), "r"(bytes), "r"(one)
+        : "memory");
+}
+
 // Untiled bulk copy of `bytes` (a multiple of 16; both addresses 16-byte aligned).
 __device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
     asm volatile(
