@@ -178,18 +178,24 @@ int sync_scalars(bsechase_ctx *ctx) {
 
 }  // namespace
 
-HopBytes hop_bytes(int64_t N, int mc, bool res, bool tri, bool bse) {
+HopBytes hop_bytes(int64_t N, int mc, bool res, bool tri, bool bse, bool gen) {
     HopBytes h;
-    h.GA = std::max(ozaki_gen_a_bytes(mc, N), ozaki_gen_a_bytes(N, mc));
     if (res) {
         h.A = residue_a_bytes(N, N);
-        h.B = std::max(residue_b_bytes(N, mc), ozaki_b_bytes(N, mc));
+        h.B = residue_b_bytes(N, mc);
         if (bse) h.B = std::max(h.B, residue_panel_bytes(N));
-        h.P = std::max({residue_r_bytes(N, N, mc), residue_work_bytes(N), ozaki_gen_partial_bytes(N, mc)});
+        h.P = std::max(residue_r_bytes(N, N, mc), residue_work_bytes(N));
+        if (gen) {
+            // residue_buffers for up to mc columns kept and not, padded separately
+            h.B = std::max(h.B, residue_right_bytes(N, mc + 64) + 1024);
+            h.P = std::max({h.P, residue_out_bytes(mc, N, mc), residue_out_bytes(N, mc, mc)});
+            h.GA = residue_left_bytes(N, mc + 256) + 1024;
+        }
     } else {
         h.A = tri ? ozaki_a_bytes_tri(N) : ozaki_a_bytes(N);
         h.B = ozaki_b_bytes(N, mc);
         h.P = ozaki_partial_bytes(N, mc);
+        h.GA = std::max(ozaki_gen_a_bytes(mc, N), ozaki_gen_a_bytes(N, mc));
     }
     return h;
 }
@@ -210,23 +216,29 @@ struct Hop {
     const BseSource *bse = nullptr;   // H not stored: its slices from the generator
     bool tri = false;    // half storage of the slices (lower triangle of H only)
     bool res = false;    // products in residues (residue.cu): the FP64 mode on full storage
+    bool gen = false;    // ... and a solve's general products too
 };
+
+// exponents and column norms of residue_buffers
+constexpr size_t kResParts = (size_t)kMaxM * kRsColParts;
+constexpr size_t kResFBytes = 2 * kResParts * sizeof(float2) + 2 * kMaxM * sizeof(int);
 
 size_t hop_f_bytes(int mc) { return ((size_t)(mc + 64) * sizeof(int) + 15) / 16 * 16; }
 
 int hop_buffers(bsechase_ctx *ctx, const Hop &op, int mc) {
     int rc;
     const int64_t Np = ozaki_padded(op.N);
-    const HopBytes hb = hop_bytes(op.N, mc, op.res, op.tri, op.bse != nullptr);
+    const HopBytes hb = hop_bytes(op.N, mc, op.res, op.tri, op.bse != nullptr, op.gen);
     if ((rc = ensure(ctx, ctx->ozA, hb.A))) return rc;
     if (op.tri && (rc = ensure(ctx, ctx->ozT, (size_t)2 * Np * sizeof(double)))) return rc;
     if ((rc = ensure(ctx, ctx->ozE, (size_t)Np * sizeof(int)))) return rc;
+    const size_t fb = hop_f_bytes(mc) + (op.res ? (size_t)mc * 32 * sizeof(float2) : 0);
     if ((rc = ensure(ctx, ctx->ozB, hb.B))) return rc;
-    if ((rc = ensure(ctx, ctx->ozF, hop_f_bytes(mc) + (op.res ? (size_t)mc * 32 * sizeof(float2) : 0)))) return rc;
+    if ((rc = ensure(ctx, ctx->ozF, std::max(fb, op.gen ? kResFBytes : 0)))) return rc;
     if ((rc = ensure(ctx, ctx->ozP, hb.P))) return rc;
     // general products of QR and Rayleigh-Ritz: op(A) is m x N (A^H) or N x m
     if ((rc = ensure(ctx, ctx->ozGA, hb.GA))) return rc;
-    return ensure(ctx, ctx->ozGE, (size_t)(Np + 512) * sizeof(int));
+    return ensure(ctx, ctx->ozGE, (size_t)(op.gen ? 2 : 1) * (Np + 512) * sizeof(int));
 }
 
 void free_product_buffers(bsechase_ctx *ctx) {
@@ -252,7 +264,7 @@ int hop_prepare(bsechase_ctx *ctx, Hop &op, int max_cols) {
     if (rc == BSE_ENOMEM && op.res) {
         // the residues take 2 N^2 bytes more than the slices: those, where only
         // they fit
-        op.res = false;
+        op.res = op.gen = false;
         free_product_buffers(ctx);
         rc = hop_buffers(ctx, op, mc);
     }
@@ -496,94 +508,6 @@ int cholqr_pass(bsechase_ctx *ctx, z_t *V, int64_t ldv, int64_t N, int m, double
     return BSE_OK;
 }
 
-// The general products in residues (residue.cu): their buffers, shared with the
-// products with H, for left operands of at most m columns of N, a kept block of
-// k columns in both roles, and right operands of m columns.
-struct ResBufs {
-    RsSide VA, VB, LA, LB;
-    void *R;
-    size_t r_bytes;
-};
-int residue_buffers(bsechase_ctx *ctx, int64_t N, int m, int k, bool tall, ResBufs *b) {
-    auto up = [](size_t x) { return (x + 1023) / 1024 * 1024; };
-    const int64_t Np = ozaki_padded(N), mk = std::max(m, k);
-    const size_t va = up(std::max(residue_left_bytes(m, N), tall ? residue_left_bytes(N, m) : 0));
-    const size_t la = k > 0 && tall ? residue_left_bytes(N, k) : 0;
-    const size_t vb = up(residue_right_bytes(N, tall ? m : k)), lb = k > 0 && tall ? residue_right_bytes(N, k) : 0;
-    size_t r = residue_out_bytes(m, N, (int)mk);
-    if (tall) r = std::max(r, residue_out_bytes(N, mk, m));
-    const size_t ne = (size_t)(Np + 512), parts = (size_t)kMaxM * kRsColParts;
-    int rc;
-    if ((rc = ensure(ctx, ctx->ozGA, va + la)) || (rc = ensure(ctx, ctx->ozB, vb + lb)) ||
-        (rc = ensure(ctx, ctx->ozP, r)) || (rc = ensure(ctx, ctx->ozGE, 2 * ne * sizeof(int))) ||
-        (rc = ensure(ctx, ctx->ozF, 2 * parts * sizeof(float2) + 2 * kMaxM * sizeof(int))))
-        return rc;
-    float2 *part = (float2 *)ctx->ozF.p;
-    int *f = (int *)(part + 2 * parts), *e = (int *)ctx->ozGE.p;
-    b->VA = RsSide{ctx->ozGA.p, va, e, part};
-    b->LA = RsSide{(char *)ctx->ozGA.p + va, la, e + ne, nullptr};
-    b->VB = RsSide{ctx->ozB.p, vb, f, part + parts};
-    b->LB = RsSide{(char *)ctx->ozB.p + vb, lb, f + kMaxM, part + parts};
-    b->R = ctx->ozP.p;
-    b->r_bytes = ctx->ozP.bytes;
-    return BSE_OK;
-}
-
-// phase_qr in residues.  L is turned into residues once for the four
-// projections, in both its roles; a projection multiplies V^H L (the wide block
-// on the left, a byte a residue) and stores its adjoint; the results go to V
-// itself.
-int phase_qr_residues(bsechase_ctx *ctx, const ResBufs &b, const z_t *L, int64_t ldl, int k, z_t *V, int64_t ldv,
-                      int64_t N, int m) {
-    cudaStream_t st = ctx->st;
-    const int sms = ctx->sms;
-    ChaseScalars *sc = ctx->sc;
-    z_t *X = (z_t *)ctx->R.p, *G = (z_t *)ctx->G.p, *Ri = (z_t *)ctx->Ri.p;
-    auto product = [&](int64_t M, int n, int64_t K, const RsSide &A, const RsSide &B, const RsOut &o) {
-        return residue_product(M, n, K, A, B, o, b.R, b.r_bytes, kDefaultWaitNs, sc, sms, st);
-    };
-    auto proj = [&]() -> int {
-        if (k <= 0) return BSE_OK;
-        RsOut x{X, k}, v{V, ldv, V, ldv};
-        x.adjoint = 1;
-        CK(residue_left(m, N, V, ldv, true, b.VA, sc, st));
-        CK(product(m, k, N, b.VA, b.LB, x));
-        CK(residue_right(k, m, X, k, nullptr, b.VB, sc, sms, st));
-        CK(product(N, m, k, b.LA, b.VB, v));
-        return BSE_OK;
-    };
-    auto cholqr = [&](double shift) -> int {
-        RsOut g{G, m}, v{V, ldv};
-        g.shift = shift;
-        g.mirror = 1;
-        CK(residue_left(m, N, V, ldv, true, b.VA, sc, st));
-        CK(residue_right(N, m, V, ldv, b.VA.part, b.VB, sc, sms, st));
-        CK(product(m, m, N, b.VA, b.VB, g));
-        CK(launch_cholesky(m, G, m, sc, st));
-        CK(launch_trinv(m, G, m, Ri, m, st));
-        CK(residue_left(N, m, V, ldv, false, b.VA, sc, st));
-        CK(residue_right(m, m, Ri, m, nullptr, b.VB, sc, sms, st));
-        CK(product(N, m, m, b.VA, b.VB, v));
-        return BSE_OK;
-    };
-    int rc;
-    Small s = small_layout(ctx, m);
-    if (k > 0) {
-        CK(residue_right(N, k, L, ldl, nullptr, b.LB, sc, sms, st));
-        CK(residue_left(N, k, L, ldl, false, b.LA, sc, st));
-    }
-    if ((rc = proj())) return rc;
-    if ((rc = proj())) return rc;
-    CK(launch_normalize_cols(N, m, V, ldv, (double *)ctx->part.p, s.norms, sc, st));
-    // columns have unit norm, so ||V||_F^2 = m
-    if ((rc = cholqr(11.0 * ((double)N * m + (double)m * (m + 1)) * kU * (double)m))) return rc;
-    for (int pass = 0; pass < 2; pass++) {
-        if ((rc = proj())) return rc;
-        if ((rc = cholqr(0.0))) return rc;
-    }
-    return BSE_OK;
-}
-
 int phase_qr(bsechase_ctx *ctx, const z_t *L, int64_t ldl, int k, z_t *V, int64_t ldv, int64_t N,
              int m) {
     int rc;
@@ -599,6 +523,126 @@ int phase_qr(bsechase_ctx *ctx, const z_t *L, int64_t ldl, int k, z_t *V, int64_
         if ((rc = project(ctx, L, ldl, k, V, ldv, N, m))) return rc;
         if ((rc = cholqr_pass(ctx, V, ldv, N, m, 0.0))) return rc;
     }
+    return BSE_OK;
+}
+
+// The general products in residues (residue.cu): their buffers, shared with the
+// products with H, for left operands of at most m columns of N, a kept block of
+// k columns in both roles, and right operands of m columns.
+struct ResBufs {
+    RsSide VA, VB, LA, LB;
+    void *R;
+    size_t r_bytes;
+    uint64_t wait_ns = kDefaultWaitNs;
+};
+cudaError_t residue_mul(bsechase_ctx *ctx, const ResBufs &b, int64_t M, int n, int64_t K, const RsSide &A,
+                        const RsSide &B, const RsOut &o) {
+    return residue_product(M, n, K, A, B, o, b.R, b.r_bytes, b.wait_ns, ctx->sc, ctx->sms, ctx->st);
+}
+int residue_buffers(bsechase_ctx *ctx, int64_t N, int m, int k, bool tall, ResBufs *b) {
+    auto up = [](size_t x) { return (x + 1023) / 1024 * 1024; };
+    const int64_t Np = ozaki_padded(N), mk = std::max(m, k);
+    const size_t va = up(std::max(residue_left_bytes(m, N), tall ? residue_left_bytes(N, m) : 0));
+    const size_t la = k > 0 && tall ? residue_left_bytes(N, k) : 0;
+    const size_t vb = up(residue_right_bytes(N, tall ? m : k)), lb = k > 0 && tall ? residue_right_bytes(N, k) : 0;
+    size_t r = residue_out_bytes(m, N, (int)mk);
+    if (tall) r = std::max(r, residue_out_bytes(N, mk, m));
+    const size_t ne = (size_t)(Np + 512), parts = kResParts;
+    int rc;
+    if ((rc = ensure(ctx, ctx->ozGA, va + la)) || (rc = ensure(ctx, ctx->ozB, vb + lb)) ||
+        (rc = ensure(ctx, ctx->ozP, r)) || (rc = ensure(ctx, ctx->ozGE, 2 * ne * sizeof(int))) ||
+        (rc = ensure(ctx, ctx->ozF, kResFBytes)))
+        return rc;
+    float2 *part = (float2 *)ctx->ozF.p;
+    int *f = (int *)(part + 2 * parts), *e = (int *)ctx->ozGE.p;
+    b->VA = RsSide{ctx->ozGA.p, va, e, part};
+    b->LA = RsSide{(char *)ctx->ozGA.p + va, la, e + ne, nullptr};
+    b->VB = RsSide{ctx->ozB.p, vb, f, part + parts};
+    b->LB = RsSide{(char *)ctx->ozB.p + vb, lb, f + kMaxM, part + parts};
+    b->R = ctx->ozP.p;
+    b->r_bytes = ctx->ozP.bytes;
+    return BSE_OK;
+}
+
+// cholqr_pass in residues; the result goes to V itself
+int cholqr_residues(bsechase_ctx *ctx, const ResBufs &b, z_t *V, int64_t ldv, int64_t N, int m, double shift) {
+    cudaStream_t st = ctx->st;
+    ChaseScalars *sc = ctx->sc;
+    z_t *G = (z_t *)ctx->G.p, *Ri = (z_t *)ctx->Ri.p;
+    RsOut g{G, m}, v{V, ldv};
+    g.shift = shift;
+    g.mirror = 1;
+    CK(residue_left(m, N, V, ldv, true, b.VA, sc, st));
+    CK(residue_right(N, m, V, ldv, b.VA.part, b.VB, sc, ctx->sms, st));
+    CK(residue_mul(ctx, b, m, m, N, b.VA, b.VB, g));
+    CK(launch_cholesky(m, G, m, sc, st));
+    CK(launch_trinv(m, G, m, Ri, m, st));
+    CK(residue_left(N, m, V, ldv, false, b.VA, sc, st));
+    CK(residue_right(m, m, Ri, m, nullptr, b.VB, sc, ctx->sms, st));
+    CK(residue_mul(ctx, b, N, m, m, b.VA, b.VB, v));
+    return BSE_OK;
+}
+
+// phase_qr in residues.  L is turned into residues once for the four
+// projections, in both its roles; a projection multiplies V^H L (the wide block
+// on the left, a byte a residue) and stores its adjoint.
+int phase_qr_residues(bsechase_ctx *ctx, const ResBufs &b, const z_t *L, int64_t ldl, int k, z_t *V, int64_t ldv,
+                      int64_t N, int m) {
+    if (m <= 0) return BSE_OK;
+    cudaStream_t st = ctx->st;
+    const int sms = ctx->sms;
+    ChaseScalars *sc = ctx->sc;
+    z_t *X = (z_t *)ctx->R.p;
+    auto proj = [&]() -> int {
+        if (k <= 0) return BSE_OK;
+        RsOut x{X, k}, v{V, ldv, V, ldv};
+        x.adjoint = 1;
+        CK(residue_left(m, N, V, ldv, true, b.VA, sc, st));
+        CK(residue_mul(ctx, b, m, k, N, b.VA, b.LB, x));
+        CK(residue_right(k, m, X, k, nullptr, b.VB, sc, sms, st));
+        CK(residue_mul(ctx, b, N, m, k, b.LA, b.VB, v));
+        return BSE_OK;
+    };
+    int rc;
+    Small s = small_layout(ctx, m);
+    if (k > 0) {
+        CK(residue_right(N, k, L, ldl, nullptr, b.LB, sc, sms, st));
+        CK(residue_left(N, k, L, ldl, false, b.LA, sc, st));
+    }
+    if ((rc = proj())) return rc;
+    if ((rc = proj())) return rc;
+    CK(launch_normalize_cols(N, m, V, ldv, (double *)ctx->part.p, s.norms, sc, st));
+    // columns have unit norm, so ||V||_F^2 = m
+    const double shift = 11.0 * ((double)N * m + (double)m * (m + 1)) * kU * (double)m;
+    if ((rc = cholqr_residues(ctx, b, V, ldv, N, m, shift))) return rc;
+    for (int pass = 0; pass < 2; pass++) {
+        if ((rc = proj())) return rc;
+        if ((rc = cholqr_residues(ctx, b, V, ldv, N, m, 0.0))) return rc;
+    }
+    return BSE_OK;
+}
+
+// phase_rr in residues
+int phase_rr_residues(bsechase_ctx *ctx, const Hop &op, const ResBufs &b, const z_t *Q, int64_t ldq, int m,
+                      double *theta, z_t *Vout, z_t *HVout) {
+    const int64_t N = op.N;
+    cudaStream_t st = ctx->st;
+    ChaseScalars *sc = ctx->sc;
+    z_t *W = (z_t *)ctx->B1.p, *G = (z_t *)ctx->G.p, *Yr = (z_t *)ctx->Yr.p;
+    GemmEpi plain{};
+    int rc;
+    if ((rc = hop_apply(ctx, op, m, Q, ldq, W, N, plain))) return rc;
+    RsOut g{G, m};
+    g.mirror = 1;
+    CK(residue_left(m, N, Q, ldq, true, b.VA, sc, st));
+    CK(residue_right(N, m, W, N, nullptr, b.VB, sc, ctx->sms, st));
+    CK(residue_mul(ctx, b, m, m, N, b.VA, b.VB, g));
+    CK(launch_heev(m, G, m, theta, Yr, m, ctx->heev.p, sc, st));
+    CK(residue_right(m, m, Yr, m, nullptr, b.VB, sc, ctx->sms, st));
+    CK(residue_left(N, m, Q, ldq, false, b.VA, sc, st));
+    CK(residue_mul(ctx, b, N, m, m, b.VA, b.VB, RsOut{Vout, N}));
+    CK(residue_left(N, m, W, N, false, b.VA, sc, st));
+    CK(residue_mul(ctx, b, N, m, m, b.VA, b.VB, RsOut{HVout, N}));
     return BSE_OK;
 }
 
@@ -628,7 +672,7 @@ int gram_residues(bsechase_ctx *ctx, const z_t *A, int64_t lda, const z_t *B, in
     CK(cudaMemsetAsync(ctx->sc, 0, sizeof(ChaseScalars), ctx->st));
     CK(residue_left(m1, K, A, lda, true, b.VA, ctx->sc, ctx->st));
     CK(residue_right(K, m2, B, ldb, same ? b.VA.part : nullptr, b.VB, ctx->sc, ctx->sms, ctx->st));
-    CK(residue_product(m1, m2, K, b.VA, b.VB, o, b.R, b.r_bytes, kDefaultWaitNs, ctx->sc, ctx->sms, ctx->st));
+    CK(residue_mul(ctx, b, m1, m2, K, b.VA, b.VB, o));
     return sync_scalars(ctx);
 }
 
@@ -743,6 +787,7 @@ int solve_device(bsechase_ctx *ctx, const z_t *H, int64_t N, int64_t ldh, int ne
     op.bse = bse;
     op.tri = o.half_storage == 1;
     op.res = ctx->residues && precision_uses_residues(precision, op.tri);
+    op.gen = op.res;
     if ((rc = hop_prepare(ctx, op, m_cap))) return rc;
     GenTcScope gen_scope(ctx, op.tc);
     if ((rc = phase_lanczos(ctx, op, m, o.lanczos_steps, o.lanczos_vecs, o.seed))) return rc;
@@ -808,9 +853,19 @@ int solve_device(bsechase_ctx *ctx, const z_t *H, int64_t N, int64_t ldh, int ne
         if (fop.level == OZ_S4) filter_mv_low += mv;
         if (fop.level == OZ_S5) filter_mv_mid += mv;
         tm.mark(3);
-        if ((rc = phase_qr(ctx, V, N, locked, Va, N, N, ma))) return rc;
+        ResBufs rb;
+        if (op.res) {
+            if ((rc = residue_buffers(ctx, N, ma, locked, true, &rb))) return rc;
+            rb.wait_ns = ctx->wait_ns;
+            rc = phase_qr_residues(ctx, rb, V, N, locked, Va, N, N, ma);
+        } else {
+            rc = phase_qr(ctx, V, N, locked, Va, N, N, ma);
+        }
+        if (rc) return rc;
         tm.mark(4);
-        if ((rc = phase_rr(ctx, op, Va, N, ma, s.theta, B2, B3))) return rc;
+        if (op.res) rc = phase_rr_residues(ctx, op, rb, Va, N, ma, s.theta, B2, B3);
+        else rc = phase_rr(ctx, op, Va, N, ma, s.theta, B2, B3);
+        if (rc) return rc;
         matvecs += ma;
         tm.mark(5);
         CK(launch_residuals(N, ma, B3, N, B2, N, s.theta, s.resid, (double *)ctx->part.p, ctx->sc,
@@ -874,7 +929,13 @@ int solve_device(bsechase_ctx *ctx, const z_t *H, int64_t N, int64_t ldh, int ne
     }
     CK(cudaMemcpyAsync(s.order, order.data(), nev * sizeof(int), cudaMemcpyHostToDevice, ctx->st));
     CK(launch_copy_cols(N, nev, V, N, d_evecs, ldz, s.order, ctx->st));
-    if (op.tc) {
+    if (op.res) {
+        // a last pass restores FP64 orthonormality across the locked blocks
+        ResBufs rb;
+        if ((rc = residue_buffers(ctx, N, nev, 0, true, &rb))) return rc;
+        rb.wait_ns = ctx->wait_ns;
+        if ((rc = cholqr_residues(ctx, rb, d_evecs, ldz, N, nev, 0.0))) return rc;
+    } else if (op.tc) {
         // The Ritz vectors went through tensor-core products whose 48-bit
         // slices leave an orthogonality error near 1e-12; one native FP64
         // Cholesky QR pass of the nev output vectors (their Gram matrix is

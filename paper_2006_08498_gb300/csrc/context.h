@@ -80,11 +80,12 @@ int solve_device(bsechase_ctx *ctx, const z_t *H, int64_t N, int64_t ldh, int ne
                  const BseSource *bse = nullptr);
 // Device bytes that the products with H of an N x N solve of up to mc columns
 // take: H's slices or residues, those of the operand, the partial results, and
-// the slices of op(A) in the general products of QR and Rayleigh-Ritz.
+// those of op(A) in the general products of QR and Rayleigh-Ritz (residues: with
+// gen, a solve).
 struct HopBytes {
     size_t A = 0, B = 0, P = 0, GA = 0;
 };
-HopBytes hop_bytes(int64_t N, int mc, bool res, bool tri, bool bse);
+HopBytes hop_bytes(int64_t N, int mc, bool res, bool tri, bool bse, bool gen);
 // Whether the products with H run in residues (residue.cu): the FP64 mode on
 // full storage.
 bool precision_uses_residues(int precision, bool half);

@@ -85,8 +85,6 @@ size_t ozaki_a_bytes_tri(int64_t N);
 size_t ozaki_b_bytes(int64_t N, int m);
 // workspace for split-K partial products of up to m columns
 size_t ozaki_partial_bytes(int64_t N, int m);
-// ... of the general products alone (ozaki_gemm) of a search space of m columns
-size_t ozaki_gen_partial_bytes(int64_t N, int m);
 
 // General FP64-accurate products on the tensor cores (same kernel and
 // slicing as the product with H): C (M x n) = out(op(A) B), op(A) = A

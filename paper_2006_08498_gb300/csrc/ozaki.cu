@@ -1364,12 +1364,6 @@ size_t ozaki_partial_bytes(int64_t N, int m) {
            std::max<int64_t>(16 * kW, std::max<int64_t>(8, sp0) * (int64_t)mp);
 }
 
-size_t ozaki_gen_partial_bytes(int64_t N, int m) {
-    // N x m outputs over K <= 512 (one split), m x m outputs over K = N
-    const int64_t nch = ozaki_padded(N) / kKC, sp = (nch + kUnitChunks - 1) / kUnitChunks + 32;
-    return (size_t)(kPartWords * 8) * m * std::max<int64_t>(N, m * sp);
-}
-
 size_t ozaki_b_bytes(int64_t N, int m) {
     const int64_t Np = ozaki_padded(N);
     const int mp = (m + kW - 1) / kW * kW;

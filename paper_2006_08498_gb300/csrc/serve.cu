@@ -89,7 +89,7 @@ size_t estimate_run_bytes(int64_t N, int m, int nev, int precision, bool own_h, 
     b += 16 * (size_t)N * nev;                              // eigenvectors
     b += (size_t)N * 8 * 3 * 16 + ((size_t)20 << 20);       // Lanczos blocks, small matrices
     if (precision != CHASE_FP64_DFMA && res) {
-        const HopBytes hb = hop_bytes(N, std::max(m, 32), true, false, !own_h);
+        const HopBytes hb = hop_bytes(N, std::max(m, 32), true, false, !own_h, true);
         b += hb.A + hb.B + hb.P + hb.GA;                    // residues of H and of the operand,
     } else if (precision != CHASE_FP64_DFMA) {              // partial results
         b += half ? ozaki_a_bytes_tri(N) + 16 * Np          // slices of H (half storage:
