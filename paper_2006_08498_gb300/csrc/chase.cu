@@ -286,7 +286,7 @@ int hop_prepare(bsechase_ctx *ctx, Hop &op, int max_cols) {
     else if (op.tri)
         CK(ozaki_prepare_h_tri(op.N, op.H, op.ldh, &ctx->oh, ctx->sc, ctx->st));
     else
-        CK(ozaki_prepare_h(op.N, op.H, op.ldh, &ctx->oh, ctx->sc, ctx->st));
+        CK(ozaki_prepare_h(op.N, op.H, op.ldh, op.level, &ctx->oh, ctx->sc, ctx->st));
     return BSE_OK;
 }
 

@@ -59,6 +59,7 @@ constexpr uint64_t kDefaultWaitNs = 2000000000ull;
 // times more accurate than OZ_S4.
 enum OzLevel { OZ_S6 = 0, OZ_S4 = 1, OZ_S5 = 2 };
 inline int oz_pairs(int level) { return level == OZ_S4 ? 10 : level == OZ_S5 ? 15 : 21; }
+inline int oz_slices(int level) { return level == OZ_S4 ? 4 : level == OZ_S5 ? 5 : 6; }
 
 // The slices of H, prepared once per solve.  Full storage: all Np x Np
 // elements, one exponent per row.  Half storage (tri): the lower-triangle
@@ -124,7 +125,8 @@ cudaError_t ozaki_prepare_bse(int Nk, int Nv, int Nc, const BseModel &md, const 
                               const z_t *u, const z_t *a, const double *Kt, bool tri, OzakiH *oh,
                               ChaseScalars *sc, cudaStream_t st);
 // Non-finite entries of H (or of a product's operand) set DEV_NONFINITE in sc.
-cudaError_t ozaki_prepare_h(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh, ChaseScalars *sc,
+// Only the slices that products up to `level` read are written.
+cudaError_t ozaki_prepare_h(int64_t N, const z_t *H, int64_t ldh, int level, OzakiH *oh, ChaseScalars *sc,
                             cudaStream_t st);
 // Half storage from the lower triangle of H (the strict upper triangle is
 // never read); oh->A >= ozaki_a_bytes_tri(N), oh->E, oh->t and oh->s hold Np

@@ -158,6 +158,36 @@ __device__ __forceinline__ void split_digits(double x, int E, int *t) {
     t[0] = (int)X;
 }
 
+// The slices p < ns of eight values (digits as split_digits, BF16 as slice_value),
+// 16 bytes each: store(p, bytes).  Balanced digits are the bytes of X plus 128 in
+// every digit's place, and a byte becomes the float digit 2^(-8(p+1)) by its
+// pattern beside 2^23 and one exact FMA: 85 instructions for 12 BF16 numbers.
+template <class Store>
+__device__ __forceinline__ void slice_run(const double *x, int E, int ns, Store store) {
+    unsigned long long X[8];
+#pragma unroll
+    for (int e = 0; e < 8; e++) X[e] = (unsigned long long)scaled_rint(x[e], kBeta * kS - E) + 0x8080808080ull;
+#pragma unroll
+    for (int p = 0; p < kS; p++) {
+        if (p >= ns) break;
+        const float f = __int_as_float((127 - kBeta * (p + 1)) << 23);
+        uint32_t o[4];
+#pragma unroll
+        for (int e = 0; e < 8; e++) {
+            const uint32_t lo = (uint32_t)X[e], hi = (uint32_t)(X[e] >> 32);
+            float v;
+            if (p == 0)                            // the top digit, signed: |X| <= 2^48
+                v = fmaf(__int_as_float(0x4B400000 + ((int)hi >> 8)), f, -12582912.f * f);
+            else                                   // p = 1: byte 4; then 3, 2, 1, 0
+                v = fmaf(__uint_as_float(__byte_perm(p == 1 ? hi : lo, 0x4B000000u, p == 1 ? 0x7650 : 0x7650 + (kS - 1 - p))),
+                         f, -8388736.f * f);
+            const uint32_t b = __float_as_uint(v);
+            o[e / 2] = e % 2 ? __byte_perm(o[e / 2], b, 0x7632) : b;
+        }
+        store(p, make_uint4(o[0], o[1], o[2], o[3]));
+    }
+}
+
 // BF16 bit pattern of v; v has at most 8 significant bits, so dropping the
 // low 16 bits of its FP32 pattern is exact.
 __device__ __forceinline__ uint16_t bf16_exact(float v) {
@@ -222,34 +252,42 @@ __host__ __device__ __forceinline__ int64_t tiled_index(int part, int64_t k, int
     return (((int64_t)part * nch + k / 64) * rows + row) * 64 + (k % 64);
 }
 
-// A slices of an M x K matrix H (rows padded to Mp, K to Kp): slice p of
-// re/im H_ik at tiled_index(p*2 + ri, k, i, Kp, Mp).  32 x 32 tiles through
-// shared memory; padded rows and columns are written as zeros.
-__global__ void k_slice_h(int64_t M, int64_t Mp, int64_t K, int64_t Kp,
-                          const z_t *__restrict__ H, int64_t ldh, const int *__restrict__ E,
-                          uint16_t *A) {
-    __shared__ z_t tile[32][33];
-    const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
-    const int64_t i0 = (int64_t)blockIdx.y * 32, k0 = (int64_t)blockIdx.x * 32;
-    for (int r = ty; r < 32; r += 8) {
-        const int64_t i = i0 + tx, k = k0 + r;       // column k, rows i: coalesced
-        tile[r][tx] = (i < M && k < K) ? H[i + k * ldh] : zmk(0.0, 0.0);
+// A slices p < ns of an M x K matrix H (rows padded to Mp, K to Kp): slice p of
+// re/im H_ik at tiled_index(p*2 + ri, k, i, Kp, Mp).  Blocks of 32 rows and 64
+// columns through shared memory, a thread eight columns of a row (16-byte stores;
+// one element a thread and 2-byte stores: 812 us at N = 8000, here 374 for four
+// slices, 1.0 + 1.0 GB).  Padded rows and columns are written as zeros.
+constexpr int kSliceRows = 32;
+__device__ __forceinline__ void slice_rows(const z_t (*tile)[kSliceRows + 1], int r, int kg, int e, int ns,
+                                           uint16_t *A, int64_t at, int64_t part) {
+    double x[8];
+#pragma unroll
+    for (int c = 0; c < 8; c++) x[c] = tile[kg * 8 + c][r].x;
+    slice_run(x, e, ns, [&](int p, uint4 v) { *(uint4 *)(A + at + 2 * p * part) = v; });
+#pragma unroll
+    for (int c = 0; c < 8; c++) x[c] = tile[kg * 8 + c][r].y;
+    slice_run(x, e, ns, [&](int p, uint4 v) { *(uint4 *)(A + at + (2 * p + 1) * part) = v; });
+}
+
+__global__ void __launch_bounds__(256)
+k_slice_h(int64_t M, int64_t Mp, int64_t K, int64_t Kp,
+          const z_t *__restrict__ H, int64_t ldh, const int *__restrict__ E, int ns,
+          uint16_t *A) {
+    __shared__ z_t tile[64][kSliceRows + 1];
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    const int64_t i0 = (int64_t)blockIdx.y * kSliceRows, k0 = (int64_t)blockIdx.x * 64;
+#pragma unroll
+    for (int c = warp; c < 64; c += 8) {
+        const int64_t i = i0 + lane, k = k0 + c;     // column k, rows i: coalesced
+        tile[c][lane] = (i < M && k < K) ? H[i + k * ldh] : zmk(0.0, 0.0);
     }
     __syncthreads();
-    for (int r = ty; r < 32; r += 8) {
-        const int64_t i = i0 + r, k = k0 + tx;       // row i, consecutive k
-        const z_t h = tile[tx][r];
-        int e = (i < M) ? E[i] : INT_MIN;
-        if (e == INT_MIN) e = 0;
-        int tr[kS], ti[kS];
-        split_digits(h.x, e, tr);
-        split_digits(h.y, e, ti);
-#pragma unroll
-        for (int p = 0; p < kS; p++) {
-            A[tiled_index(p * 2 + 0, k, i, Kp, Mp)] = bf16_exact(slice_value(tr[p], p));
-            A[tiled_index(p * 2 + 1, k, i, Kp, Mp)] = bf16_exact(slice_value(ti[p], p));
-        }
-    }
+    // eight lanes read eight rows of a column (no bank conflicts)
+    const int r = warp % 4 * 8 + lane % 8, kg = warp / 4 * 4 + lane / 8;
+    const int64_t i = i0 + r;
+    int e = (i < M) ? E[i] : INT_MIN;
+    if (e == INT_MIN) e = 0;
+    slice_rows(tile, r, kg, e, ns, A, tiled_index(0, k0 + kg * 8, i, Kp, Mp), Mp * Kp);
 }
 
 // A slices of op(A) = A^H for a K x M matrix A: op(A)_ik = conj(A_ki), read
@@ -316,25 +354,29 @@ __global__ void __launch_bounds__(256)
 k_tri_rowmax(int64_t N, const z_t *__restrict__ H, int64_t ldh, unsigned long long *Mx) {
     const int ti = blockIdx.x, tj = blockIdx.y;
     if (ti < tj) return;
-    __shared__ unsigned long long rmax[32], cmax[32];
-    const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
-    if (ty == 0) rmax[tx] = cmax[tx] = 0ull;
-    __syncthreads();
+    __shared__ unsigned long long rmax[8][32], cmax[32];
+    const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8: a warp takes whole columns
     const int64_t i = (int64_t)ti * 32 + tx;
     unsigned long long mine = 0;
+#pragma unroll
     for (int c = ty; c < 32; c += 8) {
         const int64_t k = (int64_t)tj * 32 + c;
-        if (i >= N || k >= N || k > i) continue;
-        const z_t h = H[i + k * ldh];
-        const unsigned long long mb = max(abs_bits(h.x), abs_bits(h.y));
+        unsigned long long mb = 0;
+        if (i < N && k <= i) {
+            const z_t h = H[i + k * ldh];
+            mb = max(abs_bits(h.x), abs_bits(h.y));
+        }
         mine = max(mine, mb);
-        atomicMax(&cmax[c], mb);
+        const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(mb >> 32));
+        const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(mb >> 32) == hi ? (uint32_t)mb : 0u);
+        if (tx == 0) cmax[c] = (unsigned long long)hi << 32 | lo;
     }
-    atomicMax(&rmax[tx], mine);
+    rmax[ty][tx] = mine;
     __syncthreads();
     if (ty == 0) {
         const int64_t r0 = (int64_t)ti * 32 + tx, r1 = (int64_t)tj * 32 + tx;
-        if (r0 < N && rmax[tx]) atomicMax(&Mx[r0], rmax[tx]);
+        for (int w = 1; w < 8; w++) mine = max(mine, rmax[w][tx]);
+        if (r0 < N && mine) atomicMax(&Mx[r0], mine);
         if (r1 < N && cmax[tx]) atomicMax(&Mx[r1], cmax[tx]);
     }
 }
@@ -367,40 +409,31 @@ __host__ __device__ __forceinline__ int64_t tri_index(int part, int64_t slot, in
 // kc <= 2 b + 1, is slot b (b + 1) + kc of each part (Re and Im of slice p:
 // parts 2p and 2p + 1).  The elements above the diagonal (in the tiles that
 // straddle it) are the conjugates of their mirrors, so the strict upper
-// triangle of H is never read; zeros outside N.  32 x 32 tiles through
-// shared memory (tk: column tile, ti: row tile), coalesced both ways.
+// triangle of H is never read; zeros outside N.  Blocks of 32 rows and 64
+// columns as in k_slice_h (N = 6000: 247 us with 2-byte stores, here 210: the scaling in FP64 bounds it).
 __global__ void __launch_bounds__(256)
 k_slice_tri(int64_t N, const z_t *__restrict__ H, int64_t ldh, const double *__restrict__ s,
             int64_t nslots, uint16_t *A) {
-    const int tk = blockIdx.x, ti = blockIdx.y;
-    const int b = ti / (kBM / 32), kc = tk / (kKC / 32);
+    const int kc = blockIdx.x, ti = blockIdx.y, b = ti / (kBM / kSliceRows);
     if (kc > 2 * b + 1) return;
-    __shared__ z_t tile[32][33];                   // tile[c][r] = S(i0 + r, k0 + c)
-    const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
-    const int64_t i0 = (int64_t)ti * 32, k0 = (int64_t)tk * 32;
-    for (int c = ty; c < 32; c += 8) {
-        const int64_t i = i0 + tx, k = k0 + c;
+    __shared__ z_t tile[64][kSliceRows + 1];       // tile[c][r] = S(i0 + r, k0 + c)
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    const int64_t i0 = (int64_t)ti * kSliceRows, k0 = (int64_t)kc * kKC;
+#pragma unroll
+    for (int c = warp; c < 64; c += 8) {
+        const int64_t i = i0 + lane, k = k0 + c;
         z_t h = zmk(0.0, 0.0);
         if (i < N && k < N) {
             h = (k <= i) ? H[i + k * ldh] : zconj(H[k + i * ldh]);
             h = zscale(h, s[i] * s[k]);
         }
-        tile[c][tx] = h;
+        tile[c][lane] = h;
     }
     __syncthreads();
     const int64_t slot = (int64_t)b * (b + 1) + kc;
-    for (int r = ty; r < 32; r += 8) {
-        const z_t h = tile[tx][r];                 // S(i0 + r, k0 + tx)
-        const int row = (int)(i0 + r - (int64_t)b * kBM), col = (int)(k0 + tx - (int64_t)kc * kKC);
-        int tr[kS], tim[kS];
-        split_digits(h.x, 0, tr);
-        split_digits(h.y, 0, tim);
-#pragma unroll
-        for (int p = 0; p < kS; p++) {
-            A[tri_index(2 * p, slot, nslots, row, col)] = bf16_exact(slice_value(tr[p], p));
-            A[tri_index(2 * p + 1, slot, nslots, row, col)] = bf16_exact(slice_value(tim[p], p));
-        }
-    }
+    const int r = warp % 4 * 8 + lane % 8, kg = warp / 4 * 4 + lane / 8;
+    slice_rows(tile, r, kg, 0, kS, A, tri_index(0, slot, nslots, (int)(i0 + r - (int64_t)b * kBM), kg * 8),
+               nslots * kBM * kKC);
 }
 
 // ------------------------------- slices of the synthetic H, H not stored
@@ -1370,7 +1403,7 @@ size_t ozaki_b_bytes(int64_t N, int m) {
     return (size_t)kS * 3 * mp * Np * 2;
 }
 
-cudaError_t ozaki_prepare_h(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh, ChaseScalars *sc,
+cudaError_t ozaki_prepare_h(int64_t N, const z_t *H, int64_t ldh, int level, OzakiH *oh, ChaseScalars *sc,
                             cudaStream_t st) {
     const int64_t Np = ozaki_padded(N);
     oh->N = N;
@@ -1382,8 +1415,8 @@ cudaError_t ozaki_prepare_h(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh, Ch
     dim3 g1((unsigned)((N + 255) / 256), (unsigned)((N + cpb - 1) / cpb));
     k_row_exponent<<<g1, 256, 0, st>>>(N, N, H, ldh, oh->E, cpb, sc);
     bse_count_launches(1);
-    dim3 g2((unsigned)(Np / 32), (unsigned)(Np / 32));
-    k_slice_h<<<g2, dim3(32, 8), 0, st>>>(N, Np, N, Np, H, ldh, oh->E, (uint16_t *)oh->A);
+    dim3 g2((unsigned)(Np / 64), (unsigned)(Np / kSliceRows));
+    k_slice_h<<<g2, 256, 0, st>>>(N, Np, N, Np, H, ldh, oh->E, oz_slices(level), (uint16_t *)oh->A);
     bse_count_launches(1);
     if (!make_map((CUtensorMap *)oh->tmap, oh->A, (uint64_t)Np, (uint64_t)(kS * 2 * (Np / kKC)),
                   kBM))
@@ -1400,10 +1433,10 @@ cudaError_t ozaki_prepare_h_tri(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh
     unsigned long long *Mx = (unsigned long long *)oh->s;
     cudaError_t e = cudaMemsetAsync(Mx, 0, (size_t)Np * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
-    const unsigned Tt = (unsigned)((N + 31) / 32), Tp = (unsigned)(Np / 32);
+    const unsigned Tt = (unsigned)((N + 31) / 32);
     k_tri_rowmax<<<dim3(Tt, Tt), dim3(32, 8), 0, st>>>(N, H, ldh, Mx);
     k_tri_scales<<<(unsigned)((Np + 255) / 256), 256, 0, st>>>(N, Np, Mx, oh->t, oh->s, oh->E, sc);
-    k_slice_tri<<<dim3(Tp, Tp), dim3(32, 8), 0, st>>>(N, H, ldh, oh->s, nslots, (uint16_t *)oh->A);
+    k_slice_tri<<<dim3((unsigned)(Np / kKC), (unsigned)(Np / kSliceRows)), 256, 0, st>>>(N, H, ldh, oh->s, nslots, (uint16_t *)oh->A);
     bse_count_launches(3);
     if (!make_map((CUtensorMap *)oh->tmap, oh->A, kBM, (uint64_t)(kS * 2 * nslots), kBM) ||
         !make_map((CUtensorMap *)oh->tmap2, oh->A, kBM, (uint64_t)(kS * 2 * nslots), kBM / 2))
@@ -1803,8 +1836,8 @@ cudaError_t ozaki_gemm(int64_t M, int n, int64_t K, const z_t *A, int64_t lda, i
         const int cpb = 256;
         dim3 g1((unsigned)((M + 255) / 256), (unsigned)((K + cpb - 1) / cpb));
         k_row_exponent<<<g1, 256, 0, st>>>(M, K, A, lda, w.E, cpb, sc);
-        dim3 g2((unsigned)(Kp / 32), (unsigned)(Mp / 32));
-        k_slice_h<<<g2, dim3(32, 8), 0, st>>>(M, Mp, K, Kp, A, lda, w.E, (uint16_t *)w.A);
+        dim3 g2((unsigned)(Kp / 64), (unsigned)(Mp / kSliceRows));
+        k_slice_h<<<g2, 256, 0, st>>>(M, Mp, K, Kp, A, lda, w.E, kS, (uint16_t *)w.A);
     }
     // exponents and slices of B (K x n)
     k_fill_int<<<(mp + 255) / 256, 256, 0, st>>>(w.F, mp, INT_MIN);
