@@ -142,18 +142,20 @@ k_cholesky_smem(int n, z_t *G, int64_t ld, ChaseScalars *sc) {
 }
 
 // X = R^{-1} for upper triangular R with a real positive diagonal: one warp
-// per column j (8 per CTA, as many CTAs as needed), column-oriented back
+// per column j (kTrinvW per CTA, as many CTAs as needed), column-oriented back
 // substitution of R x = e_j with x in shared memory and the reciprocals of
-// the diagonal computed once per CTA.
-__global__ void __launch_bounds__(256)
+// the diagonal computed once per CTA.  Bound by FP64 issue, so one warp a
+// scheduler: n = 100 takes 90 us, 115 with two.
+constexpr int kTrinvW = 4;
+__global__ void __launch_bounds__(32 * kTrinvW)
 k_trinv_cols(int n, const z_t *__restrict__ R, int64_t ldr, z_t *X, int64_t ldx) {
     extern __shared__ double smt[];
     double *rinv = smt;                                   // n
-    z_t *xs = (z_t *)(smt + ((n + 1) & ~1));              // 8 x n
+    z_t *xs = (z_t *)(smt + ((n + 1) & ~1));              // kTrinvW x n
     const int lane = threadIdx.x % 32, wl = threadIdx.x / 32;
     for (int k = threadIdx.x; k < n; k += blockDim.x) rinv[k] = 1.0 / R[k + (int64_t)k * ldr].x;
     __syncthreads();
-    const int j = blockIdx.x * 8 + wl;
+    const int j = blockIdx.x * kTrinvW + wl;
     if (j >= n) return;
     z_t *x = xs + (int64_t)wl * n;
     for (int r = lane; r < n; r += 32) x[r] = zmk(r == j ? 1.0 : 0.0, 0.0);
@@ -590,13 +592,18 @@ cudaError_t hh_launch(int n, const z_t *A, int64_t lda, const HeevWork &hw, cuda
 }
 
 // Cholesky G = U^H U (Sec. "QR": the Gram matrix of the filtered block) on a
-// cluster of C CTAs, right-looking: step j takes the pivot from the owner of
-// column j, forms row j of U on every CTA's own columns, publishes it, and
-// every CTA applies the rank-one update to the trailing upper triangle of
-// its columns.  The single-CTA versions are bound by FP64 issue on one SM
-// (dot products of short rows, a warp reduction each); here the work is
-// element-wise and spread over C SMs.  Column j (rows 0..j) of the upper
-// triangle lives in the shared memory of CTA j mod C.
+// cluster of C CTAs, right-looking: step j forms row j of U on every CTA's own
+// columns, publishes it, and every CTA applies the rank-one update to the
+// trailing upper triangle of its columns.  The single-CTA versions are bound by
+// FP64 issue on one SM (dot products of short rows, a warp reduction each); here
+// the work is element-wise and spread over C SMs.  Column j (rows 0..j) of the
+// upper triangle lives in the shared memory of CTA j mod C.
+// Latency of a step: one cluster barrier (published rows alternate between two
+// buffers, and each CTA keeps the whole diagonal up to date from the rows that it
+// gathers, so the pivot needs no second one) and one warp's reciprocal root (an
+// FP64 instruction occupies its scheduler for some 64 cycles whatever the lanes in
+// use; a square root and a division by all eight warps took longer than the rest).
+// n = 100: 238 us with both, 186 with two barriers, here 164.
 template <int C>
 __host__ __device__ constexpr int ch_cols(int n, int c) { return (c < n) ? (n - c + C - 1) / C : 0; }
 template <int C>
@@ -608,8 +615,9 @@ k_cholesky_cl(int n, z_t *G, int64_t ld, ChaseScalars *sc) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     extern __shared__ z_t Uc[];                 // own columns, rows 0..j
-    __shared__ z_t s_row[kMaxN];                // row j of U on the own columns (by column)
+    __shared__ z_t s_rows[2][kMaxN];            // row j of U on the own columns (by column)
     __shared__ z_t s_u[kMaxN];                  // row j of U, gathered
+    __shared__ double s_d[kMaxN];               // diagonal after j updates, the same on every CTA
     const int c = (int)cl.block_rank();
     const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
     const int ncol = ch_cols<C>(n, c);
@@ -618,28 +626,34 @@ k_cholesky_cl(int n, z_t *G, int64_t ld, ChaseScalars *sc) {
         z_t *col = Uc + ch_base<C>(c, l);
         for (int r = tid; r <= j; r += kHhT) col[r] = G[r + (int64_t)j * ld];
     }
-    cl.sync();
+    for (int i = tid; i < n; i += kHhT) s_d[i] = G[i + (int64_t)i * ld].x;
+    __syncthreads();
     for (int j = 0; j < n; j++) {
-        const int o = j % C;
-        // pivot: G(j, j) after j earlier updates, read from its owner; every
-        // CTA takes the same decision, so all leave together on a failure
-        const double d = cl.map_shared_rank(Uc, o)[ch_base<C>(o, j / C) + j].x;
+        z_t *s_row = s_rows[j & 1];
+        // every CTA takes the same decision, so all leave together on a failure
+        const double d = s_d[j];
         if (!(d > 0.0)) {
             if (c == 0 && tid == 0) set_error(sc, DEV_CHOL_FAIL, j);
             cl.sync();                          // nobody still reads this CTA's memory
             return;
         }
-        const double rjj = sqrt(d), inv = 1.0 / rjj;
         const int l0 = (j + 1 > c) ? (j + 1 - c + C - 1) / C : 0;   // own columns > j
-        for (int l = l0 + tid; l < ncol; l += kHhT) {
-            z_t *col = Uc + ch_base<C>(c, l);
-            const z_t u = zscale(col[j], inv);
-            col[j] = u;
-            s_row[l * C + c] = u;
+        if (warp == 0) {
+            const double inv = rsqrt(d);
+            if (j % C == c && lane == 0) Uc[ch_base<C>(c, j / C) + j] = zmk(d * inv, 0.0);
+            for (int l = l0 + lane; l < ncol; l += 32) {
+                z_t *col = Uc + ch_base<C>(c, l);
+                const z_t u = zscale(col[j], inv);
+                col[j] = u;
+                s_row[l * C + c] = u;
+            }
         }
-        cl.sync();                              // row j published, pivot read everywhere
-        if (o == c && tid == 0) Uc[ch_base<C>(c, j / C) + j] = zmk(rjj, 0.0);
-        for (int i = j + 1 + tid; i < n; i += kHhT) s_u[i] = cl.map_shared_rank(s_row, i % C)[i];
+        cl.sync();                              // row j published
+        for (int i = j + 1 + tid; i < n; i += kHhT) {
+            const z_t u = cl.map_shared_rank(s_row, i % C)[i];
+            s_u[i] = u;
+            s_d[i] -= u.x * u.x + u.y * u.y;
+        }
         __syncthreads();
         // G(i1, i2) -= conj(U(j, i1)) U(j, i2), j < i1 <= i2, own columns i2
         for (int l = l0 + warp; l < ncol; l += kHhW) {
@@ -654,8 +668,9 @@ k_cholesky_cl(int n, z_t *G, int64_t ld, ChaseScalars *sc) {
                 col[i1] = g;
             }
         }
-        cl.sync();                              // updates done; s_row free again
+        __syncthreads();                        // own updates done
     }
+    cl.sync();                                  // nobody still reads this CTA's rows
     for (int l = 0; l < ncol; l++) {
         const int j = l * C + c;
         const z_t *col = Uc + ch_base<C>(c, l);
@@ -674,7 +689,7 @@ size_t ch_dyn_bytes(int n) {
 // cudaErrorNotSupported otherwise.
 template <int C>
 cudaError_t ch_launch(int n, z_t *G, int64_t ld, ChaseScalars *sc, cudaStream_t st) {
-    constexpr size_t kStatic = (size_t)(2 * kMaxN) * sizeof(z_t) + 64;
+    constexpr size_t kStatic = (size_t)(3 * kMaxN) * sizeof(z_t) + kMaxN * sizeof(double) + 64;
     static std::once_flag once[kMaxDevices];
     static size_t limits[kMaxDevices];
     const int dev = current_device();
@@ -1243,15 +1258,15 @@ cudaError_t launch_cholesky(int n, z_t *G, int64_t ld, ChaseScalars *sc, cudaStr
 
 cudaError_t launch_trinv(int n, const z_t *R, int64_t ldr, z_t *X, int64_t ldx, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    const size_t bytes = (size_t)((n + 1) & ~1) * sizeof(double) + (size_t)8 * n * sizeof(z_t);
+    const size_t bytes = (size_t)((n + 1) & ~1) * sizeof(double) + (size_t)kTrinvW * n * sizeof(z_t);
     static std::once_flag once[kMaxDevices];
     static cudaError_t attr[kMaxDevices];
-    const int maxb = (int)(((kMaxN + 1) & ~1) * sizeof(double) + 8 * kMaxN * sizeof(z_t));
+    const int maxb = (int)(((kMaxN + 1) & ~1) * sizeof(double) + kTrinvW * kMaxN * sizeof(z_t));
     {
         const cudaError_t ae = smem_attr_once(once, attr, (const void *)k_trinv_cols, maxb);
         if (ae != cudaSuccess) return ae;
     }
-    k_trinv_cols<<<(n + 7) / 8, 256, bytes, st>>>(n, R, ldr, X, ldx);
+    k_trinv_cols<<<(n + kTrinvW - 1) / kTrinvW, 32 * kTrinvW, bytes, st>>>(n, R, ldr, X, ldx);
     bse_count_launches(1);
     return cudaGetLastError();
 }
