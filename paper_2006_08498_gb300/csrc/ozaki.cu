@@ -1624,12 +1624,12 @@ cudaEvent_t ready_event() {
     return ev;
 }
 
-constexpr int kRsCfg = 8;         // residue products (residue.cu)
+constexpr int kRsCfg = 8;         // residue products (residue.cu), + 1 in the three-product form
 
 // The launch of the products taken, all of one configuration.
 cudaError_t launch_taken(const std::vector<OzBatcher::Pending *> &take, int cfg, int sms, cudaStream_t st) {
     int u = 0;
-    if (cfg == kRsCfg) {
+    if (cfg >= kRsCfg) {
         static_assert(kRsMaxJobs >= kMaxJobs, "jobs of a launch");
         RsBatch bt;
         memset(&bt, 0, sizeof bt);
@@ -1737,7 +1737,7 @@ cudaError_t ozb_run(OzBatcher *b, OzBatcher::Pending &me, cudaStream_t st) {
 cudaError_t ozb_run_residue(OzBatcher *b, const RsJob &job, cudaStream_t st) {
     OzBatcher::Pending me;
     me.rjob = &job;
-    me.cfg = kRsCfg;
+    me.cfg = kRsCfg + (rs_gauss(job) ? 1 : 0);
     return ozb_run(b, me, st);
 }
 

@@ -16,12 +16,13 @@
 // Why residues.  With slices of 8 bits an FP64-accurate product takes every
 // pair of slices of the two operands (21 pairs of 48-bit operands with the
 // small ones left out); residues multiply modulus by modulus, 13 products for
-// operands of 51 and 50 bits.  And modulo p the complex product takes three
-// real ones (Gauss) instead of four, without the cancellation that the
-// three-product form has in floating point:
+// operands of 51 and 50 bits: 13 x 8 = 104 tensor flops per complex multiply-add,
+// against 168.  And modulo p the complex product can take three real ones (Gauss)
+// instead of four, without the cancellation that form has in floating point:
 //   T0 = Ar Br, T1 = Ai Bi, T2 = (Ar + Ai)(Br + Bi);
-//   Re = T0 - T1, Im = T2 - T0 - T1  (mod p).
-// 13 x 6 = 78 tensor flops per complex multiply-add, against 168.
+//   Re = T0 - T1, Im = T2 - T0 - T1  (mod p), 13 x 6 = 78.
+// Wide tiles, bound by the tensor cores (and their power), take three; narrow ones
+// take four, with fewer operands and accumulators to hand on.
 //
 // Accuracy.  The only rounding is that of the operands (and one FP64
 // rounding of the result): normwise about 2^-50 sqrt(N), without the
@@ -142,59 +143,84 @@ static_assert(kHMant >> 63 == 1 && kGMant >> 63 == 1, "normalised");
 constexpr int kRows = 128;         // rows of a CTA (TMEM lanes, MMA M)
 constexpr int kMaxW = 144;         // complex columns of a CTA at most
 constexpr int kChunk = 64;         // K elements of a stage (one swizzle row of FP16)
-constexpr int kRange = 8;          // T2 is drained every kRange chunks, T0 and T1 every 2 kRange
+constexpr int kGaussW = 112;       // three real products above this width, four up to it
+constexpr int kRange = 8;          // the exact range of an FP32 sum of two terms per K (T2, Re, Im), in chunks
 constexpr int kMaxUnitChunks = 224;           // a drain thread's packed sums
 constexpr int kAStage = 2 * kRows * kChunk;   // Re and Im residues, one byte each
 constexpr int kPack = 8192;        // a drain thread keeps Re + kPack Im in one integer
 constexpr int kDrainWarps = 8;
 constexpr int kTmemCols = 512;
-// Tensor memory holds the three accumulators of a launch's widest tile and, in
-// the rest, the ring of A operand stages (16 columns: K = 32 of one operand): 5
-// beside 144 columns, more beside fewer, which covers the latency between an
-// MMA's reading a stage and the MMA that reads its next contents.
-constexpr int kMinSlots = 5, kMaxSlots = 16;
-constexpr int kBars = 32;          // barriers of the stages, as a ring (a power of two, above kMaxSlots)
+// Tensor memory holds three accumulators of a launch's widest tile (Gauss: one per
+// product; four products: Re, Im, and the one that is being drained) and, in the
+// rest, the ring of A operand stages, which covers the latency between an MMA's
+// reading a stage and the MMA that reads its next contents.  Gauss: a stage is 16
+// columns, K = 32 of one of the three operands, 5 beside 144 columns.  Four
+// products: Re and Im of a chunk (64 columns) or of half of it.
+constexpr int kMaxSlots = 16;
+constexpr int kBars = 32;          // Gauss: barriers of the stages, as a ring (a power of two, above kMaxSlots)
 
 // Variants by the widest column tile of a launch.  Converting A costs the same
 // whatever the width, so a narrow tile is bound by the converters: it has more
 // of them, which the drain threads' registers (one packed sum per column) allow.
-// Up to 96 columns tensor memory has room for stages of a whole chunk (kH = 1):
-// half the barriers and commits, and with 4 or 5 stages of B (3: the MMA warps
-// waited 150 cycles a chunk for it) N = 8000 takes 299, 319, 361, 386 us at 16, 48,
-// 80, 96 columns against 348, 374, 404, 420 with half chunks throughout; the
-// MMA warps' own instructions, about 800 cycles a chunk, set the pace (H's
-// residues cross HBM in 248 us).
 // Warpgroups (4 warps, one per TMEM quadrant): copies and MMAs; kConv converter
 // groups; two drain groups.  Registers a thread: R0, RC, RD (setmaxnreg moves
 // them from the others to the drain groups) of RL at launch; 0: no move.
+// H: stages of A a chunk takes (four products), 0: Gauss.  N = 8000, us at 16, 48, 80,
+// 96, 112, 128, 144 columns: Gauss 295 314 351 375 443 455 481, four products 240 266
+// 324 359 407 444 508 (H's residues cross HBM in 248); twenty products of 140
+// columns at N = 20000, where the power limit counts too: 66.9 and 71.6 ms.
 template <int W, int CONV, int SA, int SB, int HOLD, int H, int RL, int R0, int RC, int RD>
 struct RsCfg {
     static constexpr int kW = W;                   // columns of a tile at most
+    static constexpr bool kGauss = H == 0;
+    static constexpr int kProducts = kGauss ? 3 : 2;   // accumulators, MMA warps and parts of B
     static constexpr int kConv = CONV;
     static constexpr int kThreads = 32 * (4 + 4 * CONV + kDrainWarps);
     static constexpr int kSA = SA, kSB = SB;       // stages of A's bytes and of B
-    static constexpr int kBStage = 3 * W * kChunk * 2;
+    static constexpr int kBStage = kProducts * W * kChunk * 2;
     static constexpr int kSmem = SA * kAStage + SB * kBStage + 1024;
     static constexpr int kHold = HOLD;             // granules of 8 columns a drain thread loads at once
-    static constexpr int kH = H, kCols = 32 / H;   // stages of A a chunk and product takes, their columns
+    static constexpr int kH = kGauss ? 2 : H, kCols = kGauss ? 16 : 64 / kH;   // stages of A and their columns
     static constexpr int kR0 = R0, kRC = RC, kRD = RD;
     static_assert(128 * (R0 + CONV * RC + 2 * RD) <= kThreads * RL && 65536 / kThreads >= RL, "register split");
-    static_assert(kSmem <= 231000 && 3 * W + kMinSlots * kCols <= kTmemCols && 2 * HOLD >= W / 16, "resources");
+    static_assert(kSmem <= 230500 && 2 * HOLD >= W / 16, "resources");
+    static constexpr int kMinSlots = (kTmemCols - 3 * W) / kCols;
+    // a converter group's step along the rings: one turn at most
+    static_assert(CONV >= 2 && (H == 1 ? (CONV + 1) / 2 : kGauss ? 3 * (CONV - 1) : CONV) <= kMinSlots && (CONV + 1) / 2 <= SA, "rings");
 };
-using RsWide = RsCfg<144, 2, 3, 3, 6, 2, 96, 48, 80, 136>;
-using RsMid = RsCfg<96, 3, 5, 4, 6, 1, 80, 48, 64, 112>;
-using RsNarrow = RsCfg<48, 4, 8, 5, 3, 1, 72, 0, 0, 0>;
+using RsGauss = RsCfg<144, 2, 3, 3, 6, 0, 96, 48, 80, 136>;
+using RsWide = RsCfg<112, 2, 5, 4, 6, 2, 96, 48, 80, 136>;
+using RsMid = RsCfg<96, 3, 7, 4, 6, 1, 80, 48, 64, 112>;
+using RsNarrow = RsCfg<48, 4, 8, 6, 3, 1, 72, 0, 0, 0>;
 static_assert((long long)kRange * kChunk * 128 * 256 <= (1ll << 24) &&
                   2ll * kRange * kChunk * 128 * 128 <= (1ll << 24), "exact FP32 sums");
-static_assert((kMaxUnitChunks / (2 * kRange) + 1) * 2 * 128 < kPack / 2, "packed sums");
-// The accumulators are drained after chunk c of a unit of nc: T0 when c % 16 is
-// 15, T1 when it is 10, T2 (whose operand Ar + Ai is twice as large) when it is
+static_assert((kMaxUnitChunks / (2 * kRange) + 1) * 2 * 128 < kPack / 2 &&
+                  (kMaxUnitChunks / kRange + 1) * 128 < kPack / 2, "packed sums");
+static_assert(kRange == 8, "drain pattern");
+// Gauss: the accumulators are drained after chunk c of a unit of nc: T0 when c % 16
+// is 15, T1 when it is 10, T2 (whose operand Ar + Ai is twice as large) when it is
 // 5 or 13, and all three after the last chunk: spread over time, so that each
 // drain is over before the next is due.
-static_assert(kRange == 8, "drain pattern");
 __device__ __forceinline__ bool range_end(int t, int c) {
     return t == 0 ? (c & 15) == 15 : t == 1 ? (c & 15) == 10 : (c & 7) == 5;
 }
+// Four products: the accumulator drained after chunk c, other than at the unit's
+// end: Re (0), Im (1) or none (-1).
+__device__ __forceinline__ int drained_after(int c, int nc) {
+    return (c & 3) == 3 && c + 1 < nc ? (c & 4 ? 0 : 1) : -1;
+}
+// Which buffer holds which accumulator: one that ends moves to the free buffer, and
+// its old one is free once it is drained.  Every role follows the same sequence.
+struct AccState {
+    uint32_t b[2] = {0, 1}, free = 2, drains = 0;  // drains: parity of each buffer's
+    __device__ __forceinline__ void end(int t) {
+        const uint32_t old = t == 0 ? b[0] : b[1];
+        if (t == 0) b[0] = free;
+        else b[1] = free;
+        free = old;
+        drains ^= 1u << old;
+    }
+};
 constexpr uint64_t kWindDownNs = 2000000000ull;
 
 // Work per CTA: one modulus, 128 rows, w <= 144 columns, the K chunks of one
@@ -203,25 +229,28 @@ constexpr uint64_t kWindDownNs = 2000000000ull;
 // read one modulus' operand (L2) and different rows of A.
 //
 //   warp 0      copies A's bytes (16 KB per chunk, untiled) into a ring of stages;
-//   warps 1-3   copy a part of B each (FP16, one TMA box per chunk) and issue the
-//               MMAs of its product: per chunk 4 K steps;
+//   warps 1-3   Gauss: copy a part of B each (FP16, one TMA box per chunk) and issue
+//               the MMAs of its product; four products: 1 and 2 issue those of
+//               Re (Ar Br, then -Ai Bi: the descriptor negates) and of Im (Ar Bi,
+//               Ai Br), 3 copies B (Re and Im in one box); per chunk 4 K steps;
 //   converters  turn A's bytes into FP16 pairs (a byte permute makes 1024 + b,
-//               one subtraction b - 128), add Re and Im for the third product
-//               and store the operands into tensor memory: one byte per
-//               residue crosses HBM and shared memory, and the MMA reads only
-//               B from shared memory;
-//   the last 8  drain an accumulator every 16 (T2: 8) chunks: reduce modulo p in FP32
+//               one subtraction b - 128), with Gauss add Re and Im for the third
+//               product, and store them into tensor memory: one byte per residue
+//               crosses HBM and shared memory, and the MMA reads only B from
+//               shared memory;
+//   the last 8  drain the accumulators within their range: reduce modulo p in FP32
 //               (exact: two FMAs and an addition, two values an instruction)
 //               and add into one packed integer per output.
 template <class Cfg>
 __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_constant__ RsBatch bt) {
     constexpr int kConvWarps = 4 * Cfg::kConv;
-    constexpr int kH = Cfg::kH, kCols = Cfg::kCols;
+    constexpr bool kGauss = Cfg::kGauss;
+    constexpr int kH = Cfg::kH, kCols = Cfg::kCols, kP = Cfg::kProducts;
     constexpr int kSA = Cfg::kSA, kSB = Cfg::kSB, kBStage = Cfg::kBStage, kConvGroups = Cfg::kConv;
     extern __shared__ uint8_t smraw[];
     uint8_t *sm = (uint8_t *)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
     uint8_t *sB = sm, *sA = sm + kSB * kBStage;
-    __shared__ uint64_t fullA[kSA], emptyA[kSA], fullB[3 * kSB], emptyB[3 * kSB];   // B: per product
+    __shared__ uint64_t fullA[kSA], emptyA[kSA], fullB[3 * kSB], emptyB[3 * kSB];   // B, Gauss: per product
     __shared__ uint64_t accFull[3], accEmpty[3], mmaDone;
     __shared__ __align__(2 * kBars * 8) uint64_t aBars[2 * kBars];   // stages of A: full, then empty
     uint64_t *aFull = aBars, *aEmpty = aBars + kBars;
@@ -239,17 +268,17 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
         }
         for (int s = 0; s < 3 * kSB; s++) {
             tc::mbar_init(&fullB[s], 1);
-            tc::mbar_init(&emptyB[s], 1);
+            tc::mbar_init(&emptyB[s], kGauss ? 1 : 2);
         }
         for (int s = 0; s < kBars; s++) {
             tc::mbar_init(&aFull[s], kH == 1 ? 8 : 4);
-            tc::mbar_init(&aEmpty[s], 1);
+            tc::mbar_init(&aEmpty[s], kGauss ? 1 : 2);
         }
         for (int t = 0; t < 3; t++) {
             tc::mbar_init(&accFull[t], 1);
             tc::mbar_init(&accEmpty[t], kDrainWarps);
         }
-        tc::mbar_init(&mmaDone, 3);
+        tc::mbar_init(&mmaDone, kP);
         abort_flag = 0;
         tc::mbar_fence_init();
     }
@@ -285,10 +314,11 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
         const bool r = tc::mbar_wait_at(b, parity, &abort_flag, wait_ns);
         return __all_sync(0xffffffffu, r) != 0;
     };
-    const uint32_t bars = tc::smem_u32(aBars);     // aligned to its size: a stage's barrier by or-ing
+    const uint32_t aF = tc::smem_u32(aFull), aE = tc::smem_u32(aEmpty);
+    const uint32_t bars = aF;                      // aligned to its size: a stage's barrier by or-ing
     constexpr uint32_t kBarMask = 8 * kBars - 1, kBarEmpty = 8 * kBars;
 
-    int fills = 0;      // copies issued, of A (warp 0) or of a part of B (warps 1-3)
+    int fills = 0;      // copies issued, of A (warp 0) or B (warps 1-3, or warp 3)
     if (warp < 4) {
       if (Cfg::kR0) tc::reg_dec<Cfg::kR0 ? Cfg::kR0 : 24>();
       if (warp == 0) {
@@ -307,7 +337,7 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                 }
             }
         }
-      } else {
+      } else if constexpr (kGauss) {
         // A warp for each product: its waits and instructions are a third (one
         // warp for all three needed 1.5 to 2 times the MMAs' own time, measured).
         // The whole warp runs the loop and one elected lane issues (predicated,
@@ -414,27 +444,110 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                 if (!load()) { ok = false; break; }
             }
         }
+      } else if (warp == 3) {
+        if (lane == 0) {
+            bool ok = true;
+            for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+                const Unit n = unit(u);
+                const RsJob &a = bt.job[n.jb];
+                const uint32_t bytes = (uint32_t)a.w * kChunk * 2 * 2;
+                const int x = n.x * a.w;
+                int z = (n.m * a.nch + n.c0) * 2;
+                for (int c = n.c0; c < n.c1; c++, z += 2) {
+                    const int s = fills % kSB, f = fills / kSB;
+                    if (f >= 1 && !tc::mbar_wait(&emptyB[s], (f - 1) & 1, &abort_flag, wait_ns)) { ok = false; break; }
+                    tc::mbar_expect_tx(&fullB[s], bytes);
+                    tc::tma_load_3d(sB + s * kBStage, &a.tmB, 0, x, z, &fullB[s]);
+                    fills++;
+                }
+            }
+        }
+      } else {
+        // A warp for each accumulator.  The whole warp runs the loop and one elected
+        // lane issues (predicated, without branches), so that the descriptors are
+        // warp-uniform (uniform registers feed tcgen05.mma).  A wait that succeeds
+        // costs a warp about 100 cycles, so the barriers of the next stage are
+        // looked at (without blocking) before this one's MMAs are issued, and waited
+        // for only if that look failed.
+        const int t = warp - 1;
+        const uint32_t one = tc::elect_one() ? 1u : 0u;
+        const uint32_t fB = tc::smem_u32(fullB), eB = tc::smem_u32(emptyB);
+        const uint32_t accF = tc::smem_u32(accFull), accE = tc::smem_u32(accEmpty);
+        const uint32_t tbeg = tmem + 3 * stride, s8end = slots * 8;
+        bool ok = true, rdy = false, rdyB = false;
+        uint32_t sB8 = 0, sph = 0;                 // stage of B (8 bytes a barrier), phase
+        AccState st;
+        uint32_t s8 = 0, bph = 0, at = tbeg;       // stage of A
+        for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
+            const Unit n = unit(u);
+            const int w = bt.job[n.jb].w;
+            const uint32_t id = tc::idesc_f16_f32(kRows, w), id2 = t == 0 ? id | tc::kIdescNegA : id;
+            const uint64_t part = (uint64_t)(w * kChunk * 2 >> 4);
+            const uint64_t bd1 = tc::sdesc_sw128(sB) + (t == 0 ? 0 : part), bd2 = tc::sdesc_sw128(sB) + (t == 0 ? part : 0);
+            const int nc = n.c1 - n.c0;
+            uint32_t fresh = 1;
+            for (int c = 0; c < nc; c++) {
+                const int dr = drained_after(c, nc);
+                const uint32_t end = c + 1 == nc || dr == t ? 1u : 0u, buf = t == 0 ? st.b[0] : st.b[1];
+                const uint32_t acc = tmem + buf * stride;
+                if (!rdyB && !wait_all(fB + sB8, sph)) { ok = false; break; }
+                // a fresh barrier passes the wait for the phase before its first
+                if (fresh && !wait_all(accE + 8 * buf, (st.drains >> buf & 1) ^ 1)) { ok = false; break; }
+                const uint64_t bo = (uint64_t)(sB8 * (kBStage / 8 >> 4));
+                const uint32_t eb = eB + sB8;
+                bool lookB = false;
+#pragma unroll
+                for (int h = 0; h < kH; h++) {
+                    if (!rdy && !wait_all(aF + s8, bph)) { ok = false; break; }
+                    tc::fence_after();
+                    const uint32_t t0 = at, e0 = aE + s8;
+                    at += kCols;
+                    s8 += 8;
+                    if (s8 == s8end) { s8 = 0; bph ^= 1; at = tbeg; }
+                    const bool look = tc::mbar_test_at(aF + s8, bph);
+                    if (h == kH - 1) {
+                        sB8 += 8;
+                        if (sB8 == 8 * kSB) { sB8 = 0; sph ^= 1; }
+                        lookB = tc::mbar_test_at(fB + sB8, sph);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4 / kH; k++) {
+                        const uint64_t ko = bo + 2 * (h * (4 / kH) + k);
+                        tc::mma_f16_ta_if(one, acc, t0 + 8 * k, bd1 + ko, id, h + k == 0 ? fresh ^ 1 : 1u);
+                        tc::mma_f16_ta_if(one, acc, t0 + kCols / 2 + 8 * k, bd2 + ko, id2, 1u);
+                    }
+                    tc::mma_commit_if(one, e0);
+                    if (h == kH - 1) {
+                        tc::mma_commit_if(one, eb);
+                        if (end) tc::mma_commit_if(one, accF + 8 * buf);
+                    }
+                    rdy = __all_sync(0xffffffffu, look) != 0;
+                }
+                if (!ok) break;
+                fresh = end;
+                if (dr >= 0) st.end(dr);
+                rdyB = __all_sync(0xffffffffu, lookB) != 0;
+            }
+            st.end(0);
+            st.end(1);
+        }
       }
     } else if (warp < 4 + kConvWarps) {
         if (Cfg::kRC) tc::reg_dec<Cfg::kRC ? Cfg::kRC : 24>();
-        // The groups take turns, half a chunk (32 K elements) each: item 2 chunk + h.
-        // (Publishing the three operands one by one costs nothing with kH = 2, whose
-        // few stages the MMAs wait for.)
-        // Its i-th operand is (with kH = 1 its half of) fill 3 item + i (3 chunk + i)
-        // of the ring of stages, and waits for the MMAs on the fill `slots` before it.
+        // The groups take turns, half a chunk (32 K elements) each: item 2 chunk + h,
+        // which is a stage, or with kH = 1 its half h.  Gauss: its i-th operand is fill
+        // 3 item + i of the ring of stages, and waits for the MMAs on the fill `slots`
+        // before it.
         const int quad = warp & 3, row = quad * 32 + lane;
         const __half2 k1152 = __floats2half2_rn(1152.f, 1152.f);
         int item = (warp - 4) >> 2;
-        const int first = kH == 1 ? item >> 1 : item;
-        uint32_t f8 = 24 * first;                  // the fill's barrier
-        uint32_t e8 = 8 * (3 * first - slots), eph = 1;   // of the fill it waits for (modulo the ring)
-        if ((int)e8 >= 0) eph = 0;
-        e8 &= kBarMask;
+        uint32_t s = kH == 1 ? item >> 1 : item, ph = 1;   // its stage; phase of the wait for it
         const uint32_t tbeg = tmem + ((uint32_t)(quad * 32) << 16) + 3 * stride, tend = tbeg + slots * kCols;
-        uint32_t ta = tbeg + 3 * first % slots * kCols;
+        uint32_t f8 = 24 * item;                   // Gauss: the fill's barrier
+        uint32_t e8 = 8 * (3 * item - slots), eph = (int)e8 >= 0 ? 0 : 1;   // of the fill it waits for (modulo the ring)
+        e8 &= kBarMask;
+        uint32_t ta = tbeg + 3 * item % slots * kCols;
         uint32_t sa8 = 8 * (item >> 1), saph = 0;  // stage of A's bytes (8 bytes a barrier), and its phase
-        static_assert((kConvGroups - 1) / 2 < kSA && (kConvGroups + 1) / 2 <= kSA && kConvGroups >= 2 &&
-                          3 * ((kH == 1 ? (kConvGroups + 1) / 2 : kConvGroups) - 1) <= kMinSlots, "one turn of the ring at most");
         const uint32_t fullA0 = tc::smem_u32(fullA), emptyA0 = tc::smem_u32(emptyA);
         auto convert = [&](const uint8_t *src, uint32_t *r) {
 #pragma unroll
@@ -451,27 +564,22 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                 }
             }
         };
-        // store an operand's columns: waits for the stage; publish tells the MMAs of
-        // the last n stored
-        auto put = [&](const uint32_t *r, int h) {
+        // Gauss: store an operand's columns and tell its product's MMAs
+        auto put = [&](const uint32_t *r) {
             // a fresh barrier passes the wait for the phase before its first
             if (!wait_all(bars | kBarEmpty | e8, eph)) return false;
             tc::fence_after();
-            tc::tmem_st16(kH == 1 ? ta + 16 * h : ta, r);
+            tc::tmem_st16(ta, r);
             ta += kCols;
             if (ta == tend) ta = tbeg;
             e8 += 8;
             if (e8 > kBarMask) { e8 = 0; eph ^= 1; }
-            return true;
-        };
-        auto publish = [&](int n) {
             tc::tmem_wait_st();
             tc::fence_before();
             __syncwarp();
-            for (int k = 0; k < n; k++) {
-                if (lane == 0) tc::mbar_arrive_at(bars | f8);
-                f8 = (f8 + 8) & kBarMask;
-            }
+            if (lane == 0) tc::mbar_arrive_at(bars | f8);
+            f8 = (f8 + 8) & kBarMask;
+            return true;
         };
         // item counts over all units; i is its number in its unit
         int done = 0;
@@ -488,27 +596,39 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                 convert(src + 4 * kRows * 16, im);
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive_at(emptyA0 + sa8);
-                if (!put(re, h)) { ok = false; break; }
-                if (kH == 2) publish(1);
-                if (!put(im, h)) { ok = false; break; }
-                if (kH == 2) publish(1);
+                const int chunks = (h + kConvGroups) / 2;
+                if constexpr (kGauss) {
+                    if (!put(re) || !put(im)) { ok = false; break; }
 #pragma unroll
-                for (int e = 0; e < 16; e++) {
-                    __half2 a, b;
-                    memcpy(&a, &re[e], 4);
-                    memcpy(&b, &im[e], 4);
-                    a = __hadd2(a, b);             // in [-256, 254]: exact
-                    memcpy(&re[e], &a, 4);
+                    for (int e = 0; e < 16; e++) {
+                        __half2 a, b;
+                        memcpy(&a, &re[e], 4);
+                        memcpy(&b, &im[e], 4);
+                        a = __hadd2(a, b);         // in [-256, 254]: exact
+                        memcpy(&re[e], &a, 4);
+                    }
+                    if (!put(re)) { ok = false; break; }
+                    // past the other groups' items
+                    constexpr uint32_t over = 3 * (kConvGroups - 1);
+                    f8 = (f8 + 8 * over) & kBarMask;
+                    e8 += 8 * over;
+                    if (e8 > kBarMask) { e8 &= kBarMask; eph ^= 1; }
+                    ta += over * kCols;            // at most one turn of the ring
+                    if (ta >= tend) ta -= slots * kCols;
+                } else {
+                    // a fresh barrier passes the wait for the phase before its first
+                    if (!wait_all(aE + 8 * s, ph)) { ok = false; break; }
+                    tc::fence_after();
+                    const uint32_t at = tbeg + s * kCols + (kH == 1 ? 16 * h : 0);
+                    tc::tmem_st16(at, re);
+                    tc::tmem_st16(at + kCols / 2, im);
+                    tc::tmem_wait_st();
+                    tc::fence_before();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive_at(aF + 8 * s);
+                    s += kH == 1 ? chunks : kConvGroups;
+                    if (s >= slots) { s -= slots; ph ^= 1; }
                 }
-                if (!put(re, h)) { ok = false; break; }
-                publish(kH == 2 ? 1 : 3);
-                // past the other groups' items
-                const int chunks = (h + kConvGroups) / 2, over = (kH == 1 ? chunks : kConvGroups) - 1;
-                f8 = (f8 + 24 * over) & kBarMask;
-                e8 += 24 * over;
-                if (e8 > kBarMask) { e8 &= kBarMask; eph ^= 1; }
-                ta += 3 * kCols * over;            // at most one turn of the ring
-                if (ta >= tend) ta -= slots * kCols;
                 sa8 += chunks * 8;
                 if (sa8 >= 8 * kSA) { sa8 -= 8 * kSA; saph ^= 1; }
             }
@@ -522,7 +642,8 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
         constexpr int kG = Cfg::kW / 16, kHold = Cfg::kHold;   // granules of 8 columns per thread, held at once
         constexpr float kMagic = 12582912.f;       // 1.5 2^23: rounds to an integer
         bool ok = true;
-        uint32_t ph = 0;                           // phases of accFull
+        AccState st;
+        uint32_t gph = 0;                          // Gauss: phases of accFull
         for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
             const Unit n = unit(u);
             const RsJob &a = bt.job[n.jb];
@@ -535,23 +656,39 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
             const int nc = n.c1 - n.c0;
             const uint64_t inv2 = tc::pin2(tc::f32x2(inv, inv)), mp2 = tc::pin2(tc::f32x2(-pf, -pf));
             const uint64_t magic2 = tc::pin2(tc::f32x2(kMagic, kMagic)), mmagic2 = tc::pin2(tc::f32x2(-kMagic, -kMagic));
-            for (int ev = 0, fin = 0; fin < 3;) {
-                // the next drain: T2, T1, T2, T0 after chunks 5, 10, 13, 15 of every
-                // 16, until the last chunk; then T0, T1, T2
+            for (int ev = 0, fin = 0; fin < kP;) {
                 int t;
-                if (fin == 0 && (ev >> 2) * 16 + ((0xFDA5 >> (ev % 4 * 4)) & 15) < nc - 1) {
-                    t = (0x0212 >> (ev % 4 * 4)) & 3;
-                    ev++;
+                uint32_t buf, phase;
+                float coef;                        // Re + kPack Im
+                if constexpr (kGauss) {
+                    // T2, T1, T2, T0 after chunks 5, 10, 13, 15 of every 16, until the
+                    // last chunk; then T0, T1, T2
+                    if (fin == 0 && (ev >> 2) * 16 + ((0xFDA5 >> (ev % 4 * 4)) & 15) < nc - 1) {
+                        t = (0x0212 >> (ev % 4 * 4)) & 3;
+                        ev++;
+                    } else {
+                        t = fin++;
+                    }
+                    buf = (uint32_t)t;
+                    phase = gph >> t & 1;
+                    gph ^= 1u << t;
+                    // T0 counts (1, -1), T1 (-1, -1), T2 (0, 1)
+                    coef = t == 0 ? (float)(1 - kPack) : t == 1 ? (float)(-1 - kPack) : (float)kPack;
                 } else {
-                    t = fin++;
+                    // Im and Re by turns after every fourth chunk, until the last
+                    // chunk; then Re, Im
+                    t = fin == 0 ? drained_after(4 * ev + 3, nc) : -1;
+                    if (t >= 0) ev++;
+                    else t = fin++;
+                    buf = t == 0 ? st.b[0] : st.b[1];
+                    phase = st.drains >> buf & 1;
+                    st.end(t);
+                    coef = t == 0 ? 1.f : (float)kPack;
                 }
-                if (!wait_all(tc::smem_u32(&accFull[t]), (ph >> t) & 1)) { ok = false; break; }
-                ph ^= 1u << t;
+                if (!wait_all(tc::smem_u32(&accFull[buf]), phase)) { ok = false; break; }
                 tc::fence_after();
-                // Re + kPack Im: T0 counts (1, -1), T1 (-1, -1), T2 (0, 1)
-                const float coef = t == 0 ? (float)(1 - kPack) : t == 1 ? (float)(-1 - kPack) : (float)kPack;
                 const uint64_t coef2 = tc::pin2(tc::f32x2(coef, coef));
-                const uint32_t col = tmem + lane_addr + t * stride + half * ng * 8;
+                const uint32_t col = tmem + lane_addr + buf * stride + half * ng * 8;
                 auto digest = [&](const uint32_t *r, int g) {
 #pragma unroll
                     for (int v = 0; v < 8; v += 2) {
@@ -579,7 +716,7 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                 tc::tmem_wait_ld();
                 tc::fence_before();
                 __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&accEmpty[t]);
+                if (lane == 0) tc::mbar_arrive(&accEmpty[buf]);
 #pragma unroll
                 for (int g = 0; g < kG; g++) {
                     const int at = g >= kHold ? g - kHold : g;
@@ -619,11 +756,15 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                 if (f > 0) drained &= tc::mbar_wait_for(&fullA[s], (f - 1) & 1, kWindDownNs);
             }
         }
-        if (warp >= 1 && warp < 4 && tc::elect_one()) {
-            for (int s = 0; s < kSB; s++) {
-                const int f = (fills - s + kSB - 1) / kSB;
-                if (f > 0) drained &= tc::mbar_wait_for(&fullB[(warp - 1) * kSB + s], (f - 1) & 1, kWindDownNs);
-            }
+        if (kGauss ? warp >= 1 && warp < 4 : warp == 3) {
+            if (tc::elect_one())
+                for (int s = 0; s < kSB; s++) {
+                    const int f = (fills - s + kSB - 1) / kSB;
+                    if (f > 0)
+                        drained &= tc::mbar_wait_for(&fullB[(kGauss ? (warp - 1) * kSB : 0) + s], (f - 1) & 1, kWindDownNs);
+                }
+        }
+        if (warp >= 1 && warp <= kP && tc::elect_one()) {
             tc::mma_commit(&mmaDone);
             drained &= tc::mbar_wait_for(&mmaDone, 0, kWindDownNs);
         }
@@ -903,14 +1044,14 @@ k_res_slice_ah(int64_t M, int64_t K, const z_t *__restrict__ A, int64_t lda, int
     residues_of_row<16>(v, h != INT_MIN ? bits - h : 0, nmod, T * nch * kAStage, dst);
 }
 
-// FP16 residues of Y, -> [modulus][chunk][Re, Im, Re + Im][column][64]: one
+// FP16 residues of Y, -> [modulus][chunk][Re, Im, and Re + Im with parts = 3][column][64]: one
 // column and 8 consecutive K elements per thread, the moduli from blockIdx.z
 // in steps of gridDim.z.  The column's norm comes from its partial sums, or with
 // npart = 0 from the column itself; F[j] receives its exponent.
 __global__ void __launch_bounds__(128)
 k_res_slice_b(int64_t N, int64_t Kp, int n, int mp, const z_t *__restrict__ Y, int64_t ldy, int npart,
-              const float2 *__restrict__ part, int *__restrict__ F, int nmod, int bits, uint16_t *__restrict__ B,
-              ChaseScalars *sc) {
+              const float2 *__restrict__ part, int *__restrict__ F, int nmod, int bits, int parts,
+              uint16_t *__restrict__ B, ChaseScalars *sc) {
     const int j = blockIdx.y;
     const int64_t k = ((int64_t)blockIdx.x * 128 + threadIdx.x) * 8;
     int h = INT_MIN;
@@ -955,13 +1096,15 @@ k_res_slice_b(int64_t N, int64_t Kp, int n, int mp, const z_t *__restrict__ Y, i
             const uint32_t wr = __byte_perm((uint32_t)a, (uint32_t)(a >> 32), 0x0400) & 0x00FF00FFu;
             const uint32_t wi = __byte_perm((uint32_t)b, (uint32_t)(b >> 32), 0x0400) & 0x00FF00FFu;
             uint32_t ws = 0;
+            if (parts == 3) {
 #pragma unroll
-            for (int e = 0; e < 2; e++) {
-                // the sum modulo p, in [-128, 127]
-                int s = (int)(wr >> (16 * e) & 255) + (int)(wi >> (16 * e) & 255) - 256;
-                s += s < -128 ? p : 0;
-                s -= s > 127 ? p : 0;
-                ws |= (uint32_t)(s + 128) << (16 * e);
+                for (int e = 0; e < 2; e++) {
+                    // the sum modulo p, in [-128, 127]
+                    int s = (int)(wr >> (16 * e) & 255) + (int)(wi >> (16 * e) & 255) - 256;
+                    s += s < -128 ? p : 0;
+                    s -= s > 127 ? p : 0;
+                    ws |= (uint32_t)(s + 128) << (16 * e);
+                }
             }
             const uint32_t w[3] = {wr, wi, ws};
 #pragma unroll
@@ -973,10 +1116,10 @@ k_res_slice_b(int64_t N, int64_t Kp, int n, int mp, const z_t *__restrict__ Y, i
                 memcpy(&o[t][q], &hh, 4);
             }
         }
-        uint16_t *d = B + (((int64_t)m * nch + c) * 3) * pstep + (int64_t)j * kChunk + k % kChunk;
+        uint16_t *d = B + (((int64_t)m * nch + c) * parts) * pstep + (int64_t)j * kChunk + k % kChunk;
 #pragma unroll
         for (int t = 0; t < 3; t++)
-            *(uint4 *)(d + t * pstep) = make_uint4(o[t][0], o[t][1], o[t][2], o[t][3]);
+            if (t < parts) *(uint4 *)(d + t * pstep) = make_uint4(o[t][0], o[t][1], o[t][2], o[t][3]);
     }
 }
 
@@ -1184,13 +1327,13 @@ k_res_out(int64_t M, int64_t Mp, int mp, int nz, const uchar2 *__restrict__ R, c
     }
 }
 
-// 3-D FP16 tensor [tiles][rows][64], box 64 x box_rows, 128-byte swizzle
-bool make_map(CUtensorMap *m, void *base, uint64_t rows, uint64_t tiles, uint32_t box_rows) {
+// 3-D FP16 tensor [tiles][rows][64], box 64 x box_rows x box_tiles, 128-byte swizzle
+bool make_map(CUtensorMap *m, void *base, uint64_t rows, uint64_t tiles, uint32_t box_rows, uint32_t box_tiles) {
     const TensorMapEncode enc = tensor_map_encode();
     if (!enc) return false;
     cuuint64_t dims[3] = {64, rows, tiles};
     cuuint64_t strides[2] = {64 * 2, rows * 64 * 2};
-    cuuint32_t box[3] = {64, box_rows, 1};
+    cuuint32_t box[3] = {64, box_rows, box_tiles};
     cuuint32_t es[3] = {1, 1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, base, dims, strides, box, es,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1203,13 +1346,16 @@ void column_tiles(int n, int *tx, int *w) {
     *w = ((n + *tx - 1) / *tx + 15) / 16 * 16;
 }
 
+// Parts of B's residues for a tile of w columns: Re and Im, and with Gauss their sum
+int b_parts(int w) { return w > kGaussW ? 3 : 2; }
+
 // Chunks per K split.  Modelled time, in cycles, of the busiest SM: a chunk
-// takes 6 w cycles of MMA, at least about 700 (its share of HBM) or 260 (its
+// takes 6 or 8 w cycles of MMA, at least about 700 (its share of HBM) or 260 (its
 // conversion) when the matrix is in L2; a unit costs about 2000 more (its first
 // copies and its last drain) and each split about 52 bytes per output.
 int choose_chunks(int64_t Mp, int nch, int mp, int tx, int w, int nmod, size_t r_bytes, int sms) {
     const double mat = 2.0 * nmod * Mp * nch * kChunk;
-    const double per_chunk = std::max(6.0 * w, mat > 1.0e8 ? 700.0 : 300.0);
+    const double per_chunk = std::max((w > kGaussW ? 6.0 : 8.0) * w, mat > 1.0e8 ? 700.0 : 300.0);
     const int64_t tiles = Mp / kRows * tx * nmod;
     int best = 0;
     double best_t = 1e300;
@@ -1324,7 +1470,11 @@ cudaError_t residue_prepare_bse(int Nk, int Nv, int Nc, const BseModel &md, cons
     return cudaGetLastError();
 }
 
-double residue_flops(int64_t M, int64_t K, int n) { return 6.0 * kNMod * (double)M * (double)K * n; }
+double residue_flops(int64_t M, int64_t K, int n) {
+    int tx, w;
+    column_tiles(n, &tx, &w);
+    return (w > kGaussW ? 6.0 : 8.0) * kNMod * (double)M * (double)K * n;
+}
 
 namespace {
 template <class Cfg>
@@ -1340,12 +1490,15 @@ cudaError_t launch_cfg(RsBatch &b, int sms, cudaStream_t st) {
 }
 }  // namespace
 
+bool rs_gauss(const RsJob &j) { return j.w > kGaussW; }
+
 cudaError_t residue_launch(RsBatch &b, int sms, cudaStream_t st) {
     b.stride = 16;
     for (int j = 0; j < b.njobs; j++) b.stride = std::max(b.stride, b.job[j].w);
     if (b.stride <= RsNarrow::kW) return launch_cfg<RsNarrow>(b, sms, st);
     if (b.stride <= RsMid::kW) return launch_cfg<RsMid>(b, sms, st);
-    return launch_cfg<RsWide>(b, sms, st);
+    if (b.stride <= kGaussW) return launch_cfg<RsWide>(b, sms, st);
+    return launch_cfg<RsGauss>(b, sms, st);
 }
 
 namespace {
@@ -1355,7 +1508,8 @@ bool single_job(RsBatch *b, const void *A, void *B, int64_t Mp, int nch, int tx,
     memset(b, 0, sizeof *b);
     RsJob &j = b->job[0];
     const int mp = tx * w;
-    if (!make_map(&j.tmB, B, (uint64_t)mp, (uint64_t)nmod * 3 * nch, (uint32_t)w)) return false;
+    if (!make_map(&j.tmB, B, (uint64_t)mp, (uint64_t)nmod * b_parts(w) * nch, (uint32_t)w, w > kGaussW ? 1 : 2))
+        return false;
     j.A = (const uint8_t *)A;
     j.R = (uchar2 *)R;
     j.sc = sc;
@@ -1396,7 +1550,7 @@ cudaError_t residue_zgemm(const OzakiH &oh, int n, const z_t *Y, int64_t ldy, z_
     const unsigned bx = (unsigned)((Kp + 1023) / 1024);
     // split the moduli over blocks while that leaves SMs idle otherwise
     const unsigned bz = (unsigned)std::max<int64_t>(1, std::min<int64_t>(kNMod, 4 * sms / ((int64_t)bx * mp)));
-    k_res_slice_b<<<dim3(bx, (unsigned)mp, bz), 128, 0, st>>>(N, Kp, n, mp, Y, ldy, npart, part, F, kNMod, kBeta,
+    k_res_slice_b<<<dim3(bx, (unsigned)mp, bz), 128, 0, st>>>(N, Kp, n, mp, Y, ldy, npart, part, F, kNMod, kBeta, b_parts(w),
                                                               (uint16_t *)B, sc);
     bse_count_launches(1);
     RsBatch b;
@@ -1479,7 +1633,7 @@ cudaError_t residue_right(int64_t K, int n, const z_t *B, int64_t ldb, const flo
     const unsigned bx = (unsigned)((Kp + 1023) / 1024);
     const unsigned bz = (unsigned)std::max<int64_t>(1, std::min<int64_t>(kGMod, 4 * sms / ((int64_t)bx * mp)));
     k_res_slice_b<<<dim3(bx, (unsigned)mp, bz), 128, 0, st>>>(K, Kp, n, mp, B, ldb, npart, norms ? norms : s.part, s.e,
-                                                              kGMod, kGBits, (uint16_t *)s.p, sc);
+                                                              kGMod, kGBits, b_parts(w), (uint16_t *)s.p, sc);
     bse_count_launches(1);
     return cudaGetLastError();
 }

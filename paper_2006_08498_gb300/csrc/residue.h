@@ -27,6 +27,8 @@ struct RsBatch {
     int njobs, units;
     int stride, slots;     // columns of an accumulator, and stages of A, in tensor memory
 };
+// Whether a job takes the three-product form: only such jobs share a launch.
+bool rs_gauss(const RsJob &j);
 inline int rs_units(const RsJob &j) { return j.tx * j.ty * j.tz * j.nmod; }
 // Run a job through the batcher; returns after `st` waits for its launch.
 struct OzBatcher;

@@ -120,6 +120,24 @@ def test_nonfinite_is_reported(ctx):
         assert ei.value.status == pkg.BSE_ENONFINITE
 
 
+@pytest.mark.parametrize("n", [111, 112, 113, 128, 129])
+def test_three_and_four_products(ctx, n):
+    """Both sides of the line between four real products and three (tiles of more
+    than 112 columns), with every drain of a long unit."""
+    A, Y = _hermitian(2100, 13), _block(2100, n, 14)
+    _check(A, Y, _hemm(ctx, A, Y))
+
+
+@pytest.mark.parametrize("n", [5, 97, 113])
+def test_largest_sums(ctx, n):
+    """Every operand's residue modulo 256 is -128 (integers 2^45 + 128 against
+    2-norms of 45.25 times that, 2^44 + 128 for Y): the FP32 sums reach 2^24."""
+    N = 1024
+    A = torch.full((N, N), 1 + 2.0 ** -38, dtype=torch.complex128, device="cuda").T * (1 + 1j)
+    Y = torch.full((n, N), 1 + 2.0 ** -37, dtype=torch.complex128, device="cuda").T * (1 + 1j)
+    _check(A, Y, _hemm(ctx, A, Y))
+
+
 # ---- the general products (Gram and QR entries)
 
 def _integers(rows, cols, seed):
