@@ -66,15 +66,18 @@ typedef enum {
                              to ||H|| ||Y||).  With half storage, and in
                              chase_rayleigh_ritz, the products are the BF16
                              Ozaki-scheme emulation of 6 slices of 8 bits per
-                             operand (~1e-12).  QR, reduced eig, residuals and
-                             locking in native FP64.                         */
+                             operand (~1e-12).  A full-storage solve's QR and
+                             Rayleigh-Ritz products take residues of 58-bit
+                             operands (15 moduli, FP64 rounding); reduced eig,
+                             residuals and locking in native FP64.           */
     CHASE_MIXED_FP32 = 1, /* filter products at FP32-level accuracy on the
                              tensor cores (first 4 slices: 32 bits relative to
                              the row/column maximum, 10 slice pairs) while
                              every unlocked residual exceeds 1e-6, then on 5
                              slices (15 pairs) while every one exceeds 1e-8,
                              then FP64-accurate filter sweeps; Lanczos, QR,
-                             Rayleigh-Ritz and residuals as in CHASE_FP64.
+                             Rayleigh-Ritz and residuals as in CHASE_FP64 with
+                             half storage.
                              In single-phase entry points it selects the
                              FP32-level product.                             */
     CHASE_MIXED_BF16X3 = 2, /* accepted and run as CHASE_MIXED_FP32, the
@@ -166,8 +169,9 @@ typedef struct {
      * timed with CUDA events around each launch on the solver's stream:    */
     double tc_kernel_ms;        /* summed launch durations                    */
     int64_t tc_kernel_launches; /* launches timed                             */
-    double tc_kernel_tflops;    /* executed BF16 tensor flops (8 per complex  */
-                                /* multiply-add per slice pair) / duration    */
+    double tc_kernel_tflops;    /* executed tensor flops / duration: per      */
+                                /* complex multiply-add 6 or 8 for each of 13 */
+                                /* moduli (FP64), 8 per slice pair otherwise  */
     int nex_used;               /* nex at the end (differs from the argument
                                    when the nex tuner grew it)                */
     int64_t filter_matvecs_mid; /* filter products on 5 slices
@@ -304,10 +308,11 @@ int chase_rayleigh_ritz(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t l
  * "RR" items): d_G (m1 x m2, ldg >= m1) = A^H B for A: K x m1 (lda), B: K x m2
  * (ldb), 1 <= m1, m2 <= 512.  Run-to-run deterministic.  For K >= 64 in
  * residue arithmetic on the tensor cores (operands of 58 bits against each
- * column's 2-norm, exact sums, one rounding; its workspace, up to 30 bytes per
- * element of the wider block and 90 of the other, stays in the context), in
- * native FP64 below, where that workspace cannot be had, and for non-finite
- * operands, whose product is what IEEE arithmetic makes of them. */
+ * column's 2-norm, exact sums, one rounding).  Its workspace (30 bytes per
+ * element of the wider block, padded to 128s, 90 of the other, padded by 64)
+ * stays in the context.  In native FP64 for smaller K, where that is more than
+ * 8 GB or cannot be had, and for non-finite operands, whose product is what
+ * IEEE arithmetic makes of them. */
 int chase_gram(bsechase_ctx *ctx, const void *d_A, int64_t lda, const void *d_B, int64_t ldb,
                int64_t K, int m1, int m2, void *d_G, int64_t ldg);
 

@@ -548,6 +548,11 @@ int residue_buffers(bsechase_ctx *ctx, int64_t N, int m, int k, bool tall, ResBu
     size_t r = residue_out_bytes(m, N, (int)mk);
     if (tall) r = std::max(r, residue_out_bytes(N, mk, m));
     const size_t ne = (size_t)(Np + 512), parts = kResParts;
+    // More than that is not allocated for them alone (a solve's buffers hold them
+    // already): native FP64, as without memory.
+    constexpr size_t kMost = (size_t)8 << 30;
+    if (va + la + vb + lb + r > kMost && (va + la > ctx->ozGA.bytes || vb + lb > ctx->ozB.bytes || r > ctx->ozP.bytes))
+        return BSE_ENOMEM;
     int rc;
     if ((rc = ensure(ctx, ctx->ozGA, va + la)) || (rc = ensure(ctx, ctx->ozB, vb + lb)) ||
         (rc = ensure(ctx, ctx->ozP, r)) || (rc = ensure(ctx, ctx->ozGE, 2 * ne * sizeof(int))) ||
