@@ -5,16 +5,15 @@ H on the device (Eq. (1) stand-in), then solve for the lowest nev
 eigenpairs (Lanczos, filter, QR, Rayleigh-Ritz, residuals/locking, output).
 Workload: N = 50000 (Nk = 3125, Nv = Nc = 4; H is 40 GB), nev = 200,
 nex = 80, deg_max = 36, tol = 1e-10, complex FP64.  The filter degrees of
-Eq. (S1) are raised in groups of 48 columns, the tile width of the
-tensor-core product (--degree-group; 0 keeps them unchanged, and the line
-also reports one solve that way).  H is far larger than L2, so no L2 flush
+Eq. (S1) are raised in groups of 48 columns (--degree-group; 0 keeps them
+unchanged, and the line also reports one solve that way).  H is far larger than L2, so no L2 flush
 is needed between steps.
 
 After the timed steps the line adds: one end-to-end solve through the
 host-buffer entry point (H copied in, eigenvectors copied out); one solve
 in the mixed precision mode with its per-eigenpair differences from the
 FP64 solve; one solve with the degrees of Eq. (S1) unchanged; one solve
-with H generated straight into its tensor-core slices (never stored); the
+with H generated straight into its tensor-core form (never stored); the
 CPU oracle timed on the host's cores on a bounded sample of the same
 workload; and the serving mix.
 
@@ -174,18 +173,20 @@ def workload(args):
 
 
 PRECISIONS = {"fp64": 0, "mixed": 1, "fp64_dfma": 3}
-DTYPES = {"fp64": "f64 (H products: bf16 slices on tensor cores, exact int + f32 accumulation)",
+DTYPES = {"fp64": "f64 (products: residues of 51-bit and wider integers on tensor cores, exact f32 accumulation)",
           "mixed": "f64 with f32-level filter sweeps (4 bf16 slices, exact accumulation)",
           "fp64_dfma": "f64"}
 def roofline(precision, st, N, workload_name):
     """Roofline of the dominant kernel, the filter's matrix product.
 
-    Tensor-core precisions: the product kernel k_ozaki_zgemm is timed by the
-    library with CUDA events around every launch on its stream, inside this
-    timed region.  Its algorithmic work per launch is 8 N^2 n real flops per
-    slice pair (21 pairs at FP64 accuracy, 10 at FP32 level) for n columns:
-    achieved = summed work / summed launch time, against the measured BF16
-    peak.  DFMA precision: the FP64-equivalent filter rate (8 N^2 per column
+    Tensor-core precisions: the product kernel (k_res_zgemm at FP64, and
+    k_ozaki_zgemm in the mixed mode) is timed by the library with CUDA events
+    around every launch on its stream, inside this timed region.  Its
+    algorithmic work per launch of n columns is, at FP64, 13 moduli of 6 or 8
+    N^2 n real FP16 flops (three real products above 112 columns a tile, four
+    up to it), in the mixed mode 8 N^2 n BF16 flops per slice pair (10, 15 or
+    21): achieved = summed work / summed launch time, against the measured
+    peak (BF16 and FP16 run at one rate).  DFMA precision: the FP64-equivalent filter rate (8 N^2 per column
     product over the filter phase) against the measured DFMA peak."""
     peaks = _peaks()
     fp64_eq = st["filter_tflops"]
@@ -201,7 +202,8 @@ def roofline(precision, st, N, workload_name):
     achieved = st["tc_kernel_tflops"]
     peak = peaks.get("bf16_tflops_sustained") or 1700.0
     launches = max(1, st["tc_kernel_launches"])
-    return {"kernel": "k_ozaki_zgemm (H*Y: BF16 slice products on tcgen05, Chebyshev epilogue)",
+    return {"kernel": "k_res_zgemm (H*Y: FP16 residue products on tcgen05)" if precision == "fp64" else
+                      "k_ozaki_zgemm (H*Y: BF16 slice products on tcgen05)",
             "bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak,
             "peak_source": ("MEASURED_PEAKS.json bf16_tflops_sustained (kernel timed inside "
@@ -469,7 +471,7 @@ def run_ours(args, rank, world, local_rank):
         extras["degree_group_0"] = {"value": t_0, "unit": UNIT, "iters": st_0["iters"],
                                     "matvecs": st_0["matvecs"], "max_resid": float(np.max(r_0))}
         del V_0
-        # the same solve with H generated straight into its tensor-core slices
+        # the same solve with H generated straight into its tensor-core form
         # (chase_solve_bse: the 16 N^2 bytes of H are never stored); generator
         # included, like the timed step
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
