@@ -314,7 +314,7 @@ int hop_apply(bsechase_ctx *ctx, const Hop &op, int n, const z_t *Y, int64_t ldy
               int64_t ldc, const GemmEpi &ep) {
     if (op.res) {
         cudaEvent_t e0 = nullptr, e1 = nullptr;
-        if (!ctx->batcher) kernel_events(ctx, residue_flops(op.N, op.N, n), &e0, &e1);
+        if (!ctx->batcher && op.gen) kernel_events(ctx, residue_flops(op.N, op.N, n), &e0, &e1);
         CK(residue_zgemm(ctx->oh, n, Y, ldy, C, ldc, ep, ctx->ozB.p, ctx->ozB.bytes, (int *)ctx->ozF.p,
                          (float2 *)((char *)ctx->ozF.p + hop_f_bytes(ctx->hop_cols)), ctx->ozP.p, ctx->ozP.bytes,
                          ctx->sc, ctx->sms, ctx->st, e0, e1, ctx->batcher));
