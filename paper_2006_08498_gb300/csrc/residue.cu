@@ -880,7 +880,8 @@ k_res_rowscale(int64_t M, int64_t Mp, int nseg, const float2 *__restrict__ part,
 // rows a block, a thread per row and segment, and the same sums in the same
 // order as the two kernels above.  For short segments only (N < 4096): 17 us
 // against 16 + 14 at N = 2000, but with one block for 8 whole rows 1056 us
-// against 940 + 17 at N = 20000.
+// against 940 + 17 at N = 20000.  Segments of 8 columns up to N = 1024 fill the
+// threads there: a product with its preparation at N = 256 47 -> 40 us.
 // With 32 rows and 8 segments at a time: the rows of a tall A of at most
 // kMaxTallCols columns (the general products).
 constexpr int kSmallSegs = 128, kMaxTallCols = 512, kTallSegs = kMaxTallCols / 32;
@@ -889,6 +890,7 @@ __global__ void __launch_bounds__(kRowsBlock *kSegThreads)
 k_res_rowexp(int64_t M, int64_t Mp, int64_t K, const z_t *__restrict__ A, int64_t lda, int seg, int nseg, int *E,
              ChaseScalars *sc) {
     __shared__ float2 part[kSegs][kRowsBlock];
+    follow();
     const int row = threadIdx.x % kRowsBlock;
     const int64_t i = (int64_t)blockIdx.x * kRowsBlock + row;
     for (int s = threadIdx.x / kRowsBlock; s < nseg; s += kSegThreads) {
@@ -1019,6 +1021,7 @@ template <int EL>   // K elements of a thread: 16, or 4 to fill the SMs from a s
 __global__ void __launch_bounds__(128, 4)
 k_res_slice_a(int64_t M, int64_t K, const z_t *__restrict__ A, int64_t lda, int64_t kbase, int64_t T,
               int64_t nch, const int *__restrict__ E, int nmod, int bits, uint8_t *__restrict__ S) {
+    follow();
     const int row = threadIdx.x;
     const int64_t i = (int64_t)blockIdx.y * kRows + row;
     const int64_t k0 = (int64_t)blockIdx.x * EL;               // within this panel
@@ -1404,7 +1407,7 @@ int choose_chunks(int64_t Mp, int nch, int mp, int tx, int w, int nmod, size_t r
     return best;
 }
 
-int norm_segment(int64_t N) { return N < 4096 ? 32 : 256; }
+int norm_segment(int64_t N) { return N <= 1024 ? 8 : N < 4096 ? 32 : 256; }
 constexpr int64_t kShortColumn = 4096;
 
 }  // namespace
@@ -1446,8 +1449,9 @@ cudaError_t residue_prepare(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh, vo
     oh->tri = false;
     const int seg = norm_segment(N), nseg = (int)((N + seg - 1) / seg);
     const unsigned rb = (unsigned)((N + 127) / 128);
-    if (seg == 32 && nseg <= kSmallSegs) {
-        k_res_rowexp<8, 64, kSmallSegs><<<(unsigned)(Np / 8), 512, 0, st>>>(N, Np, N, H, ldh, seg, nseg, oh->E, sc);
+    if (seg < 256 && nseg <= kSmallSegs) {
+        launch_next(k_res_rowexp<8, 64, kSmallSegs>, dim3((unsigned)(Np / 8)), dim3(512), 0, st, N, Np, N, H, ldh, seg,
+                    nseg, oh->E, sc);
         bse_count_launches(1);
     } else {
         k_res_rownorm<<<dim3(rb, (unsigned)nseg), 128, 0, st>>>(N, N, H, ldh, seg, 0, (float2 *)work);
@@ -1455,11 +1459,11 @@ cudaError_t residue_prepare(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh, vo
         bse_count_launches(2);
     }
     if (nch * 4 * T < 608)                         // too few blocks for four on every SM (N = 256: 9.2 us, 6.5 here)
-        k_res_slice_a<4><<<dim3((unsigned)(nch * 16), (unsigned)T), 128, 0, st>>>(N, N, H, ldh, 0, T, nch, oh->E, kNMod,
-                                                                                 kAlpha, (uint8_t *)oh->A);
+        launch_next(k_res_slice_a<4>, dim3((unsigned)(nch * 16), (unsigned)T), dim3(128), 0, st, N, N, H, ldh, (int64_t)0, T,
+                    nch, oh->E, kNMod, kAlpha, (uint8_t *)oh->A);
     else
-        k_res_slice_a<16><<<dim3((unsigned)(nch * 4), (unsigned)T), 128, 0, st>>>(N, N, H, ldh, 0, T, nch, oh->E, kNMod,
-                                                                                 kAlpha, (uint8_t *)oh->A);
+        launch_next(k_res_slice_a<16>, dim3((unsigned)(nch * 4), (unsigned)T), dim3(128), 0, st, N, N, H, ldh, (int64_t)0, T,
+                    nch, oh->E, kNMod, kAlpha, (uint8_t *)oh->A);
     bse_count_launches(1);
     return cudaGetLastError();
 }
@@ -1638,10 +1642,10 @@ cudaError_t residue_left(int64_t M, int64_t K, const z_t *A, int64_t lda, bool a
         launch_next(k_res_slice_ah, dim3((unsigned)nch, (unsigned)((M + 31) / 32)), dim3(128), 0, st, M, K, A, lda, T, nch,
                     col_parts(K), s.part, s.e, kGMod, kGBits, (uint8_t *)s.p);
     } else {
-        k_res_rowexp<32, 8, kTallSegs><<<(unsigned)(T * kRows / 32), 256, 0, st>>>(
-            M, T * kRows, K, A, lda, 32, (int)((K + 31) / 32), s.e, sc);
-        k_res_slice_a<16><<<dim3((unsigned)(nch * 4), (unsigned)T), 128, 0, st>>>(M, K, A, lda, 0, T, nch, s.e, kGMod,
-                                                                                 kGBits, (uint8_t *)s.p);
+        launch_next(k_res_rowexp<32, 8, kTallSegs>, dim3((unsigned)(T * kRows / 32)), dim3(256), 0, st, M, T * kRows, K, A,
+                    lda, 32, (int)((K + 31) / 32), s.e, sc);
+        launch_next(k_res_slice_a<16>, dim3((unsigned)(nch * 4), (unsigned)T), dim3(128), 0, st, M, K, A, lda, (int64_t)0, T,
+                    nch, s.e, kGMod, kGBits, (uint8_t *)s.p);
         bse_count_launches(1);
     }
     bse_count_launches(1);
