@@ -782,7 +782,9 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
             }
         }
         if (kGauss ? warp >= 1 && warp < 4 : warp == 3) {
-            if (tc::elect_one())
+            // lane 0 knows the copies issued: alone with four products, with
+            // Gauss every lane counts them
+            if (lane == 0)
                 for (int s = 0; s < kSB; s++) {
                     const int f = (fills - s + kSB - 1) / kSB;
                     if (f > 0)
