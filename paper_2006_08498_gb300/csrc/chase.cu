@@ -938,7 +938,7 @@ int solve_device(bsechase_ctx *ctx, const z_t *H, int64_t N, int64_t ldh, int ne
         // a last pass restores FP64 orthonormality across the locked blocks
         ResBufs rb;
         if ((rc = residue_buffers(ctx, N, nev, 0, true, &rb))) return rc;
-        rb.wait_ns = ctx->wait_ns;
+        rb.wait_ns = ctx->inject_last_wait_ns ? ctx->inject_last_wait_ns : ctx->wait_ns;
         if ((rc = cholqr_residues(ctx, rb, d_evecs, ldz, N, nev, 0.0))) return rc;
     } else if (op.tc) {
         // The Ritz vectors went through tensor-core products whose 48-bit
@@ -950,8 +950,8 @@ int solve_device(bsechase_ctx *ctx, const z_t *H, int64_t N, int64_t ldh, int ne
     }
     CK(launch_phase_normalize(N, nev, d_evecs, ldz, ctx->st));
     tm.mark(3);
-    CK(cudaStreamSynchronize(ctx->st));
-    harvest_kernel_times(ctx);
+    // the last pass reports through the scalars too (an expired wait, a failed factorisation)
+    if ((rc = sync_scalars(ctx))) return rc;
     tm.add(4, 2, 3);
     if (stats) {
         memset(stats, 0, sizeof *stats);
@@ -1068,6 +1068,14 @@ int bsechase_set_wait_limit(bsechase_ctx *ctx, double seconds) {
     ctx->wait_ns = (uint64_t)(seconds * 1e9);
     if (ctx->wait_ns == 0) ctx->wait_ns = 1;
     return BSE_OK;
+}
+
+int bsechase_inject(bsechase_ctx *ctx, int point, int64_t value) {
+    if (!ctx || value < 0) return BSE_EINVAL;
+    switch (point) {
+        case INJECT_LAST_PASS_WAIT_NS: ctx->inject_last_wait_ns = (uint64_t)value; return BSE_OK;
+        default: return BSE_EINVAL;
+    }
 }
 
 int bsechase_host_alloc(void **p, size_t bytes) {

@@ -38,6 +38,7 @@ struct bsechase_ctx {
     bool residues = true;            // solves may use the residue products (a server slot whose
                                      // request fits the budget on slices alone: not)
     int hop_cols = 0;                // columns the product buffers were sized for
+    uint64_t inject_last_wait_ns = 0;   // failure tests (bsechase_inject): wait limit of a solve's last pass
     int64_t wsN = 0;
     int wsM = 0;
     cudaEvent_t ev[kCtxEvents];   // 0..6: solve phases; 8, 9: host copies
@@ -52,6 +53,13 @@ struct bsechase_ctx {
     BseServer *server = nullptr;     // request server attached to this context
     OzBatcher *batcher = nullptr;    // a server slot's shared product batcher
 };
+
+// Failure tests of paths that no input reaches by itself; not part of the ABI.
+// 0 switches a point off.
+enum InjectPoint {
+    INJECT_LAST_PASS_WAIT_NS = 0   // wait limit, in ns, of the pass over a solve's output vectors
+};
+extern "C" int bsechase_inject(bsechase_ctx *ctx, int point, int64_t value);
 
 // Record a failure message (printf-style with one string argument).
 int fail(bsechase_ctx *c, int code, const char *fmt, const char *detail = "");

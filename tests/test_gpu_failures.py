@@ -1,11 +1,17 @@
 """Failures that a call has to report.  Every failure is made on the host: a
-short limit of the kernels' bounded waits."""
+short limit of the kernels' bounded waits, set by the caller or at one point of a
+call (bsechase_inject)."""
+import ctypes
+
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 import paper_2006_08498_gb300 as pkg  # noqa: E402
+
+LAST_PASS_WAIT_NS = 0
 
 
 @pytest.fixture
@@ -17,6 +23,12 @@ def ctx():
     c = pkg.Context(0)
     yield c
     c.close()
+
+
+def _inject(ctx, point, value):
+    f = pkg.load().bsechase_inject
+    f.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_int64]
+    assert f(ctx._h, point, value) == pkg.BSE_OK
 
 
 def _block(rows, cols, seed):
@@ -46,3 +58,18 @@ def test_expired_wait_in_every_product_kernel(ctx, n, kw):
         assert ei.value.status == pkg.BSE_ETIMEOUT
     ctx.set_wait_limit(2.0)
     assert torch.equal(ctx.hemm(A, Y, **kw), C)
+
+
+def test_solve_reports_a_failure_of_its_last_pass(ctx):
+    """The pass over the output vectors is the last thing that a solve does: a
+    wait that expires there fails the call like one before it.  (A look at a barrier
+    suspends a thread for some microseconds; the sums of this size take longer.)"""
+    H = ctx.build_hamiltonian(0, 500, 4, 4)
+    e, V, _, _ = ctx.solve(H, 100, 20)
+    _inject(ctx, LAST_PASS_WAIT_NS, 1)
+    with pytest.raises(pkg.BseError) as ei:
+        ctx.solve(H, 100, 20)
+    assert ei.value.status == pkg.BSE_ETIMEOUT
+    _inject(ctx, LAST_PASS_WAIT_NS, 0)
+    e2, V2, _, _ = ctx.solve(H, 100, 20)
+    assert np.array_equal(e, e2) and torch.equal(V, V2)
