@@ -194,9 +194,9 @@ const char *bsechase_last_error(const bsechase_ctx *ctx);
 
 /* Time limit, in seconds (0 < seconds <= 60, default 2), of every bounded
  * wait inside the context's tensor-core kernels (a wait for a copy, an MMA or
- * a drained accumulator; chase_qr and chase_gram keep the default).  When a wait runs out, the kernel stops issuing
- * work, waits for the copies and MMAs it already issued, releases its tensor
- * memory and returns; the call then fails with BSE_ETIMEOUT and the context
+ * a drained accumulator), those of chase_qr and chase_gram among them.  When a
+ * wait runs out, the kernel stops issuing work, waits for the copies and MMAs
+ * it already issued, releases its tensor memory and returns; the call then fails with BSE_ETIMEOUT and the context
  * stays usable.  A short limit makes that path run on purpose (failure
  * detection tests).  The paper has no counterpart.  Errors: BSE_EINVAL. */
 int bsechase_set_wait_limit(bsechase_ctx *ctx, double seconds);

@@ -533,7 +533,7 @@ struct ResBufs {
     RsSide VA, VB, LA, LB;
     void *R;
     size_t r_bytes;
-    uint64_t wait_ns = kDefaultWaitNs;
+    uint64_t wait_ns;
 };
 cudaError_t residue_mul(bsechase_ctx *ctx, const ResBufs &b, int64_t M, int n, int64_t K, const RsSide &A,
                         const RsSide &B, const RsOut &o) {
@@ -566,6 +566,7 @@ int residue_buffers(bsechase_ctx *ctx, int64_t N, int m, int k, bool tall, ResBu
     b->LB = RsSide{(char *)ctx->ozB.p + vb, lb, f + kMaxM, part + parts};
     b->R = ctx->ozP.p;
     b->r_bytes = ctx->ozP.bytes;
+    b->wait_ns = ctx->wait_ns;
     return BSE_OK;
 }
 
@@ -861,7 +862,6 @@ int solve_device(bsechase_ctx *ctx, const z_t *H, int64_t N, int64_t ldh, int ne
         ResBufs rb;
         if (op.res) {
             if ((rc = residue_buffers(ctx, N, ma, locked, true, &rb))) return rc;
-            rb.wait_ns = ctx->wait_ns;
             rc = phase_qr_residues(ctx, rb, V, N, locked, Va, N, N, ma);
         } else {
             rc = phase_qr(ctx, V, N, locked, Va, N, N, ma);
@@ -938,7 +938,7 @@ int solve_device(bsechase_ctx *ctx, const z_t *H, int64_t N, int64_t ldh, int ne
         // a last pass restores FP64 orthonormality across the locked blocks
         ResBufs rb;
         if ((rc = residue_buffers(ctx, N, nev, 0, true, &rb))) return rc;
-        rb.wait_ns = ctx->inject_last_wait_ns ? ctx->inject_last_wait_ns : ctx->wait_ns;
+        if (ctx->inject_last_wait_ns) rb.wait_ns = ctx->inject_last_wait_ns;
         if ((rc = cholqr_residues(ctx, rb, d_evecs, ldz, N, nev, 0.0))) return rc;
     } else if (op.tc) {
         // The Ritz vectors went through tensor-core products whose 48-bit

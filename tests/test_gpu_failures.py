@@ -73,3 +73,16 @@ def test_solve_reports_a_failure_of_its_last_pass(ctx):
     _inject(ctx, LAST_PASS_WAIT_NS, 0)
     e2, V2, _, _ = ctx.solve(H, 100, 20)
     assert np.array_equal(e, e2) and torch.equal(V, V2)
+
+
+def test_expired_wait_in_qr(ctx):
+    """The products of chase_qr are tensor-core kernels: the context's limit holds for their waits."""
+    V = _block(2000, 60, 3)
+    torch.cuda.synchronize()
+    ctx.set_wait_limit(1e-9)
+    with pytest.raises(pkg.BseError) as ei:
+        ctx.qr(V.clone(memory_format=torch.preserve_format))
+    assert ei.value.status == pkg.BSE_ETIMEOUT
+    ctx.set_wait_limit(2.0)
+    Q = ctx.qr(V)
+    assert torch.linalg.matrix_norm(Q.conj().T @ Q - torch.eye(60, device="cuda")) <= 6 * (2000 * 60 + 60 * 61) * 2.0 ** -53
