@@ -77,7 +77,8 @@ def test_solve_reports_a_failure_of_its_last_pass(ctx):
 
 def test_expired_wait_in_qr(ctx):
     """The products of chase_qr are tensor-core kernels: the context's limit holds for their waits."""
-    V = _block(2000, 60, 3)
+    N, m = 20000, 100                    # sums long enough for a wait to expire
+    V = _block(N, m, 3)
     torch.cuda.synchronize()
     ctx.set_wait_limit(1e-9)
     with pytest.raises(pkg.BseError) as ei:
@@ -85,4 +86,4 @@ def test_expired_wait_in_qr(ctx):
     assert ei.value.status == pkg.BSE_ETIMEOUT
     ctx.set_wait_limit(2.0)
     Q = ctx.qr(V)
-    assert torch.linalg.matrix_norm(Q.conj().T @ Q - torch.eye(60, device="cuda")) <= 6 * (2000 * 60 + 60 * 61) * 2.0 ** -53
+    assert torch.linalg.matrix_norm(Q.conj().T @ Q - torch.eye(m, device="cuda")) <= 6 * (N * m + m * (m + 1)) * 2.0 ** -53
