@@ -1366,9 +1366,10 @@ int chase_gram(bsechase_ctx *ctx, const void *d_A, int64_t lda, const void *d_B,
     int rc;
     if (sums_in_residues(K)) {
         rc = gram_residues(ctx, (const z_t *)d_A, lda, (const z_t *)d_B, ldb, K, m1, m2, (z_t *)d_G, ldg);
-        if (rc == BSE_OK) return rc;
-        // no memory for the residues, or non-finite operands, whose product is
-        // what IEEE arithmetic makes of them: native FP64
+        // Native FP64 without memory for the residues, and for non-finite
+        // operands, whose product is what IEEE arithmetic makes of them.  Anything
+        // else is a failure of the call.
+        if (rc != BSE_ENOMEM && rc != BSE_ENONFINITE) return rc;
         if (rc == BSE_ENOMEM) free_product_buffers(ctx);
         ctx->err.clear();
     }

@@ -87,3 +87,16 @@ def test_expired_wait_in_qr(ctx):
     ctx.set_wait_limit(2.0)
     Q = ctx.qr(V)
     assert torch.linalg.matrix_norm(Q.conj().T @ Q - torch.eye(m, device="cuda")) <= 6 * (N * m + m * (m + 1)) * 2.0 ** -53
+
+
+def test_expired_wait_in_gram(ctx):
+    """An expired wait fails the call; only missing memory and non-finite operands are for native FP64."""
+    A, B = _block(40000, 140, 4), _block(40000, 120, 5)
+    torch.cuda.synchronize()
+    G = ctx.gram(A, B)
+    ctx.set_wait_limit(1e-9)
+    with pytest.raises(pkg.BseError) as ei:
+        ctx.gram(A, B)
+    assert ei.value.status == pkg.BSE_ETIMEOUT
+    ctx.set_wait_limit(2.0)
+    assert torch.equal(ctx.gram(A, B), G)
