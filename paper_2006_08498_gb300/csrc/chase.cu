@@ -1308,7 +1308,10 @@ int chase_qr(bsechase_ctx *ctx, const void *d_L, int64_t ldl, int k, void *d_V, 
     int rc;
     if ((rc = ensure_workspace(ctx, N, k + m))) return rc;
     CK(cudaMemsetAsync(ctx->sc, 0, sizeof(ChaseScalars), ctx->st));
-    bool res = sums_in_residues(N);
+    // More columns than rows (kept ones that are zero or repeated; a block that has
+    // no basis, reported by its Cholesky factorisation): native FP64, as the
+    // residues' buffers are for tall blocks.
+    bool res = sums_in_residues(N) && m <= N && k <= N;
     ResBufs b;
     if (res && (rc = residue_buffers(ctx, N, m, k, true, &b))) {
         if (rc != BSE_ENOMEM) return rc;

@@ -100,3 +100,26 @@ def test_expired_wait_in_gram(ctx):
     assert ei.value.status == pkg.BSE_ETIMEOUT
     ctx.set_wait_limit(2.0)
     assert torch.equal(ctx.gram(A, B), G)
+
+
+@pytest.mark.parametrize("N,m,k", [(64, 5, 100), (100, 40, 129), (100, 129, 0), (64, 65, 3)])
+def test_qr_of_more_columns_than_rows(ctx, N, m, k):
+    """More kept columns than rows (zero ones, or repeated at no weight): projected like
+    fewer.  More columns than rows have no orthonormal basis: BSE_ENONFINITE."""
+    V0, L = _block(N, m, 6), None
+    if k:
+        L = torch.zeros((k, N), dtype=torch.complex128, device="cuda").T
+        L[:, :3] = torch.linalg.qr(_block(N, 3, 7))[0]
+    V = V0.clone(memory_format=torch.preserve_format)
+    torch.cuda.synchronize()
+    if m > N:
+        with pytest.raises(pkg.BseError) as ei:
+            ctx.qr(V, L)
+        assert ei.value.status == pkg.BSE_ENONFINITE
+        return
+    ctx.qr(V, L)
+    bound = 6 * (N * m + m * (m + 1)) * 2.0 ** -53
+    assert torch.linalg.matrix_norm(V.conj().T @ V - torch.eye(m, device="cuda")) <= bound
+    assert torch.linalg.matrix_norm(L.conj().T @ V) <= bound
+    P = V0 - L @ (L.conj().T @ V0)
+    assert torch.linalg.matrix_norm(V @ (V.conj().T @ P) - P) <= 2.0 ** -40 * torch.linalg.matrix_norm(P)
