@@ -207,3 +207,43 @@ def test_qr_of_sizes(ctx, N, m, k):
         assert torch.linalg.matrix_norm(L.conj().T @ V) <= bound
         P = V0 - L @ (L.conj().T @ V0)
     assert torch.linalg.matrix_norm(V @ (V.conj().T @ P) - P) <= 2.0 ** -40 * torch.linalg.matrix_norm(P)
+
+
+# ---- lines of subnormal numbers
+
+def _down(X, e):
+    """X 2^-e, exact where the result is a multiple of 2^-1074."""
+    return ((X * 2.0 ** -1000) * 2.0 ** (1000 - e)).T.contiguous().T
+
+
+@pytest.mark.parametrize("K", [300, 5000])
+def test_gram_of_the_smallest_numbers(ctx, K):
+    """Columns of entries below 2^-1042, which have no bits in a double's high word: integers of
+    18 bits times 2^-1060, exact as operands.  The result as for other integers: 2^-52 of
+    the element and 2^-70 of the norms, or a unit of 2^-1074."""
+    A, B = _integers(K, 6, 8), _integers(K, 4, 9)
+    Bt = _down(B, 1060)
+    torch.cuda.synchronize()
+    ref = A.conj().T @ B
+    norms = torch.linalg.vector_norm(A, dim=0)[:, None] * torch.linalg.vector_norm(B, dim=0)[None, :]
+    tol = 2.0 ** -52 * ref.abs() + 2.0 ** -70 * norms + 2.0 ** -13     # in units of 2^-1060
+    up = lambda G: (G * 2.0 ** 1000) * 2.0 ** 60
+    assert torch.all((up(ctx.gram(A, Bt)) - ref).abs() <= tol)
+    assert torch.all((up(ctx.gram(Bt, A)) - ref.conj().T).abs() <= tol.T)
+
+
+@pytest.mark.parametrize("N", [300, 4200])
+def test_hemm_of_the_smallest_numbers(ctx, N):
+    """A row of H, and the columns of Y, of such entries: exact as operands, so that only the
+    result's own rounding is left (2^-49 of the norms, or a unit of 2^-1074)."""
+    H, Y = _integers(N, N, 10), _integers(N, 3, 11)
+    ref = H @ Y                          # of 18 bits both: exact
+    tol = 2.0 ** -49 * torch.linalg.vector_norm(H, dim=1)[:, None] * torch.linalg.vector_norm(Y, dim=0)[None, :]
+    Ht, Yt = H.clone(memory_format=torch.preserve_format), _down(Y, 1070)
+    Ht[5] = _down(H, 1063)[5]
+    torch.cuda.synchronize()
+    C = (ctx.hemm(H, Yt) * 2.0 ** 1000) * 2.0 ** 70
+    assert torch.all((C - ref).abs() <= tol + 2.0 ** -3)
+    C = ctx.hemm(Ht, Y)
+    C[5] = (C[5] * 2.0 ** 1000) * 2.0 ** 63
+    assert torch.all((C - ref).abs() <= tol + 2.0 ** -10)
