@@ -292,8 +292,9 @@ int chase_filter(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t ldh, voi
 /* QR phase (Supplement, "QR" item): d_V (N x m) becomes an orthonormal
  * basis of span(d_V) projected off span(d_L) (d_L: N x k orthonormal, may
  * be NULL with k = 0): two projections, column scaling, shifted Cholesky QR
- * and two Cholesky QR passes each after a projection.  Its products run as
- * chase_gram's do. */
+ * and two Cholesky QR passes each after a projection.  Its products run in
+ * residues as chase_gram's do, for blocks of up to N columns, with an error
+ * relative to the norms of rows and columns (which is what Cholesky QR needs). */
 int chase_qr(bsechase_ctx *ctx, const void *d_L, int64_t ldl, int k, void *d_V, int64_t ldv,
              int64_t N, int m);
 
@@ -311,8 +312,11 @@ int chase_rayleigh_ritz(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t l
  * column's 2-norm, exact sums, one rounding).  Its workspace (30 bytes per
  * element of the wider block, padded to 128s, 90 of the other, padded by 64)
  * stays in the context.  In native FP64 for smaller K, where that is more than
- * 8 GB or cannot be had, and for non-finite operands, whose product is what
- * IEEE arithmetic makes of them. */
+ * 8 GB or cannot be had, for non-finite operands, whose product is what
+ * IEEE arithmetic makes of them, and for graded columns: where the real or
+ * imaginary part of some element has, as the sum of its products' magnitudes,
+ * less than about 1/16 of the columns' norms (and not zero).  So every element is
+ * accurate against that sum, as a sum of FP64 products is. */
 int chase_gram(bsechase_ctx *ctx, const void *d_A, int64_t lda, const void *d_B, int64_t ldb,
                int64_t K, int m1, int m2, void *d_G, int64_t ldg);
 

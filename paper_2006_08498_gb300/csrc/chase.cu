@@ -660,6 +660,10 @@ int phase_rr_residues(bsechase_ctx *ctx, const Hop &op, const ResBufs &b, const 
 // kernel is short, and the residues' padding and launches cost more.
 bool sums_in_residues(int64_t K) { return K >= 64; }
 
+// What a product that has to run in native FP64 returns: operands for which residues
+// are less accurate, or non-finite ones.
+constexpr int kWantsNative = 1;
+
 // G = A^H B in residues, the wider block on the left; synchronises.
 int gram_residues(bsechase_ctx *ctx, const z_t *A, int64_t lda, const z_t *B, int64_t ldb, int64_t K, int m1, int m2,
                   z_t *G, int64_t ldg) {
@@ -676,10 +680,15 @@ int gram_residues(bsechase_ctx *ctx, const z_t *A, int64_t lda, const z_t *B, in
     int rc;
     if ((rc = residue_buffers(ctx, K, m1, m2, false, &b))) return rc;
     CK(cudaMemsetAsync(ctx->sc, 0, sizeof(ChaseScalars), ctx->st));
-    CK(residue_left(m1, K, A, lda, true, b.VA, ctx->sc, ctx->st));
-    CK(residue_right(K, m2, B, ldb, same ? b.VA.part : nullptr, b.VB, ctx->sc, ctx->sms, ctx->st));
+    const float2 *nb = same ? b.VA.part : b.VB.part;
+    CK(residue_norms(K, m1, A, lda, b.VA.part, ctx->sc, ctx->st));
+    if (!same) CK(residue_norms(K, m2, B, ldb, b.VB.part, ctx->sc, ctx->st));
+    CK(residue_weigh(K, m1, m2, A, lda, b.VA.part, B, ldb, nb, same, b.R, b.r_bytes, ctx->sc, ctx->sms, ctx->st));
+    CK(residue_left(m1, K, A, lda, true, b.VA, ctx->sc, ctx->st, true));
+    CK(residue_right(K, m2, B, ldb, nb, b.VB, ctx->sc, ctx->sms, ctx->st));
     CK(residue_mul(ctx, b, m1, m2, K, b.VA, b.VB, o));
-    return sync_scalars(ctx);
+    rc = sync_scalars(ctx);
+    return rc && (ctx->hsc->error == DEV_GRADED || ctx->hsc->error == DEV_NONFINITE) ? kWantsNative : rc;
 }
 
 // Rayleigh-Ritz: theta (device), Vout = Q Y (ld N), HVout = H Q Y (ld N)
@@ -1369,10 +1378,11 @@ int chase_gram(bsechase_ctx *ctx, const void *d_A, int64_t lda, const void *d_B,
     int rc;
     if (sums_in_residues(K)) {
         rc = gram_residues(ctx, (const z_t *)d_A, lda, (const z_t *)d_B, ldb, K, m1, m2, (z_t *)d_G, ldg);
-        // Native FP64 without memory for the residues, and for non-finite
-        // operands, whose product is what IEEE arithmetic makes of them.  Anything
-        // else is a failure of the call.
-        if (rc != BSE_ENOMEM && rc != BSE_ENONFINITE) return rc;
+        // Native FP64 without memory for the residues; for columns with entries so
+        // far below their norm that they count and residues would lose them; for
+        // non-finite operands, whose product is what IEEE arithmetic makes of them.
+        // Anything else is a failure of the call.
+        if (rc != BSE_ENOMEM && rc != kWantsNative) return rc;
         if (rc == BSE_ENOMEM) free_product_buffers(ctx);
         ctx->err.clear();
     }

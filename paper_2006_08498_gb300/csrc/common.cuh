@@ -89,6 +89,7 @@ enum DevError : int {
     DEV_NONFINITE = 3,     // NaN or Inf met in a reduction
     DEV_BAD_ARG = 4,       // a kernel got an argument outside its limits
     DEV_TIMEOUT = 5,       // a bounded wait inside a kernel expired
+    DEV_GRADED = 6,        // a Gram product wants native FP64 (residue_weigh)
 };
 
 // Scalars shared between the kernels of one solve (device resident).

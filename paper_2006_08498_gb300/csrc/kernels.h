@@ -169,8 +169,11 @@ cudaError_t residue_zgemm(const OzakiH &oh, int n, const z_t *Y, int64_t ldy, z_
                           const GemmEpi &ep, void *B, size_t b_bytes, int *F, float2 *part, void *R,
                           size_t r_bytes, ChaseScalars *sc, int sms, cudaStream_t st, cudaEvent_t ev0,
                           cudaEvent_t ev1, OzBatcher *batcher);
-// General products C = out(op(A) B), op(A) M x K, B K x n, at native FP64's
-// accuracy or better (operands of 58 bits against each line's 2-norm): the left
+// General products C = out(op(A) B), op(A) M x K, B K x n, accurate normwise: operands
+// of 58 bits against each line's 2-norm, an error of about 2^-58 of the norms'
+// product (worst case 2^-57 sqrt(K)), which native FP64 seldom reaches.  Entries far
+// below their line's norm lose bits, though, and an element far below its norms'
+// product with them: residue_weigh tells.  The left
 // operand's rows (A, K <= 512, or A^H with ah and A K x M) and the right
 // operand's columns are turned into residues once and multiplied as often as
 // wanted.  A side's buffers: p of residue_left_bytes or residue_right_bytes, e
@@ -198,11 +201,20 @@ size_t residue_left_bytes(int64_t M, int64_t K);
 size_t residue_right_bytes(int64_t K, int n);
 size_t residue_out_bytes(int64_t M, int64_t K, int n);   // the splits' residues
 cudaError_t residue_left(int64_t M, int64_t K, const z_t *A, int64_t lda, bool ah, const RsSide &s, ChaseScalars *sc,
-                         cudaStream_t st);
+                         cudaStream_t st, bool normed = false);
 cudaError_t residue_right(int64_t K, int n, const z_t *B, int64_t ldb, const float2 *norms, const RsSide &s,
                           ChaseScalars *sc, int sms, cudaStream_t st);
 cudaError_t residue_product(int64_t M, int n, int64_t K, const RsSide &A, const RsSide &B, const RsOut &out, void *R,
                             size_t r_bytes, uint64_t wait_ns, ChaseScalars *sc, int sms, cudaStream_t st);
+// The norms of n columns (kRsColParts pairs each), for residue_left (normed: with ah,
+// left in its side's part), residue_right and residue_weigh.
+cudaError_t residue_norms(int64_t K, int n, const z_t *A, int64_t lda, float2 *part, ChaseScalars *sc, cudaStream_t st);
+// Sets DEV_GRADED in sc unless every element of A^H B (A K x m1, B K x m2) is as
+// accurate in residues as in native FP64, against its own products' magnitudes; work:
+// 8 m1 m2 bytes or a few times as many.
+cudaError_t residue_weigh(int64_t K, int m1, int m2, const z_t *A, int64_t lda, const float2 *normsA, const z_t *B,
+                          int64_t ldb, const float2 *normsB, bool same, void *work, size_t bytes, ChaseScalars *sc,
+                          int sms, cudaStream_t st);
 // Product batcher shared by the solver threads of a request server: products
 // submitted within window_s of each other (or as soon as every active solver
 // has submitted one) run in one launch of the tensor-core kernel.

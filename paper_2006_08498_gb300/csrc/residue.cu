@@ -1390,6 +1390,143 @@ k_res_out(int64_t M, int64_t Mp, int mp, int nz, const uchar2 *__restrict__ R, c
     }
 }
 
+// Whether a Gram element keeps FP64's accuracy in residues.  The operands are
+// rounded to units of 2^(h - 58), 2^h >= the column's norm, so that the rms error of Re
+// (or Im) G_ij is at most 2^-59.3 2^(hi + hj).  Native FP64 is accurate against
+//   S = sum_k |Re a||Re b| + |Im a||Im b|   (Im: |Re a||Im b| + |Im a||Re b|)
+// instead, which may lie far below the norms' product: entries far below their
+// column's norm count there (a = (1, 0, ..), b = (1e-20, 1, ..)).  Where S >= 2^-4
+// 2^(hi + hj) the residues' error is below 2^-55.3 S, less than one FP64 rounding of S
+// (rms 2^-54.8); columns of even size have S = 0.16 .. 0.64 of it.  If any element has
+// less, and not zero (whose product is exact), DEV_GRADED asks for native FP64.
+// S by FP16 magnitudes relative to 2^h (entries below 2^-26 of it count as that,
+// zero ones as zero) with FP32 sums, tiles of 64 x 64 columns over a part of the rows:
+// straight after the norms, while A and B are in L2.  K = 20000, 140 x 40: 25 us and 6 for
+// the sums, of 194 (165 without the check; native FP64: 1810).
+constexpr int kWtTile = 64, kWtRows = 32;          // columns of a tile; rows staged at once
+constexpr int kWtExp = 12;                         // 2^h becomes 2^12 in FP16
+__device__ __forceinline__ float weight(double x, int up) {
+    const uint32_t h = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
+    const int t = max((int)(h + (uint32_t)up), 113 << 20);     // FP32 exponent, 20 mantissa bits
+    return (h | (uint32_t)__double2loint(x)) == 0 ? 0.f : __uint_as_float((uint32_t)t << 3);
+}
+// The same in a column of norm below 2^-1000, whose entries may all be subnormal.
+__device__ __forceinline__ float weight_small(double x, int up) {
+    const double a = fabs(x) * 0x1.0p1022;
+    return a == 0.0 ? 0.f : fmaxf((float)ldexp(a, up / (1 << 20) - 126), 0x1.0p-14f);
+}
+constexpr int kUpSmall = (kWtExp + 1000 + 127 - 1023) * (1 << 20);
+__device__ __forceinline__ uint32_t weights(z_t v, int up) {
+    __half2 w;
+    if (up <= kUpSmall) w = __floats2half2_rn(weight(v.x, up), weight(v.y, up));
+    else w = __floats2half2_rn(weight_small(v.x, up), weight_small(v.y, up));
+    uint32_t r;
+    memcpy(&r, &w, 4);
+    return r;
+}
+__device__ __forceinline__ void mma_16816(float *d, const uint32_t *a, uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// P[z][j][i]: (Re, Im) of the rows of part z.  With upper (A = B) the tiles on and
+// above the diagonal alone.
+__global__ void __launch_bounds__(256, 2)
+k_res_weights(int64_t K, int64_t rows, int m1, int m2, const z_t *__restrict__ A, int64_t lda,
+              const float2 *__restrict__ partA, const z_t *__restrict__ B, int64_t ldb,
+              const float2 *__restrict__ partB, int npart, int upper, float2 *__restrict__ P) {
+    __shared__ uint32_t sA[kWtTile][kWtRows + 4], sB[kWtTile][kWtRows + 4];   // (Re, Im) of a row each
+    __shared__ int upA[kWtTile], upB[kWtTile];
+    follow();
+    if (upper && blockIdx.x > blockIdx.y) return;
+    const int i0 = blockIdx.x * kWtTile, j0 = blockIdx.y * kWtTile;
+    const int t = threadIdx.x, lane = t % 32, warp = t / 32;
+    if (t < 2 * kWtTile) {
+        const bool b = t >= kWtTile;
+        const int c = t % kWtTile;
+        NormAcc n;
+        if (b ? j0 + c < m2 : i0 + c < m1) {
+            const float2 *part = b ? partB + (int64_t)(j0 + c) * npart : partA + (int64_t)(i0 + c) * npart;
+            for (int s = 0; s < npart; s++) n.add(part[s]);
+        }
+        const int h = n.exponent();
+        (b ? upB : upA)[c] = h == INT_MIN ? 0 : (kWtExp - h + 127 - 1023) * (1 << 20);
+    }
+    __syncthreads();
+    const int64_t kb = (int64_t)blockIdx.z * rows, ke = min(K, kb + rows);
+    float acc[2][4][4] = {};                       // [Re, Im][8 columns of B][fragment]
+    const int wi = warp % 4 * 16, wj = warp / 4 * 32, g = lane / 4, q = lane % 4;
+    z_t va[8], vb[8];
+    auto load = [&](int64_t k) {
+#pragma unroll
+        for (int c = 0; c < 8; c++) {
+            const int col = warp + 8 * c;
+            va[c] = (k < ke && i0 + col < m1) ? A[k + (i0 + col) * lda] : zmk(0.0, 0.0);
+            vb[c] = (k < ke && j0 + col < m2) ? B[k + (j0 + col) * ldb] : zmk(0.0, 0.0);
+        }
+    };
+    load(kb + lane);
+    for (int64_t k0 = kb; k0 < ke; k0 += kWtRows) {
+        if (k0 > kb) __syncthreads();              // the step before has been read
+#pragma unroll
+        for (int c = 0; c < 8; c++) {
+            const int col = warp + 8 * c;
+            sA[col][lane] = i0 + col < m1 ? weights(va[c], upA[col]) : 0;
+            sB[col][lane] = j0 + col < m2 ? weights(vb[c], upB[col]) : 0;
+        }
+        __syncthreads();
+        load(k0 + kWtRows + lane);                 // under way during the products
+#pragma unroll
+        for (int s = 0; s < kWtRows; s += 8) {
+            const uint32_t a[4] = {sA[wi + g][s + q], sA[wi + g + 8][s + q], sA[wi + g][s + q + 4], sA[wi + g + 8][s + q + 4]};
+#pragma unroll
+            for (int n = 0; n < 4; n++) {
+                const uint32_t b0 = sB[wj + 8 * n + g][s + q], b1 = sB[wj + 8 * n + g][s + q + 4];
+                mma_16816(acc[0][n], a, b0, b1);
+                mma_16816(acc[1][n], a, __byte_perm(b0, 0, 0x1032), __byte_perm(b1, 0, 0x1032));
+            }
+        }
+    }
+    float2 *Pz = P + (int64_t)blockIdx.z * m1 * m2;
+#pragma unroll
+    for (int n = 0; n < 4; n++)
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            const int i = i0 + wi + g + (e >= 2 ? 8 : 0), j = j0 + wj + 8 * n + 2 * q + (e & 1);
+            if (i < m1 && j < m2) Pz[(int64_t)j * m1 + i] = make_float2(acc[0][n][e], acc[1][n][e]);
+        }
+}
+// 32 elements a block, their parts over 8 warps.
+__global__ void __launch_bounds__(256)
+k_res_weigh(int m1, int m2, int nz, const float2 *__restrict__ P, int upper, ChaseScalars *sc) {
+    __shared__ float2 part[8][32];
+    follow();
+    const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
+    const int64_t n = (int64_t)m1 * m2, e = (int64_t)blockIdx.x * 32 + lane;
+    const int i = (int)(e % m1), j = (int)(e / m1);
+    const bool in = e < n && !(upper && i > j);
+    float2 s = make_float2(0.f, 0.f);
+    if (in) {
+#pragma unroll 4
+        for (int z = warp; z < nz; z += 8) {
+            const float2 p = P[(int64_t)z * n + e];
+            s.x += p.x;
+            s.y += p.y;
+        }
+    }
+    part[warp][lane] = s;
+    __syncthreads();
+    if (warp != 0 || !in) return;
+    for (int w = 1; w < 8; w++) {
+        s.x += part[w][lane].x;
+        s.y += part[w][lane].y;
+    }
+    constexpr float least = (float)(1 << (2 * kWtExp - 4));
+    if (upper && i == j) s.y = 0.f;                // the diagonal is real
+    if ((s.x > 0.f && s.x < least) || (s.y > 0.f && s.y < least)) set_error(sc, DEV_GRADED, j);
+}
+
 // 3-D FP16 tensor [tiles][rows][64], box 64 x box_rows x box_tiles, 128-byte swizzle
 bool make_map(CUtensorMap *m, void *base, uint64_t rows, uint64_t tiles, uint32_t box_rows, uint32_t box_tiles) {
     const TensorMapEncode enc = tensor_map_encode();
@@ -1664,11 +1801,11 @@ void col_norms(int64_t K, int64_t n, const z_t *A, int64_t lda, float2 *part, Ch
 }  // namespace
 
 cudaError_t residue_left(int64_t M, int64_t K, const z_t *A, int64_t lda, bool ah, const RsSide &s, ChaseScalars *sc,
-                         cudaStream_t st) {
+                         cudaStream_t st, bool normed) {
     const int64_t T = (M + kRows - 1) / kRows, nch = (K + kChunk - 1) / kChunk;
     if (M < 1 || K < 1 || residue_left_bytes(M, K) > s.bytes || (!ah && K > kMaxTallCols)) return cudaErrorInvalidValue;
     if (ah) {
-        col_norms(K, M, A, lda, s.part, sc, st);
+        if (!normed) col_norms(K, M, A, lda, s.part, sc, st);
         launch_next(k_res_slice_ah, dim3((unsigned)nch, (unsigned)((M + 31) / 32)), dim3(128), 0, st, M, K, A, lda, T, nch,
                     col_parts(K), s.part, s.e, kGMod, kGBits, (uint8_t *)s.p);
     } else {
@@ -1720,5 +1857,29 @@ cudaError_t residue_product(int64_t M, int n, int64_t K, const RsSide &A, const 
         launch_next(k_res_out<4>, dim3((unsigned)((M + 511) / 512), (unsigned)n), dim3(128), 0, st, M, Mp, j.mp, j.tz, j.R,
                     A.e, B.e, out);
     bse_count_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t residue_norms(int64_t K, int n, const z_t *A, int64_t lda, float2 *part, ChaseScalars *sc, cudaStream_t st) {
+    if (n < 1 || K < 1) return cudaErrorInvalidValue;
+    col_norms(K, n, A, lda, part, sc, st);
+    return cudaGetLastError();
+}
+
+cudaError_t residue_weigh(int64_t K, int m1, int m2, const z_t *A, int64_t lda, const float2 *normsA, const z_t *B,
+                          int64_t ldb, const float2 *normsB, bool same, void *work, size_t bytes, ChaseScalars *sc,
+                          int sms, cudaStream_t st) {
+    const int64_t tx = (m1 + kWtTile - 1) / kWtTile, ty = (m2 + kWtTile - 1) / kWtTile, n = (int64_t)m1 * m2;
+    // parts of 128 rows at least, and as many as fill the SMs and `work` holds
+    int64_t nz = std::min<int64_t>((K + 127) / 128, std::max<int64_t>(1, 2 * sms / (tx * ty)));
+    nz = std::min<int64_t>(nz, (int64_t)(bytes / (n * sizeof(float2))));
+    if (nz < 1) return cudaErrorInvalidValue;
+    const int64_t rows = ((K + nz - 1) / nz + kWtRows - 1) / kWtRows * kWtRows;
+    nz = (K + rows - 1) / rows;
+    launch_next(k_res_weights, dim3((unsigned)tx, (unsigned)ty, (unsigned)nz), dim3(256), 0, st, K, rows, m1, m2, A, lda,
+                normsA, B, ldb, normsB, col_parts(K), same ? 1 : 0, (float2 *)work);
+    launch_next(k_res_weigh, dim3((unsigned)((n + 31) / 32)), dim3(256), 0, st, m1, m2, (int)nz, (const float2 *)work,
+                same ? 1 : 0, sc);
+    bse_count_launches(2);
     return cudaGetLastError();
 }

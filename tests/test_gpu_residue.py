@@ -13,6 +13,7 @@ at most 2^-49 ||A||_F ||y_j||.  The reference is an FP64 product, whose error
 (about sqrt(K) 2^-53 of the same norms) is below that."""
 import math
 
+import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -247,3 +248,49 @@ def test_hemm_of_the_smallest_numbers(ctx, N):
     C = ctx.hemm(Ht, Y)
     C[5] = (C[5] * 2.0 ** 1000) * 2.0 ** 63
     assert torch.all((C - ref).abs() <= tol + 2.0 ** -10)
+
+
+# ---- columns with entries far below their norm
+
+def _graded_cases():
+    def first(K, m, head, rest):
+        A = _block(K, m, 31) * rest
+        A[0] = head
+        return A
+    yield "one large entry against a zero", lambda K, m1, m2: (first(K, m1, 1.0, 1e-9), first(K, m2, 0.0, 1.0))
+    yield "one entry against a tiny one", lambda K, m1, m2: (first(K, m1, 1.0, 0.0), first(K, m2, 1e-20, 1.0))
+    def decay(K, m1, m2):
+        d = torch.logspace(0, -18, K, dtype=torch.float64, device="cuda")[:, None]
+        return _block(K, m1, 32) * d, _block(K, m2, 33) * d.flip(0)
+    yield "opposite decays", decay
+    def parts(K, m1, m2):
+        B = _block(K, m2, 34)
+        return _block(K, m1, 35).real.to(torch.complex128), torch.complex(B.real, 1e-15 * B.imag)
+    yield "a small imaginary part", parts
+    def one_pair(K, m1, m2):
+        A, B = _block(K, m1, 36), _block(K, m2, 37)
+        A[:, m1 - 1] = 0
+        A[3, m1 - 1] = 1
+        B[3, m2 - 1] = 1e-18
+        return A, B
+    yield "one pair among many", one_pair
+
+
+@pytest.mark.parametrize("K,m1,m2", [(64, 3, 2), (400, 7, 20), (20000, 65, 70), (4097, 1, 130)])
+@pytest.mark.parametrize("case", range(5))
+def test_gram_of_graded_columns(ctx, K, m1, m2, case):
+    """Real and imaginary part of every element to FP64 against the sum of their own
+    products' magnitudes, as a sum of FP64 products has it in the worst case (2 K
+    roundings, and as many in the reference); entries far below their column's norm
+    count."""
+    name, make = list(_graded_cases())[case]
+    A, B = (x.T.contiguous().T for x in make(K, m1, m2))
+    torch.cuda.synchronize()
+    G = ctx.gram(A, B).cpu().numpy()
+    a, b = A.cpu().numpy(), B.cpu().numpy()
+    ar, ai, br, bi = (np.asfortranarray(x) for x in (a.real, a.imag, b.real, b.imag))
+    re, im = ar.T @ br + ai.T @ bi, ar.T @ bi - ai.T @ br
+    ar, ai, br, bi = abs(ar), abs(ai), abs(br), abs(bi)
+    tol = 4 * K * 2.0 ** -53
+    assert np.all(abs(G.real - re) <= tol * (ar.T @ br + ai.T @ bi)), name
+    assert np.all(abs(G.imag - im) <= tol * (ar.T @ bi + ai.T @ br)), name
