@@ -173,7 +173,7 @@ def workload(args):
 
 
 PRECISIONS = {"fp64": 0, "mixed": 1, "fp64_dfma": 3}
-DTYPES = {"fp64": "f64 (products: residues of 51-bit and wider integers on tensor cores, exact f32 accumulation)",
+DTYPES = {"fp64": "f64 (products: residues of 54-bit and wider integers on tensor cores, exact f32 accumulation)",
           "mixed": "f64 with f32-level filter sweeps (4 bf16 slices, exact accumulation)",
           "fp64_dfma": "f64"}
 def roofline(precision, st, N, workload_name):
@@ -182,7 +182,7 @@ def roofline(precision, st, N, workload_name):
     Tensor-core precisions: the product kernel (k_res_zgemm at FP64, and
     k_ozaki_zgemm in the mixed mode) is timed by the library with CUDA events
     around every launch on its stream, inside this timed region.  Its
-    algorithmic work per launch of n columns is, at FP64, 13 moduli of 6 or 8
+    algorithmic work per launch of n columns is, at FP64, 14 moduli of 6 or 8
     N^2 n real FP16 flops (three real products above 112 columns a tile, four
     up to it), in the mixed mode 8 N^2 n BF16 flops per slice pair (10, 15 or
     21): achieved = summed work / summed launch time, against the measured

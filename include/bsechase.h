@@ -60,9 +60,9 @@ typedef enum {
     CHASE_FP64 = 0,       /* FP64 accuracy.  Products with H (Lanczos, filter,
                              the solve's Rayleigh-Ritz) run on the tensor cores
                              in residue arithmetic: operands rounded to integers
-                             of 51 and 50 bits relative to their row's or
-                             column's 2-norm, the integer product exact modulo
-                             13 coprime moduli (normwise error ~1e-13 relative
+                             of 54 bits relative to their row's or column's
+                             2-norm, the integer product exact modulo 14
+                             coprime moduli (normwise error ~1e-14 relative
                              to ||H|| ||Y||).  With half storage, and in
                              chase_rayleigh_ritz, the products are the BF16
                              Ozaki-scheme emulation of 6 slices of 8 bits per
@@ -134,8 +134,8 @@ typedef struct {
                             nex + 8), min(N, 512) - nev).  The new columns are
                             the seeded start block's next columns. */
     int half_storage;    /* 0 (default): the tensor-core operand of all of H
-                            (26 N^2 bytes, 24 N^2 in the mixed mode).  1: of its lower triangle only
-                            (12 N^2 bytes), the strict upper triangle never
+                            (28 N^2 bytes, 24 N^2 in the mixed mode).  1: of
+                            its lower triangle only (12 N^2 bytes), the strict upper triangle never
                             read (H is Hermitian; the paper's reader holds one
                             triangle, Sec. 3): rows are scaled symmetrically,
                             H = T S T with t_i = sqrt(max_k |H_ik|), so that
@@ -170,7 +170,7 @@ typedef struct {
     double tc_kernel_ms;        /* summed launch durations                    */
     int64_t tc_kernel_launches; /* launches timed                             */
     double tc_kernel_tflops;    /* executed tensor flops / duration: per      */
-                                /* complex multiply-add 6 or 8 for each of 13 */
+                                /* complex multiply-add 6 or 8 for each of 14 */
                                 /* moduli (FP64), 8 per slice pair otherwise  */
     int nex_used;               /* nex at the end (differs from the argument
                                    when the nex tuner grew it)                */
@@ -245,7 +245,7 @@ int chase_solve(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t ldh, int 
  * (same seed, Nk, Nv, Nc, model), without storing it: its elements are
  * generated straight into the tensor-core slices of H, so the N x N
  * complex128 matrix (16 N^2 bytes) never exists and the device memory the
- * solve needs drops by 16 N^2 bytes, to 26 N^2 plus workspace (24 N^2 in the
+ * solve needs drops by 16 N^2 bytes, to 28 N^2 plus workspace (24 N^2 in the
  * mixed mode, 12 N^2 with chase_opts.half_storage) (Sec. 3's
  * filter works on H only through its products).  The slices, and so every
  * result, are bit for bit those of bse_build_hamiltonian + chase_solve.

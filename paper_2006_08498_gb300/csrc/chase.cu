@@ -262,7 +262,7 @@ int hop_prepare(bsechase_ctx *ctx, Hop &op, int max_cols) {
         rc = hop_buffers(ctx, op, mc);
     }
     if (rc == BSE_ENOMEM && op.res) {
-        // the residues take 2 N^2 bytes more than the slices: those, where only
+        // the residues take 4 N^2 bytes more than the slices: those, where only
         // they fit
         op.res = op.gen = false;
         free_product_buffers(ctx);

@@ -15,18 +15,22 @@
 //
 // Why residues.  With slices of 8 bits an FP64-accurate product takes every
 // pair of slices of the two operands (21 pairs of 48-bit operands with the
-// small ones left out); residues multiply modulus by modulus, 13 products for
-// operands of 51 and 50 bits: 13 x 8 = 104 tensor flops per complex multiply-add,
+// small ones left out); residues multiply modulus by modulus, 14 products for
+// operands of 54 bits: 14 x 8 = 112 tensor flops per complex multiply-add,
 // against 168.  And modulo p the complex product can take three real ones (Gauss)
 // instead of four, without the cancellation that form has in floating point:
 //   T0 = Ar Br, T1 = Ai Bi, T2 = (Ar + Ai)(Br + Bi);
-//   Re = T0 - T1, Im = T2 - T0 - T1  (mod p), 13 x 6 = 78.
+//   Re = T0 - T1, Im = T2 - T0 - T1  (mod p), 14 x 6 = 84.
 // Wide tiles, bound by the tensor cores (and their power), take three; narrow ones
 // take four, with fewer operands and accumulators to hand on.
 //
-// Accuracy.  The only rounding is that of the operands (and one FP64
-// rounding of the result): normwise about 2^-50 sqrt(N), without the
-// truncated partial sums that the slices leave.
+// Accuracy.  The only rounding is that of the operands (and one FP64 rounding of the
+// result): an rms error of 2^-53.8 of the norms' product ||h_i|| ||y_j|| at most, measured 2^-54.1
+// from N = 256 to 40000.  The slices, which round against a line's largest entry and
+// leave partial sums out, have 2^-46.4 to 2^-46.9 on exciton matrices (one large entry a
+// row) and 2^-49.7 (N = 256) to 2^-52.1 (N = 40000) on matrices of even entries.  13 moduli
+// and operands of 51 and 50 bits, 4 to 7 % less time, have 2^-50.4 on both, less than the
+// slices on the latter.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -68,8 +72,8 @@ void launch_next(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaS
 // ------------------------------------------------------------ the moduli
 // The product with H takes the first kNMod; the general products (kGMod below),
 // which stand in for native FP64, two more and operands of kGBits bits.
-constexpr int kNMod = 13, kGMod = 15;
-constexpr int kAlpha = 51, kBeta = 50, kGBits = 58;
+constexpr int kNMod = 14, kGMod = 15;
+constexpr int kAlpha = 54, kBeta = 54, kGBits = 58;
 constexpr int kMod[kGMod] = {256, 253, 251, 249, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197};
 
 constexpr int gcd_of(int a, int b) { return b == 0 ? a : gcd_of(b, a % b); }
@@ -97,17 +101,16 @@ static_assert(modulus_product(kNMod) / 2 > ((unsigned __int128)6 << (kAlpha + kB
 // most 127 for p <= 253, and 256 divides exactly), and the low byte of r + 128 +
 // 2^23 is the residue as it is stored: b in [0, 255] stands for b - 128.
 // (The same with an integer multiply-high and multiply in place of the FP32
-// steps: 278 instructions per element of A for the 26 residues, 178 of them on one
+// steps: 278 instructions per element of A for 26 residues, 178 of them on one
 // of the two FMA pipes.)
 struct ModConst {
     uint32_t clo, chi, k0;
     float pf, inv;
-    uint32_t w[2], g[3];    // W = round(2^64 ((P/p)^-1 mod p) / p), low word first; of all kGMod with 2^96
+    uint32_t w[2][3];       // W = round(2^96 ((P/p)^-1 mod p) / p), low word first: of kNMod moduli, and of all kGMod
 };
 struct ModTable {
     ModConst m[kGMod];
-    unsigned long long bias;           // 128 sum_m W_m
-    unsigned long long gbias, gbias2;  // the same of all kGMod: low and high 64 bits
+    unsigned long long bias[2][2];     // 128 sum_m W_m of either: low and high 64 bits
 };
 constexpr unsigned inverse_of_rest(int i, int n) {     // (P / p_i)^-1 mod p_i, P of the first n
     const unsigned p = (unsigned)kMod[i];
@@ -120,7 +123,7 @@ constexpr unsigned inverse_of_rest(int i, int n) {     // (P / p_i)^-1 mod p_i, 
 }
 constexpr ModTable make_table() {
     ModTable t{};
-    unsigned __int128 gb = 0;
+    unsigned __int128 bias[2] = {};
     for (int i = 0; i < kGMod; i++) {
         const unsigned p = (unsigned)kMod[i];
         unsigned c = 1 % p, cc[8] = {};
@@ -135,31 +138,29 @@ constexpr ModTable make_table() {
         t.m[i].k0 = 0x4B400000u + (2 * p - two63 - base) % p;
         t.m[i].pf = (float)p;
         t.m[i].inv = 1.0f / (float)p;
-        if (i < kNMod) {
-            const unsigned v = inverse_of_rest(i, kNMod);
-            const unsigned long long W = (unsigned long long)((((unsigned __int128)v << 64) + p / 2) / p);
-            t.m[i].w[0] = (uint32_t)W;
-            t.m[i].w[1] = (uint32_t)(W >> 32);
-            t.bias += 128 * W;
+        for (int set = 0; set < 2; set++) {
+            const int n = set == 0 ? kNMod : kGMod;
+            if (i >= n) continue;
+            const unsigned __int128 W = (((unsigned __int128)inverse_of_rest(i, n) << 96) + p / 2) / p;
+            for (int k = 0; k < 3; k++) t.m[i].w[set][k] = (uint32_t)(W >> (32 * k));
+            bias[set] += 128 * W;
         }
-        const unsigned __int128 G = (((unsigned __int128)inverse_of_rest(i, kGMod) << 96) + p / 2) / p;
-        for (int k = 0; k < 3; k++) t.m[i].g[k] = (uint32_t)(G >> (32 * k));
-        gb += 128 * G;
     }
-    t.gbias = (unsigned long long)gb;
-    t.gbias2 = (unsigned long long)(gb >> 64);
+    for (int set = 0; set < 2; set++)
+        for (int k = 0; k < 2; k++) t.bias[set][k] = (unsigned long long)(bias[set] >> (64 * k));
     return t;
 }
 __constant__ ModTable kTab = make_table();
 
-// The element is F / 2^64 P with F = sum_m W_m r_m modulo 2^64 as a signed
-// number: the fraction of sum_m r_m inv_m / p_m, to 2^-53 of the range.  The
-// general products keep 96 bits, to 2^-84: an element far below its norms'
-// product keeps its FP64 digits.  P as a 64-bit mantissa: P = mant 2^exp.
+// The element is F / 2^96 P with F = sum_m W_m r_m modulo 2^96 as a signed
+// number: the fraction of sum_m r_m inv_m / p_m, to 2^-84 of the range, so that an
+// element far below its norms' product keeps its FP64 digits (with 64 bits the sum over
+// the K splits' residues costs up to 2^-52 of the norms' product).  P as a 64-bit
+// mantissa: P = mant 2^exp.
 constexpr unsigned long long mantissa(int n, int e) {
     return (unsigned long long)((modulus_product(n) + ((unsigned __int128)1 << (e - 1))) >> e);
 }
-constexpr int kHExp = 39, kGExp = 54;
+constexpr int kHExp = 47, kGExp = 54;
 constexpr unsigned long long kHMant = mantissa(kNMod, kHExp), kGMant = mantissa(kGMod, kGExp);
 static_assert(kHMant >> 63 == 1 && kGMant >> 63 == 1, "normalised");
 
@@ -189,7 +190,7 @@ constexpr int kBars = 32;          // Gauss: barriers of the stages, as a ring (
 // Warpgroups (4 warps, one per TMEM quadrant): copies and MMAs; kConv converter
 // groups; two drain groups.  Registers a thread: R0, RC, RD (setmaxnreg moves
 // them from the others to the drain groups) of RL at launch; 0: no move.
-// H: stages of A a chunk takes (four products), 0: Gauss.  N = 8000, us at 16, 48, 80,
+// H: stages of A a chunk takes (four products), 0: Gauss.  With 13 moduli, N = 8000, us at 16, 48, 80,
 // 96, 112, 128, 144 columns: Gauss 295 314 351 375 443 455 481, four products 240 266
 // 324 359 407 444 508 (H's residues cross HBM in 248); twenty products of 140
 // columns at N = 20000, where the power limit counts too: 66.9 and 71.6 ms.
@@ -1041,8 +1042,8 @@ __device__ __forceinline__ void residues_of_row(const z_t *v, int sh, int nmod, 
 // k0 + 16 (blockIdx.x) of the matrix, read coalesced down the rows, and for
 // each modulus 16 bytes of Re and of Im, [group of 16][row][16 bytes] of the
 // chunk's 16 KB block, so that a converter thread's row is conflict-free.
-// Bound by integer issue: about 130 instructions per element for the 26
-// residues, over 16 bytes read and 26 written.
+// Bound by integer issue: about 140 instructions per element for the 28
+// residues, over 16 bytes read and 28 written.
 template <int EL>   // K elements of a thread: 16, or 4 to fill the SMs from a small matrix
 __global__ void __launch_bounds__(128, 4)
 k_res_slice_a(int64_t M, int64_t K, const z_t *__restrict__ A, int64_t lda, int64_t kbase, int64_t T,
@@ -1237,26 +1238,15 @@ __device__ __forceinline__ double to_double(unsigned long long m, int e, bool ne
     else v = ldexp((double)m, e);
     return neg ? -v : v;
 }
-struct WithH {                                     // the product with H
-    static constexpr int kMods = kNMod, kWords = 2, kBits = kAlpha + kBeta;
-    static __device__ __forceinline__ unsigned long long word(int m, int i) { return kTab.m[m].w[i]; }
-    // F P 2^(x - 64)
+template <int MODS, int BITS, int EXP, unsigned long long MANT, int SET>
+struct Recombine {
+    static constexpr int kMods = MODS, kWords = 3, kBits = BITS;
+    static __device__ __forceinline__ unsigned long long word(int m, int i) { return kTab.m[m].w[SET][i]; }
+    // F P 2^(x - 96): |F| P in integers, 64 bits of each, and one rounding to FP64
+    // (whose issue is scarce: with conversions and products in FP64 these took longer
+    // than the loads)
     static __device__ __forceinline__ double value(const unsigned long long *s, int nz, int x) {
-        const unsigned long long t = s[0] + (s[1] << 32) - kTab.bias * (unsigned)nz;
-        if (t == 0) return 0.0;
-        const bool neg = t >> 63;
-        const unsigned long long a = neg ? 0 - t : t;
-        const int lz = __clzll((long long)a);
-        return to_double(__umul64hi(a << lz, kHMant), kHExp - lz + x, neg);
-    }
-};
-struct General {                                   // the general products
-    static constexpr int kMods = kGMod, kWords = 3, kBits = 2 * kGBits;
-    static __device__ __forceinline__ unsigned long long word(int m, int i) { return kTab.m[m].g[i]; }
-    // |F| P in integers, 64 bits of each, and one rounding to FP64 (whose issue
-    // is scarce: with conversions and products in FP64 these took longer than the loads)
-    static __device__ __forceinline__ double value(const unsigned long long *s, int nz, int x) {
-        const unsigned __int128 b = ((unsigned __int128)kTab.gbias2 << 64 | kTab.gbias) * (unsigned)nz;
+        const unsigned __int128 b = ((unsigned __int128)kTab.bias[SET][1] << 64 | kTab.bias[SET][0]) * (unsigned)nz;
         unsigned __int128 t = s[0] + ((unsigned __int128)s[1] << 32) + ((unsigned __int128)s[2] << 64) - b;
         const bool neg = (uint32_t)(t >> 64) >> 31;            // F: 96 bits, signed
         if (neg) t = 0 - t;
@@ -1272,9 +1262,11 @@ struct General {                                   // the general products
         } else if (lz > 0) {
             hi = hi << lz | lo >> (64 - lz);
         }
-        return to_double(__umul64hi(hi, kGMant), kGExp - lz + x, neg);   // |F| = hi 2^(32 - lz)
+        return to_double(__umul64hi(hi, MANT), EXP - lz + x, neg);   // |F| = hi 2^(32 - lz)
     }
 };
+using WithH = Recombine<kNMod, kAlpha + kBeta, kHExp, kHMant, 0>;    // the product with H
+using General = Recombine<kGMod, 2 * kGBits, kGExp, kGMant, 1>;      // the general products
 // v[e]: elements (i + e, j), e < ROWS, where i + e < M (i a multiple of ROWS).
 // The loads of kAhead moduli are in flight together: all of them where one row
 // a thread leaves few threads, four with four rows, whose sums need the registers.

@@ -315,7 +315,7 @@ int chase_server_submit(bsechase_ctx *ctx, const chase_request *req, uint64_t *t
     q->rq.precision = precision_mode(req->precision);
     q->N = N;
     if (req->d_H && req->ldh < N) return fail(ctx, BSE_EINVAL, "request H: ldh < N%s");
-    // residue products where they fit the budget, else the slices (2 N^2 bytes less)
+    // residue products where they fit the budget, else the slices (4 N^2 bytes less)
     for (q->residues = precision_uses_residues(q->rq.precision, req->half_storage == 1);; q->residues = false) {
         q->run_bytes = estimate_run_bytes(N, m, req->nev, q->rq.precision, req->d_H == nullptr && !req->h_free,
                                           req->half_storage == 1, q->residues);

@@ -294,3 +294,30 @@ def test_gram_of_graded_columns(ctx, K, m1, m2, case):
     tol = 4 * K * 2.0 ** -53
     assert np.all(abs(G.real - re) <= tol * (ar.T @ br + ai.T @ bi)), name
     assert np.all(abs(G.imag - im) <= tol * (ar.T @ bi + ai.T @ br)), name
+
+
+# ---- the operands' precision
+
+def test_flat_matrix_keeps_the_precision_of_48_bit_slices(ctx):
+    """Entries of even size.  An operand's unit is at most 2^-53 of its norm, a rounding
+    moves a real number by a uniform half unit at most (variance 1/12): the two
+    operands give an element's complex error an rms of at most sqrt(1/6 + 1/6)
+    2^-53 = 2^-53.8 of the norms' product.  The reference sums FP64 products of 200
+    columns (2^-56.8).  48-bit slices have about 2^-50.4 at this size."""
+    N, n = 3000, 24
+    A, Y = _hermitian(N, 15), _block(N, n, 16)
+    torch.cuda.synchronize()
+    C = ctx.hemm(A, Y)
+    ref = sum(A[:, k:k + 200] @ Y[k:k + 200] for k in range(0, N, 200))
+    e = (C - ref).abs() / (torch.linalg.vector_norm(A, dim=1)[:, None] * torch.linalg.vector_norm(Y, dim=0)[None, :])
+    assert e.square().mean().sqrt() <= 2.0 ** -53.7
+
+
+@pytest.mark.parametrize("n", [5, 97, 113])
+def test_largest_sums_of_54_bits(ctx, n):
+    """Every operand's residue modulo 256 is -128 (integers 2^48 + 128 against
+    2-norms of 45.25 times that, both sides): the FP32 sums reach 2^24."""
+    N = 1024
+    A = torch.full((N, N), 1 + 2.0 ** -41, dtype=torch.complex128, device="cuda").T * (1 + 1j)
+    Y = torch.full((n, N), 1 + 2.0 ** -41, dtype=torch.complex128, device="cuda").T * (1 + 1j)
+    _check(A, Y, _hemm(ctx, A, Y))
