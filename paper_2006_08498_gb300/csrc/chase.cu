@@ -539,7 +539,11 @@ cudaError_t residue_mul(bsechase_ctx *ctx, const ResBufs &b, int64_t M, int n, i
                         const RsSide &B, const RsOut &o) {
     return residue_product(M, n, K, A, B, o, b.R, b.r_bytes, b.wait_ns, ctx->sc, ctx->sms, ctx->st);
 }
-int residue_buffers(bsechase_ctx *ctx, int64_t N, int m, int k, bool tall, ResBufs *b) {
+// What a product that has to run in native FP64 returns: residues that would take too
+// much memory or be less accurate, non-finite operands.
+constexpr int kWantsNative = 1;
+
+int residue_buffers(bsechase_ctx *ctx, int64_t N, int m, int k, bool tall, bool single, ResBufs *b) {
     auto up = [](size_t x) { return (x + 1023) / 1024 * 1024; };
     const int64_t Np = ozaki_padded(N), mk = std::max(m, k);
     const size_t va = up(std::max(residue_left_bytes(m, N), tall ? residue_left_bytes(N, m) : 0));
@@ -548,11 +552,10 @@ int residue_buffers(bsechase_ctx *ctx, int64_t N, int m, int k, bool tall, ResBu
     size_t r = residue_out_bytes(m, N, (int)mk);
     if (tall) r = std::max(r, residue_out_bytes(N, mk, m));
     const size_t ne = (size_t)(Np + 512), parts = kResParts;
-    // More than that is not allocated for them alone (a solve's buffers hold them
-    // already): native FP64, as without memory.
+    // More than that is not allocated for a single call (a solve's buffers hold them
+    // already), nor used if it is there: a call's bits follow its sizes.
     constexpr size_t kMost = (size_t)8 << 30;
-    if (va + la + vb + lb + r > kMost && (va + la > ctx->ozGA.bytes || vb + lb > ctx->ozB.bytes || r > ctx->ozP.bytes))
-        return BSE_ENOMEM;
+    if (single && va + la + vb + lb + r > kMost) return kWantsNative;
     int rc;
     if ((rc = ensure(ctx, ctx->ozGA, va + la)) || (rc = ensure(ctx, ctx->ozB, vb + lb)) ||
         (rc = ensure(ctx, ctx->ozP, r)) || (rc = ensure(ctx, ctx->ozGE, 2 * ne * sizeof(int))) ||
@@ -660,10 +663,6 @@ int phase_rr_residues(bsechase_ctx *ctx, const Hop &op, const ResBufs &b, const 
 // kernel is short, and the residues' padding and launches cost more.
 bool sums_in_residues(int64_t K) { return K >= 64; }
 
-// What a product that has to run in native FP64 returns: operands for which residues
-// are less accurate, or non-finite ones.
-constexpr int kWantsNative = 1;
-
 // G = A^H B in residues, the wider block on the left; synchronises.
 int gram_residues(bsechase_ctx *ctx, const z_t *A, int64_t lda, const z_t *B, int64_t ldb, int64_t K, int m1, int m2,
                   z_t *G, int64_t ldg) {
@@ -678,7 +677,7 @@ int gram_residues(bsechase_ctx *ctx, const z_t *A, int64_t lda, const z_t *B, in
     }
     ResBufs b;
     int rc;
-    if ((rc = residue_buffers(ctx, K, m1, m2, false, &b))) return rc;
+    if ((rc = residue_buffers(ctx, K, m1, m2, false, true, &b))) return rc;
     CK(cudaMemsetAsync(ctx->sc, 0, sizeof(ChaseScalars), ctx->st));
     const float2 *nb = same ? b.VA.part : b.VB.part;
     CK(residue_norms(K, m1, A, lda, b.VA.part, ctx->sc, ctx->st));
@@ -870,7 +869,7 @@ int solve_device(bsechase_ctx *ctx, const z_t *H, int64_t N, int64_t ldh, int ne
         tm.mark(3);
         ResBufs rb;
         if (op.res) {
-            if ((rc = residue_buffers(ctx, N, ma, locked, true, &rb))) return rc;
+            if ((rc = residue_buffers(ctx, N, ma, locked, true, false, &rb))) return rc;
             rc = phase_qr_residues(ctx, rb, V, N, locked, Va, N, N, ma);
         } else {
             rc = phase_qr(ctx, V, N, locked, Va, N, N, ma);
@@ -946,7 +945,7 @@ int solve_device(bsechase_ctx *ctx, const z_t *H, int64_t N, int64_t ldh, int ne
     if (op.res) {
         // a last pass restores FP64 orthonormality across the locked blocks
         ResBufs rb;
-        if ((rc = residue_buffers(ctx, N, nev, 0, true, &rb))) return rc;
+        if ((rc = residue_buffers(ctx, N, nev, 0, true, false, &rb))) return rc;
         if (ctx->inject_last_wait_ns) rb.wait_ns = ctx->inject_last_wait_ns;
         if ((rc = cholqr_residues(ctx, rb, d_evecs, ldz, N, nev, 0.0))) return rc;
     } else if (op.tc) {
@@ -1322,9 +1321,9 @@ int chase_qr(bsechase_ctx *ctx, const void *d_L, int64_t ldl, int k, void *d_V, 
     // residues' buffers are for tall blocks.
     bool res = sums_in_residues(N) && m <= N && k <= N;
     ResBufs b;
-    if (res && (rc = residue_buffers(ctx, N, m, k, true, &b))) {
-        if (rc != BSE_ENOMEM) return rc;
-        free_product_buffers(ctx);      // native FP64 needs no more workspace
+    if (res && (rc = residue_buffers(ctx, N, m, k, true, true, &b))) {
+        if (rc != BSE_ENOMEM && rc != kWantsNative) return rc;
+        if (rc == BSE_ENOMEM) free_product_buffers(ctx);      // native FP64 needs no more workspace
         res = false;
     }
     if (res) rc = phase_qr_residues(ctx, b, (const z_t *)d_L, ldl, k, (z_t *)d_V, ldv, N, m);
@@ -1378,7 +1377,8 @@ int chase_gram(bsechase_ctx *ctx, const void *d_A, int64_t lda, const void *d_B,
     int rc;
     if (sums_in_residues(K)) {
         rc = gram_residues(ctx, (const z_t *)d_A, lda, (const z_t *)d_B, ldb, K, m1, m2, (z_t *)d_G, ldg);
-        // Native FP64 without memory for the residues; for columns with entries so
+        // Native FP64 without memory for the residues, or where they would take more
+        // than a single call should; for columns with entries so
         // far below their norm that they count and residues would lose them; for
         // non-finite operands, whose product is what IEEE arithmetic makes of them.
         // Anything else is a failure of the call.

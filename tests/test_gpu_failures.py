@@ -123,3 +123,17 @@ def test_qr_of_more_columns_than_rows(ctx, N, m, k):
     assert torch.linalg.matrix_norm(L.conj().T @ V) <= bound
     P = V0 - L @ (L.conj().T @ V0)
     assert torch.linalg.matrix_norm(V @ (V.conj().T @ P) - P) <= 2.0 ** -40 * torch.linalg.matrix_norm(P)
+
+
+def test_gram_does_not_depend_on_earlier_calls(ctx):
+    """Above 8 GB of workspace chase_gram stays in native FP64, whatever buffers
+    other calls have left in the context: the same call gives the same bits."""
+    A, B = _block(870000, 4, 41), _block(870000, 4, 42)   # 3.3 + 5.3 GB of residues
+    torch.cuda.synchronize()
+    fresh = ctx.gram(A, B)
+    with pkg.Context(0) as other:
+        other.gram(_block(291000, 300, 43), _block(291000, 1, 44))     # 3.4 GB of left operands
+        X = _block(103000, 512, 45)
+        torch.cuda.synchronize()
+        other.gram(X, X.clone(memory_format=torch.preserve_format))    # 5.3 GB of right ones
+        assert torch.equal(other.gram(A, B), fresh)
