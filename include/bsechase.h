@@ -66,7 +66,11 @@ typedef enum {
                              to ||H|| ||Y||).  With half storage, and in
                              chase_rayleigh_ritz, the products are the BF16
                              Ozaki-scheme emulation of 6 slices of 8 bits per
-                             operand (~1e-12).  A full-storage solve's QR and
+                             operand (~1e-12), and so they are where the
+                             device (or a server's budget) has no room for the
+                             residues, 4 N^2 bytes more than the slices: tensor
+                             flops per product in chase_stats tell (84 to 112
+                             for residues, 168 for slices).  A full-storage solve's QR and
                              Rayleigh-Ritz products take residues of 58-bit
                              operands (15 moduli, FP64 rounding); reduced eig,
                              residuals and locking in native FP64.           */
@@ -169,7 +173,8 @@ typedef struct {
      * timed with CUDA events around each launch on the solver's stream:    */
     double tc_kernel_ms;        /* summed launch durations                    */
     int64_t tc_kernel_launches; /* launches timed                             */
-    double tc_kernel_tflops;    /* executed tensor flops / duration: per      */
+    double tc_kernel_tflops;    /* executed tensor flops / duration (of
+                                   N^2 matvecs multiply-adds in all): per     */
                                 /* complex multiply-add 6 or 8 for each of 14 */
                                 /* moduli (FP64), 8 per slice pair otherwise  */
     int nex_used;               /* nex at the end (differs from the argument
@@ -248,7 +253,8 @@ int chase_solve(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t ldh, int 
  * solve needs drops by 16 N^2 bytes, to 28 N^2 plus workspace (24 N^2 in the
  * mixed mode, 12 N^2 with chase_opts.half_storage) (Sec. 3's
  * filter works on H only through its products).  The slices, and so every
- * result, are bit for bit those of bse_build_hamiltonian + chase_solve.
+ * result, are bit for bit those of bse_build_hamiltonian + chase_solve (where
+ * both find the memory for the residues: see CHASE_FP64).
  * Tensor-core precisions only (CHASE_FP64, CHASE_MIXED_FP32, value 2);
  * CHASE_FP64_DFMA needs the stored H: BSE_EINVAL.  Other errors as
  * chase_solve. */
@@ -360,7 +366,9 @@ int chase_hemm_slices(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t ldh
  * stream, so admitted requests run concurrently; results (eigenvalues,
  * residuals, stats, latency stamps) stay with the server until released, and
  * eigenvectors stay on the device (LRU-evicted under the budget) so later
- * requests can warm-start from them. */
+ * requests can warm-start from them.  A result is bit for bit the direct
+ * solve's; a CHASE_FP64 request whose residues exceed the budget (28 N^2 bytes
+ * for 24) runs on the slices instead of being refused. */
 
 typedef struct {
     uint64_t seed;           /* synthetic Hamiltonian: bse_build_hamiltonian   */

@@ -227,6 +227,10 @@ size_t hop_f_bytes(int mc) { return ((size_t)(mc + 64) * sizeof(int) + 15) / 16 
 
 int hop_buffers(bsechase_ctx *ctx, const Hop &op, int mc) {
     int rc;
+    if (ctx->inject_refusals > 0) {
+        ctx->inject_refusals--;
+        return fail(ctx, BSE_ENOMEM, "refused%s");
+    }
     const int64_t Np = ozaki_padded(op.N);
     const HopBytes hb = hop_bytes(op.N, mc, op.res, op.tri, op.bse != nullptr, op.gen);
     if ((rc = ensure(ctx, ctx->ozA, hb.A))) return rc;
@@ -1082,6 +1086,7 @@ int bsechase_inject(bsechase_ctx *ctx, int point, int64_t value) {
     if (!ctx || value < 0) return BSE_EINVAL;
     switch (point) {
         case INJECT_LAST_PASS_WAIT_NS: ctx->inject_last_wait_ns = (uint64_t)value; return BSE_OK;
+        case INJECT_PRODUCT_REFUSALS: ctx->inject_refusals = value; return BSE_OK;
         default: return BSE_EINVAL;
     }
 }

@@ -38,7 +38,8 @@ struct bsechase_ctx {
     bool residues = true;            // solves may use the residue products (a server slot whose
                                      // request fits the budget on slices alone: not)
     int hop_cols = 0;                // columns the product buffers were sized for
-    uint64_t inject_last_wait_ns = 0;   // failure tests (bsechase_inject): wait limit of a solve's last pass
+    uint64_t inject_last_wait_ns = 0;   // failure tests (bsechase_inject): see InjectPoint
+    int64_t inject_refusals = 0;
     int64_t wsN = 0;
     int wsM = 0;
     cudaEvent_t ev[kCtxEvents];   // 0..6: solve phases; 8, 9: host copies
@@ -57,7 +58,8 @@ struct bsechase_ctx {
 // Failure tests of paths that no input reaches by itself; not part of the ABI.
 // 0 switches a point off.
 enum InjectPoint {
-    INJECT_LAST_PASS_WAIT_NS = 0   // wait limit, in ns, of the pass over a solve's output vectors
+    INJECT_LAST_PASS_WAIT_NS = 0,  // wait limit, in ns, of the pass over a solve's output vectors
+    INJECT_PRODUCT_REFUSALS = 1    // the next so many tries to allocate the products' buffers have no memory
 };
 extern "C" int bsechase_inject(bsechase_ctx *ctx, int point, int64_t value);
 

@@ -1,6 +1,6 @@
-"""Failures that a call has to report.  Every failure is made on the host: a
-short limit of the kernels' bounded waits, set by the caller or at one point of a
-call (bsechase_inject)."""
+"""Failures that a call has to report, and what it does where memory is short.  Every
+failure is made on the host: a short limit of the kernels' bounded waits, set by the
+caller or at one point of a call, an allocation that is refused (bsechase_inject)."""
 import ctypes
 
 import numpy as np
@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 import paper_2006_08498_gb300 as pkg  # noqa: E402
 
-LAST_PASS_WAIT_NS = 0
+LAST_PASS_WAIT_NS, PRODUCT_REFUSALS = 0, 1      # bsechase_inject
 
 
 @pytest.fixture
@@ -137,3 +137,67 @@ def test_gram_does_not_depend_on_earlier_calls(ctx):
         torch.cuda.synchronize()
         other.gram(X, X.clone(memory_format=torch.preserve_format))    # 5.3 GB of right ones
         assert torch.equal(other.gram(A, B), fresh)
+
+
+def test_products_without_memory_for_the_residues(ctx):
+    """One refused allocation: the buffers are given back and taken anew, the same
+    product.  Two: the product on slices, to its own bound (5e-11), and solves too; the
+    solve without the stored H takes the same bits."""
+    A, Y = _hermitian(1000, 51), _block(1000, 40, 52)
+    torch.cuda.synchronize()
+    C = ctx.hemm(A, Y)
+    _inject(ctx, PRODUCT_REFUSALS, 1)
+    assert torch.equal(ctx.hemm(A, Y), C)
+    _inject(ctx, PRODUCT_REFUSALS, 2)
+    D = ctx.hemm(A, Y)
+    assert not torch.equal(D, C)
+    norm = torch.linalg.matrix_norm(A, 2) * torch.linalg.vector_norm(Y, dim=0)
+    assert torch.all(torch.linalg.vector_norm(D - C, dim=0) <= 5e-11 * norm)
+    H = ctx.build_hamiltonian(3, 63, 4, 4)
+    e, _, _, st = ctx.solve(H, 20, 10, seed=3)
+    assert _flops(st, 1008) < 8 * 21
+    _inject(ctx, PRODUCT_REFUSALS, 2)
+    e2, V2, _, st = ctx.solve(H, 20, 10, seed=3)
+    assert abs(_flops(st, 1008) - 8 * 21) < 1e-6 * 8 * 21
+    assert np.max(np.abs(e2 - e) / np.abs(e)) <= 1e-10
+    _inject(ctx, PRODUCT_REFUSALS, 2)
+    e3, V3, _, _ = ctx.solve_bse(3, 63, 4, 4, 20, 10, seed_start=3)
+    assert np.array_equal(e2, e3) and torch.equal(V2, V3)
+
+
+def _flops(st, N):
+    """Tensor flops per complex multiply-add of a solve's products with H."""
+    return st["tc_kernel_tflops"] * st["tc_kernel_ms"] * 1e9 / (float(N) * N * st["matvecs"])
+
+
+def test_request_whose_residues_exceed_the_budget(ctx):
+    """The smallest budget that admits a request runs it on slices; one that holds
+    the residues runs it as the direct solve, bit for bit."""
+    R = dict(seed=3, Nk=63, Nv=4, Nc=4, nev=20, nex=10)
+    H = ctx.build_hamiltonian(3, 63, 4, 4)
+    e, _, _, _ = ctx.solve(H, 20, 10, seed=3)
+
+    def run(budget):
+        ctx.server_create(budget, 1)
+        try:
+            return ctx.wait(ctx.submit(**R))
+        except pkg.BseError as err:
+            assert err.status == pkg.BSE_ENOMEM
+            return None
+        finally:
+            ctx.server_destroy()
+
+    lo, hi = 1 << 20, 1 << 30                       # refused, admitted
+    assert run(lo) is None
+    full = run(hi)
+    assert np.array_equal(full["evals"], e) and _flops(full["stats"], 1008) < 8 * 21
+    while hi - lo > 1 << 16:
+        mid = (lo + hi) // 2
+        r = run(mid)
+        if r is None:
+            lo = mid
+        else:
+            hi, least = mid, r
+    assert least["status"] == pkg.BSE_OK
+    assert abs(_flops(least["stats"], 1008) - 8 * 21) < 1e-6 * 8 * 21
+    assert np.max(np.abs(least["evals"] - e) / np.abs(e)) <= 1e-10
