@@ -348,8 +348,9 @@ int chase_gram_noalloc(const void *d_A, int64_t lda, const void *d_B, int64_t ld
 int chase_hemm(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t ldh, const void *d_Y,
                int64_t ldy, int n, void *d_C, int64_t ldc, int precision);
 /* As chase_hemm on the tensor cores with the first `slices` 8-bit slices of
- * each operand (4, 5 or 6; slice pairs p + q <= slices + 1): 6 is CHASE_FP64's
- * product, 4 the FP32-level product of CHASE_MIXED_FP32, 5 the intermediate
+ * each operand (4 or 5, and 6 with half storage; slice pairs p + q <= slices + 1).
+ * 6 is CHASE_FP64's product of the same storage, bit for bit: of all of H in
+ * residues.  4 is the FP32-level product of CHASE_MIXED_FP32, 5 the intermediate
  * level that mode uses between them (about 40 bits per operand relative to
  * its row or column maximum).  half_storage = 1: the product on the slices
  * of H's lower triangle (chase_opts.half_storage; the strict upper triangle

@@ -443,7 +443,8 @@ class Context:
         """C = H Y (the filter's product) as a new column-major tensor; with
         `slices` (4, 5 or 6) or half_storage, the tensor-core product on that
         many slices (default 6) of all of H or of its lower triangle
-        (chase_hemm_slices) instead of `precision`'s."""
+        (chase_hemm_slices; 6 of all of H: CHASE_FP64's product) instead of
+        `precision`'s."""
         N, n = Y.shape
         C = colmajor_empty(N, n, device=Y.device) if out is None else out
         if slices is None and not half_storage:

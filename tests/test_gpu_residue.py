@@ -321,3 +321,18 @@ def test_largest_sums_of_54_bits(ctx, n):
     A = torch.full((N, N), 1 + 2.0 ** -41, dtype=torch.complex128, device="cuda").T * (1 + 1j)
     Y = torch.full((n, N), 1 + 2.0 ** -41, dtype=torch.complex128, device="cuda").T * (1 + 1j)
     _check(A, Y, _hemm(ctx, A, Y))
+
+
+# ---- the product on slices of all of H, which chase_hemm no longer reaches
+
+@pytest.mark.parametrize("N,m", [(63, 1), (129, 33), (333, 7), (640, 96), (1000, 97), (2050, 40)])
+def test_product_on_six_slices(ctx, N, m):
+    """Rayleigh-Ritz keeps the products on six slices: H V of its vectors V = Q Y against its
+    own H V = (H Q) Y.  An error of 2^-49.7 of ||h_i|| ||v_j|| (rms, entries of even size) in
+    each of three products; a slice less costs 8 bits: 2^-42."""
+    A = _hermitian(N, 61)
+    Q = torch.linalg.qr(_block(N, m, 62))[0].T.contiguous().T
+    torch.cuda.synchronize()
+    _, V, HV, _ = ctx.rayleigh_ritz(A, Q)
+    e = (HV - A @ V).abs() / torch.linalg.vector_norm(A, dim=1)[:, None]
+    assert e.square().mean().sqrt() <= 2.0 ** -46
