@@ -283,7 +283,7 @@ int hop_prepare(bsechase_ctx *ctx, Hop &op, int max_cols) {
         CK(residue_prepare_bse(op.bse->Nk, op.bse->Nv, op.bse->Nc, op.bse->md, op.bse->dE, op.bse->u, op.bse->a,
                                op.bse->Kt, &ctx->oh, ctx->ozP.p, ctx->ozB.p, ctx->sc, ctx->st));
     else if (op.res)
-        CK(residue_prepare(op.N, op.H, op.ldh, &ctx->oh, ctx->ozP.p, ctx->sc, ctx->st));
+        CK(residue_prepare(op.N, op.H, op.ldh, &ctx->oh, ctx->ozP.p, ctx->sc, ctx->sms, ctx->st));
     else if (op.bse)
         CK(ozaki_prepare_bse(op.bse->Nk, op.bse->Nv, op.bse->Nc, op.bse->md, op.bse->dE, op.bse->u,
                              op.bse->a, op.bse->Kt, op.tri, &ctx->oh, ctx->sc, ctx->st));

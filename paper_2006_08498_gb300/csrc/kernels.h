@@ -160,7 +160,7 @@ size_t residue_r_bytes(int64_t M, int64_t K, int n);
 size_t residue_work_bytes(int64_t N);
 size_t residue_panel_bytes(int64_t N);
 double residue_flops(int64_t M, int64_t K, int n);   // tensor flops of a product
-cudaError_t residue_prepare(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh, void *work, ChaseScalars *sc,
+cudaError_t residue_prepare(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh, void *work, ChaseScalars *sc, int sms,
                             cudaStream_t st);
 cudaError_t residue_prepare_bse(int Nk, int Nv, int Nc, const BseModel &md, const double *dE, const z_t *u,
                                 const z_t *a, const double *Kt, OzakiH *oh, void *work, void *panel,
@@ -187,8 +187,9 @@ struct RsSide {
     float2 *part = nullptr;
 };
 // S = op(A) B goes to C as D - S (D may be C) or as its conjugate transpose; with
-// mirror (S = A^H A) its upper triangle gives both halves and the diagonal is
-// real.  shift is added to the diagonal.
+// mirror, for an S that is Hermitian (A^H A) or would be without rounding (the
+// projected matrix Q^H (H Q)), its upper triangle gives both halves and the diagonal
+// is real.  shift is added to the diagonal.
 struct RsOut {
     z_t *C;
     int64_t ldc;

@@ -1600,7 +1600,7 @@ size_t residue_work_bytes(int64_t N) {
 
 size_t residue_panel_bytes(int64_t N) { return (size_t)N * 256 * sizeof(z_t); }
 
-cudaError_t residue_prepare(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh, void *work, ChaseScalars *sc,
+cudaError_t residue_prepare(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh, void *work, ChaseScalars *sc, int sms,
                             cudaStream_t st) {
     const int64_t Np = ozaki_padded(N), T = Np / kRows, nch = (N + kChunk - 1) / kChunk;
     oh->N = N;
@@ -1617,7 +1617,7 @@ cudaError_t residue_prepare(int64_t N, const z_t *H, int64_t ldh, OzakiH *oh, vo
         k_res_rowscale<<<(unsigned)T, 128, 0, st>>>(N, Np, nseg, (const float2 *)work, oh->E, sc);
         bse_count_launches(2);
     }
-    if (nch * 4 * T < 608)                         // too few blocks for four on every SM (N = 256: 9.2 us, 6.5 here)
+    if (nch * 4 * T < 4 * sms)                     // too few blocks for four on every SM (N = 256: 9.2 us, 6.5 here)
         launch_next(k_res_slice_a<4>, dim3((unsigned)(nch * 16), (unsigned)T), dim3(128), 0, st, N, N, H, ldh, (int64_t)0, T,
                     nch, oh->E, kNMod, kAlpha, (uint8_t *)oh->A);
     else
