@@ -93,10 +93,11 @@ bse_tile_kernel(int Nk, int nb, int N, BseModel md, const double *__restrict__ d
     for (int c = ty; c < kGT; c += 8) {
         if (diag && tx < c) continue;            // above the diagonal: the mirror pass
         const int J = j0 + c;
+        if (I >= N || J >= N) continue;          // no such element: its ring distance may be negative
         const z_t h = bse_element(I, J, R, sai + tx, saj + c, kGT, ui[tx], uj[c], dEi[tx], Nk, nb,
                                   md.w0, Kt);
         tile[c][tx] = h;
-        if (I < N && J < N) H[I + (int64_t)J * ldh] = h;
+        H[I + (int64_t)J * ldh] = h;
     }
     __syncthreads();
     for (int c = ty; c < kGT; c += 8) {

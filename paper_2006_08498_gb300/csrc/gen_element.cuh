@@ -10,7 +10,7 @@
 #include "common.cuh"
 #include "kernels.h"
 
-// H(I, J) for I >= J: dE_I [I = J] + 2 sum_r a_r(I) conj(a_r(J))
+// H(I, J) for N > I >= J: dE_I [I = J] + 2 sum_r a_r(I) conj(a_r(J))
 //                     - w0 Kt[d(k_I, k_J)] [b_I = b_J] u_I conj(u_J)
 // with k = I / nb, b = I % nb (nb = Nv Nc band pairs), d the ring distance.
 __device__ __forceinline__ z_t bse_element(int I, int J, int R, const z_t *ai, const z_t *aj,

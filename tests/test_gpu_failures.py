@@ -9,6 +9,7 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
+import oracle  # noqa: E402
 import paper_2006_08498_gb300 as pkg  # noqa: E402
 
 LAST_PASS_WAIT_NS, PRODUCT_REFUSALS = 0, 1      # bsechase_inject
@@ -201,3 +202,13 @@ def test_request_whose_residues_exceed_the_budget(ctx):
     assert least["status"] == pkg.BSE_OK
     assert abs(_flops(least["stats"], 1008) - 8 * 21) < 1e-6 * 8 * 21
     assert np.max(np.abs(least["evals"] - e) / np.abs(e)) <= 1e-10
+
+
+@pytest.mark.parametrize("model", [None, dict(rank_x=0), dict(rank_x=1)])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 1, 1), (1, 2, 3), (3, 1, 2), (31, 1, 1), (33, 1, 1)])
+def test_generator_of_the_smallest_matrices(ctx, shape, model):
+    """Matrices within one tile: the elements that the tile has beyond them have no ring distance (the
+    generator read the distance table at down to -31 for them, before the tables' memory for N < 7)."""
+    H = ctx.build_hamiltonian(5, *shape, model).cpu().numpy()
+    ref = oracle.build_h(5, *shape, model)
+    assert np.max(np.abs(H - ref)) <= 4e-15 * np.max(np.abs(ref))
