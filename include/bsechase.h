@@ -300,7 +300,10 @@ int chase_filter(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t ldh, voi
  * be NULL with k = 0): two projections, column scaling, shifted Cholesky QR
  * and two Cholesky QR passes each after a projection.  Its products run in
  * residues as chase_gram's do, for blocks of up to N columns, with an error
- * relative to the norms of rows and columns (which is what Cholesky QR needs). */
+ * relative to the norms of rows and columns (which is what Cholesky QR needs).
+ * Columns that depend on others get directions of their own (2^-40 of each
+ * column is added in a random direction where a factorisation fails); a zero
+ * column, or m > N, fails with BSE_ENONFINITE. */
 int chase_qr(bsechase_ctx *ctx, const void *d_L, int64_t ldl, int k, void *d_V, int64_t ldv,
              int64_t N, int m);
 

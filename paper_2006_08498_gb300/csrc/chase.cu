@@ -500,33 +500,15 @@ int project(bsechase_ctx *ctx, const z_t *L, int64_t ldl, int k, z_t *V, int64_t
 }
 
 // one Cholesky QR pass: G = V^H V + shift I = R^H R, V <- V R^{-1}
-int cholqr_pass(bsechase_ctx *ctx, z_t *V, int64_t ldv, int64_t N, int m, double shift) {
+int cholqr_pass(bsechase_ctx *ctx, z_t *V, int64_t ldv, int64_t N, int m, double shift, double weak = 0.0) {
     z_t *G = (z_t *)ctx->G.p, *Ri = (z_t *)ctx->Ri.p, *B1 = (z_t *)ctx->B1.p;
     int rc;
     if ((rc = gemm_cn(ctx, m, m, N, V, ldv, V, ldv, G, m, shift, 1))) return rc;
-    CK(launch_cholesky(m, G, m, ctx->sc, ctx->st));
+    CK(launch_cholesky(m, G, m, ctx->sc, ctx->st, weak));
     CK(launch_trinv(m, G, m, Ri, m, ctx->st));
     // R^{-1} is upper triangular
     if ((rc = gemm_nn(ctx, N, m, m, V, ldv, Ri, m, B1, N, nullptr, 0, true))) return rc;
     CK(launch_copy_cols(N, m, B1, N, V, ldv, nullptr, ctx->st));
-    return BSE_OK;
-}
-
-int phase_qr(bsechase_ctx *ctx, const z_t *L, int64_t ldl, int k, z_t *V, int64_t ldv, int64_t N,
-             int m) {
-    int rc;
-    if (m <= 0) return BSE_OK;
-    Small s = small_layout(ctx, m);
-    if ((rc = project(ctx, L, ldl, k, V, ldv, N, m))) return rc;
-    if ((rc = project(ctx, L, ldl, k, V, ldv, N, m))) return rc;
-    CK(launch_normalize_cols(N, m, V, ldv, (double *)ctx->part.p, s.norms, ctx->sc, ctx->st));
-    // columns have unit norm, so ||V||_F^2 = m
-    const double shift = 11.0 * ((double)N * m + (double)m * (m + 1)) * kU * (double)m;
-    if ((rc = cholqr_pass(ctx, V, ldv, N, m, shift))) return rc;
-    for (int pass = 0; pass < 2; pass++) {
-        if ((rc = project(ctx, L, ldl, k, V, ldv, N, m))) return rc;
-        if ((rc = cholqr_pass(ctx, V, ldv, N, m, 0.0))) return rc;
-    }
     return BSE_OK;
 }
 
@@ -578,7 +560,8 @@ int residue_buffers(bsechase_ctx *ctx, int64_t N, int m, int k, bool tall, bool 
 }
 
 // cholqr_pass in residues; the result goes to V itself
-int cholqr_residues(bsechase_ctx *ctx, const ResBufs &b, z_t *V, int64_t ldv, int64_t N, int m, double shift) {
+int cholqr_residues(bsechase_ctx *ctx, const ResBufs &b, z_t *V, int64_t ldv, int64_t N, int m, double shift,
+                    double weak = 0.0) {
     cudaStream_t st = ctx->st;
     ChaseScalars *sc = ctx->sc;
     z_t *G = (z_t *)ctx->G.p, *Ri = (z_t *)ctx->Ri.p;
@@ -588,7 +571,7 @@ int cholqr_residues(bsechase_ctx *ctx, const ResBufs &b, z_t *V, int64_t ldv, in
     CK(residue_left(m, N, V, ldv, true, b.VA, sc, st));
     CK(residue_right(N, m, V, ldv, b.VA.part, b.VB, sc, ctx->sms, st));
     CK(residue_mul(ctx, b, m, m, N, b.VA, b.VB, g));
-    CK(launch_cholesky(m, G, m, sc, st));
+    CK(launch_cholesky(m, G, m, sc, st, weak));
     CK(launch_trinv(m, G, m, Ri, m, st));
     CK(residue_left(N, m, V, ldv, false, b.VA, sc, st));
     CK(residue_right(m, m, Ri, m, nullptr, b.VB, sc, ctx->sms, st));
@@ -596,11 +579,21 @@ int cholqr_residues(bsechase_ctx *ctx, const ResBufs &b, z_t *V, int64_t ldv, in
     return BSE_OK;
 }
 
-// phase_qr in residues.  L is turned into residues once for the four
-// projections, in both its roles; a projection multiplies V^H L (the wide block
-// on the left, a byte a residue) and stores its adjoint.
-int phase_qr_residues(bsechase_ctx *ctx, const ResBufs &b, const z_t *L, int64_t ldl, int k, z_t *V, int64_t ldv,
-                      int64_t N, int m) {
+// The QR phase, its products in residues with b (native FP64, or on slices in a solve's
+// scope, without).  Residues: L is turned once for the four projections, in both its
+// roles; a projection multiplies V^H L (the wide block on the left, a byte a residue)
+// and stores its adjoint.  `keep` (N x m) holds a copy of V.  Synchronises.
+//
+// Columns that depend on others: the shifted pass leaves its products' rounding errors
+// of them, which the next passes turn into directions of their own.  Residues make
+// hardly any (equal columns stay exactly parallel), FP64 products some, so that a later
+// factorisation may fail.  The phase starts again from the copy then, with 2^-40 of each
+// normalised column (as much of a kept direction was lost to FP64's rounding before) added
+// in a random direction.  And where the last factorisation has a pivot far from 1, its
+// block was far from orthonormal: one pass more.  The copy and the wait take about 25 us at
+// N = 20000, 100 columns, of 2.8 ms.
+int phase_qr(bsechase_ctx *ctx, const ResBufs *b, const z_t *L, int64_t ldl, int k, z_t *V, int64_t ldv, int64_t N, int m,
+             z_t *keep) {
     if (m <= 0) return BSE_OK;
     cudaStream_t st = ctx->st;
     const int sms = ctx->sms;
@@ -608,31 +601,49 @@ int phase_qr_residues(bsechase_ctx *ctx, const ResBufs &b, const z_t *L, int64_t
     z_t *X = (z_t *)ctx->R.p;
     auto proj = [&]() -> int {
         if (k <= 0) return BSE_OK;
+        if (!b) return project(ctx, L, ldl, k, V, ldv, N, m);
         RsOut x{X, k}, v{V, ldv, V, ldv};
         x.adjoint = 1;
-        CK(residue_left(m, N, V, ldv, true, b.VA, sc, st));
-        CK(residue_mul(ctx, b, m, k, N, b.VA, b.LB, x));
-        CK(residue_right(k, m, X, k, nullptr, b.VB, sc, sms, st));
-        CK(residue_mul(ctx, b, N, m, k, b.LA, b.VB, v));
+        CK(residue_left(m, N, V, ldv, true, b->VA, sc, st));
+        CK(residue_mul(ctx, *b, m, k, N, b->VA, b->LB, x));
+        CK(residue_right(k, m, X, k, nullptr, b->VB, sc, sms, st));
+        CK(residue_mul(ctx, *b, N, m, k, b->LA, b->VB, v));
         return BSE_OK;
+    };
+    auto pass = [&](double shift, double weak) {
+        return b ? cholqr_residues(ctx, *b, V, ldv, N, m, shift, weak) : cholqr_pass(ctx, V, ldv, N, m, shift, weak);
     };
     int rc;
     Small s = small_layout(ctx, m);
-    if (k > 0) {
-        CK(residue_right(N, k, L, ldl, nullptr, b.LB, sc, sms, st));
-        CK(residue_left(N, k, L, ldl, false, b.LA, sc, st));
+    if (k > 0 && b) {
+        CK(residue_right(N, k, L, ldl, nullptr, b->LB, sc, sms, st));
+        CK(residue_left(N, k, L, ldl, false, b->LA, sc, st));
     }
-    if ((rc = proj())) return rc;
-    if ((rc = proj())) return rc;
-    CK(launch_normalize_cols(N, m, V, ldv, (double *)ctx->part.p, s.norms, sc, st));
+    CK(launch_copy_cols(N, m, V, ldv, keep, N, nullptr, st));
     // columns have unit norm, so ||V||_F^2 = m
     const double shift = 11.0 * ((double)N * m + (double)m * (m + 1)) * kU * (double)m;
-    if ((rc = cholqr_residues(ctx, b, V, ldv, N, m, shift))) return rc;
-    for (int pass = 0; pass < 2; pass++) {
+    for (int attempt = 0;; attempt++) {
         if ((rc = proj())) return rc;
-        if ((rc = cholqr_residues(ctx, b, V, ldv, N, m, 0.0))) return rc;
+        if ((rc = proj())) return rc;
+        CK(launch_normalize_cols(N, m, V, ldv, (double *)ctx->part.p, s.norms, sc, st));
+        if (attempt > 0) CK(launch_nudge(N, m, V, ldv, s.norms, 0x1.0p-40 / sqrt((double)N), st));
+        if ((rc = pass(shift, 0.0))) return rc;
+        if ((rc = proj())) return rc;
+        if ((rc = pass(0.0, 0.0))) return rc;
+        if ((rc = proj())) return rc;
+        if ((rc = pass(0.0, 0.5))) return rc;
+        rc = sync_scalars(ctx);
+        if (rc == BSE_OK) break;
+        if (attempt > 0 || ctx->hsc->error != DEV_CHOL_FAIL) return rc;
+        ctx->err.clear();
+        CK(cudaMemsetAsync(&sc->error, 0, sizeof sc->error, st));
+        CK(launch_copy_cols(N, m, keep, N, V, ldv, nullptr, st));
     }
-    return BSE_OK;
+    if (!ctx->hsc->weak) return BSE_OK;
+    CK(cudaMemsetAsync(&sc->weak, 0, sizeof sc->weak, st));
+    if ((rc = proj())) return rc;
+    if ((rc = pass(0.0, 0.0))) return rc;
+    return sync_scalars(ctx);
 }
 
 // phase_rr in residues
@@ -872,13 +883,9 @@ int solve_device(bsechase_ctx *ctx, const z_t *H, int64_t N, int64_t ldh, int ne
         if (fop.level == OZ_S5) filter_mv_mid += mv;
         tm.mark(3);
         ResBufs rb;
-        if (op.res) {
-            if ((rc = residue_buffers(ctx, N, ma, locked, true, false, &rb))) return rc;
-            rc = phase_qr_residues(ctx, rb, V, N, locked, Va, N, N, ma);
-        } else {
-            rc = phase_qr(ctx, V, N, locked, Va, N, N, ma);
-        }
-        if (rc) return rc;
+        if (op.res && (rc = residue_buffers(ctx, N, ma, locked, true, false, &rb))) return rc;
+        // B3 is free until Rayleigh-Ritz
+        if ((rc = phase_qr(ctx, op.res ? &rb : nullptr, V, N, locked, Va, N, N, ma, B3))) return rc;
         tm.mark(4);
         if (op.res) rc = phase_rr_residues(ctx, op, rb, Va, N, ma, s.theta, B2, B3);
         else rc = phase_rr(ctx, op, Va, N, ma, s.theta, B2, B3);
@@ -1331,10 +1338,7 @@ int chase_qr(bsechase_ctx *ctx, const void *d_L, int64_t ldl, int k, void *d_V, 
         if (rc == BSE_ENOMEM) free_product_buffers(ctx);      // native FP64 needs no more workspace
         res = false;
     }
-    if (res) rc = phase_qr_residues(ctx, b, (const z_t *)d_L, ldl, k, (z_t *)d_V, ldv, N, m);
-    else rc = phase_qr(ctx, (const z_t *)d_L, ldl, k, (z_t *)d_V, ldv, N, m);
-    if (rc) return rc;
-    return sync_scalars(ctx);
+    return phase_qr(ctx, res ? &b : nullptr, (const z_t *)d_L, ldl, k, (z_t *)d_V, ldv, N, m, (z_t *)ctx->B3.p);
 }
 
 int chase_rayleigh_ritz(bsechase_ctx *ctx, const void *d_H, int64_t N, int64_t ldh,

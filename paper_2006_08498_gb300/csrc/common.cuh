@@ -99,7 +99,7 @@ struct ChaseScalars {
     int locked;        // number of locked pairs
     int new_locked;    // pairs locked by the last Rayleigh-Ritz step
     int m_act;         // active (unlocked) columns
-    int pad0;
+    int weak;          // the last factorisation with a `weak` bound had a pivot below it
     double alpha;      // lower end of the damped interval
     double beta;       // upper bound of the spectrum (Lanczos)
     double lower;      // normalisation point of the filter (min Ritz value)

@@ -256,13 +256,16 @@ cudaError_t launch_lanczos_step(int64_t N, int nl, z_t *V, z_t *Vprev, z_t *W, i
 cudaError_t launch_phase_normalize(int64_t N, int nc, z_t *X, int64_t ldx, cudaStream_t st);
 cudaError_t launch_normalize_cols(int64_t N, int nc, z_t *X, int64_t ldx, double *work,
                                   double *norms, ChaseScalars *sc, cudaStream_t st);
+// X(i, j) += size (u + i v), u and v uniform in [-1, 1] by (i, j), where norms[j] > 0
+cudaError_t launch_nudge(int64_t N, int nc, z_t *X, int64_t ldx, const double *norms, double size, cudaStream_t st);
 // out[:, j] = sel[j] ? B[:, j] : A[:, j]   (gather of filter results)
 cudaError_t launch_select_cols(int64_t N, int nc, const z_t *A, const z_t *B, int64_t ld,
                                const int *deg, int parity, z_t *out, cudaStream_t st);
 
 // ---- single-CTA small dense kernels (small.cu)
-// In-place Cholesky G = R^H R (upper R, n x n); failure recorded in sc.
-cudaError_t launch_cholesky(int n, z_t *G, int64_t ld, ChaseScalars *sc, cudaStream_t st);
+// In-place Cholesky G = R^H R (upper R, n x n); failure recorded in sc, and sc->weak
+// set if a pivot (the square of R's diagonal) is below `weak`.
+cudaError_t launch_cholesky(int n, z_t *G, int64_t ld, ChaseScalars *sc, cudaStream_t st, double weak = 0.0);
 // X = R^{-1} for upper-triangular R (n x n)
 cudaError_t launch_trinv(int n, const z_t *R, int64_t ldr, z_t *X, int64_t ldx, cudaStream_t st);
 // Eigen-decomposition of Hermitian A (n x n, may be overwritten): ascending w, vectors Y.

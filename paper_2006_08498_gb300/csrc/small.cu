@@ -43,7 +43,7 @@ __device__ double block_sum(double v, double *red) {
 }
 
 // ------------------------------------------------------------ Cholesky
-__global__ void __launch_bounds__(kST) k_cholesky(int n, z_t *G, int64_t ld, ChaseScalars *sc) {
+__global__ void __launch_bounds__(kST) k_cholesky(int n, z_t *G, int64_t ld, double weak, ChaseScalars *sc) {
     __shared__ int failed;
     __shared__ double rjj_s;
     const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
@@ -61,6 +61,7 @@ __global__ void __launch_bounds__(kST) k_cholesky(int n, z_t *G, int64_t ld, Cha
                     set_error(sc, DEV_CHOL_FAIL, j);
                 } else {
                     rjj_s = sqrt(d);
+                    if (d < weak) sc->weak = 1;
                     G[j + (int64_t)j * ld] = zmk(rjj_s, 0.0);
                 }
             }
@@ -94,7 +95,7 @@ constexpr int kCholSmemN = 160;
 __device__ __forceinline__ int upk(int i, int j) { return j * (j + 1) / 2 + i; }
 
 __global__ void __launch_bounds__(kST)
-k_cholesky_smem(int n, z_t *G, int64_t ld, ChaseScalars *sc) {
+k_cholesky_smem(int n, z_t *G, int64_t ld, double weak, ChaseScalars *sc) {
     extern __shared__ z_t U[];
     __shared__ int failed;
     __shared__ double rjj_s;
@@ -118,6 +119,7 @@ k_cholesky_smem(int n, z_t *G, int64_t ld, ChaseScalars *sc) {
                     set_error(sc, DEV_CHOL_FAIL, j);
                 } else {
                     rjj_s = sqrt(d);
+                    if (d < weak) sc->weak = 1;
                     U[upk(j, j)] = zmk(rjj_s, 0.0);
                 }
             }
@@ -611,7 +613,7 @@ __host__ __device__ constexpr int ch_base(int c, int l) { return C * l * (l - 1)
 
 template <int C>
 __global__ void __launch_bounds__(kHhT)
-k_cholesky_cl(int n, z_t *G, int64_t ld, ChaseScalars *sc) {
+k_cholesky_cl(int n, z_t *G, int64_t ld, double weak, ChaseScalars *sc) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     extern __shared__ z_t Uc[];                 // own columns, rows 0..j
@@ -640,6 +642,7 @@ k_cholesky_cl(int n, z_t *G, int64_t ld, ChaseScalars *sc) {
         const int l0 = (j + 1 > c) ? (j + 1 - c + C - 1) / C : 0;   // own columns > j
         if (warp == 0) {
             const double inv = rsqrt(d);
+            if (c == 0 && lane == 0 && d < weak) sc->weak = 1;
             if (j % C == c && lane == 0) Uc[ch_base<C>(c, j / C) + j] = zmk(d * inv, 0.0);
             for (int l = l0 + lane; l < ncol; l += 32) {
                 z_t *col = Uc + ch_base<C>(c, l);
@@ -688,7 +691,7 @@ size_t ch_dyn_bytes(int n) {
 // Launches the clustered Cholesky with C CTAs if the cluster fits;
 // cudaErrorNotSupported otherwise.
 template <int C>
-cudaError_t ch_launch(int n, z_t *G, int64_t ld, ChaseScalars *sc, cudaStream_t st) {
+cudaError_t ch_launch(int n, z_t *G, int64_t ld, double weak, ChaseScalars *sc, cudaStream_t st) {
     constexpr size_t kStatic = (size_t)(3 * kMaxN) * sizeof(z_t) + kMaxN * sizeof(double) + 64;
     static std::once_flag once[kMaxDevices];
     static size_t limits[kMaxDevices];
@@ -701,7 +704,7 @@ cudaError_t ch_launch(int n, z_t *G, int64_t ld, ChaseScalars *sc, cudaStream_t 
     });
     const size_t bytes = ch_dyn_bytes<C>(n);
     if (limit == 0 || bytes > limit) return cudaErrorNotSupported;
-    return cluster_launch<C>(k_cholesky_cl<C>, bytes, st, n, G, ld, sc);
+    return cluster_launch<C>(k_cholesky_cl<C>, bytes, st, n, G, ld, weak, sc);
 }
 
 // Deflation test shared by every path: e_k is negligible next to its
@@ -1232,11 +1235,11 @@ __global__ void k_chase_update(int m_act, int nev, double tol, int deg_max,
 
 }  // namespace
 
-cudaError_t launch_cholesky(int n, z_t *G, int64_t ld, ChaseScalars *sc, cudaStream_t st) {
+cudaError_t launch_cholesky(int n, z_t *G, int64_t ld, ChaseScalars *sc, cudaStream_t st, double weak) {
     if (n <= 0) return cudaSuccess;
     if (n <= kMaxN) {
-        cudaError_t ce = ch_launch<16>(n, G, ld, sc, st);
-        if (ce == cudaErrorNotSupported) ce = ch_launch<8>(n, G, ld, sc, st);
+        cudaError_t ce = ch_launch<16>(n, G, ld, weak, sc, st);
+        if (ce == cudaErrorNotSupported) ce = ch_launch<8>(n, G, ld, weak, sc, st);
         if (ce != cudaErrorNotSupported) {
             bse_count_launches(1);
             return ce;
@@ -1248,9 +1251,9 @@ cudaError_t launch_cholesky(int n, z_t *G, int64_t ld, ChaseScalars *sc, cudaStr
         static cudaError_t attr[kMaxDevices];
         const cudaError_t ae = smem_attr_once(once, attr, (const void *)k_cholesky_smem, bytes);
         if (ae != cudaSuccess) return ae;
-        k_cholesky_smem<<<1, kST, (size_t)(n * (n + 1) / 2) * sizeof(z_t), st>>>(n, G, ld, sc);
+        k_cholesky_smem<<<1, kST, (size_t)(n * (n + 1) / 2) * sizeof(z_t), st>>>(n, G, ld, weak, sc);
     } else {
-        k_cholesky<<<1, kST, 0, st>>>(n, G, ld, sc);
+        k_cholesky<<<1, kST, 0, st>>>(n, G, ld, weak, sc);
     }
     bse_count_launches(1);
     return cudaGetLastError();

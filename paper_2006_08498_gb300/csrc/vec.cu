@@ -107,6 +107,15 @@ __global__ void k_random_block(uint64_t seed, uint64_t stream, int64_t n, int co
     V[i + (int64_t)j * ldv] = zmk(re, im);
 }
 
+__global__ void k_nudge(int64_t n, z_t *X, int64_t ldx, const double *__restrict__ norms, double size) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.y;
+    if (i >= n || !(norms[j] > 0.0)) return;
+    const uint64_t idx = 2 * (uint64_t)((int64_t)j * n + i);
+    z_t &x = X[i + (int64_t)j * ldx];
+    x = zadd(x, zmk(size * (2.0 * unif(0, 6, idx) - 1.0), size * (2.0 * unif(0, 6, idx + 1) - 1.0)));
+}
+
 // Lanczos, per column l: dot partials of Re(v^H w)
 __global__ void __launch_bounds__(kVT)
 k_lz_dot(int64_t N, int nl, const z_t *__restrict__ V, const z_t *__restrict__ W, int64_t ld,
@@ -265,6 +274,13 @@ cudaError_t launch_random_block(uint64_t seed, uint64_t stream, int64_t n, int m
     if (m <= 0 || n <= 0) return cudaSuccess;
     dim3 grid((unsigned)((n + 255) / 256), (unsigned)m);
     k_random_block<<<grid, 256, 0, st>>>(seed, stream, n, col0, V, ldv);
+    bse_count_launches(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_nudge(int64_t N, int nc, z_t *X, int64_t ldx, const double *norms, double size, cudaStream_t st) {
+    if (nc <= 0 || N <= 0) return cudaSuccess;
+    k_nudge<<<dim3((unsigned)((N + 255) / 256), (unsigned)nc), 256, 0, st>>>(N, X, ldx, norms, size);
     bse_count_launches(1);
     return cudaGetLastError();
 }

@@ -2,6 +2,7 @@
 failure is made on the host: a short limit of the kernels' bounded waits, set by the
 caller or at one point of a call, an allocation that is refused (bsechase_inject)."""
 import ctypes
+import math
 
 import numpy as np
 import pytest
@@ -212,3 +213,48 @@ def test_generator_of_the_smallest_matrices(ctx, shape, model):
     H = ctx.build_hamiltonian(5, *shape, model).cpu().numpy()
     ref = oracle.build_h(5, *shape, model)
     assert np.max(np.abs(H - ref)) <= 4e-15 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("N,m,k", [(400, 20, 0), (400, 20, 9), (2000, 75, 30), (129, 60, 0), (63, 12, 4)])
+@pytest.mark.parametrize("kind", ["equal", "half equal", "rank 5", "nearly equal", "kept"])
+def test_qr_of_dependent_columns(ctx, N, m, k, kind):
+    """Columns that depend on others (or on kept ones) get directions of their own: the basis is
+    orthonormal to rounding, 2^-50 a column, and holds the columns to what is added to
+    them, 2^-40 of each (2^-38 with the passes).  Native FP64 (N < 64) may keep a
+    direction of less than its rounding over the square root of the first pass' shift
+    without failing, and holds the columns to that."""
+    V0 = _block(N, m, 71)
+    L = torch.linalg.qr(_block(N, k, 72))[0].T.contiguous().T if k else None
+    if kind == "equal":
+        V0[:, 4] = V0[:, 5]
+    elif kind == "half equal":
+        V0[:, m // 2:] = V0[:, :m - m // 2].clone()
+    elif kind == "rank 5":
+        V0 = (_block(N, 5, 73) @ _block(5, m, 74)).T.contiguous().T
+    elif kind == "nearly equal":
+        V0[:, 4] = V0[:, 5] + 1e-10 * V0[:, 6]
+    elif k:
+        V0[:, 2] = L[:, 1]
+    V = V0.clone(memory_format=torch.preserve_format)
+    torch.cuda.synchronize()
+    ctx.qr(V, L)
+    assert torch.linalg.matrix_norm(V.conj().T @ V - torch.eye(m, device="cuda")) <= m * 2.0 ** -50
+    P = V0
+    if k:
+        assert torch.linalg.matrix_norm(L.conj().T @ V) <= m * 2.0 ** -50
+        P = V0 - L @ (L.conj().T @ V0)
+    span = 2.0 ** -38 if N >= 64 else 2.0 ** -53 / math.sqrt(11 * (N * m + m * (m + 1)) * 2.0 ** -53 * m)
+    assert torch.linalg.matrix_norm(V @ (V.conj().T @ P) - P) <= span * torch.linalg.matrix_norm(P)
+
+
+@pytest.mark.parametrize("kw", [{}, dict(precision=pkg.CHASE_MIXED_FP32), dict(half_storage=True),
+                                dict(precision=pkg.CHASE_FP64_DFMA)])
+def test_solve_from_a_dependent_start_block(ctx, kw):
+    H = ctx.build_hamiltonian(0, 63, 4, 4)
+    e, _, _, _ = ctx.solve(H, 20, 10)
+    X = _block(1008, 30, 75)
+    X[:, 10:20] = X[:, :10].clone()
+    torch.cuda.synchronize()
+    e2, V, _, _ = ctx.solve(H, 20, 10, V0=X, **kw)
+    assert np.max(np.abs(e2 - e) / np.abs(e)) <= 1e-10
+    assert torch.linalg.matrix_norm(V.conj().T @ V - torch.eye(20, device="cuda")) <= 20 * 2.0 ** -50
