@@ -41,6 +41,7 @@
 #include "gen_element.cuh"
 #include "kernels.h"
 #include "residue.h"
+#include "rotation.h"
 #include "tc_common.cuh"
 
 namespace {
@@ -229,23 +230,6 @@ static_assert(kRange == 8, "drain pattern");
 __device__ __forceinline__ bool range_end(int t, int c) {
     return t == 0 ? (c & 15) == 15 : t == 1 ? (c & 15) == 10 : (c & 7) == 5;
 }
-// Four products: the accumulator drained after chunk c, other than at the unit's
-// end: Re (0), Im (1) or none (-1).
-__device__ __forceinline__ int drained_after(int c, int nc) {
-    return (c & 3) == 3 && c + 1 < nc ? (c & 4 ? 0 : 1) : -1;
-}
-// Which buffer holds which accumulator: one that ends moves to the free buffer, and
-// its old one is free once it is drained.  Every role follows the same sequence.
-struct AccState {
-    uint32_t b[2] = {0, 1}, free = 2, drains = 0;  // drains: parity of each buffer's
-    __device__ __forceinline__ void end(int t) {
-        const uint32_t old = t == 0 ? b[0] : b[1];
-        if (t == 0) b[0] = free;
-        else b[1] = free;
-        free = old;
-        drains ^= 1u << old;
-    }
-};
 constexpr uint64_t kWindDownNs = 2000000000ull;
 
 // Work per CTA: one modulus, 128 rows, w <= 144 columns, the K chunks of one
@@ -276,7 +260,7 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
     uint8_t *sm = (uint8_t *)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
     uint8_t *sB = sm, *sA = sm + kSB * kBStage;
     __shared__ uint64_t fullA[kSA], emptyA[kSA], fullB[3 * kSB], emptyB[3 * kSB];   // B, Gauss: per product
-    __shared__ uint64_t accFull[3], accEmpty[3], mmaDone;
+    __shared__ uint64_t accFull[3], accEmpty[AccState::kEnds], mmaDone;   // empty, Gauss: per product; else per end
     __shared__ __align__(2 * kBars * 8) uint64_t aBars[2 * kBars];   // stages of A: full, then empty
     uint64_t *aFull = aBars, *aEmpty = aBars + kBars;
     __shared__ uint32_t tmem_base;
@@ -299,10 +283,8 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
             tc::mbar_init(&aFull[s], kH == 1 ? 8 : 4);
             tc::mbar_init(&aEmpty[s], kGauss ? 1 : 2);
         }
-        for (int t = 0; t < 3; t++) {
-            tc::mbar_init(&accFull[t], 1);
-            tc::mbar_init(&accEmpty[t], kDrainWarps);
-        }
+        for (int t = 0; t < 3; t++) tc::mbar_init(&accFull[t], 1);
+        for (uint32_t t = 0; t < AccState::kEnds; t++) tc::mbar_init(&accEmpty[t], kDrainWarps);
         tc::mbar_init(&mmaDone, kP);
         abort_flag = 0;
         tc::mbar_fence_init();
@@ -518,7 +500,7 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                 const uint32_t acc = tmem + buf * stride;
                 if (!rdyB && !wait_all(fB + sB8, sph)) { ok = false; break; }
                 // a fresh barrier passes the wait for the phase before its first
-                if (fresh && !wait_all(accE + 8 * buf, (st.drains >> buf & 1) ^ 1)) { ok = false; break; }
+                if (fresh && !wait_all(accE + 8 * st.wait_on(buf), st.wait_parity(buf))) { ok = false; break; }
                 const uint64_t bo = (uint64_t)(sB8 * (kBStage / 8 >> 4));
                 const uint32_t eb = eB + sB8;
                 bool lookB = false;
@@ -684,7 +666,7 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
             const uint64_t magic2 = tc::pin2(tc::f32x2(kMagic, kMagic)), mmagic2 = tc::pin2(tc::f32x2(-kMagic, -kMagic));
             for (int ev = 0, fin = 0; fin < kP;) {
                 int t;
-                uint32_t buf, phase;
+                uint32_t buf, phase, done;
                 float coef;                        // Re + kPack Im
                 if constexpr (kGauss) {
                     // T2, T1, T2, T0 after chunks 5, 10, 13, 15 of every 16, until the
@@ -695,7 +677,7 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                     } else {
                         t = fin++;
                     }
-                    buf = (uint32_t)t;
+                    buf = done = (uint32_t)t;
                     phase = gph >> t & 1;
                     gph ^= 1u << t;
                     // T0 counts (1, -1), T1 (-1, -1), T2 (0, 1)
@@ -708,6 +690,7 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                     else t = fin++;
                     buf = t == 0 ? st.b[0] : st.b[1];
                     phase = st.drains >> buf & 1;
+                    done = st.signal();
                     st.end(t);
                     coef = t == 0 ? 1.f : (float)kPack;
                 }
@@ -742,7 +725,7 @@ __global__ void __launch_bounds__(Cfg::kThreads, 1) k_res_zgemm(const __grid_con
                 tc::tmem_wait_ld();
                 tc::fence_before();
                 __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&accEmpty[buf]);
+                if (lane == 0) tc::mbar_arrive(&accEmpty[done]);
 #pragma unroll
                 for (int g = 0; g < kG; g++) {
                     const int at = g >= kHold ? g - kHold : g;

@@ -247,3 +247,35 @@ def test_request_with_caller_hamiltonian(ctx):
     w, _ = oracle.eigh(A, 0)
     assert np.max(np.abs(r["evals"] - w[:30]) / np.abs(w[:30])) <= 1e-10
     assert np.max(np.abs(r["evals"] - lam[:30]) / lam[:30]) <= 1e-10
+
+
+def test_products_are_the_same_under_contention(ctx):
+    """Products of three contexts at once, in units of 12 to 44 chunks: each keeps the bits that it
+    has alone (a wait answered too early by the rotating accumulators shows under such load)."""
+    import threading
+    jobs = []
+    for i, (N, n) in enumerate([(2736, 4), (2784, 48), (2784, 100)]):
+        g = torch.Generator(device="cuda").manual_seed(i)
+        A = torch.randn((N, N), dtype=torch.complex128, device="cuda", generator=g)
+        Y = torch.randn((n, N), dtype=torch.complex128, device="cuda", generator=g).T
+        jobs.append(((A + A.conj().T).T.contiguous().T, Y))
+    torch.cuda.synchronize()
+    alone = [ctx.hemm(A, Y) for A, Y in jobs]
+    wrong = []
+
+    def work(i):
+        stream = torch.cuda.Stream()
+        with pkg.Context(0, stream=stream) as c:
+            out = pkg.colmajor_empty(*jobs[i][1].shape)
+            for _ in range(150):
+                c.hemm(*jobs[i], out=out)
+                stream.synchronize()
+                if not torch.equal(out, alone[i]):
+                    wrong.append(i)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(3)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
