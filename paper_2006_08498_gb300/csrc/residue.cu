@@ -211,6 +211,11 @@ struct RsCfg {
     static_assert(128 * (R0 + CONV * RC + 2 * RD) <= kThreads * RL && 65536 / kThreads >= RL, "register split");
     static_assert(kSmem <= 230500 && 2 * HOLD >= W / 16, "resources");
     static constexpr int kMinSlots = (kTmemCols - 3 * W) / kCols;
+    // H = 1: with an odd number of groups a stage of A's bytes goes to different ones in
+    // turn.  A group at chunk m has seen those up to m - 2 - slots used, which covers the
+    // stage's last contents (chunk m - SA), so no older phase answers its wait; such
+    // variants have tiles above 48 columns.
+    static_assert(H != 1 || CONV % 2 == 0 || SA >= 2 + (kTmemCols - 3 * 64) / 64, "phases of A's stages");
     // a converter group's step along the rings: one turn at most
     static_assert(CONV >= 2 && (H == 1 ? (CONV + 1) / 2 : kGauss ? 3 * (CONV - 1) : CONV) <= kMinSlots && (CONV + 1) / 2 <= SA, "rings");
 };
