@@ -670,12 +670,13 @@ int phase_rr_residues(bsechase_ctx *ctx, const Hop &op, const ResBufs &b, const 
     return BSE_OK;
 }
 
-// Sums over K = N of a chunk or more go in residues, whatever the widths.  us,
-// native FP64 against residues: Gram K = 7 (3 x 2) 70, 73; K = 64 (1 x 1) 104,
-// 74; K = 2000 (40 x 20) 309, 87; K = 20000 (140 x 40) 1816, 214; QR N = 7 (3
-// after 2) 467, 503; N = 64 (1) 340, 285; N = 2000 (40 after 20) 3247, 1049;
-// N = 20000 (100 after 40) 21832, 3714.  Below one chunk every split of the FP64
-// kernel is short, and the residues' padding and launches cost more.
+// Sums over K = N of a chunk or more go in residues, whatever the widths.  us a call,
+// native FP64 against residues (Gram with the check of its weights): Gram K = 64
+// (1 x 1) 90, 55, (40 x 40) 92, 68; K = 2000 (40 x 20) 294, 77; K = 20000 (140 x 40) 1798,
+// 201; K = 50000 (512 x 512) 100800, 3330; QR N = 64 (1) 345, 208; N = 2000 (40 after
+// 20) 3257, 734; N = 20000 (100 after 40) 21850, 2820.  Below one chunk (K = 7: Gram 57, QR
+// 480) every split of the FP64 kernel is short, and the residues' padding and launches
+// cost more (73 and 503 when they were tried there).
 bool sums_in_residues(int64_t K) { return K >= 64; }
 
 // G = A^H B in residues, the wider block on the left; synchronises.

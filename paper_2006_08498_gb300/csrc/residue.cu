@@ -49,8 +49,9 @@ namespace {
 // The kernels of a product follow one another without the gap of a launch: each
 // may be set up while the one before it drains (programmatic dependent launch),
 // waits for that one's end before it touches memory, and lets the next one be set up.
-// (No timing events between them either, outside solves.)  N = 256, 30 columns: 55 -> 47 us
-// a product with its preparation; filter N = 2000, 75 columns: 2.05 -> 1.78 ms.
+// (No timing events between them either, outside solves.)  With 13 moduli: N = 256, 30
+// columns 55 -> 47 us a product with its preparation; filter N = 2000, 75 columns
+// 2.05 -> 1.78 ms.
 __device__ __forceinline__ void follow() {
     cudaGridDependencySynchronize();
     cudaTriggerProgrammaticLaunchCompletion();
@@ -887,7 +888,7 @@ k_res_rowscale(int64_t M, int64_t Mp, int nseg, const float2 *__restrict__ part,
 // order as the two kernels above.  For short segments only (N < 4096): 17 us
 // against 16 + 14 at N = 2000, but with one block for 8 whole rows 1056 us
 // against 940 + 17 at N = 20000.  Segments of 8 columns up to N = 1024 fill the
-// threads there: a product with its preparation at N = 256 47 -> 40 us.
+// threads there: a product with its preparation at N = 256 47 -> 40 us (13 moduli; 42 with 14).
 // With 32 rows and 8 segments at a time: the rows of a tall A of at most
 // kMaxTallCols columns (the general products).
 constexpr int kSmallSegs = 128, kMaxTallCols = 512, kTallSegs = kMaxTallCols / 32;
@@ -1208,11 +1209,11 @@ k_res_panel(int Nk, int nb, int N, int jbase, int cols, BseModel md, const doubl
 // Element (i, j) from the residues of all moduli and splits, ROWS consecutive
 // rows per thread (4, or 1 to fill the SMs from a small result).  The splits' bytes (residue + 128) are summed two to a
 // word first, then F = sum_m W_m u_m - nz bias, a multiply-add per word of W:
-// 10 us at N = 2000, 75 columns (15 with four rows per thread, and 20 with a
-// 64-bit product per split and value before; 23 with the moduli shared out over
-// four warps), 7 us at N = 256 (14).  At N = 20000, 140 columns four rows take 65
-// us (82 with the loads of two moduli in flight, and the conversion and the
-// scaling on the FP64 pipe).
+// 14 us at N = 2000, 75 columns, and with four rows a thread 88 us at N = 20000, 140 columns
+// (from HBM).  With 13 moduli and 64-bit fractions: 10 us at N = 2000 (15 with four rows per
+// thread, and 20 with a 64-bit product per split and value before; 23 with the moduli
+// shared out over four warps), 7 us at N = 256 (14); 65 at N = 20000 (82 with the loads
+// of two moduli in flight, and the conversion and the scaling on the FP64 pipe).
 // m 2^e, m >= 2^62, rounded once
 __device__ __forceinline__ double to_double(unsigned long long m, int e, bool neg) {
     if (!(m >> 63)) {
@@ -1760,8 +1761,8 @@ cudaError_t residue_zgemm(const OzakiH &oh, int n, const z_t *Y, int64_t ldy, z_
 // ------------------------------------------------------------ general products
 // A^H B and A B of the QR and Gram entries, for tall A and B.  In native FP64
 // (1.2 TFLOP/s on this part) they were bound by its issue: Gram K = 20000,
-// 140 x 40: 1805 us, here 187 (55 left residues, 24 right, 23 norms, 47 product,
-// 17 result); QR N = 20000, 100 columns after 40: 21.8 ms, here 3.5.
+// 140 x 40: 1805 us, here 197 (55 left residues, 23 right, 21 norms, 31 their weights'
+// check, 39 product, 8 result); QR N = 20000, 100 columns after 40: 21.8 ms, here 2.8.
 size_t residue_left_bytes(int64_t M, int64_t K) { return a_bytes_of(M, K, kGMod); }
 size_t residue_right_bytes(int64_t K, int n) { return b_bytes_of(K, n, kGMod); }
 size_t residue_out_bytes(int64_t M, int64_t K, int n) {
