@@ -14,14 +14,14 @@ struct Use {
 };
 
 int main(int argc, char **argv) {
-    const int rounds = argc > 1 ? atoi(argv[1]) : 1000;
+    const int trials = argc > 1 ? atoi(argv[1]) : 1000;
     std::mt19937 rng(1);
-    for (int round = 0; round < rounds; round++) {
-        const int top = (const int[]){2, 6, 20, 48}[round % 4], ring = (const int[]){4, 6, 7, 16}[rng() % 4];
+    for (int trial = 0; trial < trials; trial++) {
+        const int top = (const int[]){2, 6, 20, 48}[trial % 4], ring = (const int[]){4, 6, 7, 16}[rng() % 4];
         std::vector<int> nc(2 + rng() % 12);
         for (int &n : nc) n = 1 + rng() % top;
-        if (round == 0) nc = {16, 16, 12, 16, 16, 12};
-        if (round == 1) nc = {44, 44, 44};
+        if (trial == 0) nc = {16, 16, 12, 16, 16, 12};
+        if (trial == 1) nc = {44, 44, 44};
         // the ends in the drains' order, as the kernel's drain warps take them
         std::vector<Use> ends;
         std::vector<uint32_t> signal;
@@ -58,7 +58,7 @@ int main(int argc, char **argv) {
         const unsigned seldom = (const unsigned[]){3, 12, 60}[rng() % 3];   // the drains move once in so many steps
         long idle = 0;
         while (drained < ends.size()) {
-            if (++idle > 100000) return printf("round %d: nothing moves\n", round), 1;
+            if (++idle > 100000) return printf("trial %d: nothing moves\n", trial), 1;
             if (rng() % seldom == 0) {                          // the next end, once its MMAs are done
                 const Use &u = ends[drained];
                 size_t i = 0;
@@ -79,7 +79,7 @@ int main(int argc, char **argv) {
                 if ((uint32_t)((phases[on] + 1) & 1) != a.st.wait_parity(buf)) continue;   // not the last phase
                 const long need = last_before(t, a.uses);
                 if ((int)buf != ends[use_of[t][a.uses]].buf || (need >= 0 && (size_t)need >= drained))
-                    return printf("round %d: warp %d took buffer %u at chunk %d before end %ld was drained\n", round, t, buf,
+                    return printf("trial %d: warp %d took buffer %u at chunk %d before end %ld was drained\n", trial, t, buf,
                                   a.chunk, need), 1;
             }
             idle = 0;
